@@ -163,19 +163,21 @@ __global__ void __launch_bounds__(kApassThreads, 1) apass_kernel(const ApassKArg
             if (tid == 0) loss += 0.5 * rr * rr;
           } else if (a.mode == MODE_LGRAD) {
             const double td = (double)t;
-            const double sg = sigmoid_d(td);
+            const double e = exp(-fabs(td));
+            const double sg = sigmoid_of(td, e);
             const double b01 = 0.5 * (1.0 + a.b[i]);
             u[r] = (C)(sg - b01);
-            if (tid == 0) loss += fmax(td, 0.0) + log1p(exp(-fabs(td))) - b01 * td;
+            if (tid == 0 && a.loss_part) loss += fmax(td, 0.0) + log1p(e) - b01 * td;
           } else {  // MODE_LOGIT
             const double td = (double)t;
-            const double sg = sigmoid_d(td);
+            const double e = exp(-fabs(td));
+            const double sg = sigmoid_of(td, e);
             const double wv = sg * (1.0 - sg);
             const double b01 = 0.5 * (1.0 + a.b[i]);
             u[r] = (C)(wv * td + b01 - sg);
             if (tid == 0) {
               if (a.D_out) a.D_out[i] = wv;
-              loss += fmax(td, 0.0) + log1p(exp(-fabs(td))) - b01 * td;
+              if (a.loss_part) loss += fmax(td, 0.0) + log1p(e) - b01 * td;
             }
           }
           if (tid == 0 && a.t_out) a.t_out[i] = (double)t;

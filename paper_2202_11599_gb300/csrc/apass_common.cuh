@@ -77,16 +77,12 @@ __device__ __forceinline__ void timer_end(const ApassKArgs& a, int slot, int dty
   }
 }
 
-__device__ __forceinline__ double sigmoid_d(double t) {
-  // stable logistic function
-  if (t >= 0) {
-    const double e = exp(-t);
-    return 1.0 / (1.0 + e);
-  }
-  const double e = exp(t);
-  return e / (1.0 + e);
-}
+// sigma(t) given e = exp(-|t|): the stable form of the logistic function.
+__device__ __forceinline__ double sigmoid_of(double t, double e) { return (t >= 0 ? 1.0 : e) / (1.0 + e); }
 
+// Whether a row mode evaluates exp and a division in FP64: one such instruction holds an SM
+// quarter's FP64 pipe for 64 clocks however few lanes take part.
+__device__ __forceinline__ bool mode_is_heavy(int mode) { return mode == MODE_LOGIT || mode == MODE_LGRAD; }
 
 // Two consecutive stored elements (pair q of a 16-byte vector) as FP32 values.
 template <int DT>
@@ -162,19 +158,19 @@ __device__ __forceinline__ float row_phi(const ApassKArgs& a, int64_t i, float t
       return (float)rr;
     }
     case MODE_LGRAD: {
-      const double td = (double)t;
-      const double sg = sigmoid_d(td);
+      const double td = (double)t, e = exp(-fabs(td));
+      const double sg = sigmoid_of(td, e);
       const double b01 = 0.5 * (1.0 + in);
-      loss += fmax(td, 0.0) + log1p(exp(-fabs(td))) - b01 * td;
+      if (a.loss_part) loss += fmax(td, 0.0) + log1p(e) - b01 * td;
       return (float)(sg - b01);
     }
     default: {  // MODE_LOGIT
-      const double td = (double)t;
-      const double sg = sigmoid_d(td);
+      const double td = (double)t, e = exp(-fabs(td));
+      const double sg = sigmoid_of(td, e);
       const double wv = sg * (1.0 - sg);
       const double b01 = 0.5 * (1.0 + in);
       if (a.D_out) a.D_out[i] = wv;
-      loss += fmax(td, 0.0) + log1p(exp(-fabs(td))) - b01 * td;
+      if (a.loss_part) loss += fmax(td, 0.0) + log1p(e) - b01 * td;
       return (float)(wv * td + b01 - sg);
     }
   }
@@ -193,17 +189,19 @@ __device__ __forceinline__ double row_phi_d(const ApassKArgs& a, int64_t i, doub
       return rr;
     }
     case MODE_LGRAD: {
-      const double sg = sigmoid_d(t);
+      const double e = exp(-fabs(t));
+      const double sg = sigmoid_of(t, e);
       const double b01 = 0.5 * (1.0 + in);
-      loss += fmax(t, 0.0) + log1p(exp(-fabs(t))) - b01 * t;
+      if (a.loss_part) loss += fmax(t, 0.0) + log1p(e) - b01 * t;
       return sg - b01;
     }
     default: {  // MODE_LOGIT
-      const double sg = sigmoid_d(t);
+      const double e = exp(-fabs(t));
+      const double sg = sigmoid_of(t, e);
       const double wv = sg * (1.0 - sg);
       const double b01 = 0.5 * (1.0 + in);
       if (a.D_out) a.D_out[i] = wv;
-      loss += fmax(t, 0.0) + log1p(exp(-fabs(t))) - b01 * t;
+      if (a.loss_part) loss += fmax(t, 0.0) + log1p(e) - b01 * t;
       return wv * t + b01 - sg;
     }
   }

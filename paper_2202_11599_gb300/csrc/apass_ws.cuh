@@ -109,46 +109,64 @@ __device__ __forceinline__ int ws_produce(const ApassKArgs& a, WsBars& b, unsign
 
 // Finisher warp: u_i = phi(t_i) for the rows of each stage, t_i summed over the G dot
 // warps' partials in a fixed order.  Returns this lane's share of the pass's loss term.
+//
+// The logistic modes take two stages per step: exp and the division are ~40 FP64 warp
+// instructions of 64 pipe clocks each whether one lane or all take part, so with one wide
+// row per stage (R = 1) the finisher, not the FP64 dot products beside it, set the pace
+// (200,000 x 5,000 FP64, logistic mode: 6.9 -> 5.6 ms a pass; before, one row at a time with a
+// second exp and the log1p of an unwanted loss).  Lane q R + r takes row r of stage k + q.
 template <typename C, int R, int G>
 __device__ __forceinline__ double ws_finish(const ApassKArgs& a, WsBars& b, const C (*red)[G][R], C (*us)[R],
                                             int nsteps, int S, int64_t r0, int64_t r1, volatile int* abort_flag,
                                             int kbase = 0) {
   const int lane = threadIdx.x & 31;
   const bool nodot = a.mode == MODE_CONST;
+  const int NQ = mode_is_heavy(a.mode) && S > 2 ? 2 : 1;
+  const int q = lane / R, r = lane % R;   // this lane's stage of the step and row of the stage
   double loss = 0.0;
   int st = kbase % S;
   uint32_t ph = (uint32_t)((kbase / S) & 1);
-  for (int k = 0; k < nsteps; ++k, st = st + 1 == S ? 0 : st + 1, ph ^= st == 0 ? 1u : 0u) {
-    const int64_t row0 = r0 + (int64_t)k * R;
-    const int rows_here = (int)min((int64_t)R, r1 - row0);
+  for (int k = 0; k < nsteps; k += NQ) {
+    const int nq = min(NQ, nsteps - k);
+    const int64_t row = r0 + (int64_t)(k + q) * R + r;
+    const bool mine = q < nq, live = mine && row < r1;
     // the row's mode input (D_i or b_i) is loaded before the waits
-    const double rin = (lane < R && lane < rows_here) ? row_input(a, row0 + lane) : 0.0;
+    const double rin = live ? row_input(a, row) : 0.0;
     // waiting for the stage itself orders the writes of us[st] after its previous use
     // (the stage was re-armed only after the update warps released it)
-    if (!warp_wait(&b.full[st], ph) || (!nodot && !warp_wait(&b.dotted[st], ph))) {
+    const int st1 = st + 1 == S ? 0 : st + 1;
+    const uint32_t ph1 = st1 == 0 ? ph ^ 1u : ph;
+    bool ok = warp_wait(&b.full[st], ph) && (nodot || warp_wait(&b.dotted[st], ph));
+    if (ok && nq == 2) ok = warp_wait(&b.full[st1], ph1) && (nodot || warp_wait(&b.dotted[st1], ph1));
+    if (!ok) {
       *abort_flag = 1;
       break;
     }
-    if (lane < R) {
+    if (mine) {
+      const int sq = q == 0 ? st : st1;
       C u = C(0);
-      if (lane < rows_here) {
-        const int64_t i = row0 + lane;
+      if (live) {
         C t = C(0);
         if (!nodot) {
 #pragma unroll
-          for (int w = 0; w < G; ++w) t += red[st][w][lane];
+          for (int w = 0; w < G; ++w) t += red[sq][w][r];
         }
         if constexpr (sizeof(C) == 4) {
-          u = row_phi(a, i, t, rin, loss);
+          u = row_phi(a, row, t, rin, loss);
         } else {
-          u = (C)row_phi_d(a, i, (double)t, rin, loss);
+          u = (C)row_phi_d(a, row, (double)t, rin, loss);
         }
-        if (!nodot && a.t_out) a.t_out[i] = (double)t;
+        if (!nodot && a.t_out) a.t_out[row] = (double)t;
       }
-      us[st][lane] = u;
+      us[sq][r] = u;
     }
     __syncwarp();
-    if (lane == 0) mbar_arrive(&b.ready[st]);
+    if (lane < nq) mbar_arrive(&b.ready[lane == 0 ? st : st1]);
+    // the ring moves on by nq stages
+    st = nq == 2 ? st1 : st;
+    ph = nq == 2 ? ph1 : ph;
+    st = st + 1 == S ? 0 : st + 1;
+    ph ^= st == 0 ? 1u : 0u;
   }
   return loss;
 }

@@ -382,7 +382,7 @@ nys_status aux_pass(const nys_matrix* A, int mode, const void* p, const double* 
   a.D_out = D_out;
   a.t_out = t_out;
   a.mode = mode;
-  NYS_CU(apass_run(a, plan, part, lp, dstat, st));
+  NYS_CU(apass_run(a, plan, part, loss_h ? lp : nullptr, dstat, st));   // no buffer: the loss is not formed
   ApassArgs ar = a;
   ar.p = nullptr;
   NYS_CU(apass_reduce(ar, plan, part, 0.0, y, nullptr, 0, st));
