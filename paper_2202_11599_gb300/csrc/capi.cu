@@ -272,6 +272,21 @@ void precond_free(nys_precond_s* P) {
   delete P;
 }
 
+// U in the compute type: the FP64 factor, or its FP32 copy (made on first use).
+template <typename C>
+nys_status precond_u(nys_precond_s* P, cudaStream_t st, const C** out) {
+  if constexpr (sizeof(C) == 8) {
+    *out = P->U64;
+  } else {
+    if (!P->U32) {
+      if (cudaMalloc(&P->U32, (size_t)P->d * P->s * sizeof(float)) != cudaSuccess) return NYS_ENOMEM;
+      NYS_CU(convert_f64_to_f32(P->U64, P->U32, P->d * P->s, st));
+    }
+    *out = P->U32;
+  }
+  return NYS_OK;
+}
+
 // Device view of P^{-1} for one rho in the PCG compute type.
 template <typename C>
 nys_status precond_view(nys_precond_s* P, double rho, C* c, cudaStream_t st, PrecondView* out) {
@@ -285,17 +300,29 @@ nys_status precond_view(nys_precond_s* P, double rho, C* c, cudaStream_t st, Pre
   for (int i = 0; i < s; ++i) ch[i] = (C)((lam_s + rho) / (P->lam[i] + rho) - 1.0);
   NYS_CU(cudaMemcpyAsync(c, ch.data(), s * sizeof(C), cudaMemcpyHostToDevice, st));
   NYS_CU(cudaStreamSynchronize(st));  // ch goes out of scope
-  if constexpr (sizeof(C) == 8) {
-    out->U = P->U64;
-  } else {
-    if (!P->U32) {
-      if (cudaMalloc(&P->U32, (size_t)P->d * s * sizeof(float)) != cudaSuccess) return NYS_ENOMEM;
-      NYS_CU(convert_f64_to_f32(P->U64, P->U32, P->d * s, st));
-    }
-    out->U = P->U32;
-  }
+  const C* U = nullptr;
+  NYS_TRY(precond_u<C>(P, st, &U));
+  out->U = U;
   out->c = c;
   out->s = s;
+  return NYS_OK;
+}
+
+// Y = P^{-1} V for a d x k block (Y may be V), in panels of at most 4,096 columns.
+template <typename C>
+nys_status precond_apply_block(nys_precond_s* P, double rho, const C* V, C* Y, int64_t k, cudaStream_t st) {
+  const C* U = nullptr;
+  NYS_TRY(precond_u<C>(P, st, &U));
+  constexpr int64_t kPanel = 4096;
+  Pool pool(st);
+  size_t elems = precond_block_work<C>(P->d, P->s, (int)std::min(k, kPanel));
+  if (k > kPanel && k % kPanel) elems = std::max(elems, precond_block_work<C>(P->d, P->s, (int)(k % kPanel)));
+  C* work = pool.alloc<C>(elems);
+  if (!pool.ok()) return NYS_ENOMEM;
+  for (int64_t c0 = 0; c0 < k; c0 += kPanel)
+    NYS_CU(precond_block<C>(U, nullptr, P->lam_d, rho, P->d, P->s, (int)std::min(kPanel, k - c0), V + c0 * P->d,
+                            Y + c0 * P->d, work, st));
+  NYS_CU(cudaStreamSynchronize(st));
   return NYS_OK;
 }
 
@@ -1254,16 +1281,8 @@ nys_status nys_precond_apply(nys_precond P, double rho, const void* V, void* Yv,
   if (!P || !V || !Yv || k < 1 || !(rho > 0) || !is_fin(rho)) return NYS_EINVAL;
   if (dtype != NYS_F64 && dtype != NYS_F32) return NYS_EINVAL;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  Pool pool(st);
-  void* cbuf = pool.alloc<double>(P->s);
-  if (!pool.ok()) return NYS_ENOMEM;
-  PrecondView view;
-  if (dtype == NYS_F64) {
-    NYS_TRY(precond_view<double>(P, rho, (double*)cbuf, st, &view));
-    return precond_apply_run<double>(view, P->d, (const double*)V, (double*)Yv, k, st);
-  }
-  NYS_TRY(precond_view<float>(P, rho, (float*)cbuf, st, &view));
-  return precond_apply_run<float>(view, P->d, (const float*)V, (float*)Yv, k, st);
+  if (dtype == NYS_F64) return precond_apply_block<double>(P, rho, (const double*)V, (double*)Yv, k, st);
+  return precond_apply_block<float>(P, rho, (const float*)V, (float*)Yv, k, st);
 }
 
 nys_status pcg_solve(const nys_matrix* A, const double* D, double rho, nys_precond P, const void* r, void* x,

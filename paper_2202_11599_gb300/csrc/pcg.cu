@@ -509,47 +509,6 @@ template nys_status pcg_run<double>(const PcgProblem&, const PrecondView&, const
 template nys_status pcg_run<float>(const PcgProblem&, const PrecondView&, const float*, float*, const PcgParams&,
                                    cudaStream_t, int*, double*);
 
-// ------------------------------------------------------------------ P^{-1} on k vectors (standalone apply)
-template <typename C>
-nys_status precond_apply_run(const PrecondView& P, int64_t d, const C* V, C* Y, int64_t k, cudaStream_t stream) {
-  Pool pool(stream);
-  const int s = P.s;
-  const int chunk = upd_chunk(d);
-  const int nb3 = (int)((d + chunk - 1) / chunk);
-  const int nb5 = reduce_blocks(d);
-  C* w = pool.alloc<C>(d);
-  C* gs = pool.alloc<C>(std::max(1, s));
-  double* part_w2 = pool.alloc<double>(nb3);
-  double* part_r2 = pool.alloc<double>(nb3);
-  double* part_g = pool.alloc<double>((size_t)nb3 * std::max(1, s));
-  double* wy_part = pool.alloc<double>(nb5);
-  PcgState* st = pool.alloc<PcgState>(1);
-  if (!pool.ok()) return NYS_ENOMEM;
-  for (int64_t c = 0; c < k; ++c) {
-    count_launch();
-    pcg_reset_kernel<<<1, 1, 0, stream>>>(st, 0.0, 1, 1, -1, nullptr);
-    // init-mode update copies V[:, c] into w and forms the partials of U^T w
-    count_launch();
-    pcg_update_kernel<C><<<nb3, kVecThreads, (size_t)chunk * sizeof(C), stream>>>(
-        1, d, chunk, nullptr, w, V + c * d, nullptr, nullptr, reinterpret_cast<const C*>(P.U), s, nullptr, 0,
-        nullptr, 0, part_w2, part_r2, part_g, st, (C*)nullptr, reinterpret_cast<const C*>(P.c), gs, 0ull, 0, nullptr,
-        nullptr, nullptr, 0.0, (C*)nullptr);
-    // the scalar step may mark the state done (||w|| <= 0 threshold); force the tail to run
-    count_launch();
-    pcg_reset_kernel<<<1, 1, 0, stream>>>(st, 0.0, 1, 1, -1, nullptr);
-    count_launch();
-    pcg_tail_kernel<C><<<nb5, kVecThreads, (size_t)std::max(1, s) * sizeof(C), stream>>>(
-        d, w, Y + c * d, reinterpret_cast<const C*>(P.U), s, gs, wy_part, st, 1, (C*)nullptr);
-    if (cudaGetLastError() != cudaSuccess) return NYS_ECUDA;
-  }
-  if (cudaStreamSynchronize(stream) != cudaSuccess) return NYS_ECUDA;
-  return NYS_OK;
-}
-
-template nys_status precond_apply_run<double>(const PrecondView&, int64_t, const double*, double*, int64_t,
-                                              cudaStream_t);
-template nys_status precond_apply_run<float>(const PrecondView&, int64_t, const float*, float*, int64_t, cudaStream_t);
-
 // ------------------------------------------------------------------ ADMM vector kernels (FP64 state)
 
 // r = q + rho (z - u)   or, for the refined x-step, the residual of Eq. ADMMSubProb at x:

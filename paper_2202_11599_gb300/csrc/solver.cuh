@@ -93,8 +93,14 @@ template <typename C>
 nys_status pcg_run(const PcgProblem& pb, const PrecondView& P, const C* r, C* x, const PcgParams& prm,
                    cudaStream_t stream, int* iters_out, double* resnorm_out);
 
-template <typename C>
-nys_status precond_apply_run(const PrecondView& P, int64_t d, const C* V, C* Y, int64_t k, cudaStream_t stream);
+// Y = V + U diag(c) U^T V for a d x k block, column-major (precond_block.cu); Y may be V.
+// c_i from `cvec`, or (lam_s + rho) / (lam_i + rho) - 1 from the device eigenvalues when it is
+// null.  work: precond_block_work elements of T.
+template <typename T>
+size_t precond_block_work(int64_t d, int s, int k);
+template <typename T>
+cudaError_t precond_block(const T* U, const T* cvec, const double* lam, double rho, int64_t d, int s, int k,
+                          const T* V, T* Y, T* work, cudaStream_t st);
 
 template <typename C>
 cudaError_t admm_rhs(int64_t d, const double* q, const double* z, const double* u, double rho, const double* x,
