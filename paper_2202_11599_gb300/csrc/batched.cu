@@ -19,11 +19,22 @@
 namespace nys {
 namespace {
 
+// Per-column scalars of the k PCG solves.  Every kernel below that changes them reads one copy
+// and writes another (its blocks with chunk 0), so that the blocks of a column all see the
+// same values.
 struct BCol {
-  double wy, wy_new, pv, w2, r2, thresh2;
+  double wy, pv, w2, r2, thresh2;
   float alpha, beta;
   int iters, done, status, pad;
 };
+
+// Vector kernels: block (b, c) of kVecThreads threads owns rows [1024 b, 1024 b + 1024) of
+// column c, four elements per thread, and leaves one partial sum per block, so a column's dot
+// product is nb partials added in increasing b.  (One block per 1,024 rows over all columns
+// left four blocks for a 4,000 x 64 panel: 62 us per dot and 206 us per prox step.)
+constexpr int kColChunk = 1024;
+constexpr int kColPer = kColChunk / kVecThreads;
+int col_blocks(int64_t d) { return (int)((d + kColChunk - 1) / kColChunk); }
 
 template <typename C>
 __global__ void b_matvec_finish_kernel(const C* __restrict__ part, int nz, int64_t len, C rho, const C* __restrict__ P,
@@ -35,117 +46,165 @@ __global__ void b_matvec_finish_kernel(const C* __restrict__ part, int nz, int64
   }
 }
 
-// per-column partial dot products over a chunk of rows: warp w takes columns w, w+8, ...
-template <typename C>
-__global__ void __launch_bounds__(kVecThreads) b_coldot_kernel(const C* __restrict__ X, const C* __restrict__ Y,
-                                                               int64_t d, int k, int chunk, double* part) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t j0 = (int64_t)blockIdx.x * chunk;
-  const int64_t j1 = min(d, j0 + chunk);
-  for (int c = warp; c < k; c += kVecThreads / 32) {
-    const C* x = X + (int64_t)c * d;
-    const C* y = Y + (int64_t)c * d;
-    double acc = 0.0;
-    for (int64_t j = j0 + lane; j < j1; j += 32) acc += (double)x[j] * (double)y[j];
-    acc = warp_sum(acc);
-    if (lane == 0) part[(int64_t)blockIdx.x * k + c] = acc;
-  }
-}
-
-__global__ void b_colsum_kernel(const double* part, int nb, int k, double* out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= k) return;
+// Sum of a column's partials part[b * k + c] (increasing b; nb is small).
+__device__ __forceinline__ double col_sum(const double* __restrict__ part, int nb, int k, int c) {
   double s = 0.0;
   for (int b = 0; b < nb; ++b) s += part[(int64_t)b * k + c];
-  out[c] = s;
+  return s;
 }
 
-// phase 0: init (r2, w2 -> threshold, done);  1: alpha from wy / pv;  2: stop test after the
-// update (w2);  3: beta = wy_new / wy.  `sums` holds the column sums of the current dot.
-__global__ void b_scalar_kernel(int phase, int k, BCol* col, const double* sums, const double* sums2, double tol,
-                                int tol_abs, int maxit, int* ndone) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= k) return;
-  BCol& s = col[c];
-  if (phase == 0) {
-    s.r2 = sums[c];
-    s.w2 = sums2[c];
-    s.thresh2 = tol_abs ? tol * tol : tol * tol * s.r2;
-    s.iters = 0;
-    s.status = 0;
-    s.wy = 0.0;
-    s.done = !(s.w2 > s.thresh2);
-    s.alpha = 0.f;
-    s.beta = 0.f;
-  } else if (phase == 1) {
-    s.pv = sums[c];
-    if (s.done) {
-      s.alpha = 0.f;
-    } else if (!(s.pv > 0.0) || !isfinite(s.pv)) {
-      s.alpha = 0.f;
-      s.done = 1;
-      s.status = s.iters == 0 ? NYS_EBREAKDOWN : NYS_ENOCONV;
-    } else {
-      s.alpha = (float)(s.wy / s.pv);
-    }
-  } else if (phase == 2) {
+// part[b][c] = the block's share of x_c . y_c.  With `in` the column's stop test runs first
+// (||w||^2 from w2_part, the iteration counted): the dot is w . y of the same iteration.
+template <typename C>
+__global__ void __launch_bounds__(kVecThreads) b_dot_kernel(const C* __restrict__ X, const C* __restrict__ Y,
+                                                            int64_t d, int k, double* part,
+                                                            const double* __restrict__ w2_part, int maxit,
+                                                            const BCol* __restrict__ in, BCol* __restrict__ out) {
+  __shared__ double sh[kVecThreads / 32];
+  const int c = blockIdx.y;
+  const int64_t j0 = (int64_t)blockIdx.x * kColChunk + threadIdx.x;
+  double acc = 0.0;
+#pragma unroll
+  for (int q = 0; q < kColPer; ++q) {
+    const int64_t j = j0 + q * kVecThreads;
+    if (j < d) acc += (double)X[(int64_t)c * d + j] * (double)Y[(int64_t)c * d + j];
+  }
+  const double t = block_sum_t0<kVecThreads>(acc, sh);
+  if (threadIdx.x != 0) return;
+  part[(int64_t)blockIdx.x * k + c] = t;
+  if (in && blockIdx.x == 0) {
+    BCol s = in[c];
     if (!s.done) {
-      s.w2 = sums[c];
+      s.w2 = col_sum(w2_part, gridDim.x, k, c);
       s.iters += 1;
-      if (!(s.w2 > s.thresh2)) s.done = 1;
-      else if (s.iters >= maxit) {
+      if (!(s.w2 > s.thresh2)) {
+        s.done = 1;
+      } else if (s.iters >= maxit) {
         s.done = 1;
         s.status = NYS_ENOCONV;
       }
     }
-  } else {  // phase 3
-    s.wy_new = sums[c];
-    s.beta = s.wy > 0.0 ? (float)(s.wy_new / s.wy) : 0.f;
-    s.wy = s.wy_new;
-  }
-  if (ndone && phase == 2) {
-    // count converged columns (one writer per column; the host reads after the launch)
-    if (s.done) atomicAdd(ndone, 1);
+    out[c] = s;
   }
 }
 
+// w = r - v (v = (H + rho I) x0, or x0 = 0) with the partials of ||r||^2 and ||w||^2.
 template <typename C>
-__global__ void b_init_w_kernel(int64_t len, const C* __restrict__ R, const C* __restrict__ V, C* __restrict__ W) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
-    W[i] = V ? R[i] - V[i] : R[i];
-}
-
-template <typename C>
-__global__ void b_update_kernel(int64_t d, int k, C* __restrict__ X, C* __restrict__ W, const C* __restrict__ P,
-                                const C* __restrict__ V, const BCol* col) {
-  const int64_t len = d * k;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x) {
-    const C a = (C)col[i / d].alpha;
-    X[i] = fma(a, P[i], X[i]);
-    W[i] = fma(-a, V[i], W[i]);
+__global__ void __launch_bounds__(kVecThreads) b_init_w_kernel(int64_t d, int k, const C* __restrict__ R,
+                                                               const C* __restrict__ V, C* __restrict__ W,
+                                                               double* r2_part, double* w2_part) {
+  __shared__ double sh[kVecThreads / 32];
+  const int c = blockIdx.y;
+  const int64_t j0 = (int64_t)blockIdx.x * kColChunk + threadIdx.x;
+  double lr = 0.0, lw = 0.0;
+#pragma unroll
+  for (int q = 0; q < kColPer; ++q) {
+    const int64_t j = j0 + q * kVecThreads;
+    if (j < d) {
+      const int64_t e = (int64_t)c * d + j;
+      const C r = R[e], w = V ? r - V[e] : r;
+      W[e] = w;
+      lr += (double)r * (double)r;
+      lw += (double)w * (double)w;
+    }
+  }
+  const double tr = block_sum_t0<kVecThreads>(lr, sh);
+  const double tw = block_sum_t0<kVecThreads>(lw, sh);
+  if (threadIdx.x == 0) {
+    r2_part[(int64_t)blockIdx.x * k + c] = tr;
+    w2_part[(int64_t)blockIdx.x * k + c] = tw;
   }
 }
 
-template <typename C>
-__global__ void b_pupdate_kernel(int64_t d, int k, const C* __restrict__ Y, C* __restrict__ P, const BCol* col,
-                                 int init) {
-  const int64_t len = d * k;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
-    P[i] = init ? Y[i] : fma((C)col[i / d].beta, P[i], Y[i]);
+// Thresholds and first stop test of every column.
+__global__ void b_start_kernel(int k, int nb, const double* r2_part, const double* w2_part, double tol, int tol_abs,
+                               BCol* out) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= k) return;
+  BCol s = {};
+  s.r2 = col_sum(r2_part, nb, k, c);
+  s.w2 = col_sum(w2_part, nb, k, c);
+  s.thresh2 = tol_abs ? tol * tol : tol * tol * s.r2;
+  s.done = !(s.w2 > s.thresh2);
+  out[c] = s;
 }
 
-// G (s x k) *= c_i row-wise
+// alpha = w . y / p . v of each column (0 for a finished one), x += alpha p, w -= alpha v and
+// the partials of ||w||^2.
 template <typename C>
-__global__ void b_scale_rows_kernel(C* G, int s, int k, const C* __restrict__ cvec) {
-  const int64_t len = (int64_t)s * k;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
-    G[i] *= cvec[i % s];
+__global__ void __launch_bounds__(kVecThreads) b_update_kernel(int64_t d, int k, C* __restrict__ X, C* __restrict__ W,
+                                                               const C* __restrict__ P, const C* __restrict__ V,
+                                                               const double* __restrict__ pv_part, double* w2_part,
+                                                               const BCol* __restrict__ in, BCol* __restrict__ out) {
+  __shared__ double sh[kVecThreads / 32];
+  __shared__ float s_alpha;
+  const int c = blockIdx.y;
+  if (threadIdx.x == 0) {
+    BCol s = in[c];
+    s.pv = col_sum(pv_part, gridDim.x, k, c);
+    s.alpha = 0.f;
+    if (!s.done) {
+      if (!(s.pv > 0.0) || !isfinite(s.pv)) {
+        s.done = 1;
+        s.status = s.iters == 0 ? NYS_EBREAKDOWN : NYS_ENOCONV;
+      } else {
+        s.alpha = (float)(s.wy / s.pv);
+      }
+    }
+    s_alpha = s.alpha;
+    if (blockIdx.x == 0) out[c] = s;
+  }
+  __syncthreads();
+  const C a = (C)s_alpha;
+  const int64_t j0 = (int64_t)blockIdx.x * kColChunk + threadIdx.x;
+  double acc = 0.0;
+#pragma unroll
+  for (int q = 0; q < kColPer; ++q) {
+    const int64_t j = j0 + q * kVecThreads;
+    if (j < d) {
+      const int64_t e = (int64_t)c * d + j;
+      X[e] = fma(a, P[e], X[e]);
+      const C w = fma(-a, V[e], W[e]);
+      W[e] = w;
+      acc += (double)w * (double)w;
+    }
+  }
+  const double t = block_sum_t0<kVecThreads>(acc, sh);
+  if (threadIdx.x == 0) w2_part[(int64_t)blockIdx.x * k + c] = t;
 }
 
+// beta = (w . y)_new / (w . y)_old of each column, p = y + beta p (init: p = y).  Counts the
+// finished columns in *ndone (zeroed by the caller).
 template <typename C>
-__global__ void b_add_kernel(int64_t len, const C* __restrict__ W, C* __restrict__ Y) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
-    Y[i] += W[i];
+__global__ void __launch_bounds__(kVecThreads) b_direction_kernel(int64_t d, int k, const C* __restrict__ Y,
+                                                                  C* __restrict__ P,
+                                                                  const double* __restrict__ wy_part, int init,
+                                                                  const BCol* __restrict__ in, BCol* __restrict__ out,
+                                                                  int* ndone) {
+  __shared__ float s_beta;
+  const int c = blockIdx.y;
+  if (threadIdx.x == 0) {
+    BCol s = in[c];
+    const double wy = col_sum(wy_part, gridDim.x, k, c);
+    s.beta = s.wy > 0.0 ? (float)(wy / s.wy) : 0.f;
+    s.wy = wy;
+    s_beta = s.beta;
+    if (blockIdx.x == 0) {
+      out[c] = s;
+      if (s.done) atomicAdd(ndone, 1);
+    }
+  }
+  __syncthreads();
+  const C b = (C)s_beta;
+  const int64_t j0 = (int64_t)blockIdx.x * kColChunk + threadIdx.x;
+#pragma unroll
+  for (int q = 0; q < kColPer; ++q) {
+    const int64_t j = j0 + q * kVecThreads;
+    if (j < d) {
+      const int64_t e = (int64_t)c * d + j;
+      P[e] = init ? Y[e] : fma(b, P[e], Y[e]);
+    }
+  }
 }
 
 unsigned grid_for(int64_t len) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>(8192, (len + 255) / 256)); }
@@ -153,29 +212,31 @@ unsigned grid_for(int64_t len) { return (unsigned)std::max<int64_t>(1, std::min<
 }  // namespace
 
 template <typename C>
-nys_status batched_pcg_run(const PcgProblem& pb, const PrecondView& P, const C* R, C* X, int k, const PcgParams& prm,
-                           cudaStream_t st, std::vector<int>* iters_out) {
+nys_status batched_pcg_run(const PcgProblem& pb, const TcPrepared* tcp, const PrecondView& P, const C* R, C* X, int k,
+                           const PcgParams& prm, cudaStream_t st, std::vector<int>* iters_out) {
   const int64_t d = pb.A->d, n = pb.A->n;
   const int s = P.s;
   const int64_t len = d * k;
-  const int chunk = 1024;
-  const int nbd = (int)((d + chunk - 1) / chunk);
+  const int nb = col_blocks(d);
+  const bool use_tc = tcp != nullptr;
   Pool pool(st);
   C* W = pool.alloc<C>(len);
   C* Y = pool.alloc<C>(len);
   C* Pd = pool.alloc<C>(len);
   C* V = pool.alloc<C>(len);
-  C* Wn = pool.alloc<C>((size_t)n * k);
-  const size_t atw_bytes = sketch_atw_work_bytes(pb.A, k);
-  void* atw = pool.alloc<unsigned char>(atw_bytes);
-  C* G = pool.alloc<C>((size_t)std::max(1, s) * k);
-  C* gwork = pool.alloc<C>(std::max<size_t>(1, gemm_tn_work_elems<C>(d, std::max(1, s), k)));
-  double* part = pool.alloc<double>((size_t)nbd * k);
-  double* sums = pool.alloc<double>(k);
-  double* sums2 = pool.alloc<double>(k);
-  BCol* col = pool.alloc<BCol>(k);
-  int* ndone = pool.alloc<int>(1);
+  C* Wn = use_tc ? nullptr : pool.alloc<C>((size_t)n * k);
+  const size_t atw_bytes = use_tc ? 0 : sketch_atw_work_bytes(pb.A, k);
+  void* atw = use_tc ? nullptr : pool.alloc<unsigned char>(atw_bytes);
+  void* tcw = use_tc ? pool.alloc<unsigned char>(tc_hmm_work_bytes(pb.A, *tcp, k)) : nullptr;
+  C* gwork = s > 0 ? pool.alloc<C>(precond_block_work<C>(d, s, k)) : nullptr;
+  double* pv_part = pool.alloc<double>((size_t)nb * k);
+  double* w2_part = pool.alloc<double>((size_t)nb * k);
+  double* wy_part = pool.alloc<double>((size_t)nb * k);
+  BCol* cols = pool.alloc<BCol>(2 * (size_t)k);
+  int* ndone = pool.alloc<int>(2);   // finished columns; status of the tensor-core products
   if (!pool.ok()) return NYS_ENOMEM;
+  BCol *cin = cols, *cout = cols + k;
+  int* tc_status = ndone + 1;
   const C* U = reinterpret_cast<const C*>(P.U);
   const C* cvec = reinterpret_cast<const C*>(P.c);
 #define B_OK(x)                             \
@@ -183,24 +244,14 @@ nys_status batched_pcg_run(const PcgProblem& pb, const PrecondView& P, const C* 
     if ((x) != cudaSuccess) return NYS_ECUDA; \
   } while (0)
   auto launch_ok = [&]() { return cudaGetLastError() == cudaSuccess; };
-  // BF16 storage: the k-column products run on the tensor cores (the same tcgen05 GEMMs
-  // as the sketch, FP32 operand as three BF16 terms), with a transposed copy of A made
-  // once for the whole solve
-  TcPrepared tcp;
-  bool use_tc = false;
-  if constexpr (sizeof(C) == 4) {
-    if (sketch_tc_supported(pb.A)) {
-      void* tcs = pool.alloc<unsigned char>(tc_prepare_bytes(pb.A));
-      if (!pool.ok()) return NYS_ENOMEM;
-      if (tc_prepare(pb.A, tcs, &tcp, st) != cudaSuccess) return NYS_ECUDA;
-      use_tc = true;
-    }
-  }
+  const dim3 cgrid((unsigned)nb, (unsigned)k);
+  // BF16 and FP32 storage: the k-column products run on the tensor cores (the same tcgen05
+  // GEMMs as the sketch, FP32 operand as three BF16 terms) from operands prepared once per solve.
   // V = A^T (A P) + rho P for the k columns of P (reads A once)
   auto bmatvec = [&](const C* Pin, C* Vout) -> bool {
     if constexpr (sizeof(C) == 4) {
-      if (use_tc) return tc_hmm(pb.A, tcp, pb.D, reinterpret_cast<const float*>(Pin), k, pb.rho,
-                                reinterpret_cast<float*>(Vout), st) == cudaSuccess;
+      if (use_tc) return tc_hmm(pb.A, *tcp, pb.D, reinterpret_cast<const float*>(Pin), k, pb.rho,
+                                reinterpret_cast<float*>(Vout), tcw, tc_status, st) == cudaSuccess;
     }
     if (sketch_aw(pb.A, Pin, k, pb.D, Wn, st) != cudaSuccess) return false;
     int nz = 0;
@@ -209,61 +260,57 @@ nys_status batched_pcg_run(const PcgProblem& pb, const PrecondView& P, const C* 
     b_matvec_finish_kernel<C><<<grid_for(len), 256, 0, st>>>((const C*)atw, nz, len, (C)pb.rho, Pin, Vout);
     return launch_ok();
   };
-  auto coldot = [&](const C* A_, const C* B_, double* out) -> bool {
-    count_launch();
-    b_coldot_kernel<C><<<nbd, kVecThreads, 0, st>>>(A_, B_, d, k, chunk, part);
-    count_launch();
-    b_colsum_kernel<<<(k + 127) / 128, 128, 0, st>>>(part, nbd, k, out);
-    return launch_ok();
-  };
   // Y = P^{-1} W = U diag(c) U^T W + W
   auto precond = [&]() -> bool {
     if (s == 0) return cudaMemcpyAsync(Y, W, len * sizeof(C), cudaMemcpyDeviceToDevice, st) == cudaSuccess;
-    if (gemm_tn<C>(U, W, d, s, k, G, gwork, st) != cudaSuccess) return false;
-    count_launch();
-    b_scale_rows_kernel<C><<<grid_for((int64_t)s * k), 256, 0, st>>>(G, s, k, cvec);
-    if (gemm_nn_t<C>(U, d, s, G, k, Y, st) != cudaSuccess) return false;
-    count_launch();
-    b_add_kernel<C><<<grid_for(len), 256, 0, st>>>(len, W, Y);
-    return launch_ok();
+    return precond_block<C>(U, cvec, nullptr, 0.0, d, s, k, W, Y, gwork, st) == cudaSuccess;
   };
-  auto scalar = [&](int phase, const double* s1, const double* s2, int* nd) -> bool {
+  auto direction = [&](int init) -> bool {
     count_launch();
-    b_scalar_kernel<<<(k + 127) / 128, 128, 0, st>>>(phase, k, col, s1, s2, prm.tol, prm.tol_abs, prm.maxit, nd);
+    b_direction_kernel<C><<<cgrid, kVecThreads, 0, st>>>(d, k, Y, Pd, wy_part, init, cin, cout, ndone);
+    std::swap(cin, cout);
     return launch_ok();
   };
 
   // init: W = R - (H + rho I) X0, thresholds, Y = P^{-1} W, P = Y
+  B_OK(cudaMemsetAsync(ndone, 0, 2 * sizeof(int), st));
   if (!prm.x0_zero) {
     if (!bmatvec(X, V)) return NYS_ECUDA;
   }
   count_launch();
-  b_init_w_kernel<C><<<grid_for(len), 256, 0, st>>>(len, R, prm.x0_zero ? nullptr : V, W);
-  if (!coldot(R, R, sums) || !coldot(W, W, sums2) || !scalar(0, sums, sums2, nullptr)) return NYS_ECUDA;
-  if (!precond() || !coldot(W, Y, sums) || !scalar(3, sums, nullptr, nullptr)) return NYS_ECUDA;
+  b_init_w_kernel<C><<<cgrid, kVecThreads, 0, st>>>(d, k, R, prm.x0_zero ? nullptr : V, W, pv_part, w2_part);
   count_launch();
-  b_pupdate_kernel<C><<<grid_for(len), 256, 0, st>>>(d, k, Y, Pd, col, 1);
+  b_start_kernel<<<(k + 127) / 128, 128, 0, st>>>(k, nb, pv_part, w2_part, prm.tol, prm.tol_abs, cin);
+  if (!launch_ok() || !precond()) return NYS_ECUDA;
+  count_launch();
+  b_dot_kernel<C><<<cgrid, kVecThreads, 0, st>>>(W, Y, d, k, wy_part, nullptr, 0, nullptr, nullptr);
+  if (!launch_ok() || !direction(1)) return NYS_ECUDA;
   std::vector<BCol> hc(k);
-  B_OK(cudaMemcpyAsync(hc.data(), col, k * sizeof(BCol), cudaMemcpyDeviceToHost, st));
+  int host2[2] = {0, 0};
+  B_OK(cudaMemcpyAsync(host2, ndone, sizeof(host2), cudaMemcpyDeviceToHost, st));
   B_OK(cudaStreamSynchronize(st));
-  int done_h = 0;
-  for (const BCol& c : hc) done_h += c.done;
   const int cap = prm.fixed >= 0 ? prm.fixed : prm.maxit;
-  for (int it = 0; it < cap && done_h < k; ++it) {
-    if (!bmatvec(Pd, V) || !coldot(Pd, V, sums) || !scalar(1, sums, nullptr, nullptr)) return NYS_ECUDA;
+  for (int it = 0; it < cap && host2[0] < k && !host2[1]; ++it) {
+    if (!bmatvec(Pd, V)) return NYS_ECUDA;
     count_launch();
-    b_update_kernel<C><<<grid_for(len), 256, 0, st>>>(d, k, X, W, Pd, V, col);
+    b_dot_kernel<C><<<cgrid, kVecThreads, 0, st>>>(Pd, V, d, k, pv_part, nullptr, 0, nullptr, nullptr);
+    count_launch();
+    b_update_kernel<C><<<cgrid, kVecThreads, 0, st>>>(d, k, X, W, Pd, V, pv_part, w2_part, cin, cout);
+    std::swap(cin, cout);
     B_OK(cudaMemsetAsync(ndone, 0, sizeof(int), st));
-    if (!coldot(W, W, sums) || !scalar(2, sums, nullptr, ndone)) return NYS_ECUDA;
-    if (!precond() || !coldot(W, Y, sums) || !scalar(3, sums, nullptr, nullptr)) return NYS_ECUDA;
+    if (!launch_ok() || !precond()) return NYS_ECUDA;
     count_launch();
-    b_pupdate_kernel<C><<<grid_for(len), 256, 0, st>>>(d, k, Y, Pd, col, 0);
-    B_OK(cudaMemcpyAsync(&done_h, ndone, sizeof(int), cudaMemcpyDeviceToHost, st));
+    b_dot_kernel<C><<<cgrid, kVecThreads, 0, st>>>(W, Y, d, k, wy_part, w2_part, prm.maxit, cin, cout);
+    std::swap(cin, cout);
+    if (!launch_ok() || !direction(0)) return NYS_ECUDA;
+    B_OK(cudaMemcpyAsync(host2, ndone, sizeof(host2), cudaMemcpyDeviceToHost, st));
     B_OK(cudaStreamSynchronize(st));
   }
-  B_OK(cudaMemcpyAsync(hc.data(), col, k * sizeof(BCol), cudaMemcpyDeviceToHost, st));
+  B_OK(cudaMemcpyAsync(hc.data(), cin, k * sizeof(BCol), cudaMemcpyDeviceToHost, st));
+  B_OK(cudaMemcpyAsync(host2, ndone, sizeof(host2), cudaMemcpyDeviceToHost, st));
   B_OK(cudaStreamSynchronize(st));
 #undef B_OK
+  if (host2[1]) return NYS_ECUDA;   // a bounded wait of a tensor-core product ran out
   nys_status res = NYS_OK;
   if (iters_out) iters_out->assign(k, 0);
   for (int c = 0; c < k; ++c) {
@@ -273,52 +320,60 @@ nys_status batched_pcg_run(const PcgProblem& pb, const PrecondView& P, const C* 
   }
   return res;
 }
-template nys_status batched_pcg_run<float>(const PcgProblem&, const PrecondView&, const float*, float*, int,
-                                           const PcgParams&, cudaStream_t, std::vector<int>*);
-template nys_status batched_pcg_run<double>(const PcgProblem&, const PrecondView&, const double*, double*, int,
-                                            const PcgParams&, cudaStream_t, std::vector<int>*);
+template nys_status batched_pcg_run<float>(const PcgProblem&, const TcPrepared*, const PrecondView&, const float*,
+                                           float*, int, const PcgParams&, cudaStream_t, std::vector<int>*);
+template nys_status batched_pcg_run<double>(const PcgProblem&, const TcPrepared*, const PrecondView&, const double*,
+                                            double*, int, const PcgParams&, cudaStream_t, std::vector<int>*);
 
 // ------------------------------------------------------------------ ADMM steps on d x k blocks
 namespace {
 template <typename C>
-__global__ void b_rhs_kernel(int64_t d, int k, const double* __restrict__ q, const double* __restrict__ Z,
-                             const double* __restrict__ Uu, double rho, C* __restrict__ R) {
-  const int64_t len = d * k;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
-    R[i] = (C)fma(rho, Z[i] - Uu[i], q[i % d]);
+__global__ void __launch_bounds__(kVecThreads) b_rhs_kernel(int64_t d, const double* __restrict__ q,
+                                                            const double* __restrict__ Z,
+                                                            const double* __restrict__ Uu, double rho,
+                                                            C* __restrict__ R) {
+  const int64_t j0 = (int64_t)blockIdx.x * kColChunk + threadIdx.x, base = (int64_t)blockIdx.y * d;
+#pragma unroll
+  for (int t = 0; t < kColPer; ++t) {
+    const int64_t j = j0 + t * kVecThreads;
+    if (j < d) R[base + j] = (C)fma(rho, Z[base + j] - Uu[base + j], q[j]);
+  }
 }
 
 // column c: z = S_{kappa_c}(x + u), u += x - z; partials of ||x - z||^2 and ||z - z_old||^2
 template <typename C>
-__global__ void __launch_bounds__(kVecThreads) b_zu_kernel(int64_t d, int k, int chunk, const C* __restrict__ Xc,
+__global__ void __launch_bounds__(kVecThreads) b_zu_kernel(int64_t d, int k, const C* __restrict__ Xc,
                                                            double* __restrict__ X, double* __restrict__ Z,
                                                            double* __restrict__ Uu, const double* __restrict__ kappa,
                                                            double* part) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t j0 = (int64_t)blockIdx.x * chunk;
-  const int64_t j1 = min(d, j0 + chunk);
-  for (int c = warp; c < k; c += kVecThreads / 32) {
-    const double kap = kappa[c];
-    double a0 = 0.0, a1 = 0.0;
-    for (int64_t j = j0 + lane; j < j1; j += 32) {
+  __shared__ double sh[kVecThreads / 32];
+  const int c = blockIdx.y;
+  const int64_t j0 = (int64_t)blockIdx.x * kColChunk + threadIdx.x;
+  const double kap = kappa[c];
+  double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+  for (int t = 0; t < kColPer; ++t) {
+    const int64_t j = j0 + t * kVecThreads;
+    if (j < d) {
       const int64_t i = (int64_t)c * d + j;
       const double xj = (double)Xc[i];
       const double zo = Z[i];
-      const double vj = xj + Uu[i];
+      const double uo = Uu[i];
+      const double vj = xj + uo;
       const double mag = fabs(vj) - kap;
       const double zj = mag > 0.0 ? copysign(mag, vj) : 0.0;
       X[i] = xj;
       Z[i] = zj;
-      Uu[i] += xj - zj;
+      Uu[i] = uo + (xj - zj);
       a0 += (xj - zj) * (xj - zj);
       a1 += (zj - zo) * (zj - zo);
     }
-    a0 = warp_sum(a0);
-    a1 = warp_sum(a1);
-    if (lane == 0) {
-      part[((int64_t)blockIdx.x * k + c) * 2] = a0;
-      part[((int64_t)blockIdx.x * k + c) * 2 + 1] = a1;
-    }
+  }
+  const double t0 = block_sum_t0<kVecThreads>(a0, sh);
+  const double t1 = block_sum_t0<kVecThreads>(a1, sh);
+  if (threadIdx.x == 0) {
+    part[((int64_t)blockIdx.x * k + c) * 2] = t0;
+    part[((int64_t)blockIdx.x * k + c) * 2 + 1] = t1;
   }
 }
 }  // namespace
@@ -327,20 +382,19 @@ template <typename C>
 cudaError_t batched_rhs(int64_t d, int k, const double* q, const double* Z, const double* Uu, double rho, C* R,
                         cudaStream_t st) {
   count_launch();
-  b_rhs_kernel<C><<<grid_for(d * k), 256, 0, st>>>(d, k, q, Z, Uu, rho, R);
+  b_rhs_kernel<C><<<dim3((unsigned)col_blocks(d), (unsigned)k), kVecThreads, 0, st>>>(d, q, Z, Uu, rho, R);
   return cudaGetLastError();
 }
 template <typename C>
 cudaError_t batched_zu(int64_t d, int k, const C* Xc, double* X, double* Z, double* Uu, const double* kappa,
                        double* part, int* nb_out, cudaStream_t st) {
-  const int chunk = 1024;
-  const int nb = (int)((d + chunk - 1) / chunk);
+  const int nb = col_blocks(d);
   count_launch();
-  b_zu_kernel<C><<<nb, kVecThreads, 0, st>>>(d, k, chunk, Xc, X, Z, Uu, kappa, part);
+  b_zu_kernel<C><<<dim3((unsigned)nb, (unsigned)k), kVecThreads, 0, st>>>(d, k, Xc, X, Z, Uu, kappa, part);
   *nb_out = nb;
   return cudaGetLastError();
 }
-int batched_zu_blocks(int64_t d) { return (int)((d + 1023) / 1024); }
+int batched_zu_blocks(int64_t d) { return col_blocks(d); }
 template cudaError_t batched_rhs<float>(int64_t, int, const double*, const double*, const double*, double, float*,
                                         cudaStream_t);
 template cudaError_t batched_rhs<double>(int64_t, int, const double*, const double*, const double*, double, double*,

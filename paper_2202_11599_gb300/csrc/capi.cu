@@ -785,9 +785,19 @@ nys_status lasso_path(const nys_matrix* A, const nys_matrix* Ain, const double* 
   double* Om = pool.alloc<double>((size_t)d * rank);
   double* Y = pool.alloc<double>((size_t)d * rank);
   if (!pool.ok()) return NYS_ENOMEM;
+  // the tensor-core operands of A (FP32: three BF16 terms and their transposes), made once for
+  // the sketch and every matvec of the path (50,000 x 4,000: 1.05 ms each time)
+  TcPrepared tcp;
+  const TcPrepared* tcpp = nullptr;
+  if (sizeof(C) == 4 && sketch_tc_supported(Ain)) {
+    void* tcs = pool.alloc<unsigned char>(tc_prepare_bytes(Ain));
+    if (!pool.ok()) return NYS_ENOMEM;
+    NYS_CU(tc_prepare(Ain, tcs, &tcp, st));
+    tcpp = &tcp;
+  }
   NYS_TRY(omega_panel(Omega, o.seed, d, rank, Om, st));
   NYS_TRY(cholqr2(Om, d, rank, st, Ain->dtype != NYS_F64));
-  NYS_TRY(sketch_panel(Ain, nullptr, 0.0, Om, rank, Y, st));
+  NYS_TRY(sketch_panel(Ain, nullptr, 0.0, Om, rank, Y, st, tcpp));
   const double shs = o.shift_scale > 0 ? o.shift_scale : std::sqrt((double)d);
   NYS_TRY(precond_from_panels(Om, Y, d, rank, shs, mant_bits_of(Ain), &P, st));
   C* cbuf = pool.alloc<C>(rank);
@@ -831,7 +841,7 @@ nys_status lasso_path(const nys_matrix* A, const nys_matrix* Ain, const double* 
     prm.maxit = maxit;
     prm.x0_zero = it == 0;
     if (o.pcg_fixed_iters) prm.fixed = o.pcg_fixed_iters[it];
-    nys_status s = batched_pcg_run<C>(pb, view, Rc, Xc, k, prm, st, &its);
+    nys_status s = batched_pcg_run<C>(pb, tcpp, view, Rc, Xc, k, prm, st, &its);
     if (s == NYS_ENOCONV) result = NYS_ENOCONV;
     else if (s != NYS_OK) return s;
     for (int c = 0; c < k; ++c) tot[c] += its[c];

@@ -139,19 +139,14 @@ cudaError_t sketch_tc_with(const nys_matrix* A, const TcPrepared& prep, const do
 // X (n values, FP64) <- each entry rounded to the nearest BF16 value through FP32 (to nearest,
 // ties to even): the test matrix of an FP32-class sketch.
 cudaError_t round_panel_bf16(double* X, int64_t n, cudaStream_t st);
-// Y (d x k) = A^T diag(D) A X + rho X, FP32 X and Y column-major (multi-RHS H-matvec).
+// Y (d x k) = A^T diag(D) A X + rho X, FP32 X and Y column-major (multi-RHS H-matvec), enqueued
+// on `st`: no allocation or synchronisation.  work: tc_hmm_work_bytes; status: a device int the
+// caller zeroes, set to NYS_ETIMEOUT when a bounded wait of a product ran out.
+size_t tc_hmm_work_bytes(const nys_matrix* A, const TcPrepared& prep, int k);
 cudaError_t tc_hmm(const nys_matrix* A, const TcPrepared& prep, const double* D, const float* X, int k, double rho,
-                   float* Y, cudaStream_t st);
+                   float* Y, void* work, int* status, cudaStream_t st);
 cudaError_t sketch_atw_partials(const nys_matrix* A, const void* W, int s, void* work, size_t work_bytes, int* nz_out,
                                 cudaStream_t st);
-// small dense GEMMs in compute type T (column-major)
-template <typename T>
-cudaError_t gemm_tn(const T* X, const T* Y, int64_t K, int M, int N, T* C, T* work, cudaStream_t st);
-template <typename T>
-size_t gemm_tn_work_elems(int64_t K, int M, int N);
-template <typename T>
-cudaError_t gemm_nn_t(const T* B, int64_t M, int K, const T* V, int N, T* C, cudaStream_t st);
-
 // ---------------------------------------------------------------- helpers
 // Omega (d x s column-major FP64) ~ N(0,1) from Philox-4x32-10 + Box-Muller (random.cu).
 cudaError_t gaussian_panel(uint64_t seed, int64_t d, int s, double* Omega, cudaStream_t st);

@@ -32,6 +32,7 @@
 #include "device_util.cuh"
 #include "nys_internal.cuh"
 #include "solver.cuh"
+#include "tc_ptx.cuh"
 
 #include <algorithm>
 #include <cstdio>
@@ -68,65 +69,7 @@ struct TcArgs {
   int* status;
 };
 
-// ---- PTX wrappers (tcgen05, cp.async, proxy fences)
-__device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
-               "r"(ncols)
-               : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish() {
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// Shared-memory matrix descriptor, no swizzle: start address, leading (K) and stride
-// (M/N) byte offsets, all in 16-byte units; bits 46-48 hold the fixed value 1.  The
-// swizzled form below sets the layout field (bits 61-63; 4 = 64-byte swizzle) and takes
-// only the 8-row-group stride (the leading offset is unused there, encoded as 1).
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
-}
-// Instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16 (bits 7-9 and
-// 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bit 17, M >> 4 at bit 24.
-__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr, uint32_t sbo) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46) |
-         (4ull << 61);
-}
-__host__ __device__ constexpr uint32_t mma_idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-__device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(dtmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
-// 32 lanes x 8 columns of 32 bits: thread l of the warp gets lane (base + l), 8 columns.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-               : "r"(taddr)
-               : "memory");
-}
-// the registers are operands so that no use of them is scheduled before the wait
-__device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[8]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7])
-               :
-               : "memory");
-}
+// ---- PTX wrappers (cp.async; tcgen05 in tc_ptx.cuh)
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
@@ -655,51 +598,54 @@ __global__ void split_matrix_kernel(const float* __restrict__ A, int64_t n, int6
 
 
 namespace {
+// Sizes and scratch of one product Y = A^T diag(D) A X with m columns.
+struct TcShape {
+  int64_t dP, mt2, kt2, kslice2;
+  int NPmax, rows1, rows2, Zeff;
+  size_t ot, wt, p;   // bytes of the operand terms of X, the terms of W and the partials of Y
+};
+TcShape tc_shape(const nys_matrix* A, const TcPrepared& prep, int m, int xterms) {
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  TcShape h;
+  h.dP = (A->d + TC_BK - 1) / TC_BK * TC_BK;
+  h.NPmax = std::min(TC_NMAX, (m + 15) / 16 * 16);
+  h.rows1 = tc_cta_rows(prep.at, xterms);
+  h.rows2 = tc_cta_rows(prep.at, TC_TERMS);
+  h.mt2 = (A->d + h.rows2 - 1) / h.rows2;
+  h.kt2 = prep.nP / TC_BK;
+  const int Z = pick_slices(h.mt2, h.kt2, sm_count_tc());
+  h.kslice2 = (h.kt2 + Z - 1) / Z;
+  h.Zeff = (int)((h.kt2 + h.kslice2 - 1) / h.kslice2);
+  h.ot = up((size_t)xterms * h.NPmax * h.dP * sizeof(uint16_t));
+  h.wt = up((size_t)TC_TERMS * h.NPmax * prep.nP * sizeof(uint16_t));
+  h.p = (size_t)h.Zeff * h.NPmax * A->d * sizeof(float);
+  return h;
+}
+
 // Y (d x m, column-major) = A^T diag(D) A X (+ rho X) on the tensor cores, given the
 // transposed copy At (d x nP) of A.  X and Y are FP64 (sketch) or FP32 (batched PCG).
 // xterms = 1: X holds BF16 values (the sketch's rounded test matrix), so the first product
-// takes one MMA term of X instead of three.
-template <typename TX, typename TY>
-cudaError_t tc_product(const nys_matrix* A, const TcPrepared& prep, const double* D, const TX* X, int m,
-                       double rho, TY* Y, cudaStream_t st, bool trace, int xterms) {
+// takes one MMA term of X instead of three.  Enqueues on `st` only: work (tc_shape's bytes) and
+// status (a device int the caller zeroed; NYS_ETIMEOUT when a wait ran out) are the caller's.
+template <typename TX, typename TY, typename Mark>
+cudaError_t tc_enqueue(const nys_matrix* A, const TcPrepared& prep, const double* D, const TX* X, int m, double rho,
+                       TY* Y, const TcShape& h, void* work, int* status, cudaStream_t st, int xterms, Mark mark) {
   const int64_t n = A->n, d = A->d;
   const int64_t nP = prep.nP;
-  const int64_t dP = (d + TC_BK - 1) / TC_BK * TC_BK;
-  const int NPmax = std::min(TC_NMAX, (m + 15) / 16 * 16);
   const uint32_t swap = std::getenv("NYS_TC_DESC_SWAP") ? (uint32_t)std::atoi(std::getenv("NYS_TC_DESC_SWAP")) : 0u;
-  const int sms = sm_count_tc();
-  const int rows1 = tc_cta_rows(prep.at, xterms), rows2 = tc_cta_rows(prep.at, TC_TERMS);
-  const int64_t mt2 = (d + rows2 - 1) / rows2;
-  const int64_t kt2 = nP / TC_BK;
-  const int Z = pick_slices(mt2, kt2, sms);
-  const int64_t kslice2 = (kt2 + Z - 1) / Z;
-  const int Zeff = (int)((kt2 + kslice2 - 1) / kslice2);
-
-  cudaEvent_t ev[8] = {};
-  int nev = 0;
-  auto mark = [&]() {
-    if (!trace || nev >= 8) return;
-    if (cudaEventCreate(&ev[nev]) == cudaSuccess) cudaEventRecord(ev[nev], st);
-    ++nev;
-  };
-  mark();
-  Pool pool(st);
-  uint16_t* Ot = pool.alloc<uint16_t>((size_t)xterms * NPmax * dP);
-  uint16_t* Wt = pool.alloc<uint16_t>((size_t)TC_TERMS * NPmax * nP);
-  float* P = pool.alloc<float>((size_t)Zeff * NPmax * d);
-  int* status = pool.alloc<int>(1);
-  if (!pool.ok()) return cudaErrorMemoryAllocation;
-  NYS_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), st));
-  mark();
+  unsigned char* wb = reinterpret_cast<unsigned char*>(work);
+  uint16_t* Ot = reinterpret_cast<uint16_t*>(wb);
+  uint16_t* Wt = reinterpret_cast<uint16_t*>(wb + h.ot);
+  float* P = reinterpret_cast<float*>(wb + h.ot + h.wt);
   for (int c0 = 0; c0 < m; c0 += TC_NMAX) {
     const int mp = std::min(TC_NMAX, m - c0);
     const int NP = (mp + 15) / 16 * 16;
     count_launch();
-    const unsigned sgrid = (unsigned)std::min<int64_t>(4096, ((int64_t)NP * dP + 255) / 256);
+    const unsigned sgrid = (unsigned)std::min<int64_t>(4096, ((int64_t)NP * h.dP + 255) / 256);
     if (xterms == 1)
-      split_operand_kernel<TX, 1><<<sgrid, 256, 0, st>>>(X, d, c0, mp, NP, dP, Ot);
+      split_operand_kernel<TX, 1><<<sgrid, 256, 0, st>>>(X, d, c0, mp, NP, h.dP, Ot);
     else
-      split_operand_kernel<TX, TC_TERMS><<<sgrid, 256, 0, st>>>(X, d, c0, mp, NP, dP, Ot);
+      split_operand_kernel<TX, TC_TERMS><<<sgrid, 256, 0, st>>>(X, d, c0, mp, NP, h.dP, Ot);
     NYS_CUDA_TRY(cudaGetLastError());
     if (c0 == 0) mark();
 
@@ -710,10 +656,10 @@ cudaError_t tc_product(const nys_matrix* A, const TcPrepared& prep, const double
     g1.Mrows = n;
     g1.Kvalid = d;
     g1.B = Ot;
-    g1.ldb = dP;
-    g1.bterm = (int64_t)NP * dP;
+    g1.ldb = h.dP;
+    g1.bterm = (int64_t)NP * h.dP;
     g1.NP = NP;
-    g1.ktiles = dP / TC_BK;
+    g1.ktiles = h.dP / TC_BK;
     g1.kslice = g1.ktiles;
     g1.D = D;
     g1.Wt = Wt;
@@ -722,7 +668,7 @@ cudaError_t tc_product(const nys_matrix* A, const TcPrepared& prep, const double
     g1.wrows = nP;
     g1.desc_swap = swap;
     g1.status = status;
-    NYS_CUDA_TRY(launch_tc_at<0>(prep.at, xterms, g1, dim3((unsigned)((n + rows1 - 1) / rows1), 1), st));
+    NYS_CUDA_TRY(launch_tc_at<0>(prep.at, xterms, g1, dim3((unsigned)((n + h.rows1 - 1) / h.rows1), 1), st));
     if (c0 == 0) mark();
 
     TcArgs g2 = {};
@@ -735,21 +681,44 @@ cudaError_t tc_product(const nys_matrix* A, const TcPrepared& prep, const double
     g2.ldb = nP;
     g2.bterm = (int64_t)NP * nP;
     g2.NP = NP;
-    g2.ktiles = kt2;
-    g2.kslice = kslice2;
+    g2.ktiles = h.kt2;
+    g2.kslice = h.kslice2;
     g2.P = P;
     g2.ldp = d;
     g2.desc_swap = swap;
     g2.status = status;
-    NYS_CUDA_TRY(launch_tc_at<1>(prep.at, TC_TERMS, g2, dim3((unsigned)mt2, (unsigned)Zeff), st));
+    NYS_CUDA_TRY(launch_tc_at<1>(prep.at, TC_TERMS, g2, dim3((unsigned)h.mt2, (unsigned)h.Zeff), st));
     if (c0 == 0) mark();
 
     count_launch();
     sum_slices_kernel<TY, TX><<<(unsigned)std::min<int64_t>(4096, ((int64_t)mp * d + 255) / 256), 256, 0, st>>>(
-        P, Zeff, NP, d, c0, mp, rho, X, Y);
+        P, h.Zeff, NP, d, c0, mp, rho, X, Y);
     NYS_CUDA_TRY(cudaGetLastError());
     if (c0 == 0) mark();
   }
+  return cudaSuccess;
+}
+
+// The sketch's product: own scratch, checked on return.
+cudaError_t tc_product(const nys_matrix* A, const TcPrepared& prep, const double* D, const double* X, int m, double* Y,
+                       cudaStream_t st, bool trace) {
+  constexpr int xterms = 1;   // the rounded test matrix
+  cudaEvent_t ev[8] = {};
+  int nev = 0;
+  auto mark = [&]() {
+    if (!trace || nev >= 8) return;
+    if (cudaEventCreate(&ev[nev]) == cudaSuccess) cudaEventRecord(ev[nev], st);
+    ++nev;
+  };
+  mark();
+  const TcShape h = tc_shape(A, prep, m, xterms);
+  Pool pool(st);
+  void* work = pool.alloc<unsigned char>(h.ot + h.wt + h.p);
+  int* status = pool.alloc<int>(1);
+  if (!pool.ok()) return cudaErrorMemoryAllocation;
+  NYS_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), st));
+  mark();
+  NYS_CUDA_TRY((tc_enqueue<double, double>(A, prep, D, X, m, 0.0, Y, h, work, status, st, xterms, mark)));
   int status_h = 0;
   NYS_CUDA_TRY(cudaMemcpyAsync(&status_h, status, sizeof(int), cudaMemcpyDeviceToHost, st));
   NYS_CUDA_TRY(cudaStreamSynchronize(st));
@@ -760,7 +729,7 @@ cudaError_t tc_product(const nys_matrix* A, const TcPrepared& prep, const double
       if (ev[i - 1] && ev[i]) cudaEventElapsedTime(&ms, ev[i - 1], ev[i]);
       std::fprintf(stderr, "[nys]   tc %-18s %8.3f ms\n", names[i - 1], ms);
     }
-    std::fprintf(stderr, "[nys]   tc split-K slices %d, NP %d\n", Zeff, NPmax);
+    std::fprintf(stderr, "[nys]   tc split-K slices %d, NP %d\n", h.Zeff, h.NPmax);
   }
   for (auto& e : ev)
     if (e) cudaEventDestroy(e);
@@ -860,19 +829,25 @@ cudaError_t sketch_tc(const nys_matrix* A, const double* D, const double* Om, in
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
   }
-  return tc_product<double, double>(A, prep, D, Om, m, 0.0, Y, st, trace, 1);
+  return tc_product(A, prep, D, Om, m, Y, st, trace);
 }
 
 cudaError_t sketch_tc_with(const nys_matrix* A, const TcPrepared& prep, const double* D, const double* Om, int m,
                            double* Y, cudaStream_t st) {
   if (m <= 0) return cudaErrorInvalidValue;
-  return tc_product<double, double>(A, prep, D, Om, m, 0.0, Y, st, std::getenv("NYS_TRACE") != nullptr, 1);
+  return tc_product(A, prep, D, Om, m, Y, st, std::getenv("NYS_TRACE") != nullptr);
+}
+
+size_t tc_hmm_work_bytes(const nys_matrix* A, const TcPrepared& prep, int k) {
+  const TcShape h = tc_shape(A, prep, k, TC_TERMS);
+  return h.ot + h.wt + h.p;
 }
 
 cudaError_t tc_hmm(const nys_matrix* A, const TcPrepared& prep, const double* D, const float* X, int k, double rho,
-                   float* Y, cudaStream_t st) {
+                   float* Y, void* work, int* status, cudaStream_t st) {
   if (k <= 0) return cudaErrorInvalidValue;
-  return tc_product<float, float>(A, prep, D, X, k, rho, Y, st, false, TC_TERMS);
+  return tc_enqueue<float, float>(A, prep, D, X, k, rho, Y, tc_shape(A, prep, k, TC_TERMS), work, status, st, TC_TERMS,
+                                  [] {});
 }
 
 }  // namespace nys

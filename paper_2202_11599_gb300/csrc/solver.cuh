@@ -115,9 +115,10 @@ int pcg_nb3(int64_t d);
 
 PcgState* host_state();
 
-// Multi-RHS PCG (k columns sharing H + rho I and P); R, X: d x k column-major.
+// Multi-RHS PCG (k columns sharing H + rho I and P); R, X: d x k column-major.  tcp: tensor-core
+// operands of pb.A (the matvecs then run there), or NULL.
 template <typename C>
-nys_status batched_pcg_run(const PcgProblem& pb, const PrecondView& P, const C* R, C* X, int k, const PcgParams& prm,
+nys_status batched_pcg_run(const PcgProblem& pb, const TcPrepared* tcp, const PrecondView& P, const C* R, C* X, int k, const PcgParams& prm,
                            cudaStream_t st, std::vector<int>* iters_out);
 template <typename C>
 cudaError_t batched_rhs(int64_t d, int k, const double* q, const double* Z, const double* Uu, double rho, C* R,
