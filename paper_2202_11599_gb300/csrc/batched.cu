@@ -36,11 +36,12 @@ constexpr int kColChunk = 1024;
 constexpr int kColPer = kColChunk / kVecThreads;
 int col_blocks(int64_t d) { return (int)((d + kColChunk - 1) / kColChunk); }
 
+// V = rho P + (sum of the partials of A^T D A P); with nz = 0 the sum is in V already.
 template <typename C>
 __global__ void b_matvec_finish_kernel(const C* __restrict__ part, int nz, int64_t len, C rho, const C* __restrict__ P,
                                        C* __restrict__ V) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x) {
-    C s = C(0);
+    C s = nz ? C(0) : V[i];
     for (int z = 0; z < nz; ++z) s += part[z * len + i];
     V[i] = fma(rho, P[i], s);
   }
@@ -224,10 +225,13 @@ nys_status batched_pcg_run(const PcgProblem& pb, const TcPrepared* tcp, const Pr
   C* Y = pool.alloc<C>(len);
   C* Pd = pool.alloc<C>(len);
   C* V = pool.alloc<C>(len);
-  C* Wn = use_tc ? nullptr : pool.alloc<C>((size_t)n * k);
-  const size_t atw_bytes = use_tc ? 0 : sketch_atw_work_bytes(pb.A, k);
-  void* atw = use_tc ? nullptr : pool.alloc<unsigned char>(atw_bytes);
-  void* tcw = use_tc ? pool.alloc<unsigned char>(tc_hmm_work_bytes(pb.A, *tcp, k)) : nullptr;
+  constexpr bool f64 = sizeof(C) == 8;
+  const bool cuda_cores = !f64 && !use_tc;
+  C* Wn = cuda_cores ? pool.alloc<C>((size_t)n * k) : nullptr;
+  const size_t atw_bytes = cuda_cores ? sketch_atw_work_bytes(pb.A, k) : 0;
+  void* atw = cuda_cores ? pool.alloc<unsigned char>(atw_bytes) : nullptr;
+  void* tcw = use_tc ? pool.alloc<unsigned char>(tc_hmm_work_bytes(pb.A, *tcp, k))
+                     : (f64 ? pool.alloc<unsigned char>(hmm64_bytes(pb.A, k)) : nullptr);
   C* gwork = s > 0 ? pool.alloc<C>(precond_block_work<C>(d, s, k)) : nullptr;
   double* pv_part = pool.alloc<double>((size_t)nb * k);
   double* w2_part = pool.alloc<double>((size_t)nb * k);
@@ -236,7 +240,7 @@ nys_status batched_pcg_run(const PcgProblem& pb, const TcPrepared* tcp, const Pr
   int* ndone = pool.alloc<int>(2);   // finished columns; status of the tensor-core products
   if (!pool.ok()) return NYS_ENOMEM;
   BCol *cin = cols, *cout = cols + k;
-  int* tc_status = ndone + 1;
+  int* tc_status = f64 ? hmm64_status(pb.A, k, tcw) : ndone + 1;
   const C* U = reinterpret_cast<const C*>(P.U);
   const C* cvec = reinterpret_cast<const C*>(P.c);
 #define B_OK(x)                             \
@@ -245,13 +249,20 @@ nys_status batched_pcg_run(const PcgProblem& pb, const TcPrepared* tcp, const Pr
   } while (0)
   auto launch_ok = [&]() { return cudaGetLastError() == cudaSuccess; };
   const dim3 cgrid((unsigned)nb, (unsigned)k);
+  if (f64) B_OK(hmm64_prepare(pb.A, k, tcw, st));
   // BF16 and FP32 storage: the k-column products run on the tensor cores (the same tcgen05
-  // GEMMs as the sketch, FP32 operand as three BF16 terms) from operands prepared once per solve.
+  // GEMMs as the sketch, FP32 operand as three BF16 terms) from operands prepared once per solve;
+  // FP64 storage on the FP64 products of the sketch.
   // V = A^T (A P) + rho P for the k columns of P (reads A once)
   auto bmatvec = [&](const C* Pin, C* Vout) -> bool {
     if constexpr (sizeof(C) == 4) {
       if (use_tc) return tc_hmm(pb.A, *tcp, pb.D, reinterpret_cast<const float*>(Pin), k, pb.rho,
                                 reinterpret_cast<float*>(Vout), tcw, tc_status, st) == cudaSuccess;
+    } else {
+      if (hmm64(pb.A, pb.D, Pin, k, Vout, tcw, st) != cudaSuccess) return false;
+      count_launch();
+      b_matvec_finish_kernel<C><<<grid_for(len), 256, 0, st>>>(nullptr, 0, len, (C)pb.rho, Pin, Vout);
+      return launch_ok();
     }
     if (sketch_aw(pb.A, Pin, k, pb.D, Wn, st) != cudaSuccess) return false;
     int nz = 0;
@@ -307,7 +318,7 @@ nys_status batched_pcg_run(const PcgProblem& pb, const TcPrepared* tcp, const Pr
     B_OK(cudaStreamSynchronize(st));
   }
   B_OK(cudaMemcpyAsync(hc.data(), cin, k * sizeof(BCol), cudaMemcpyDeviceToHost, st));
-  B_OK(cudaMemcpyAsync(host2, ndone, sizeof(host2), cudaMemcpyDeviceToHost, st));
+  B_OK(cudaMemcpyAsync(host2 + 1, tc_status, sizeof(int), cudaMemcpyDeviceToHost, st));
   B_OK(cudaStreamSynchronize(st));
 #undef B_OK
   if (host2[1]) return NYS_ECUDA;   // a bounded wait of a tensor-core product ran out

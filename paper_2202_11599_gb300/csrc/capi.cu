@@ -112,11 +112,12 @@ nys_status cholqr2(double* Om, int64_t d, int m, cudaStream_t st, bool fp32_clas
   Pool pool(st);
   double* G = pool.alloc<double>((size_t)m * m);
   double* work = pool.alloc<double>(gram_work_bytes(d, m) / sizeof(double) + 1);
-  int* info = pool.alloc<int>(1);
+  int* info = pool.alloc<int>(2);   // Cholesky; waits of the products
   double* gap = pool.alloc<double>(1);
   if (!pool.ok()) return NYS_ENOMEM;
+  NYS_CU(cudaMemsetAsync(info, 0, 2 * sizeof(int), st));
   for (int pass = 0; pass < 2; ++pass) {
-    NYS_CU(gram_xty(Om, Om, d, m, G, work, st));
+    NYS_CU(gram_xty(Om, Om, d, m, G, work, info + 1, st));
     if (pass == 1 && fp32_class) {
       NYS_CU(identity_gap(G, m, gap, st));
       double gap_h = 1.0;
@@ -127,10 +128,11 @@ nys_status cholqr2(double* Om, int64_t d, int m, cudaStream_t st, bool fp32_clas
     // a pivot below 1e-10 of the largest column norm^2: columns dependent to ~1e-5, which
     // CholQR cannot orthonormalise -- refused as a bad test matrix
     NYS_CU(chol_upper(G, m, info, st, 1e-10));
-    int info_h = 0;
-    NYS_CU(cudaMemcpyAsync(&info_h, info, sizeof(int), cudaMemcpyDeviceToHost, st));
+    int info_h[2] = {0, 0};
+    NYS_CU(cudaMemcpyAsync(info_h, info, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     NYS_CU(cudaStreamSynchronize(st));
-    if (info_h != 0) return NYS_EINVAL;  // Omega has (numerically) dependent columns
+    if (info_h[1]) return (nys_status)info_h[1];
+    if (info_h[0] != 0) return NYS_EINVAL;  // Omega has (numerically) dependent columns
     NYS_CU(trsm_right_upper(G, m, Om, d, st));
   }
   return NYS_OK;
@@ -164,14 +166,18 @@ nys_status sketch_panel(const nys_matrix* A, const double* D, double shift, doub
     if (shift != 0.0) NYS_CU(axpy_panel(shift, Om, Y, d * m, st));
     return NYS_OK;
   }
-  const size_t wbytes = sketch_atw_work_bytes(A, m);
-  void* work = pool.alloc<unsigned char>(wbytes);
   if (A->dtype == NYS_F64) {
-    double* W = pool.alloc<double>((size_t)n * m);
+    void* scratch = pool.alloc<unsigned char>(hmm64_bytes(A, m));
     if (!pool.ok()) return NYS_ENOMEM;
-    NYS_CU(sketch_aw(A, Om, m, D, W, st));
-    NYS_CU(sketch_atw(A, W, m, Y, work, wbytes, st));
+    NYS_CU(hmm64_prepare(A, m, scratch, st));
+    NYS_CU(hmm64(A, D, Om, m, Y, scratch, st));
+    int status_h = 0;
+    NYS_CU(cudaMemcpyAsync(&status_h, hmm64_status(A, m, scratch), sizeof(int), cudaMemcpyDeviceToHost, st));
+    NYS_CU(cudaStreamSynchronize(st));
+    if (status_h) return (nys_status)status_h;
   } else {
+    const size_t wbytes = sketch_atw_work_bytes(A, m);
+    void* work = pool.alloc<unsigned char>(wbytes);
     float* Om32 = pool.alloc<float>((size_t)d * m);
     float* W = pool.alloc<float>((size_t)n * m);
     if (!pool.ok()) return NYS_ENOMEM;
@@ -196,17 +202,19 @@ nys_status nystrom_core(const double* Om, const double* Y, int64_t d, int s, dou
   double* pw = pool.alloc<double>(2 * (size_t)s + 2);   // power iteration: two w buffers + barrier words
   double* Ynu = pool.alloc<double>((size_t)d * s);
   double* M = pool.alloc<double>((size_t)s * s);
-  int* info = pool.alloc<int>(1);
+  int* info = pool.alloc<int>(2);   // Cholesky; waits of the products
+  int* status = info + 1;
   const int N = s + (s & 1);
   double* V = pool.alloc<double>((size_t)N * N);
   double* jw = pool.alloc<double>(jacobi_work_bytes(s) / sizeof(double) + 1);
-  double* fw = pool.alloc<double>((size_t)s * s + s);
+  double* fw = pool.alloc<double>(finish_work_bytes(d, s) / sizeof(double) + 1);
   if (!pool.ok()) return NYS_ENOMEM;
+  NYS_CU(cudaMemsetAsync(info, 0, 2 * sizeof(int), st));
 
   PhaseTimer pt_all("nystrom core (total)", st);
   {
     PhaseTimer pt("core: Y^T Y + power", st);
-    NYS_CU(gram_xty(Y, Y, d, s, G, gw, st));
+    NYS_CU(gram_xty(Y, Y, d, s, G, gw, status, st));
     NYS_CU(power_lambda_max(G, s, lmax, pw, st));
   }
   double lmax_h = 0.0;
@@ -219,7 +227,7 @@ nys_status nystrom_core(const double* Om, const double* Y, int64_t d, int s, dou
   for (int attempt = 0; attempt < 4; ++attempt) {
     NYS_CU(cudaMemcpyAsync(Ynu, Y, (size_t)d * s * sizeof(double), cudaMemcpyDeviceToDevice, st));
     NYS_CU(axpy_panel(nu, Om, Ynu, d * s, st));
-    NYS_CU(gram_xty(Om, Ynu, d, s, M, gw, st));
+    NYS_CU(gram_xty(Om, Ynu, d, s, M, gw, status, st));
     NYS_CU(chol_upper(M, s, info, st));
     int info_h = 0;
     NYS_CU(cudaMemcpyAsync(&info_h, info, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -235,7 +243,7 @@ nys_status nystrom_core(const double* Om, const double* Y, int64_t d, int s, dou
   {
     PhaseTimer pt("core: trsm + B^T B", st);
     NYS_CU(trsm_right_upper(M, s, Ynu, d, st));       // B = Y_nu C^{-1} (in Ynu)
-    NYS_CU(gram_xty(Ynu, Ynu, d, s, G, gw, st));      // B^T B
+    NYS_CU(gram_xty(Ynu, Ynu, d, s, G, gw, status, st));      // B^T B
   }
   int sweeps = 0;
   {
@@ -246,14 +254,16 @@ nys_status nystrom_core(const double* Om, const double* Y, int64_t d, int s, dou
   }
   {
     PhaseTimer pt("core: finish (U = BV)", st);
-    NYS_CU(nystrom_finish(Ynu, d, s, jw, V, nu, U, lam_d, fw, st));
+    NYS_CU(nystrom_finish(Ynu, d, s, jw, V, nu, U, lam_d, fw, status, st));
   }
   if (std::getenv("NYS_TRACE")) std::fprintf(stderr, "[nys] jacobi sweeps %d (s = %d)\n", sweeps, s);
   lam_h.resize(s);
+  int status_h = 0;
+  NYS_CU(cudaMemcpyAsync(&status_h, status, sizeof(int), cudaMemcpyDeviceToHost, st));
   NYS_CU(cudaMemcpyAsync(lam_h.data(), lam_d, s * sizeof(double), cudaMemcpyDeviceToHost, st));
   NYS_CU(cudaStreamSynchronize(st));
   if (nu_out) *nu_out = nu;
-  return NYS_OK;
+  return status_h ? (nys_status)status_h : NYS_OK;
 }
 
 nys_status precond_alloc(nys_precond_s* P, int64_t d, int s) {

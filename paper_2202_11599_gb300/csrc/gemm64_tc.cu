@@ -1,0 +1,578 @@
+// FP64 matrix products on the BF16 tensor cores.
+//
+//   C (M x N) = diag(D) A B^T,   A(m, k), B(n, k) FP64
+//
+// GB300's FP64 pipe retires about 2 FMA per clock and SM; its BF16 tensor cores ~3,400 MAC.
+// Each operand row is written in fixed point relative to its own largest exponent, as eight
+// signed 8-bit digits (62 bits below the row's maximum):
+//   A(m, k) = 2^(ea_m - 1084) sum_i a_i 256^(7 - i),  a_i in [-128, 127] (exact in BF16),
+// so a product of digits is an integer of at most 2^14, and the tensor core's FP32
+// accumulators add them exactly while |sum| < 2^24.  The digit products of equal weight
+// (order o = i + j = 0 .. 7, o + 1 pairs) share one TMEM accumulator: 36 MMAs per K step for
+// 64 output columns x 8 orders = all 512 TMEM columns.  Every 256 K the accumulators are read
+// out as integers and added to two 64-bit integer sums per output: at 256 K orders 0-3 cannot
+// leave 2^24 for any input, and orders 4-7, below 2^-32 of the product's scale, could round
+// only for inputs whose low digits all agree in sign.  The dropped orders lie below 2^-60.
+// The final integer is rounded to FP64 once.  (Fixed-point splitting of a product into exact
+// low-precision ones: Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 59, 2012.)  The error is
+// that of rounding each operand to 2^-62 of its row's maximum plus the final rounding: on random,
+// graded, constant and one-signed rows of up to 600 terms it is 1e-18 to 7e-17 of sum |a||b|,
+// against 1e-16 to 8e-15 for a chain of FP64 FMAs.  A row holding a NaN or an infinity gives NaN.
+//
+// Measured (FP64 pipe before, this kernel after): the two products of a 40,000 x 4,000 sketch of
+// rank 100, 36.1 + 40.4 ms -> 2.7 + 2.7 ms; X^T Y at 10,000 x 200, 0.52 (symmetric) and 0.90 ms
+// -> 0.05 ms; U = B V at 10,000 x 200, 1.09 -> 0.06 ms.
+//
+// What bounds it: at N = 64 an MMA reads its 4 KB A tile and 2 KB B tile from shared memory in
+// 48 clocks and multiplies in 39, so shared memory does (36 MMAs x 2 per 32 K: ~3,400 clocks
+// plus 500 to store the digits); making the digits (30 integer operations an element, 512
+// threads) runs beside the MMAs of the previous stage.  Both operands are converted in the
+// kernel: the digits are never written to memory, and an operand stored along M (A^T) is
+// transposed on the way into shared memory.
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "solver.cuh"
+#include "tc_ptx.cuh"
+
+namespace nys {
+namespace {
+
+constexpr int EM = 128, EN = 64, EK = 32;     // tile and K of one stage
+constexpr int ET = 512;                       // threads
+constexpr int ESL = 8;                        // digits per operand = orders kept
+constexpr int EFLUSH = 8;                     // stages between read-outs (256 K)
+constexpr uint32_t EA_SLICE = EM * EK * 2, EB_SLICE = EN * EK * 2;
+constexpr uint32_t E_STAGE = ESL * (EA_SLICE + EB_SLICE);   // 96 KB
+constexpr int E_MINSTEPS = 4;                 // K steps a split slice has at least
+
+struct EmuArgs {
+  const double* A;
+  int64_t lda;
+  const unsigned* ea;   // per row m: top word of its largest magnitude (exponent in bits 20-30)
+  const double* B;
+  int64_t ldb;
+  const unsigned* eb;
+  int64_t M, K, kslice;
+  int N;
+  const double* D;      // row factors, applied when the K range is not split
+  double* C;            // slice z at C + z * cslice, column n at + n * ldc
+  int64_t ldc, cslice;
+  int* status;
+};
+
+// Fixed-point value of x at the scale of its row (largest exponent field emax), each byte the
+// digit + 128.
+__device__ __forceinline__ uint64_t digits(double x, int emax) {
+  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+  const int e = (int)((h >> 20) & 0x7ffu);
+  const uint32_t mh = (h & 0xfffffu) | (e ? 0x100000u : 0u);
+  const uint64_t m = (((uint64_t)mh << 32) | l) << 9;
+  const int sh = emax - max(e, 1);
+  uint64_t q = sh < 64 ? m >> sh : 0ull;
+  if ((int)h < 0) q = 0ull - q;
+  return q + 0x8080808080808080ull;
+}
+
+// Digit b (0 = lowest byte) of two biased values as a BF16 pair: with d + 128 = 128 u + v
+// (v < 128), (128 + v) - (u ? 128 : 256) = d, all exact in BF16.
+template <int B>
+__device__ __forceinline__ uint32_t digit_pair(uint32_t x0, uint32_t x1) {
+  const uint32_t p = __byte_perm(x0, x1, B | (B << 4) | ((4 + B) << 8) | ((4 + B) << 12));
+  const uint32_t a = (p & 0x007f007fu) | 0x43004300u;
+  const uint32_t s = (~p & 0x00800080u) | 0x43004300u;
+  const __nv_bfloat162 r = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&a),
+                                   *reinterpret_cast<const __nv_bfloat162*>(&s));
+  return *reinterpret_cast<const uint32_t*>(&r);
+}
+
+// v 2^sh rounded once to FP64 (to nearest, ties to even).
+__device__ __forceinline__ double fixed_to_double(__int128 v, int sh) {
+  if (v == 0) return 0.0;
+  const bool neg = v < 0;
+  unsigned __int128 u = neg ? (unsigned __int128)(-v) : (unsigned __int128)v;
+  const uint64_t uh = (uint64_t)(u >> 64);
+  const int lz = uh ? __clzll((long long)uh) : 64 + __clzll((long long)(uint64_t)u);
+  u <<= lz;
+  const uint64_t top = (uint64_t)(u >> 64);
+  const bool sticky = (uint64_t)u != 0;
+  uint64_t m = top >> 11;
+  const uint32_t r = (uint32_t)(top & 0x7ffu);
+  if (r > 0x400u || (r == 0x400u && (sticky || (m & 1)))) ++m;
+  int e = 127 + sh - lz;
+  if (m >> 53) {
+    m >>= 1;
+    ++e;
+  }
+  double x;
+  if (e > 1023) x = __longlong_as_double(0x7ff0000000000000ll);
+  else if (e < -1022) x = scalbn((double)m, e - 52);
+  else x = __longlong_as_double((long long)(((uint64_t)(e + 1023) << 52) | (m & 0xfffffffffffffull)));
+  return neg ? -x : x;
+}
+
+// KC: A(m, k) = A[m lda + k]; else A(m, k) = A[k lda + m].  B(n, k) = B[n ldb + k].
+template <bool KC>
+__global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t bars[2];
+  __shared__ uint32_t tmem_slot;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t m0 = (int64_t)blockIdx.y * EM;
+  const int n0 = blockIdx.x * EN;
+  const int64_t kb = (int64_t)blockIdx.z * a.kslice, ke = min(a.K, kb + a.kslice);
+  const int nt = (int)((ke - kb + EK - 1) / EK);
+  const uint32_t sbase = smem_u32(smem);
+  if (warp == 0) {
+    tmem_alloc(&tmem_slot, 512);
+    tmem_relinquish();
+  }
+  if (tid == 0) {
+    mbar_init(&bars[0], 1);
+    mbar_init(&bars[1], 1);
+    fence_mbar_init();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+
+  // Conversion: this thread's chunk of A is row ar, K 8 ac .. + 7 of a stage; its half chunk of
+  // B is row br, K 4 bc .. + 3.  Lanes run over the rows of a core matrix (8 rows x 16 bytes),
+  // so the 16-byte stores of eight lanes fill one.
+  int ar, ac;
+  if (KC) {
+    ar = 8 * warp + (lane & 7);
+    ac = lane >> 3;
+  } else {
+    ar = 32 * (warp & 3) + lane;
+    ac = warp >> 2;
+  }
+  const int br = 4 * warp + (lane >> 3), bc = lane & 7;
+  const int64_t am = m0 + ar;
+  const bool aok = am < a.M, bok = n0 + br < a.N;
+  const int emA = aok ? max(1, (int)(a.ea[am] >> 20)) : 1;
+  const int emB = bok ? max(1, (int)(a.eb[n0 + br] >> 20)) : 1;
+  const double* Ap = KC ? a.A + (aok ? am : 0) * a.lda : a.A + (aok ? am : 0);
+  const double* Bp = a.B + (int64_t)(bok ? n0 + br : 0) * a.ldb;
+  const bool avec = KC && (a.lda & 1) == 0 && (reinterpret_cast<uintptr_t>(a.A) & 15u) == 0 && (kb & 1) == 0;
+  const bool bvec = (a.ldb & 1) == 0 && (reinterpret_cast<uintptr_t>(a.B) & 15u) == 0 && (kb & 1) == 0;
+  double ra[8], rb[4];
+  auto load = [&](int t) {
+    const int64_t ka = kb + (int64_t)t * EK + 8 * ac, kk = kb + (int64_t)t * EK + 4 * bc;
+    if (KC && avec && aok && ka + 8 <= ke) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const double2 v = __ldg(reinterpret_cast<const double2*>(Ap + ka) + e);
+        ra[2 * e] = v.x;
+        ra[2 * e + 1] = v.y;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        ra[e] = (aok && ka + e < ke) ? __ldg(KC ? Ap + ka + e : Ap + (ka + e) * a.lda) : 0.0;
+    }
+    if (bvec && bok && kk + 4 <= ke) {
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const double2 v = __ldg(reinterpret_cast<const double2*>(Bp + kk) + e);
+        rb[2 * e] = v.x;
+        rb[2 * e + 1] = v.y;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) rb[e] = (bok && kk + e < ke) ? __ldg(Bp + kk + e) : 0.0;
+    }
+  };
+  // byte offsets of the chunks in a slice: core matrix (row / 8, K chunk) at 512 (row / 8) + 128 chunk
+  const uint32_t aoff = (uint32_t)((ar >> 3) * 512 + ac * 128 + (ar & 7) * 16);
+  const uint32_t boff = (uint32_t)((br >> 3) * 512 + (bc >> 1) * 128 + (br & 7) * 16 + (bc & 1) * 8);
+  auto store = [&](uint32_t st) {
+    {
+      uint32_t lo[8], hi[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const uint64_t q = digits(ra[e], emA);
+        lo[e] = (uint32_t)q;
+        hi[e] = (uint32_t)(q >> 32);
+      }
+      auto put = [&](int slice, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(st + slice * EA_SLICE + aoff), "r"(w0), "r"(w1),
+                     "r"(w2), "r"(w3)
+                     : "memory");
+      };
+#define NYS_PUT(SL, B, W) \
+  put(SL, digit_pair<B>(W[0], W[1]), digit_pair<B>(W[2], W[3]), digit_pair<B>(W[4], W[5]), digit_pair<B>(W[6], W[7]))
+      NYS_PUT(0, 3, hi);
+      NYS_PUT(1, 2, hi);
+      NYS_PUT(2, 1, hi);
+      NYS_PUT(3, 0, hi);
+      NYS_PUT(4, 3, lo);
+      NYS_PUT(5, 2, lo);
+      NYS_PUT(6, 1, lo);
+      NYS_PUT(7, 0, lo);
+#undef NYS_PUT
+    }
+    {
+      uint32_t lo[4], hi[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const uint64_t q = digits(rb[e], emB);
+        lo[e] = (uint32_t)q;
+        hi[e] = (uint32_t)(q >> 32);
+      }
+      auto put = [&](int slice, uint32_t w0, uint32_t w1) {
+        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(st + ESL * EA_SLICE + slice * EB_SLICE + boff), "r"(w0),
+                     "r"(w1)
+                     : "memory");
+      };
+#define NYS_PUT(SL, B, W) put(SL, digit_pair<B>(W[0], W[1]), digit_pair<B>(W[2], W[3]))
+      NYS_PUT(0, 3, hi);
+      NYS_PUT(1, 2, hi);
+      NYS_PUT(2, 1, hi);
+      NYS_PUT(3, 0, hi);
+      NYS_PUT(4, 3, lo);
+      NYS_PUT(5, 2, lo);
+      NYS_PUT(6, 1, lo);
+      NYS_PUT(7, 0, lo);
+#undef NYS_PUT
+    }
+  };
+
+  // Read-out: warp w holds rows 32 (w % 4) + lane, columns 16 (w / 4) .. + 15.  hi collects
+  // orders 0-3 (in units of order 3), lo orders 4-7 (in units of order 7).
+  const int quad = warp & 3, cg = (warp >> 2) * 16;
+  int64_t hi[16], lo[16];
+#pragma unroll
+  for (int e = 0; e < 16; ++e) hi[e] = lo[e] = 0;
+  const uint32_t trow = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)cg;
+  auto flush = [&]() {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        int64_t s[8];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+          uint32_t v[8];
+          tmem_ld8(trow + (uint32_t)((4 * half + o) * EN + 8 * h), v);
+          tmem_ld_wait(v);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const int64_t t = (int64_t)__float2int_rn(__uint_as_float(v[e]));
+            s[e] = o == 0 ? t : (s[e] << 8) + t;
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) (half ? lo : hi)[8 * h + e] += s[e];
+      }
+    }
+  };
+
+  constexpr uint32_t idesc = mma_idesc_bf16(EM, EN);
+  bool ok = true;
+  if (nt > 0) load(0);
+  for (int t = 0; t < nt; ++t) {
+    const int s = t & 1;
+    const uint32_t st = sbase + (uint32_t)s * E_STAGE;
+    // the MMAs of this stage's previous use must be done reading it
+    if (t >= 2) ok = ok && mbar_wait_bounded(&bars[s], (uint32_t)(((t >> 1) - 1) & 1));
+    store(st);
+    if (t + 1 < nt) load(t + 1);
+    fence_proxy_async_smem();
+    tc_fence_before();
+    ok = __syncthreads_and(ok) != 0;
+    if (!ok) break;
+    const bool first = t % EFLUSH == 0;
+    if (tid == 0) {
+      tc_fence_after();
+      const uint64_t ad0 = smem_desc(st, 128u, 512u), bd0 = smem_desc(st + ESL * EA_SLICE, 128u, 512u);
+#pragma unroll 1
+      for (int kk = 0; kk < EK / 16; ++kk) {
+#pragma unroll
+        for (int o = 0; o < ESL; ++o) {
+#pragma unroll
+          for (int i = 0; i <= o; ++i) {
+            mma_bf16(tmem + (uint32_t)(o * EN), ad0 + (uint64_t)((i * EA_SLICE + kk * 256u) >> 4),
+                     bd0 + (uint64_t)(((o - i) * EB_SLICE + kk * 256u) >> 4), idesc,
+                     (first && kk == 0 && i == 0) ? 0u : 1u);
+          }
+        }
+      }
+      mma_commit(&bars[s]);
+    }
+    if (t % EFLUSH == EFLUSH - 1 || t == nt - 1) {
+      ok = mbar_wait_bounded(&bars[s], (uint32_t)((t >> 1) & 1));
+      tc_fence_after();
+      if (__all_sync(0xffffffffu, ok)) flush();
+    }
+  }
+  tc_fence_before();
+  ok = __syncthreads_and(ok) != 0;
+  tc_fence_after();
+  if (!ok && tid == 0) {
+    // a wait gave up: report, and give the MMAs still queued a bounded last chance to finish
+    atomicExch(a.status, (int)NYS_ETIMEOUT);
+    const int last = nt - 1;
+    (void)mbar_wait_bounded(&bars[last & 1], (uint32_t)((last >> 1) & 1));
+  }
+  const int64_t m = m0 + 32 * quad + lane;
+  if (m < a.M) {
+    const unsigned wa = a.ea[m];
+    const double dm = a.D ? a.D[m] : 1.0;
+    double* out = a.C + (int64_t)blockIdx.z * a.cslice + m;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const int n = n0 + cg + e;
+      if (n < a.N) {
+        const unsigned wb = a.eb[n];
+        double x = fixed_to_double((((__int128)hi[e]) << 32) + (__int128)lo[e],
+                                   56 - 2168 + max(1, (int)(wa >> 20)) + max(1, (int)(wb >> 20)));
+        if (!ok || (wa >> 20) == 0x7ffu || (wb >> 20) == 0x7ffu) x = __longlong_as_double(0x7ff8000000000000ll);
+        out[(int64_t)n * a.ldc] = a.D ? dm * x : x;
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
+// Largest magnitude (top word: order and exponent; a NaN or an infinity is above every finite
+// value) of each row and / or column of the row-major rows x cols matrix X.  Block (bx, by):
+// columns 512 bx .. + 511 (two per thread), `slab` rows from by * slab; rowmax and colmax are
+// zeroed by the caller.  Bound by the one read of X.
+constexpr int kAbsCols = 512;
+constexpr int kAbsMaxSlab = 256;
+__global__ void __launch_bounds__(256) absmax_kernel(const double* __restrict__ X, int64_t rows, int64_t cols,
+                                                     int64_t ld, int slab, unsigned* rowmax, unsigned* colmax) {
+  __shared__ unsigned rm[kAbsMaxSlab][8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t c = (int64_t)blockIdx.x * kAbsCols + 2 * threadIdx.x;
+  const int64_t r0 = (int64_t)blockIdx.y * slab;
+  const int nr = (int)min((int64_t)slab, rows - r0);
+  const bool vec = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0 && c + 1 < cols;
+  unsigned m0 = 0u, m1 = 0u;
+  for (int b = 0; b < nr; b += 8) {
+    unsigned h0[8], h1[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      h0[q] = h1[q] = 0u;
+      if (b + q < nr) {
+        const double* p = X + (r0 + b + q) * ld + c;
+        if (vec) {
+          const double2 v = __ldg(reinterpret_cast<const double2*>(p));
+          h0[q] = (unsigned)__double2hiint(v.x) & 0x7fffffffu;
+          h1[q] = (unsigned)__double2hiint(v.y) & 0x7fffffffu;
+        } else {
+          if (c < cols) h0[q] = (unsigned)__double2hiint(__ldg(p)) & 0x7fffffffu;
+          if (c + 1 < cols) h1[q] = (unsigned)__double2hiint(__ldg(p + 1)) & 0x7fffffffu;
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      m0 = max(m0, h0[q]);
+      m1 = max(m1, h1[q]);
+      if (rowmax) {
+        const unsigned r = __reduce_max_sync(0xffffffffu, max(h0[q], h1[q]));
+        if (lane == 0 && b + q < nr) rm[b + q][warp] = r;
+      }
+    }
+  }
+  if (colmax) {
+    if (c < cols && m0) atomicMax(colmax + c, m0);
+    if (c + 1 < cols && m1) atomicMax(colmax + c + 1, m1);
+  }
+  if (rowmax) {
+    __syncthreads();
+    for (int r = threadIdx.x; r < nr; r += 256) {
+      unsigned v = 0u;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) v = max(v, rm[r][w]);
+      if (v) atomicMax(rowmax + r0 + r, v);
+    }
+  }
+}
+
+// C (column-major, ldc) = diag(D) sum_z part[z] (column-major, ld M), increasing z.
+__global__ void emu_sum_kernel(const double* __restrict__ part, int nz, int64_t M, int64_t len,
+                               const double* __restrict__ D, double* __restrict__ C, int64_t ldc) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x) {
+    double s = 0.0;
+    for (int z0 = 0; z0 < nz; z0 += 8) {
+      double v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = z0 + q < nz ? part[(z0 + q) * len + i] : 0.0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (z0 + q < nz) s += v[q];
+    }
+    const int64_t n = i / M, m = i - n * M;
+    C[m + n * ldc] = D ? D[m] * s : s;
+  }
+}
+
+// Split of K: the slice count (at most 64, each of at least E_MINSTEPS stages) whose CTAs take
+// the fewest stages in all, counting three stages for a CTA's read-out and start-up.  For 152
+// SMs whatever the device, so that the summation order does not depend on it.
+int emu_slices(int64_t tiles, int64_t steps) {
+  int best = 1;
+  int64_t best_cost = INT64_MAX;
+  for (int z = 1; z <= 64; ++z) {
+    if (z > 1 && steps / z < E_MINSTEPS) break;
+    const int64_t waves = (tiles * z + 151) / 152;
+    const int64_t cost = waves * ((steps + z - 1) / z + 3);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = z;
+    }
+  }
+  return best;
+}
+struct EmuPlan {
+  int64_t mt, steps, kslice;
+  int ntl, nz;
+};
+EmuPlan emu_plan(int64_t M, int N, int64_t K) {
+  EmuPlan p;
+  p.mt = (M + EM - 1) / EM;
+  p.ntl = (N + EN - 1) / EN;
+  p.steps = std::max<int64_t>(1, (K + EK - 1) / EK);
+  const int z = emu_slices(p.mt * p.ntl, p.steps);
+  const int64_t per = (p.steps + z - 1) / z;
+  p.kslice = per * EK;
+  p.nz = (int)((p.steps + per - 1) / per);
+  return p;
+}
+
+}  // namespace
+
+cudaError_t absmax_f64(const double* X, int64_t rows, int64_t cols, int64_t ld, unsigned* rowmax, unsigned* colmax,
+                       cudaStream_t st) {
+  if (rowmax) NYS_CUDA_TRY(cudaMemsetAsync(rowmax, 0, rows * sizeof(unsigned), st));
+  if (colmax) NYS_CUDA_TRY(cudaMemsetAsync(colmax, 0, cols * sizeof(unsigned), st));
+  // slabs of 8 .. 256 rows, a multiple of 8: at least ~600 blocks where the matrix allows
+  const int64_t cb = (cols + kAbsCols - 1) / kAbsCols;
+  int64_t slab = (rows * cb + 607) / 608;
+  slab = std::min<int64_t>(kAbsMaxSlab, std::max<int64_t>(8, (slab + 7) / 8 * 8));
+  while ((rows + slab - 1) / slab > 65535 && slab < kAbsMaxSlab) slab += 8;
+  for (int64_t r0 = 0; r0 < rows; r0 += 65535 * slab) {
+    const int64_t nr = std::min<int64_t>(65535 * slab, rows - r0);
+    count_launch();
+    absmax_kernel<<<dim3((unsigned)cb, (unsigned)((nr + slab - 1) / slab)), 256, 0, st>>>(
+        X + r0 * ld, nr, cols, ld, (int)slab, rowmax ? rowmax + r0 : nullptr, colmax);
+    NYS_CUDA_TRY(cudaGetLastError());
+  }
+  return cudaSuccess;
+}
+
+size_t gemm64_work_bytes(int64_t M, int N, int64_t K) {
+  const EmuPlan p = emu_plan(M, N, K);
+  return p.nz > 1 ? (size_t)p.nz * M * N * sizeof(double) : 0;
+}
+
+cudaError_t gemm64(const double* A, bool k_contiguous, int64_t lda, const unsigned* ea, int64_t M, const double* B,
+                   int64_t ldb, const unsigned* eb, int N, int64_t K, const double* D, double* C, int64_t ldc,
+                   void* work, int* status, cudaStream_t st) {
+  if (M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
+  const EmuPlan p = emu_plan(M, N, K);
+  if (p.ntl > INT32_MAX) return cudaErrorInvalidValue;
+  EmuArgs a;
+  a.A = A;
+  a.lda = lda;
+  a.B = B;
+  a.ldb = ldb;
+  a.K = K;
+  a.kslice = p.kslice;
+  a.N = N;
+  a.eb = eb;
+  a.status = status;
+  a.D = p.nz == 1 ? D : nullptr;
+  a.ldc = p.nz == 1 ? ldc : M;
+  a.cslice = M * (int64_t)N;
+  const void* fn = k_contiguous ? (const void*)gemm64_tc_kernel<true> : (const void*)gemm64_tc_kernel<false>;
+  NYS_CUDA_TRY(ensure_max_dyn_smem(fn, 2 * E_STAGE));
+  // row tiles in launches of at most 65,535
+  for (int64_t t0 = 0; t0 < p.mt; t0 += 65535) {
+    const int64_t nt = std::min<int64_t>(65535, p.mt - t0), m0 = t0 * EM;
+    a.A = A + (k_contiguous ? m0 * lda : m0);
+    a.ea = ea + m0;
+    a.M = std::min<int64_t>(M - m0, nt * EM);
+    a.C = (p.nz == 1 ? C : reinterpret_cast<double*>(work)) + m0;
+    a.D = p.nz == 1 && D ? D + m0 : nullptr;
+    const dim3 grid((unsigned)p.ntl, (unsigned)nt, (unsigned)p.nz);
+    count_launch();
+    if (k_contiguous) gemm64_tc_kernel<true><<<grid, ET, 2 * E_STAGE, st>>>(a);
+    else gemm64_tc_kernel<false><<<grid, ET, 2 * E_STAGE, st>>>(a);
+    NYS_CUDA_TRY(cudaGetLastError());
+  }
+  if (p.nz > 1) {
+    const int64_t len = M * (int64_t)N;
+    count_launch();
+    emu_sum_kernel<<<(unsigned)std::min<int64_t>(4096, (len + 127) / 128), 128, 0, st>>>(
+        reinterpret_cast<const double*>(work), p.nz, M, len, D, C, ldc);
+    NYS_CUDA_TRY(cudaGetLastError());
+  }
+  return cudaSuccess;
+}
+
+}  // namespace nys
+
+namespace nys {
+
+// ------------------------------------------------------------------ Y = A^T diag(D) A X
+namespace {
+struct HmmShape {
+  size_t row, col, ex, ew, w, status, total;   // byte offsets in the scratch; the products' work last
+};
+HmmShape hmm_shape(const nys_matrix* A, int m) {
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  HmmShape h;
+  h.row = 0;
+  h.col = h.row + up((size_t)A->n * sizeof(unsigned));
+  h.ex = h.col + up((size_t)A->d * sizeof(unsigned));
+  h.ew = h.ex + up((size_t)m * sizeof(unsigned));
+  h.status = h.ew + up((size_t)m * sizeof(unsigned));
+  h.w = h.status + 256;
+  h.total = h.w + up((size_t)A->n * m * sizeof(double)) +
+            std::max(gemm64_work_bytes(A->n, m, A->d), gemm64_work_bytes(A->d, m, A->n));
+  return h;
+}
+}  // namespace
+
+size_t hmm64_bytes(const nys_matrix* A, int m) { return hmm_shape(A, m).total; }
+
+cudaError_t hmm64_prepare(const nys_matrix* A, int m, void* scratch, cudaStream_t st) {
+  const HmmShape h = hmm_shape(A, m);
+  unsigned char* b = reinterpret_cast<unsigned char*>(scratch);
+  NYS_CUDA_TRY(cudaMemsetAsync(b + h.status, 0, sizeof(int), st));
+  return absmax_f64(reinterpret_cast<const double*>(A->data), A->n, A->d, A->ld, reinterpret_cast<unsigned*>(b + h.row),
+                    reinterpret_cast<unsigned*>(b + h.col), st);
+}
+
+int* hmm64_status(const nys_matrix* A, int m, void* scratch) {
+  return reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(scratch) + hmm_shape(A, m).status);
+}
+
+cudaError_t hmm64(const nys_matrix* A, const double* D, const double* X, int m, double* Y, void* scratch,
+                  cudaStream_t st) {
+  const HmmShape h = hmm_shape(A, m);
+  unsigned char* b = reinterpret_cast<unsigned char*>(scratch);
+  const double* Ad = reinterpret_cast<const double*>(A->data);
+  unsigned* row = reinterpret_cast<unsigned*>(b + h.row);
+  unsigned* col = reinterpret_cast<unsigned*>(b + h.col);
+  unsigned* ex = reinterpret_cast<unsigned*>(b + h.ex);
+  unsigned* ew = reinterpret_cast<unsigned*>(b + h.ew);
+  double* W = reinterpret_cast<double*>(b + h.w);
+  int* status = reinterpret_cast<int*>(b + h.status);
+  void* work = b + h.w + ((size_t)A->n * m * sizeof(double) + 255) / 256 * 256;
+  const int64_t n = A->n, d = A->d;
+  NYS_CUDA_TRY(absmax_f64(X, m, d, d, ex, nullptr, st));
+  NYS_CUDA_TRY(gemm64(Ad, true, A->ld, row, n, X, d, ex, m, d, D, W, n, work, status, st));
+  NYS_CUDA_TRY(absmax_f64(W, m, n, n, ew, nullptr, st));
+  return gemm64(Ad, false, A->ld, col, d, W, n, ew, m, n, nullptr, Y, d, work, status, st);
+}
+
+}  // namespace nys

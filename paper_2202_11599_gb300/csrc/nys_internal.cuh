@@ -85,8 +85,27 @@ cudaError_t apass_reduce(const ApassArgs& a, const ApassPlan& plan, const void* 
 int reduce_blocks(int64_t d);
 
 // ---------------------------------------------------------------- small dense FP64 kernels
+// FP64 products on the tensor cores (gemm64_tc.cu).  absmax_f64: per row and / or column of the
+// row-major rows x cols matrix X, the top word of its largest magnitude.
+cudaError_t absmax_f64(const double* X, int64_t rows, int64_t cols, int64_t ld, unsigned* rowmax, unsigned* colmax,
+                       cudaStream_t st);
+// C (M x N, column-major, ldc) = diag(D) A B^T with A(m, k) = A[m lda + k] (k_contiguous) or
+// A[k lda + m], B(n, k) = B[n ldb + k]; ea / eb: absmax of A over k for each m, of B for each n.
+// D (length M) may be NULL.  *status (device, caller-zeroed): NYS_ETIMEOUT when a bounded wait ran
+// out (the outputs are then NaN).
+size_t gemm64_work_bytes(int64_t M, int N, int64_t K);
+cudaError_t gemm64(const double* A, bool k_contiguous, int64_t lda, const unsigned* ea, int64_t M, const double* B,
+                   int64_t ldb, const unsigned* eb, int N, int64_t K, const double* D, double* C, int64_t ldc,
+                   void* work, int* status, cudaStream_t st);
+// Y (d x m, column-major) = A^T diag(D) A X for an FP64 matrix; scratch of hmm64_bytes, prepared
+// once per matrix and m (the exponents of A; zeroes the status word).
+size_t hmm64_bytes(const nys_matrix* A, int m);
+cudaError_t hmm64_prepare(const nys_matrix* A, int m, void* scratch, cudaStream_t st);
+int* hmm64_status(const nys_matrix* A, int m, void* scratch);
+cudaError_t hmm64(const nys_matrix* A, const double* D, const double* X, int m, double* Y, void* scratch,
+                  cudaStream_t st);
 // C (s x s, col-major, ldc = s) = X^T Y for X, Y d x s col-major FP64 (ld = d); deterministic.
-cudaError_t gram_xty(const double* X, const double* Y, int64_t d, int s, double* C, double* work,
+cudaError_t gram_xty(const double* X, const double* Y, int64_t d, int s, double* C, double* work, int* status,
                      cudaStream_t st);
 size_t gram_work_bytes(int64_t d, int s);
 // In-place upper Cholesky of a symmetric s x s matrix (col-major): C^T C = M. info[0] = 0 ok,
@@ -108,9 +127,11 @@ size_t jacobi_work_bytes(int s);
 cudaError_t identity_gap(const double* G, int m, double* out, cudaStream_t st);
 // After Jacobi: sort eigenpairs descending, U = B V Sigma^{-1}, lam = max(0, sigma^2 - nu).
 cudaError_t nystrom_finish(const double* B, int64_t d, int s, const double* G, const double* V,
-                           double nu, double* U, double* lam, double* work, cudaStream_t st);
+                           double nu, double* U, double* lam, double* work, int* status, cudaStream_t st);
+size_t finish_work_bytes(int64_t d, int s);
 
 // ---------------------------------------------------------------- sketch GEMMs
+// FP32 and BF16 storage, CUDA cores (FP64: hmm64).
 // W (n x s, col-major, ld n) = diag(D) (A Omega) with Omega d x s col-major (ld d) in compute type
 cudaError_t sketch_aw(const nys_matrix* A, const void* Omega, int s, const double* D, void* W,
                       cudaStream_t st);

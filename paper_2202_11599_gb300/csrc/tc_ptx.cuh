@@ -1,5 +1,5 @@
 // PTX wrappers of the 5th-generation tensor core shared by the tensor-core kernels
-// (sketch_tc.cu): TMEM allocation, tcgen05.mma / commit / ld, fences, and the
+// (sketch_tc.cu, gemm64_tc.cu): TMEM allocation, tcgen05.mma / commit / ld, fences, and the
 // shared-memory and instruction descriptors.
 #pragma once
 #include "device_util.cuh"
