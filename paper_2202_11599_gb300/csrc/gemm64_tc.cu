@@ -45,7 +45,7 @@ constexpr int ESL = 8;                        // digits per operand = orders kep
 constexpr int EFLUSH = 8;                     // stages between read-outs (256 K)
 constexpr uint32_t EA_SLICE = EM * EK * 2, EB_SLICE = EN * EK * 2;
 constexpr uint32_t E_STAGE = ESL * (EA_SLICE + EB_SLICE);   // 96 KB
-constexpr int E_MINSTEPS = 4;                 // K steps a split slice has at least
+constexpr int E_MINSTEPS = 2;                 // K steps a split slice has at least
 
 struct EmuArgs {
   const double* A;
@@ -70,7 +70,7 @@ __device__ __forceinline__ uint64_t digits(double x, int emax) {
   const uint32_t mh = (h & 0xfffffu) | (e ? 0x100000u : 0u);
   const uint64_t m = (((uint64_t)mh << 32) | l) << 9;
   const int sh = emax - max(e, 1);
-  uint64_t q = sh < 64 ? m >> sh : 0ull;
+  uint64_t q = (unsigned)sh < 64u ? m >> sh : 0ull;
   if ((int)h < 0) q = 0ull - q;
   return q + 0x8080808080808080ull;
 }

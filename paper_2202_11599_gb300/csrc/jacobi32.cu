@@ -1,0 +1,423 @@
+// FP32 start of the symmetric eigensolve of the Nystrom core: an orthogonal V0 that makes
+// V0^T G V0 diagonal to FP32 accuracy, from which the FP64 Jacobi sweeps (core.cu) need one or two
+// sweeps instead of six to eleven.
+//
+// A round of the FP64 sweeps costs ~4.3 us whatever the size (grid barrier, L2 loads, the FP64
+// square root of the rotation), so a 200 x 200 eigensolve took 9 x 199 of them, 8.1 ms.  Here
+// everything stays on chip in FP32: L L^T = G + eps I (one CTA, packed in shared memory), then
+// one-sided Jacobi (Hestenes) on the columns of L in one thread-block cluster, one warp per pair
+// of columns, the columns in registers.  A round is three dot products, a rotation and the
+// systolic exchange of the round-robin order (each warp passes one column to each neighbour
+// through the neighbour's shared memory, across CTAs through distributed shared memory), with one
+// cluster barrier.  The left singular vectors of L -- the normalised columns at the end -- are the
+// eigenvectors of G, so no V is carried, and starting from the Cholesky factor saves a third of
+// the sweeps (Drmac and Veselic, SIAM J. Matrix Anal. Appl. 29, 2008).  eps = 1e-3 trace(G)
+// leaves the eigenvectors as they are and keeps the small columns above FP32 rounding.
+// V0 is then orthonormalised in FP64 (three Newton-Schulz steps: the columns leave the FP32
+// stage orthogonal to 1e-6 .. 3e-4 over spectra from flat to (1 + j)^-4) and checked on the
+// device: if V0^T V0 is off the identity by more than 1e-13 the sweeps start from the identity
+// instead, as they do without this stage.  The accuracy of the result is that of the sweeps.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+#include "device_util.cuh"
+#include "nys_internal.cuh"
+
+namespace nys {
+namespace {
+namespace cg = cooperative_groups;
+
+constexpr float kJacRidge = 1e-3f;   // eps / trace(G)
+constexpr float kJacSkip = 1e-8f;    // entries of L^T L (largest diagonal of G: 1) below rounding
+constexpr float kJacAgain = 1e-5f;   // a sweep that met none above this was the last (quadratic)
+
+// L (N x N FP32, column-major, lower) with L L^T = 2^-ex (G + eps I), G symmetrised, 2^ex the
+// scale of its largest diagonal entry; zero when that is zero or not finite.  Rows and columns
+// from s on are those of the identity times sqrt(eps).  Right-looking, packed by columns.
+__global__ void __launch_bounds__(1024) chol32_kernel(const double* __restrict__ G, int s, int N, float* __restrict__ L) {
+  extern __shared__ float lo[];
+  __shared__ double smx[32], str[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  auto at = [N](int i, int c) { return c * N - c * (c - 1) / 2 + (i - c); };
+  double mx = 0.0, tr = 0.0;
+  for (int i = tid; i < s; i += blockDim.x) {
+    const double g = G[i + (int64_t)i * s];
+    tr += g;
+    mx = fabs(g) > mx || g != g ? fabs(g) : mx;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double m2 = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = m2 > mx || m2 != m2 ? m2 : mx;
+    tr += __shfl_xor_sync(0xffffffffu, tr, o);
+  }
+  if (lane == 0) {
+    smx[warp] = mx;
+    str[warp] = tr;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    mx = tr = 0.0;
+    for (int w = 0; w < nw; ++w) {
+      mx = smx[w] > mx || smx[w] != smx[w] ? smx[w] : mx;
+      tr += str[w];
+    }
+    smx[0] = mx;
+    str[0] = tr;
+  }
+  __syncthreads();
+  mx = smx[0];
+  tr = str[0];
+  const bool plain = mx > 0.0 && isfinite(mx) && isfinite(tr);
+  int ex = 0;
+  if (plain) frexp(mx, &ex);
+  const float eps = plain ? kJacRidge * (float)scalbn(tr, -ex) : 0.f;
+  for (int c = warp; c < N; c += nw)
+    for (int i = c + lane; i < N; i += 32) {
+      float v = (plain && i < s && c < s)
+                    ? (float)scalbn(0.5 * (G[i + (int64_t)c * s] + G[c + (int64_t)i * s]), -ex) : 0.f;
+      if (i == c) v += eps;
+      lo[at(i, c)] = v;
+    }
+  __syncthreads();
+  for (int j = 0; j < N && plain; ++j) {
+    // pivots stay above eps / 4: G is positive semidefinite up to rounding
+    const float r = rsqrtf(fmaxf(lo[at(j, j)], 0.25f * eps));
+    const float* col = lo + at(j, j) - j;   // col[i] = entry (i, j), not yet scaled
+    for (int c = j + 1 + warp; c < N; c += nw) {
+      const float f = col[c] * r * r;
+      float* dst = lo + at(c, c) - c;
+      for (int i = c + lane; i < N; i += 32) dst[i] = fmaf(-f, col[i], dst[i]);
+    }
+    __syncthreads();
+    for (int i = j + tid; i < N; i += blockDim.x) lo[at(i, j)] *= r;   // nobody reads column j again
+  }
+  __syncthreads();
+  for (int c = warp; c < N; c += nw)
+    for (int i = lane; i < N; i += 32) L[i + (int64_t)c * N] = i >= c && plain ? lo[at(i, c)] : 0.f;
+}
+
+// Warp sums of three values, in every lane: a reduce-scatter over the first two lane bits, one
+// value per lane after that, and a broadcast of each (9 exchanges for 15).
+__device__ __forceinline__ void sum3(float& a, float& b, float& c, int lane) {
+  constexpr unsigned F = 0xffffffffu;
+  const bool h4 = (lane & 16) != 0, h3 = (lane & 8) != 0;
+  // lanes 0-15 go on with (a, b), lanes 16-31 with (c, -)
+  float x = (h4 ? c : a) + __shfl_xor_sync(F, h4 ? a : c, 16);
+  float y = b + __shfl_xor_sync(F, b, 16);
+  // then lanes with bit 3 clear keep x (a or c), the others y (b)
+  float v = (h3 ? y : x) + __shfl_xor_sync(F, h3 ? x : y, 8);
+  v += __shfl_xor_sync(F, v, 4);
+  v += __shfl_xor_sync(F, v, 2);
+  v += __shfl_xor_sync(F, v, 1);
+  a = __shfl_sync(F, v, 0);
+  b = __shfl_sync(F, v, 8);
+  c = __shfl_sync(F, v, 16);
+}
+
+// One-sided Jacobi on the columns of L.  N even; warp m of the cluster holds pair m of H = N / 2;
+// NL elements per lane (32 NL >= N).  Shared memory: [2][warps][2][32 NL] exchange buffers
+// (t, b).  V (N x N FP64 out, column-major): the normalised columns.
+template <int NL>
+__global__ void jacobi32_kernel(const float* __restrict__ L, int N, double* __restrict__ V, int max_sweeps) {
+  extern __shared__ __align__(16) float xbuf[];
+  __shared__ int flag[3];
+  cg::cluster_group cl = cg::this_cluster();
+  const int wpc = blockDim.x >> 5;
+  const int rank = (int)cl.block_rank();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int H = N / 2, m = rank * wpc + warp;
+  const bool on = m < H;
+  constexpr int LEN = 32 * NL;
+  if (threadIdx.x < 3) flag[threadIdx.x] = 0;
+  // pair m starts with columns m and N - 1 - m
+  float t[NL], b[NL];
+#pragma unroll
+  for (int l = 0; l < NL; ++l) {
+    const int i = l * 32 + lane;
+    t[l] = on && i < N ? L[i + (int64_t)m * N] : 0.f;
+    b[l] = on && i < N ? L[i + (int64_t)(N - 1 - m) * N] : 0.f;
+  }
+  // where this warp's columns go after a round: t to pair m + 1's t (pair 0 keeps it; the last
+  // pair's becomes its own b), b to pair m - 1's b (pair 0's becomes pair 1's t)
+  // (the CTA's own buffers by their plain address: only the edge warps write across CTAs)
+  auto slot = [&](int pair, int buf, int part) -> float* {
+    float* base = pair / wpc == rank ? xbuf : cl.map_shared_rank(xbuf, pair / wpc);
+    return base + ((buf * wpc + pair % wpc) * 2 + part) * LEN;
+  };
+  int* flags0 = cl.map_shared_rank(flag, 0);
+  cl.sync();
+  int buf = 0;
+  for (int sweep = 0; sweep < max_sweeps && H > 1; ++sweep) {
+    if (rank == 0 && threadIdx.x == 0) flag[(sweep + 1) % 3] = 0;
+    bool again = false;
+    for (int r = 0; r < N - 1; ++r) {
+      if (on) {
+        float a = 0.f, c2 = 0.f, g = 0.f;
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+          a = fmaf(t[l], t[l], a);
+          c2 = fmaf(b[l], b[l], c2);
+          g = fmaf(t[l], b[l], g);
+        }
+        sum3(a, c2, g, lane);
+        if (fabsf(g) > kJacSkip) {
+          if (fabsf(g) > kJacAgain) again = true;
+          // the smaller root, by h = |b|^2 - |t|^2, r = sqrt(h^2 + 4 g^2): c^2 = (1 + |h| / r) / 2,
+          // s = sign(h g) |g| / (r c): two reciprocal square roots and a reciprocal
+          const float h = c2 - a, g2 = 2.f * g;
+          const float ir = rsqrtf(fmaf(h, h, g2 * g2));
+          const float cc = fmaf(0.5f * fabsf(h), ir, 0.5f);
+          const float ic = rsqrtf(cc);
+          const float sn = 0.5f * ic * ir * (h < 0.f ? -g2 : g2);
+          // Rutishauser's form: the rounding of a rotation shrinks with its angle, so the
+          // columns' lengths do not drift over the two thousand rounds
+          const float tau = __fdividef(sn, fmaf(cc, ic, 1.f));
+#pragma unroll
+          for (int l = 0; l < NL; ++l) {
+            const float x = t[l], y = b[l];
+            t[l] = fmaf(-sn, fmaf(tau, x, y), x);
+            b[l] = fmaf(sn, fmaf(-tau, y, x), y);
+          }
+        }
+        if (m >= 1) {
+          float* d = slot(m - 1, buf, 1);
+#pragma unroll
+          for (int l = 0; l < NL; ++l) d[l * 32 + lane] = b[l];
+        }
+        if (m == 0 || m < H - 1) {
+          float* d = slot(m + 1, buf, 0);
+#pragma unroll
+          for (int l = 0; l < NL; ++l) d[l * 32 + lane] = m == 0 ? b[l] : t[l];
+        }
+      }
+      if (r == N - 2 && again && lane == 0) flags0[sweep % 3] = 1;
+      cl.sync();
+      if (on) {
+        const float* base = xbuf + (size_t)(buf * wpc + warp) * 2 * LEN;
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+          b[l] = m == H - 1 ? t[l] : base[LEN + l * 32 + lane];
+          if (m >= 1) t[l] = base[l * 32 + lane];
+        }
+      }
+      buf ^= 1;
+    }
+    if (*(volatile int*)(flags0 + sweep % 3) == 0) break;
+  }
+  if (on) {
+    float a = 0.f, c2 = 0.f;
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+      a = fmaf(t[l], t[l], a);
+      c2 = fmaf(b[l], b[l], c2);
+    }
+    a = warp_sum(a);
+    c2 = warp_sum(c2);
+    const float ia = a > 0.f ? rsqrtf(a) : 0.f, ib = c2 > 0.f ? rsqrtf(c2) : 0.f;
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+      const int i = l * 32 + lane;
+      if (i < N) {
+        V[i + (int64_t)(2 * m) * N] = (double)(t[l] * ia);
+        V[i + (int64_t)(2 * m + 1) * N] = (double)(b[l] * ib);
+      }
+    }
+  }
+  cl.sync();   // no CTA leaves while another may still read its flag
+}
+
+// S <- 1.5 I - 0.5 S (the factor of the Newton-Schulz step V <- V (1.5 I - 0.5 V^T V))
+__global__ void schulz_kernel(double* __restrict__ S, int N) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)N * N; e += (int64_t)gridDim.x * blockDim.x)
+    S[e] = (e % N == e / N ? 1.5 : 0.0) - 0.5 * S[e];
+}
+// *bad |= any |S - I| > tol (or NaN)
+__global__ void gap_kernel(const double* __restrict__ S, int N, double tol, int* bad) {
+  int b = 0;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)N * N; e += (int64_t)gridDim.x * blockDim.x)
+    b |= !(fabs(S[e] - (e % N == e / N ? 1.0 : 0.0)) <= tol);
+  if (__syncthreads_or(b) && threadIdx.x == 0) atomicOr(bad, 1);
+}
+// A <- (T + T^T) / 2, V <- Vn; when Vn failed its check A stays, and V too (V = I with `reset`).
+// Vn may be V.
+__global__ void accept_kernel(const double* __restrict__ T, int N, const int* __restrict__ bad, int reset,
+                              double* __restrict__ A, const double* Vn, double* V) {
+  const bool no = *bad != 0;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)N * N; e += (int64_t)gridDim.x * blockDim.x) {
+    const int i = (int)(e % N), j = (int)(e / N);
+    if (no) {
+      if (reset) V[e] = i == j ? 1.0 : 0.0;
+    } else {
+      A[e] = 0.5 * (T[i + (int64_t)j * N] + T[j + (int64_t)i * N]);
+      if (Vn != V) V[e] = Vn[e];
+    }
+  }
+}
+__global__ void fill_kernel(unsigned* x, int n, unsigned v) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) x[i] = v;
+}
+
+// E <- E_ij = A_ij / (A_jj - A_ii), antisymmetric, zero where it is not small (a near-degenerate pair)
+__global__ void first_order_kernel(const double* __restrict__ A, int N, double* __restrict__ E) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)N * N; e += (int64_t)gridDim.x * blockDim.x) {
+    const int i = (int)(e % N), j = (int)(e / N);
+    const double h = A[j + (int64_t)j * N] - A[i + (int64_t)i * N];
+    const double g = 0.5 * (A[e] + A[j + (int64_t)i * N]);
+    E[e] = i != j && fabs(g) <= 2e-3 * fabs(h) && h != 0.0 ? g / h : 0.0;
+  }
+}
+// U = I + E + E2 / 2
+__global__ void exp2_kernel(const double* __restrict__ E, const double* __restrict__ E2, int N, double* __restrict__ U) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)N * N; e += (int64_t)gridDim.x * blockDim.x)
+    U[e] = (e % N == e / N ? 1.0 : 0.0) + E[e] + 0.5 * E2[e];
+}
+// Cluster shape: one CTA while its 32 warps hold every pair, else eight CTAs.
+int jac_ctas(int H) { return H <= 32 ? 1 : 8; }
+
+template <int NL>
+cudaError_t launch_jacobi32(const float* L, int N, double* V, cudaStream_t st, bool* ran) {
+  const int H = N / 2, C = jac_ctas(H), wpc = (H + C - 1) / C;
+  const size_t smem = (size_t)2 * wpc * 2 * 32 * NL * sizeof(float);
+  NYS_CUDA_TRY(ensure_max_dyn_smem((const void*)jacobi32_kernel<NL>, 200 * 1024));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)C);
+  cfg.blockDim = dim3((unsigned)(32 * wpc));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n_clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&n_clusters, jacobi32_kernel<NL>, &cfg) != cudaSuccess || n_clusters < 1) {
+    (void)cudaGetLastError();
+    *ran = false;   // the cluster does not fit this device: the FP64 sweeps start from the identity
+    return cudaSuccess;
+  }
+  count_launch();
+  *ran = true;
+  return cudaLaunchKernelEx(&cfg, jacobi32_kernel<NL>, L, N, V, 12);
+}
+
+size_t up256(size_t b) { return (b + 255) / 256 * 256; }
+
+}  // namespace
+
+// Ranks the start covers: the packed factor of 320 columns takes 205 KB of shared memory.
+bool jacobi_start_supported(int s) { return s >= 8 && s <= 320; }
+
+// Scratch of the start and of the correction: two N x N matrices, exponents, the products' own.
+namespace {
+struct StartWork {
+  double *S, *P;
+  unsigned *e1, *eg, *et;   // exponents: of entries below 4, of G's rows, of a product's columns
+  int* bad;
+  void* gw;
+  StartWork(void* work, int N) {
+    unsigned char* b = reinterpret_cast<unsigned char*>(work);
+    const size_t m = up256((size_t)N * N * sizeof(double));
+    S = reinterpret_cast<double*>(b);
+    P = reinterpret_cast<double*>(b + m);
+    e1 = reinterpret_cast<unsigned*>(b + 2 * m);
+    eg = e1 + N;
+    et = eg + N;
+    bad = reinterpret_cast<int*>(et + N);
+    gw = b + 2 * m + up256(3 * (size_t)N * sizeof(unsigned) + sizeof(int));
+  }
+};
+}  // namespace
+
+size_t jacobi_start_work_bytes(int s) {
+  const size_t N = s + (s & 1);
+  return 2 * up256(N * N * sizeof(double)) + up256(3 * N * sizeof(unsigned) + sizeof(int)) +
+         gemm64_work_bytes(N, (int)N, N);
+}
+
+cudaError_t jacobi_start(const double* G, int s, double* A, double* V, void* work, int* status, cudaStream_t st,
+                         bool* ran) {
+  const int N = s + (s & 1);
+  const int64_t nn = (int64_t)N * N;
+  const StartWork w(work, N);
+  float* L = reinterpret_cast<float*>(w.S);
+  const size_t tri = (size_t)N * (N + 1) / 2 * sizeof(float);
+  NYS_CUDA_TRY(ensure_max_dyn_smem((const void*)chol32_kernel, 206 * 1024));
+  count_launch();
+  chol32_kernel<<<1, 1024, tri, st>>>(G, s, N, L);
+  NYS_CUDA_TRY(cudaGetLastError());
+  // three orthonormalisation steps alternate between P and V, so V0 goes to P
+  if (N <= 64) NYS_CUDA_TRY(launch_jacobi32<2>(L, N, w.P, st, ran));
+  else if (N <= 128) NYS_CUDA_TRY(launch_jacobi32<4>(L, N, w.P, st, ran));
+  else if (N <= 224) NYS_CUDA_TRY(launch_jacobi32<7>(L, N, w.P, st, ran));
+  else NYS_CUDA_TRY(launch_jacobi32<10>(L, N, w.P, st, ran));
+  if (!*ran) return cudaSuccess;
+  const unsigned grid = (unsigned)std::min<int64_t>(1024, (nn + 255) / 256);
+  count_launch();
+  fill_kernel<<<(N + 127) / 128, 128, 0, st>>>(w.e1, N, 0x40000000u);
+  NYS_CUDA_TRY(cudaMemsetAsync(w.bad, 0, sizeof(int), st));
+  // Z = op(X) Y (columns of Y are K-contiguous); ex, ey: exponents of X's rows, of Y's columns
+  auto mul = [&](const double* X, bool kc, const unsigned* ex, const double* Y, const unsigned* ey, double* Z) {
+    return gemm64(X, kc, N, ex, N, Y, N, ey, N, N, nullptr, Z, N, w.gw, status, st);
+  };
+  double *cur = w.P, *nxt = V;
+  for (int k = 0; k < 3; ++k) {
+    NYS_CUDA_TRY(mul(cur, true, w.e1, cur, w.e1, w.S));
+    count_launch();
+    schulz_kernel<<<grid, 256, 0, st>>>(w.S, N);
+    NYS_CUDA_TRY(cudaGetLastError());
+    NYS_CUDA_TRY(mul(cur, false, w.e1, w.S, w.e1, nxt));
+    std::swap(cur, nxt);
+  }
+  NYS_CUDA_TRY(mul(V, true, w.e1, V, w.e1, w.S));
+  count_launch();
+  gap_kernel<<<grid, 256, 0, st>>>(w.S, N, 1e-13, w.bad);
+  NYS_CUDA_TRY(cudaGetLastError());
+  // A <- V^T A V
+  NYS_CUDA_TRY(absmax_f64(A, N, N, N, w.eg, nullptr, st));
+  NYS_CUDA_TRY(mul(A, true, w.eg, V, w.e1, w.S));
+  NYS_CUDA_TRY(absmax_f64(w.S, N, N, N, w.et, nullptr, st));
+  NYS_CUDA_TRY(mul(V, true, w.e1, w.S, w.et, w.P));
+  count_launch();
+  accept_kernel<<<grid, 256, 0, st>>>(w.P, N, w.bad, 1, A, V, V);
+  return cudaGetLastError();
+}
+
+cudaError_t jacobi_polish(const double* G, int N, double* A, double* T, double* V, void* work, int* status,
+                          cudaStream_t st) {
+  const int64_t nn = (int64_t)N * N;
+  const StartWork w(work, N);   // e1 and eg as jacobi_start left them
+  const unsigned grid = (unsigned)std::min<int64_t>(1024, (nn + 255) / 256);
+  auto mul = [&](const double* X, bool kc, const unsigned* ex, const double* Y, const unsigned* ey, double* Z) {
+    return gemm64(X, kc, N, ex, N, Y, N, ey, N, N, nullptr, Z, N, w.gw, status, st);
+  };
+  // exp(E) to second order, its departure from orthogonality (E^4 / 4) squared away by one
+  // Newton-Schulz step; checked like the start's V, and left out when it fails
+  NYS_CUDA_TRY(cudaMemsetAsync(w.bad, 0, sizeof(int), st));
+  count_launch();
+  first_order_kernel<<<grid, 256, 0, st>>>(A, N, w.S);
+  NYS_CUDA_TRY(mul(w.S, false, w.e1, w.S, w.e1, w.P));
+  count_launch();
+  exp2_kernel<<<grid, 256, 0, st>>>(w.S, w.P, N, w.S);
+  NYS_CUDA_TRY(mul(V, false, w.e1, w.S, w.e1, w.P));
+  NYS_CUDA_TRY(mul(w.P, true, w.e1, w.P, w.e1, w.S));
+  count_launch();
+  schulz_kernel<<<grid, 256, 0, st>>>(w.S, N);
+  NYS_CUDA_TRY(cudaGetLastError());
+  NYS_CUDA_TRY(mul(w.P, false, w.e1, w.S, w.e1, T));
+  NYS_CUDA_TRY(mul(T, true, w.e1, T, w.e1, w.S));
+  count_launch();
+  gap_kernel<<<grid, 256, 0, st>>>(w.S, N, 1e-13, w.bad);
+  NYS_CUDA_TRY(cudaGetLastError());
+  NYS_CUDA_TRY(mul(G, true, w.eg, T, w.e1, w.S));
+  NYS_CUDA_TRY(absmax_f64(w.S, N, N, N, w.et, nullptr, st));
+  NYS_CUDA_TRY(mul(T, true, w.e1, w.S, w.et, w.P));
+  count_launch();
+  accept_kernel<<<grid, 256, 0, st>>>(w.P, N, w.bad, 0, A, T, V);
+  return cudaGetLastError();
+}
+
+}  // namespace nys

@@ -118,10 +118,23 @@ cudaError_t trsm_right_upper(const double* C, int s, double* Y, int64_t d, cudaS
 cudaError_t axpy_panel(double nu, const double* X, double* Y, int64_t n, cudaStream_t st);
 // lambda_max of a symmetric s x s matrix by power iteration (device scalar out)
 cudaError_t power_lambda_max(const double* G, int s, double* out, double* work, cudaStream_t st);
-// Symmetric eigendecomposition by parallel cyclic Jacobi: G (s x s, overwritten) -> V (s x s),
-// eigenvalues in the diagonal.  Sweeps stop once off(A) <= tol ||A||_F.  Returns sweeps used
-// in *sweeps (host).
-cudaError_t jacobi_eig(double* G, double* V, int s, double* work, int* sweeps, cudaStream_t st, double tol = 1e-12);
+// Symmetric eigendecomposition by parallel cyclic Jacobi: G (s x s, overwritten) -> V (N x N),
+// eigenvalues in the diagonal of the first N x N of work.  Sweeps stop once off(A) <= tol ||A||_F.
+// Returns the FP64 sweeps used in *sweeps (host); *status as for gemm64.
+cudaError_t jacobi_eig(double* G, double* V, int s, double* work, int* sweeps, int* status, cudaStream_t st,
+                       double tol = 1e-12);
+// FP32 start of the sweeps (jacobi32.cu): V = an orthogonal matrix that makes V^T G V diagonal to
+// FP32 accuracy and A <- V^T A V, for A = the zero-padded symmetrised G.  *ran = false: nothing
+// was changed; a V that fails its orthogonality check on the device leaves V = I and A alone.
+bool jacobi_start_supported(int s);
+size_t jacobi_start_work_bytes(int s);
+cudaError_t jacobi_start(const double* G, int s, double* A, double* V, void* work, int* status, cudaStream_t st,
+                         bool* ran);
+// First-order correction of a nearly diagonal A = V^T G V: V <- V exp(E) with E_ij = A_ij / (A_jj -
+// A_ii) where that is below 2e-3, A <- V^T G V; nothing changes when the new V fails its
+// orthogonality check.  G: N x N symmetric; T: N x N scratch; work of jacobi_start.
+cudaError_t jacobi_polish(const double* G, int N, double* A, double* T, double* V, void* work, int* status,
+                          cudaStream_t st);
 size_t jacobi_work_bytes(int s);
 // *out (device) = max_ij |G_ij - delta_ij| of the m x m matrix G.
 cudaError_t identity_gap(const double* G, int m, double* out, cudaStream_t st);
