@@ -6,8 +6,8 @@
 // sides A^T b (lasso) and A^T (w t + b01 - sigma(t)) (logistic, Sec. 3.2) and the
 // residual A^T (A x - b) for the objective / KKT measures (Eq. 2, Eq. 31).
 //
-// GB300 design (one CTA of 512 threads per SM, persistent over a contiguous
-// slab of rows):
+// GB300 design of the float kernel (one CTA of 512 threads per SM, persistent over a
+// contiguous slab of rows):
 //   * rows are streamed HBM -> shared memory by 1-D TMA bulk copies
 //     (cp.async.bulk + mbarrier transaction counts), S stages of R rows each,
 //     S-1 stages in flight while the CTA computes on the current one;
@@ -30,206 +30,7 @@
 
 namespace nys {
 
-template <int DT, int VPT>
-__global__ void __launch_bounds__(kApassThreads, 1) apass_kernel(const ApassKArgs a) {
-  using C = typename Stor<DT>::C;
-  constexpr int VEC = Stor<DT>::VEC;
-  constexpr int ESZ = Stor<DT>::ESZ;
-  constexpr int T = kApassThreads;
-  constexpr int NW = T / 32;
-
-  extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ __align__(8) uint64_t bars[kMaxStages];
-  __shared__ C red[2][NW][kRMax];
-
-  if (a.skip && *a.skip) return;
-  if (a.executed && blockIdx.x == 0 && threadIdx.x == 0) *a.executed = 1;
-  const int ts_slot = timer_begin(a);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t nvec = (a.d + VEC - 1) / VEC;
-  const int64_t rowbytes = a.ld * ESZ;
-  const int R = a.R, S = a.S;
-  const int64_t stage_bytes = (int64_t)R * rowbytes;
-  const int64_t r0 = a.n * (int64_t)blockIdx.x / gridDim.x;
-  const int64_t r1 = a.n * (int64_t)(blockIdx.x + 1) / gridDim.x;
-  const int nsteps = (int)((r1 - r0 + R - 1) / R);
-  const int64_t tail_vec = a.d / VEC;           // vector holding the ragged end (if any)
-  const int tail_n = (int)(a.d % VEC);          // valid elements in it
-
-  const C* p = reinterpret_cast<const C*>(a.p);
-  C pr[VPT][VEC];
-  C acc[VPT][VEC];
-#pragma unroll
-  for (int k = 0; k < VPT; ++k) {
-    const int64_t v = tid + (int64_t)k * T;
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) {
-      const int64_t j = v * VEC + e;
-      pr[k][e] = (a.mode != MODE_CONST && v < nvec && j < a.d) ? p[j] : C(0);
-      acc[k][e] = C(0);
-    }
-  }
-
-  if (tid == 0) {
-    for (int s = 0; s < S; ++s) mbar_init(&bars[s], 1);
-    fence_mbar_init();
-  }
-  __syncthreads();
-
-  const uint64_t pol = l2_evict_first_policy();  // A is streamed once per pass
-  auto issue = [&](int step) {
-    const int stage = step % S;
-    const int64_t row = r0 + (int64_t)step * R;
-    const int rows = (int)min((int64_t)R, r1 - row);
-    const uint32_t bytes = (uint32_t)(rows * rowbytes);
-    mbar_arrive_expect_tx(&bars[stage], bytes);
-    tma_load_1d_hint(smem + stage * stage_bytes, a.A + row * rowbytes, bytes, &bars[stage], pol);
-  };
-  int issued = 0;
-  if (tid == 0) {
-    for (int st = 0; st < S && st < nsteps; ++st) issue(st);
-    issued = min(S, nsteps);
-  }
-
-  double loss = 0.0;
-  bool aborted = false;
-  int k = 0;
-  for (; k < nsteps; ++k) {
-    const int stage = k % S;
-    const unsigned char* sb = smem + stage * stage_bytes;
-    const int64_t row0 = r0 + (int64_t)k * R;
-    const int rows_here = (int)min((int64_t)R, r1 - row0);
-    const bool ok = mbar_wait_bounded(&bars[stage], (uint32_t)((k / S) & 1));
-
-    C dot[kRMax];
-#pragma unroll
-    for (int r = 0; r < kRMax; ++r) dot[r] = C(0);
-    if (ok && a.mode != MODE_CONST) {
-#pragma unroll
-      for (int r = 0; r < kRMax; ++r) {
-        if (r < rows_here) {
-#pragma unroll
-          for (int kk = 0; kk < VPT; ++kk) {
-            const int64_t v = tid + (int64_t)kk * T;
-            if (v < nvec) {
-              const uint4 raw = *reinterpret_cast<const uint4*>(sb + r * rowbytes + v * 16);
-              C val[VEC];
-              unpack16<DT>(raw, val);
-              if (v == tail_vec) {
-#pragma unroll
-                for (int e = 0; e < VEC; ++e)
-                  if (e >= tail_n) val[e] = C(0);
-              }
-#pragma unroll
-              for (int e = 0; e < VEC; ++e) dot[r] = fma(val[e], pr[kk][e], dot[r]);
-            }
-          }
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < kRMax; ++r) {
-        const C s = warp_sum(dot[r]);
-        if (lane == 0) red[k & 1][warp][r] = s;
-      }
-    }
-    if (__syncthreads_or(!ok)) {
-      aborted = true;
-      break;
-    }
-    // Stage (k-1) % S has been fully consumed by every thread: refill it.
-    if (tid == 0 && k >= 1 && (k - 1 + S) < nsteps) {
-      issue(k - 1 + S);
-      ++issued;
-    }
-    C u[kRMax];
-#pragma unroll
-    for (int r = 0; r < kRMax; ++r) {
-      u[r] = C(0);
-      if (r < rows_here) {
-        const int64_t i = row0 + r;
-        if (a.mode == MODE_CONST) {
-          u[r] = (C)a.b[i];
-        } else {
-          C t = C(0);
-#pragma unroll
-          for (int w = 0; w < NW; ++w) t += red[k & 1][w][r];
-          if (a.mode == MODE_ID) {
-            u[r] = t;
-          } else if (a.mode == MODE_DIAG) {
-            u[r] = (C)(a.D[i] * (double)t);
-          } else if (a.mode == MODE_RESID) {
-            const double rr = (double)t - a.b[i];
-            u[r] = (C)rr;
-            if (tid == 0) loss += 0.5 * rr * rr;
-          } else if (a.mode == MODE_LGRAD) {
-            const double td = (double)t;
-            const double e = exp(-fabs(td));
-            const double sg = sigmoid_of(td, e);
-            const double b01 = 0.5 * (1.0 + a.b[i]);
-            u[r] = (C)(sg - b01);
-            if (tid == 0 && a.loss_part) loss += fmax(td, 0.0) + log1p(e) - b01 * td;
-          } else {  // MODE_LOGIT
-            const double td = (double)t;
-            const double e = exp(-fabs(td));
-            const double sg = sigmoid_of(td, e);
-            const double wv = sg * (1.0 - sg);
-            const double b01 = 0.5 * (1.0 + a.b[i]);
-            u[r] = (C)(wv * td + b01 - sg);
-            if (tid == 0) {
-              if (a.D_out) a.D_out[i] = wv;
-              if (a.loss_part) loss += fmax(td, 0.0) + log1p(e) - b01 * td;
-            }
-          }
-          if (tid == 0 && a.t_out) a.t_out[i] = (double)t;
-        }
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < kRMax; ++r) {
-      if (r < rows_here) {
-#pragma unroll
-        for (int kk = 0; kk < VPT; ++kk) {
-          const int64_t v = tid + (int64_t)kk * T;
-          if (v < nvec) {
-            const uint4 raw = *reinterpret_cast<const uint4*>(sb + r * rowbytes + v * 16);
-            C val[VEC];
-            unpack16<DT>(raw, val);
-            if (v == tail_vec) {
-#pragma unroll
-              for (int e = 0; e < VEC; ++e)
-                if (e >= tail_n) val[e] = C(0);
-            }
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) acc[kk][e] = fma(val[e], u[r], acc[kk][e]);
-          }
-        }
-      }
-    }
-  }
-
-  if (aborted) {
-    // Drain the copies still in flight into this CTA's shared memory (bounded), then report.
-    if (tid == 0) {
-      for (int st = k; st < issued; ++st) (void)mbar_wait_bounded(&bars[st % S], (uint32_t)((st / S) & 1));
-      atomicExch(a.status, (int)NYS_ETIMEOUT);
-    }
-    return;
-  }
-
-  C* part = reinterpret_cast<C*>(a.partial) + (int64_t)blockIdx.x * a.dpad;
-#pragma unroll
-  for (int kk = 0; kk < VPT; ++kk) {
-    const int64_t v = tid + (int64_t)kk * T;
-    if (v < nvec) {
-#pragma unroll
-      for (int e = 0; e < VEC; ++e) part[v * VEC + e] = acc[kk][e];
-    }
-  }
-  if (tid == 0 && a.loss_part) a.loss_part[blockIdx.x] = loss;
-  timer_end(a, ts_slot, DT);
-}
-
-// Float-compute variant (FP32 / BF16 storage).  Same streaming scheme, tuned for
+// Float-compute kernel (FP32 / BF16 / FP8 storage; FP64: apass_rows64.cu), tuned for
 // the instruction budget of a bandwidth-bound pass:
 //   * the R rows of a stage are loaded from shared memory ONCE into registers (raw
 //     16-byte vectors) and reused by both the dot product and the rank-1 update, so a
@@ -606,11 +407,16 @@ int apass_row_candidates(const nys_matrix* A, int* out) {
     }
     return n;
   }
+  if (A->dtype == NYS_F64) {
+    // narrow FP64 rows: the stage depth follows from the rows per CTA; a warp takes four rows
+    out[n++] = 4;
+    return n;
+  }
   int threads = kApassThreads, vpt = vpt_bucket(nvec);
-  if (A->dtype != NYS_F64) float_layout(A, nvec, &threads, &vpt);
+  float_layout(A, nvec, &threads, &vpt);
   for (int r : {1, 2, 4}) {
     if (2 * r * rowbytes > kSmemBudget) continue;
-    if (A->dtype != NYS_F64 && !float_rows_ok(r, vpt)) continue;
+    if (!float_rows_ok(r, vpt)) continue;
     out[n++] = r;
   }
   return n;
@@ -653,31 +459,45 @@ bool apass_plan(const nys_matrix* A, ApassPlan* plan) {
   }
   if (vkey < 0) return false;
   if (A->dtype == NYS_F64 && vkey > 12) return false;
-  int vpt = vkey;
-  int R = (int)std::max<int64_t>(1, std::min<int64_t>(kRMax, (48 * 1024) / rowbytes));
   if (A->dtype == NYS_F64) {
-    if (const int tr = tuned_rows(A->dtype, vkey, rowbytes)) R = tr;
+    if (2 * rowbytes > kSmemBudget) return false;
+    // stages of at most 64 KB and 32 rows, evened out over a CTA's slab (2,000 rows on 152
+    // SMs: one stage of 14); one stage needs no ring
+    const int64_t slab = (A->n + sm_count() - 1) / sm_count();
+    const int64_t rmax = std::max<int64_t>(1, std::min<int64_t>(kRows64Max, 64 * 1024 / rowbytes));
+    const int64_t steps = (slab + rmax - 1) / rmax;
+    plan->ws = false;
+    plan->rows_per_step = (int)((slab + steps - 1) / steps);
+    plan->stages = (int)std::min<int64_t>(std::min<int64_t>(kMaxStages, steps),
+                                          kSmemBudget / (plan->rows_per_step * rowbytes));
+    plan->threads = 0;   // fixed by the kernel
+    plan->vpt = apass_rows64_vpt(A->d);
+    plan->onebar = false;
+    plan->smem = (size_t)plan->stages * plan->rows_per_step * rowbytes;
+    plan->dpad = nvec * vec;
+    plan->grid = (int)std::max<int64_t>(1, std::min<int64_t>(sm_count(), (A->n + plan->rows_per_step - 1) / plan->rows_per_step));
+    plan->fused = true;
+    return plan->vpt > 0;
   }
+  int vpt = vkey, R = 1;
   int threads = kApassThreads;
   bool onebar = false;
-  if (A->dtype != NYS_F64) {
-    float_layout(A, nvec, &threads, &vpt);
-    // float path: R is a template parameter bounded by the register budget of raw[R][VPT]
-    R = vpt <= 3 ? 4 : (vpt <= 6 ? 2 : 1);
-    if (const int tr = tuned_rows(A->dtype, vkey, rowbytes)) R = tr;
-    // FP32: one barrier per step (every warp finishes the R row sums itself); BF16: two
-    // barriers (its raw registers leave no room for R row sums in every warp: measured
-    // 4.0 -> 3.1 TB/s with one barrier).  Tuning overrides: NYS_APASS_ROWS (rows per
-    // stage; kept only if the instantiation exists for this width), NYS_APASS_ONEBAR (0/1).
-    onebar = A->dtype == NYS_F32;
-    if (const char* env = std::getenv("NYS_APASS_ROWS")) {
-      const int r = std::atoi(env);
-      if (float_rows_ok(r, vpt)) R = r;
-    }
-    if (const char* env = std::getenv("NYS_APASS_ONEBAR")) onebar = std::atoi(env) != 0;
-    if (!float_rows_ok(R, vpt)) R = 1;
-    while (R > 1 && 2 * R * rowbytes > kSmemBudget) R /= 2;
+  float_layout(A, nvec, &threads, &vpt);
+  // float path: R is a template parameter bounded by the register budget of raw[R][VPT]
+  R = vpt <= 3 ? 4 : (vpt <= 6 ? 2 : 1);
+  if (const int tr = tuned_rows(A->dtype, vkey, rowbytes)) R = tr;
+  // FP32: one barrier per step (every warp finishes the R row sums itself); BF16: two
+  // barriers (its raw registers leave no room for R row sums in every warp: measured
+  // 4.0 -> 3.1 TB/s with one barrier).  Tuning overrides: NYS_APASS_ROWS (rows per
+  // stage; kept only if the instantiation exists for this width), NYS_APASS_ONEBAR (0/1).
+  onebar = A->dtype == NYS_F32;
+  if (const char* env = std::getenv("NYS_APASS_ROWS")) {
+    const int r = std::atoi(env);
+    if (float_rows_ok(r, vpt)) R = r;
   }
+  if (const char* env = std::getenv("NYS_APASS_ONEBAR")) onebar = std::atoi(env) != 0;
+  if (!float_rows_ok(R, vpt)) R = 1;
+  while (R > 1 && 2 * R * rowbytes > kSmemBudget) R /= 2;
   int S = (int)std::min<int64_t>(kMaxStages, kSmemBudget / (R * rowbytes));
   if (S < 2) {
     R = 1;
@@ -704,16 +524,6 @@ size_t apass_partial_bytes(const nys_matrix* A, const ApassPlan& plan) {
 }
 
 static thread_local bool g_prepare_only = false;
-
-template <int DT, int VPT>
-static cudaError_t launch_vpt(const ApassKArgs& k, const ApassPlan& plan, cudaStream_t st) {
-  auto fn = apass_kernel<DT, VPT>;
-  NYS_CUDA_TRY(ensure_max_dyn_smem((const void*)fn, kSmemBudget));
-  if (g_prepare_only) return cudaSuccess;
-  count_launch();
-  fn<<<plan.grid, kApassThreads, plan.smem, st>>>(k);
-  return cudaGetLastError();
-}
 
 template <int DT, int VPT, int R, int T, bool OB>
 static cudaError_t launch_f(const ApassKArgs& k, const ApassPlan& plan, cudaStream_t st) {
@@ -769,27 +579,6 @@ static cudaError_t launch_float(const ApassKArgs& k, const ApassPlan& plan, cuda
   }
 }
 
-template <int DT>
-static cudaError_t launch_dt(const ApassKArgs& k, const ApassPlan& plan, cudaStream_t st) {
-  constexpr int VEC = Stor<DT>::VEC;
-  const int64_t nvec = (k.d + VEC - 1) / VEC;
-  switch (vpt_bucket(nvec)) {
-    case 1: return launch_vpt<DT, 1>(k, plan, st);
-    case 2: return launch_vpt<DT, 2>(k, plan, st);
-    case 3: return launch_vpt<DT, 3>(k, plan, st);
-    case 4: return launch_vpt<DT, 4>(k, plan, st);
-    case 5: return launch_vpt<DT, 5>(k, plan, st);
-    case 6: return launch_vpt<DT, 6>(k, plan, st);
-    case 8: return launch_vpt<DT, 8>(k, plan, st);
-    case 10: return launch_vpt<DT, 10>(k, plan, st);
-    case 12: return launch_vpt<DT, 12>(k, plan, st);
-    case 16:
-      if constexpr (DT != NYS_F64) return launch_vpt<DT, 16>(k, plan, st);
-      return cudaErrorInvalidValue;
-    default: return cudaErrorInvalidValue;
-  }
-}
-
 cudaError_t apass_run(const ApassArgs& a, const ApassPlan& plan, void* partial, double* loss_part,
                       int* dev_status, cudaStream_t st, bool allow_stats) {
   ApassKArgs k;
@@ -839,7 +628,7 @@ cudaError_t apass_run(const ApassArgs& a, const ApassPlan& plan, void* partial, 
   if (plan.ws) {
     err = apass_ws_launch(k, plan, a.dtype, st, g_prepare_only);
   } else switch (a.dtype) {
-    case NYS_F64: err = launch_dt<NYS_F64>(k, plan, st); break;
+    case NYS_F64: err = apass_rows64_launch(k, plan, st, g_prepare_only); break;
     case NYS_F32: err = launch_float<NYS_F32>(k, plan, st); break;
     case NYS_BF16: err = launch_float<NYS_BF16>(k, plan, st); break;
     case NYS_FP8E4M3: err = launch_float<NYS_FP8E4M3>(k, plan, st); break;

@@ -10,9 +10,9 @@
 namespace nys {
 
 constexpr int kMaxStages = 8;
-constexpr int kRMax = 4;
 constexpr int kSmemBudget = 200 * 1024;
 constexpr int kWsGroupWarps = 8;   // warp-specialised float pass: dot warps = update warps
+constexpr int kRows64Max = 32;     // FP64 pass for narrow rows: rows per stage
 constexpr int kWs64DotWarps = 8;   // warp-specialised FP64 pass: dot warps (update warps: twice as many)
 
 struct ApassKArgs {
@@ -24,7 +24,7 @@ struct ApassKArgs {
   double* D_out;
   double* t_out;
   int mode;
-  int R;          // rows per stage (<= kRMax)
+  int R;          // rows per stage
   int S;          // stages
   int64_t dpad;   // partial stride
   void* partial;
@@ -218,5 +218,9 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity) {
 bool apass_ws_layout(int dtype, int64_t d, int* threads, int* vpt);
 cudaError_t apass_ws_launch(const ApassKArgs& k, const ApassPlan& plan, int dtype, cudaStream_t st,
                             bool prepare_only);
+// FP64 pass for the widths the warp-specialised one does not take (apass_rows64.cu): column
+// vectors per thread (-1: too wide), and the launch.
+int apass_rows64_vpt(int64_t d);
+cudaError_t apass_rows64_launch(const ApassKArgs& k, const ApassPlan& plan, cudaStream_t st, bool prepare_only);
 
 }  // namespace nys

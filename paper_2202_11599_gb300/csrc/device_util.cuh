@@ -33,33 +33,6 @@ template <> struct Stor<NYS_FP8E4M3> {
   static constexpr int ESZ = 1;
 };
 
-// Unpack one 16-byte vector of stored elements into compute values.
-template <int DT>
-__device__ __forceinline__ void unpack16(const uint4 r, typename Stor<DT>::C* o);
-template <>
-__device__ __forceinline__ void unpack16<NYS_F64>(const uint4 r, double* o) {
-  o[0] = __hiloint2double((int)r.y, (int)r.x);
-  o[1] = __hiloint2double((int)r.w, (int)r.z);
-}
-template <>
-__device__ __forceinline__ void unpack16<NYS_F32>(const uint4 r, float* o) {
-  o[0] = __uint_as_float(r.x);
-  o[1] = __uint_as_float(r.y);
-  o[2] = __uint_as_float(r.z);
-  o[3] = __uint_as_float(r.w);
-}
-template <>
-__device__ __forceinline__ void unpack16<NYS_BF16>(const uint4 r, float* o) {
-  o[0] = __uint_as_float(r.x << 16);
-  o[1] = __uint_as_float(r.x & 0xffff0000u);
-  o[2] = __uint_as_float(r.y << 16);
-  o[3] = __uint_as_float(r.y & 0xffff0000u);
-  o[4] = __uint_as_float(r.z << 16);
-  o[5] = __uint_as_float(r.z & 0xffff0000u);
-  o[6] = __uint_as_float(r.w << 16);
-  o[7] = __uint_as_float(r.w & 0xffff0000u);
-}
-
 // Load element j of a stored row as a compute value (scalar path for tails / GEMMs).
 template <int DT>
 __device__ __forceinline__ typename Stor<DT>::C load_elem(const void* base, int64_t idx);
