@@ -26,6 +26,7 @@
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 #include <vector>
 
 namespace nys {
@@ -258,30 +259,56 @@ __global__ void __launch_bounds__(T, 1) apass_f_kernel(const ApassKArgs a) {
   timer_end(a, ts_slot, DT);
 }
 
-// y_j = sum_g partial[g][j] (fixed order) + rho p_j; optional per-block partials of p^T y.
-template <typename C>
+// y_j = sum_g partial[g][j] (fixed order) + rho p_j for the block's `chunk` columns; optional
+// partial of p^T y per block.  NT tiles of 32 columns at a time.
+template <typename C, int NT>
 __global__ void __launch_bounds__(kVecThreads) apass_reduce_kernel(const C* __restrict__ partial, int G,
-                                                                   int64_t d, int64_t dpad, C rho,
+                                                                   int64_t d, int64_t dpad, int chunk, C rho,
                                                                    const C* __restrict__ p, C* __restrict__ y,
                                                                    double* dot_part, const int* skip,
                                                                    const float* __restrict__ cscale) {
   if (skip && *skip) return;
-  __shared__ double sh[kVecThreads / 32];
+  static_assert(kVecThreads == 256, "pass_column_sums takes eight warps");
+  __shared__ C sh[8][NT][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t j0 = (int64_t)blockIdx.x * chunk, j1 = min(d, j0 + chunk);
   double dacc = 0.0;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d; j += (int64_t)gridDim.x * blockDim.x) {
-    // fixed order over the CTAs' partials (increasing g)
-    C s = sum_strided_fixed<false>(partial, G, dpad, j, C(0));
-    if (cscale) s *= (C)cscale[j];  // FP8: sum_i q_ij u_i -> sum_i A_ij u_i
-    const C pj = p ? p[j] : C(0);
-    const C yj = fma(rho, pj, s);
-    y[j] = yj;
-    dacc += (double)pj * (double)yj;
+  for (int64_t t0 = j0; t0 < j1; t0 += 32 * NT) {
+    C sum[NT];
+    pass_column_sums<C, NT>(partial, G, dpad, t0 + lane, j1, sum, sh);
+    if (warp == 0) {
+#pragma unroll
+      for (int t = 0; t < NT; ++t) {
+        const int64_t j = t0 + lane + 32 * t;
+        if (j < j1) {
+          C sj = sum[t];
+          if (cscale) sj *= (C)cscale[j];  // FP8: sum_i q_ij u_i -> sum_i A_ij u_i
+          const C pj = p ? p[j] : C(0);
+          const C yj = fma(rho, pj, sj);
+          y[j] = yj;
+          if (dot_part) dacc += (double)pj * (double)yj;
+        }
+      }
+    }
   }
-  if (dot_part) {
-    const double t = block_sum_t0<kVecThreads>(dacc, sh);
-    if (threadIdx.x == 0) dot_part[blockIdx.x] = t;
+  if (dot_part && warp == 0) {
+    const double t = warp_sum(dacc);
+    if (lane == 0) dot_part[blockIdx.x] = t;
   }
 }
+
+// Elements per block of the PCG / ADMM vector steps.  Up to 2,048 elements: at most eight blocks,
+// so that the fused steps run as one cluster (its barrier costs a fraction of the grid's
+// 1.6 us), but never under 64; up to 19,456: 128, for up to 152 blocks; beyond: 256 and
+// more, at most 304 blocks.
+int vec_chunk(int64_t d) {
+  int64_t c;
+  if (d <= 256 * kClusterBlocks) c = std::max<int64_t>(64, (d + kClusterBlocks - 1) / kClusterBlocks);
+  else if (d <= 128 * 152) c = 128;
+  else c = std::max<int64_t>(256, (d + 303) / 304);
+  return (int)((c + 31) / 32 * 32);
+}
+int vec_blocks(int64_t d) { return (int)((d + vec_chunk(d) - 1) / vec_chunk(d)); }
 
 // Blocks of the vector kernels over d elements: one element per thread, at most 4 blocks
 // per SM (measured: spreading a 10,000-element vector over 4x more blocks made the
@@ -783,20 +810,21 @@ cudaError_t apass_prepare(const nys_matrix* A, const ApassPlan& plan) {
 }
 
 cudaError_t apass_reduce(const ApassArgs& a, const ApassPlan& plan, const void* partial, double rho,
-                         void* y, double* dot_part, int dot_blocks, cudaStream_t st) {
-  const int nb = dot_blocks > 0 ? dot_blocks : reduce_blocks(a.d);
-  if (compute_is_f64(a.dtype)) {
+                         void* y, double* dot_part, cudaStream_t st) {
+  // without the dot product every 32 columns take a block of their own
+  const int chunk = dot_part ? vec_chunk(a.d) : 32;
+  const unsigned nb = (unsigned)((a.d + chunk - 1) / chunk);
+  auto run = [&](auto zero, auto nt) {
+    using C = decltype(zero);
     count_launch();
-    apass_reduce_kernel<double><<<nb, kVecThreads, 0, st>>>(
-        reinterpret_cast<const double*>(partial), plan.grid, a.d, plan.dpad, rho,
-        reinterpret_cast<const double*>(a.p), reinterpret_cast<double*>(y), dot_part, a.skip, nullptr);
-  } else {
-    count_launch();
-    apass_reduce_kernel<float><<<nb, kVecThreads, 0, st>>>(
-        reinterpret_cast<const float*>(partial), plan.grid, a.d, plan.dpad, (float)rho,
-        reinterpret_cast<const float*>(a.p), reinterpret_cast<float*>(y), dot_part, a.skip,
-        a.dtype == NYS_FP8E4M3 ? a.col_scale : nullptr);
-  }
+    apass_reduce_kernel<C, decltype(nt)::value><<<nb, kVecThreads, 0, st>>>(
+        reinterpret_cast<const C*>(partial), plan.grid, a.d, plan.dpad, chunk, (C)rho, reinterpret_cast<const C*>(a.p),
+        reinterpret_cast<C*>(y), dot_part, a.skip, a.dtype == NYS_FP8E4M3 ? a.col_scale : nullptr);
+  };
+  using One = std::integral_constant<int, 1>;
+  using Four = std::integral_constant<int, kSumTiles>;
+  if (compute_is_f64(a.dtype)) dot_part ? run(0.0, Four{}) : run(0.0, One{});
+  else dot_part ? run(0.f, Four{}) : run(0.f, One{});
   return cudaGetLastError();
 }
 

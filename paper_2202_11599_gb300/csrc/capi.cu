@@ -387,7 +387,7 @@ nys_status hmatvec_t(const nys_matrix* A, const double* D, double rho, const voi
   a.t_out = nullptr;
   a.mode = D ? MODE_DIAG : MODE_ID;
   NYS_CU(apass_run(a, plan, part, nullptr, dstat, st));
-  NYS_CU(apass_reduce(a, plan, part, rho, y, nullptr, 0, st));
+  NYS_CU(apass_reduce(a, plan, part, rho, y, nullptr, st));
   int h = 0;
   NYS_CU(cudaMemcpyAsync(&h, dstat, sizeof(int), cudaMemcpyDeviceToHost, st));
   NYS_CU(cudaStreamSynchronize(st));
@@ -422,7 +422,7 @@ nys_status aux_pass(const nys_matrix* A, int mode, const void* p, const double* 
   NYS_CU(apass_run(a, plan, part, loss_h ? lp : nullptr, dstat, st));   // no buffer: the loss is not formed
   ApassArgs ar = a;
   ar.p = nullptr;
-  NYS_CU(apass_reduce(ar, plan, part, 0.0, y, nullptr, 0, st));
+  NYS_CU(apass_reduce(ar, plan, part, 0.0, y, nullptr, st));
   if (loss_h) {
     std::vector<double> h(plan.grid);
     NYS_CU(cudaMemcpyAsync(h.data(), lp, plan.grid * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -529,7 +529,7 @@ struct SidePass {
     }
     NYS_CU(apass_run(a, plan, part, lp, dstat, side));
     ApassArgs ar = a;
-    NYS_CU(apass_reduce(ar, plan, part, 0.0, y, nullptr, 0, side));
+    NYS_CU(apass_reduce(ar, plan, part, 0.0, y, nullptr, side));
     if (side != st) NYS_CU(cudaEventRecord(join, side));
     return NYS_OK;
   }
@@ -608,7 +608,7 @@ nys_status lasso_admm(const nys_matrix* A, const nys_matrix* Ain, const double* 
   C* rc = pool.alloc<C>(d);
   float* xA32 = pool.alloc<float>(d);
   const int K = std::max(1, o.admm_maxit);
-  const int nb = admm_blocks(d);
+  const int nb = vec_blocks(d);
   double* part5 = pool.alloc<double>((size_t)nb * 5);
   double* rp = pool.alloc<double>(K);
   double* rd = pool.alloc<double>(K);
@@ -1026,7 +1026,7 @@ nys_status logistic_admm(const nys_matrix* A, const nys_matrix* Ain, const doubl
   void* ytmp = pool.alloc<unsigned char>(d * 8);
   float* xA32 = pool.alloc<float>(d);
   const int K = std::max(1, o.admm_maxit);
-  const int nb = admm_blocks(d);
+  const int nb = vec_blocks(d);
   double* part5 = pool.alloc<double>((size_t)nb * 5);
   double* rp = pool.alloc<double>(K);
   double* rd = pool.alloc<double>(K);

@@ -177,6 +177,12 @@ __device__ __forceinline__ bool grid_barrier_mono(unsigned* count, unsigned targ
   return __syncthreads_and(ok) != 0;
 }
 
+// Barrier of the blocks of one cluster: orders their global writes before it against reads
+// after it, like the grid barriers (data of other blocks is read through L2).
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
@@ -239,6 +245,49 @@ __device__ __forceinline__ T sum_strided_fixed(const T* a, int n, int64_t stride
       if (g + q < n) s += v[q];
   }
   return s;
+}
+
+// Column sums of the A-pass partials [G][dpad] by a block of 256 threads, for NT (four, or one) tiles
+// of 32 columns (tile t: columns j + 32 t, j = first column + lane): warp w adds the partials g = w,
+// w + 8, ... in increasing g, then warp 0 adds the eight warps' sums in order and holds the
+// result (one FP64 addition per 64 clocks and SM quarter: 152 partials added by one thread
+// each took 10 us).  Every use of the partials goes through here, so they agree bit for bit.
+constexpr int kSumTiles = 4;
+template <typename C, int NT>
+__device__ __forceinline__ void pass_column_sums(const C* partial, int G, int64_t dpad, int64_t j, int64_t j1,
+                                                 C (&sum)[NT], C (*sh)[NT][32]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int U = NT == 1 ? 20 : (sizeof(C) == 4 ? 10 : 5);   // partials per tile in flight
+#pragma unroll
+  for (int t = 0; t < NT; ++t) sum[t] = C(0);
+  for (int g0 = warp; g0 < G; g0 += 8 * U) {
+    C v[U][NT];
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+#pragma unroll
+      for (int t = 0; t < NT; ++t)
+        v[q][t] = (g0 + 8 * q < G && j + 32 * t < j1) ? partial[(int64_t)(g0 + 8 * q) * dpad + j + 32 * t] : C(0);
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+      if (g0 + 8 * q < G) {
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+          if (j - lane + 32 * t < j1) sum[t] += v[q][t];
+      }
+  }
+#pragma unroll
+  for (int t = 0; t < NT; ++t) sh[warp][t][lane] = sum[t];
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int t = 0; t < NT; ++t)
+      if (j - lane + 32 * t < j1) {
+        sum[t] = sh[0][t][lane];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) sum[t] += sh[w][t][lane];
+      }
+  }
+  __syncthreads();
 }
 
 // acc + sum_{i < s} U[i * d + j] g[i] as one fma chain in increasing i (the row of U g, for

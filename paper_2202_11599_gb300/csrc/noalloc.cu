@@ -71,7 +71,7 @@ extern "C" nys_status nys_hmatvec_noalloc(const nys_matrix* A, const double* D, 
   a.t_out = nullptr;
   a.mode = D ? MODE_DIAG : MODE_ID;
   if (apass_run(a, plan, scratch, nullptr, dstat, st, /*allow_stats=*/false) != cudaSuccess) return NYS_ECUDA;
-  if (apass_reduce(a, plan, scratch, rho, y, nullptr, 0, st) != cudaSuccess) return NYS_ECUDA;
+  if (apass_reduce(a, plan, scratch, rho, y, nullptr, st) != cudaSuccess) return NYS_ECUDA;
   int h = 0;
   if (cudaMemcpyAsync(&h, dstat, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return NYS_ECUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return NYS_ECUDA;

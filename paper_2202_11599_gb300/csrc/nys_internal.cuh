@@ -77,13 +77,19 @@ cudaError_t apass_balance_rows(const nys_matrix* A, const void* p, void* part, i
                                double* ms_equal, double* ms_split);
 
 // y = sum of partials + rho * p (+ beta * y_prev?) -- y in compute type.
-// dot_part (optional): per-block partials of p^T y (double), count returned via nblk.
+// dot_part (optional): partials of p^T y (double), one per block of vec_blocks(d).
 // allow_stats = false keeps the launch off the instrumentation path (which may allocate).
 cudaError_t apass_run(const ApassArgs& a, const ApassPlan& plan, void* partial, double* loss_part,
                       int* dev_status, cudaStream_t st, bool allow_stats = true);
 cudaError_t apass_reduce(const ApassArgs& a, const ApassPlan& plan, const void* partial, double rho,
-                         void* y, double* dot_part, int dot_blocks, cudaStream_t st);
+                         void* y, double* dot_part, cudaStream_t st);
 int reduce_blocks(int64_t d);
+// The vector steps of PCG and ADMM: block b owns elements [b c, b c + c) of a d-vector, c =
+// vec_chunk(d), in every kernel, so that a kernel that fuses two steps needs no exchange of
+// vector data between blocks, only of sums.
+int vec_chunk(int64_t d);
+int vec_blocks(int64_t d);
+constexpr int kClusterBlocks = 8;   // vec_blocks(d) up to this: the fused kernels run as one cluster
 
 // ---------------------------------------------------------------- small dense FP64 kernels
 // FP64 products on the tensor cores (gemm64_tc.cu).  absmax_f64: per row and / or column of the

@@ -2,7 +2,7 @@
 // steps of Alg. NysADMM (z-prox by soft-thresholding, scaled dual update,
 // primal/dual residuals of Sec. 2.1).
 //
-// One PCG iteration is six stream-ordered launches; every scalar (alpha, beta,
+// In the host-driven loop one PCG iteration is four stream-ordered launches; every scalar (alpha, beta,
 // ||w||, the stop test) lives in a device PcgState, so the host only reads the
 // state once per chunk of iterations.  Kernels launched past convergence see
 // `done` and return at once, which keeps the iterate sequence identical to a
@@ -19,34 +19,16 @@
 
 namespace nys {
 
-// Fixed-order sum of n doubles by one warp; all lanes get the result.
-__device__ __forceinline__ double warp_fixed_sum(const double* a, int n) {
-  const int lane = threadIdx.x & 31;
-  double s = 0.0;
-  for (int i = lane; i < n; i += 32) s += a[i];
-  return warp_sum(s);
-}
-
-// Block-wide broadcast of warp 0's fixed-order sum.
-__device__ __forceinline__ double block_fixed_sum(const double* a, int n, double* slot) {
-  if (threadIdx.x < 32) {
-    const double s = warp_fixed_sum(a, n);
-    if (threadIdx.x == 0) *slot = s;
-  }
-  __syncthreads();
-  const double r = *slot;
-  __syncthreads();
-  return r;
-}
-
-// Same sums reading through L2 (__ldcg): for partials written by other blocks of the
-// running kernel, which this block's L1 may not see.
+// Fixed-order sum of n doubles by one warp, all lanes get the result; read through L2 (__ldcg):
+// the partials may have been written by other blocks of the running kernel, which this block's
+// L1 may not see.
 __device__ __forceinline__ double warp_fixed_sum_cg(const double* a, int n) {
   const int lane = threadIdx.x & 31;
   double s = 0.0;
   for (int i = lane; i < n; i += 32) s += __ldcg(a + i);
   return warp_sum(s);
 }
+// Block-wide broadcast of warp 0's fixed-order sum.
 __device__ __forceinline__ double block_fixed_sum_cg(const double* a, int n, double* slot) {
   if (threadIdx.x < 32) {
     const double s = warp_fixed_sum_cg(a, n);
@@ -58,26 +40,21 @@ __device__ __forceinline__ double block_fixed_sum_cg(const double* a, int n, dou
   return r;
 }
 
-// Two fixed-order sums of the same kind as block_fixed_sum_cg in one pass (same values).
-__device__ __forceinline__ void block_fixed_sum2_cg(const double* a, const double* b, int n, double* out_a,
-                                                    double* out_b, double* slot2) {
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x & 31;
-    double sa = 0.0, sb = 0.0;
-    for (int i = lane; i < n; i += 32) {
-      sa += __ldcg(a + i);
-      sb += __ldcg(b + i);
+// Up to three sums of block_fixed_sum_cg's kind at once, one warp each (same values; the FP64
+// chains run side by side).  Every thread gets the results.
+template <int N>
+__device__ __forceinline__ void block_fixed_sums_cg(const double* const (&a)[N], int n, double (&out)[N],
+                                                    double* slots) {
+  const int warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    if (warp == q) {
+      const double s = warp_fixed_sum_cg(a[q], n);
+      if ((threadIdx.x & 31) == 0) slots[q] = s;
     }
-    sa = warp_sum(sa);
-    sb = warp_sum(sb);
-    if (threadIdx.x == 0) {
-      slot2[0] = sa;
-      slot2[1] = sb;
-    }
-  }
   __syncthreads();
-  *out_a = slot2[0];
-  *out_b = slot2[1];
+#pragma unroll
+  for (int q = 0; q < N; ++q) out[q] = slots[q];
   __syncthreads();
 }
 
@@ -139,51 +116,85 @@ __global__ void pcg_reset_kernel(PcgState* st, double tol, int tol_abs, int maxi
   st->ticket[1] = 0u;
 }
 
-// K4 body (run by the last block of K3): ||w||^2, stop test, iteration count,
+// Warp sums of eight per-lane values by a reduce-scatter over the lane bits: nine additions
+// instead of forty (the exchanges pair the same lanes in the same order as warp_sum, so each
+// sum has its bits).  Lane 4 r holds the sum of v[r].
+template <typename T>
+__device__ __forceinline__ T warp_sum8(const T (&v)[8], int lane) {
+  constexpr unsigned F = 0xffffffffu;
+  T a[4], c[2];
+  const bool h4 = (lane & 16) != 0, h3 = (lane & 8) != 0, h2 = (lane & 4) != 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) a[i] = (h4 ? v[i + 4] : v[i]) + __shfl_xor_sync(F, h4 ? v[i] : v[i + 4], 16);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) c[i] = (h3 ? a[i + 2] : a[i]) + __shfl_xor_sync(F, h3 ? a[i] : a[i + 2], 8);
+  T t = (h2 ? c[1] : c[0]) + __shfl_xor_sync(F, h2 ? c[0] : c[1], 4);
+  t += __shfl_xor_sync(F, t, 2);
+  t += __shfl_xor_sync(F, t, 1);
+  return t;
+}
+
 // Partials of U^T w over one block's chunk of w (in shared memory, len elements from j0):
 // out[i] = sum over the chunk of U[i, j] w_j, each lane adding its lane-strided elements in
-// increasing j, then a warp sum.  Eight rows of U per warp pass keep 64 loads in flight.
+// increasing j, then a warp sum.  Eight rows of U per warp pass.
 template <typename C>
 __device__ __forceinline__ void utw_partials(const C* wch, int len, const C* __restrict__ U, int64_t d, int64_t j0,
-                                             int s, double* out) {
+                                             int s, C* out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int RW = 8;
   for (int i0 = warp * RW; i0 < s; i0 += (kVecThreads / 32) * RW) {
     C acc[RW];
 #pragma unroll
     for (int q = 0; q < RW; ++q) acc[q] = C(0);
-#pragma unroll 8
+#pragma unroll 4
     for (int jj = lane; jj < len; jj += 32) {
       const C wv = wch[jj];
 #pragma unroll
       for (int q = 0; q < RW; ++q)
         if (i0 + q < s) acc[q] = fma(U[(int64_t)(i0 + q) * d + j0 + jj], wv, acc[q]);
     }
-#pragma unroll
-    for (int q = 0; q < RW; ++q) acc[q] = warp_sum(acc[q]);
-    if (lane == 0) {
-#pragma unroll
-      for (int q = 0; q < RW; ++q)
-        if (i0 + q < s) out[i0 + q] = (double)acc[q];
-    }
+    const C t = warp_sum8(acc, lane);
+    if ((lane & 3) == 0 && i0 + (lane >> 2) < s) out[i0 + (lane >> 2)] = t;
   }
 }
 
-// g_i = c_i (U^T w)_i.
+// g_i = c_i sum_b part[b][i], the partials read through L2 and added in increasing b: in FP64, or
+// for FP32 partials as an error-compensated FP32 pair (two-sum; 48 bits of the sum for values
+// of 24), which keeps FP64 accuracy after the rounding to FP32 without the FP64 pipe (79
+// blocks x 200 rows: 4.4 us of FP64 additions in every block).
 template <typename C>
-__device__ void pcg_scalar_body(int init, int nb3, const double* part_w2, const double* part_r2,
-                                const double* part_g, int s, const C* __restrict__ cvec, C* __restrict__ gs,
-                                const double* pv_part, int npv, const double* wy_part, int nwy, PcgState* st,
-                                cudaGraphConditionalHandle cond, int use_cond) {
-  __shared__ double slot;
-  const double w2 = block_fixed_sum_cg(part_w2, nb3, &slot);
-  double r2 = 0.0, pv = 1.0, wy = 0.0;
-  if (init) {
-    r2 = block_fixed_sum_cg(part_r2, nb3, &slot);
+__device__ __forceinline__ C g_entry(const C* part, int nb, int s, int i, C ci) {
+  if constexpr (sizeof(C) == 8) {
+    return ci * sum_strided_fixed<true>(part, nb, s, i, 0.0);
   } else {
-    pv = block_fixed_sum(pv_part, npv, &slot);
-    wy = block_fixed_sum(wy_part, nwy, &slot);
+    constexpr int B = 32;
+    float hi = 0.f, lo = 0.f;
+    for (int b = 0; b < nb; b += B) {
+      float v[B];
+#pragma unroll
+      for (int q = 0; q < B; ++q) v[q] = b + q < nb ? __ldcg(part + (int64_t)(b + q) * s + i) : 0.f;
+#pragma unroll
+      for (int q = 0; q < B; ++q) {
+        const float t = hi + v[q], z = t - hi;
+        lo += (hi - (t - z)) + (v[q] - z);
+        hi = t;
+      }
+    }
+    return (float)((double)ci * ((double)hi + (double)lo));
   }
+}
+
+// Scalar step of a PCG iteration (run by the last block of the update): ||w||^2, stop test,
+// iteration count, g = c o U^T w.
+template <typename C>
+__device__ void pcg_scalar_body(int init, int nb, const double* part_w2, const double* part_r2, const C* part_g, int s,
+                                const C* __restrict__ cvec, C* __restrict__ gs, const double* pv_part,
+                                const double* wy_part, PcgState* st, cudaGraphConditionalHandle cond, int use_cond) {
+  __shared__ double slots[3];
+  double v[3];
+  const double* src[3] = {part_w2, init ? part_r2 : pv_part, init ? part_w2 : wy_part};
+  block_fixed_sums_cg<3>(src, nb, v, slots);
+  const double w2 = v[0], r2 = v[1], pv = v[1], wy = v[2];
   if (threadIdx.x == 0) {
     if (init) {
       st->r2 = r2;
@@ -213,10 +224,7 @@ __device__ void pcg_scalar_body(int init, int nb3, const double* part_w2, const 
       }
     }
   }
-  for (int i = threadIdx.x; i < s; i += kVecThreads) {
-    const double g = sum_strided_fixed<true>(part_g, nb3, s, i, 0.0);
-    gs[i] = (C)((double)cvec[i] * g);
-  }
+  for (int i = threadIdx.x; i < s; i += kVecThreads) gs[i] = g_entry<C>(part_g, nb, s, i, cvec[i]);
   __syncthreads();
   if (use_cond && threadIdx.x == 0) cudaGraphSetConditional(cond, st->done ? 0u : 1u);
 }
@@ -230,9 +238,9 @@ __global__ void __launch_bounds__(kVecThreads) pcg_update_kernel(int init, int64
                                                                  C* __restrict__ w, const C* __restrict__ r,
                                                                  const C* __restrict__ v, const C* __restrict__ p,
                                                                  const C* __restrict__ U, int s,
-                                                                 const double* __restrict__ pv_part, int npv,
-                                                                 const double* __restrict__ wy_part, int nwy,
-                                                                 double* part_w2, double* part_r2, double* part_g,
+                                                                 const double* __restrict__ pv_part,
+                                                                 const double* __restrict__ wy_part,
+                                                                 double* part_w2, double* part_r2, C* part_g,
                                                                  PcgState* st, C* __restrict__ hx,
                                                                  const C* __restrict__ cvec, C* __restrict__ gs,
                                                                  cudaGraphConditionalHandle cond, int use_cond,
@@ -247,16 +255,19 @@ __global__ void __launch_bounds__(kVecThreads) pcg_update_kernel(int init, int64
   extern __shared__ __align__(16) unsigned char sm_raw[];
   C* wch = reinterpret_cast<C*>(sm_raw);
   __shared__ double sh[kVecThreads / 32];
-  __shared__ double slot;
+  __shared__ double slots[2];
   const int64_t j0 = (int64_t)blockIdx.x * chunk;
   const int64_t j1 = min(d, j0 + chunk);
   double alpha = 0.0;
   bool bad = false;
   if (!init) {
-    const double pv = block_fixed_sum(pv_part, npv, &slot);
-    const double wy = block_fixed_sum(wy_part, nwy, &slot);
-    bad = !(pv > 0.0) || !isfinite(pv);  // breakdown: flagged by the scalar step
-    if (!bad) alpha = wy / pv;
+    const double* const src[2] = {pv_part, wy_part};
+    double v2[2];
+    block_fixed_sums_cg<2>(src, (int)gridDim.x, v2, slots);
+    bad = !(v2[0] > 0.0) || !isfinite(v2[0]);  // breakdown: flagged by the scalar step
+    if (threadIdx.x == 0) slots[0] = v2[1] / v2[0];   // one division (the FP64 pipe is narrow), shared
+    __syncthreads();
+    if (!bad) alpha = slots[0];
   }
   if (!bad) {
     const C a = (C)alpha;
@@ -294,15 +305,16 @@ __global__ void __launch_bounds__(kVecThreads) pcg_update_kernel(int init, int64
     utw_partials<C>(wch, (int)(j1 - j0), U, d, j0, s, part_g + (int64_t)blockIdx.x * s);
   }
   if (!last_block_done(&st->ticket[0])) return;
-  pcg_scalar_body<C>(init, (int)gridDim.x, part_w2, part_r2, part_g, s, cvec, gs, pv_part, npv, wy_part, nwy, st,
-                     cond, use_cond);
+  pcg_scalar_body<C>(init, (int)gridDim.x, part_w2, part_r2, part_g, s, cvec, gs, pv_part, wy_part, st, cond,
+                     use_cond);
 }
 
 // K5: y = w + U gs (= P^{-1} w), partial w^T y; when p is given, the last block to finish
 // runs K6 over the whole vector: beta = (w^T y)_new / (w^T y)_old, p = y + beta p
 // (init: p = y).
 template <typename C>
-__global__ void __launch_bounds__(kVecThreads) pcg_tail_kernel(int64_t d, const C* __restrict__ w, C* __restrict__ y,
+__global__ void __launch_bounds__(kVecThreads) pcg_tail_kernel(int64_t d, int chunk, const C* __restrict__ w,
+                                                               C* __restrict__ y,
                                                                const C* __restrict__ U, int s,
                                                                const C* __restrict__ gs, double* part_wy,
                                                                PcgState* st, int init, C* __restrict__ p) {
@@ -314,7 +326,8 @@ __global__ void __launch_bounds__(kVecThreads) pcg_tail_kernel(int64_t d, const 
   for (int i = threadIdx.x; i < s; i += kVecThreads) g[i] = gs[i];
   __syncthreads();
   double lwy = 0.0;
-  for (int64_t j = blockIdx.x * (int64_t)kVecThreads + threadIdx.x; j < d; j += (int64_t)gridDim.x * kVecThreads) {
+  const int64_t j1 = min(d, (int64_t)(blockIdx.x + 1) * chunk);
+  for (int64_t j = blockIdx.x * (int64_t)chunk + threadIdx.x; j < j1; j += kVecThreads) {
     const C wj = w[j];
     const C acc = urow_dot(U, d, j, s, g, wj);
     y[j] = acc;
@@ -334,22 +347,22 @@ __global__ void __launch_bounds__(kVecThreads) pcg_tail_kernel(int64_t d, const 
 }
 
 // Row-sharded matvec, after the sum over ranks of the local A_g^T D_g A_g p (in v):
-// v = rho p + v and the per-block partials of p^T v, with the loop and order of
+// v = rho p + v and the partials of p^T v, one warp per chunk with the order of
 // apass_reduce_kernel (so an unsharded run and a one-rank sharded run agree bitwise).
 template <typename C>
-__global__ void __launch_bounds__(kVecThreads) shard_finish_kernel(int64_t d, C rho, const C* __restrict__ p,
-                                                                   C* __restrict__ v, double* dot_part, const int* skip) {
+__global__ void __launch_bounds__(32) shard_finish_kernel(int64_t d, int chunk, C rho, const C* __restrict__ p,
+                                                          C* __restrict__ v, double* dot_part, const int* skip) {
   if (skip && *skip) return;
-  __shared__ double sh[kVecThreads / 32];
   double dacc = 0.0;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d; j += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t j1 = min(d, (int64_t)(blockIdx.x + 1) * chunk);
+  for (int64_t j = (int64_t)blockIdx.x * chunk + threadIdx.x; j < j1; j += 32) {
     const C pj = p ? p[j] : C(0);
     const C yj = fma(rho, pj, v[j]);
     v[j] = yj;
     dacc += (double)pj * (double)yj;
   }
   if (dot_part) {
-    const double t = block_sum_t0<kVecThreads>(dacc, sh);
+    const double t = warp_sum(dacc);
     if (threadIdx.x == 0) dot_part[blockIdx.x] = t;
   }
 }
@@ -357,29 +370,20 @@ __global__ void __launch_bounds__(kVecThreads) shard_finish_kernel(int64_t d, C 
 // v = (A^T D A + rho I) p with the row sum completed over the ranks of a sharded solve.
 template <typename C>
 static cudaError_t sharded_reduce(const ApassArgs& aa, const ApassPlan& plan, const void* apart, double rho, C* v,
-                                  double* dot_part, int nblk, cudaStream_t stream, nys_status* comm_status) {
-  NYS_CUDA_TRY(apass_reduce(aa, plan, apart, 0.0, v, nullptr, 0, stream));  // local sum, no shift
+                                  double* dot_part, cudaStream_t stream, nys_status* comm_status) {
+  NYS_CUDA_TRY(apass_reduce(aa, plan, apart, 0.0, v, nullptr, stream));  // local sum, no shift
   const nys_status cs = shard_sum(v, aa.d, sizeof(C) == 8 ? NYS_F64 : NYS_F32, stream);
   if (cs != NYS_OK) {
     *comm_status = cs;
     return cudaErrorUnknown;
   }
   count_launch();
-  shard_finish_kernel<C><<<nblk, kVecThreads, 0, stream>>>(aa.d, (C)rho, reinterpret_cast<const C*>(aa.p), v, dot_part,
-                                                             aa.skip);
+  shard_finish_kernel<C><<<vec_blocks(aa.d), 32, 0, stream>>>(aa.d, vec_chunk(aa.d), (C)rho,
+                                                              reinterpret_cast<const C*>(aa.p), v, dot_part, aa.skip);
   return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ host driver
-
-static int upd_chunk(int64_t d) {
-  // ~2 blocks per SM at large d, >= 256 elements per block
-  int64_t ch = std::max<int64_t>(256, (d + 303) / 304);
-  ch = (ch + 31) / 32 * 32;
-  return (int)ch;
-}
-
-int pcg_nb3(int64_t d) { return (int)((d + upd_chunk(d) - 1) / upd_chunk(d)); }
 
 template <typename C>
 nys_status pcg_run(const PcgProblem& pb, const PrecondView& P, const C* r, C* x, const PcgParams& prm,
@@ -389,21 +393,19 @@ nys_status pcg_run(const PcgProblem& pb, const PrecondView& P, const C* r, C* x,
   const int s = P.s;
   const C* U = reinterpret_cast<const C*>(P.U);
   const C* cvec = reinterpret_cast<const C*>(P.c);
-  const int chunk = upd_chunk(d);
-  const int nb3 = (int)((d + chunk - 1) / chunk);
-  const int nbr = reduce_blocks(d);
-  const int nb5 = nbr;
+  const int chunk = vec_chunk(d);
+  const int nb = vec_blocks(d);
 
   C* w = pool.alloc<C>(d);
   C* y = pool.alloc<C>(d);
   C* p = pool.alloc<C>(d);
   C* v = pool.alloc<C>(d);
   C* gs = pool.alloc<C>(std::max(1, s));
-  double* part_w2 = pool.alloc<double>(nb3);
-  double* part_r2 = pool.alloc<double>(nb3);
-  double* part_g = pool.alloc<double>((size_t)nb3 * std::max(1, s));
-  double* pv_part = pool.alloc<double>(nbr);
-  double* wy_part = pool.alloc<double>(nb5);
+  double* part_w2 = pool.alloc<double>(nb);
+  double* part_r2 = pool.alloc<double>(nb);
+  C* part_g = pool.alloc<C>((size_t)nb * std::max(1, s));
+  double* pv_part = pool.alloc<double>(nb);
+  double* wy_part = pool.alloc<double>(nb);
   void* apart = pool.alloc<unsigned char>(apass_partial_bytes(pb.A, pb.plan));
   PcgState* st = pool.alloc<PcgState>(1);
   int* dstat = pool.alloc<int>(1);
@@ -438,14 +440,14 @@ nys_status pcg_run(const PcgProblem& pb, const PrecondView& P, const C* r, C* x,
   LAUNCH_OK(cudaGetLastError());
   const bool sharded = shard_comm().fn != nullptr;
   nys_status comm_status = NYS_OK;
-#define MATVEC_REDUCE(rho_, dots_, nd_)                                                                  \
+#define MATVEC_REDUCE(rho_, dots_)                                                                       \
   do {                                                                                                  \
     if (sharded) {                                                                                      \
-      e = sharded_reduce<C>(aa, pb.plan, apart, (rho_), v, (dots_), nbr, stream, &comm_status);          \
+      e = sharded_reduce<C>(aa, pb.plan, apart, (rho_), v, (dots_), stream, &comm_status);               \
       if (comm_status != NYS_OK) return comm_status;                                                    \
       if (e != cudaSuccess) return NYS_ECUDA;                                                           \
     } else {                                                                                            \
-      LAUNCH_OK(apass_reduce(aa, pb.plan, apart, (rho_), v, (dots_), (nd_), stream));                  \
+      LAUNCH_OK(apass_reduce(aa, pb.plan, apart, (rho_), v, (dots_), stream));                          \
     }                                                                                                   \
   } while (0)
   const C* v0 = nullptr;
@@ -454,18 +456,18 @@ nys_status pcg_run(const PcgProblem& pb, const PrecondView& P, const C* r, C* x,
     const int* skip0 = aa.skip;
     aa.skip = nullptr;
     LAUNCH_OK(apass_run(aa, pb.plan, apart, nullptr, dstat, stream));
-    MATVEC_REDUCE(pb.rho, nullptr, 0);
+    MATVEC_REDUCE(pb.rho, nullptr);
     aa.skip = skip0;
     v0 = v;
   }
   count_launch();
-  pcg_update_kernel<C><<<nb3, kVecThreads, sm_upd, stream>>>(1, d, chunk, x, w, r, v0, p, U, s, pv_part, nbr,
-                                                             wy_part, nb5, part_w2, part_r2, part_g, st, (C*)nullptr,
+  pcg_update_kernel<C><<<nb, kVecThreads, sm_upd, stream>>>(1, d, chunk, x, w, r, v0, p, U, s, pv_part,
+                                                             wy_part, part_w2, part_r2, part_g, st, (C*)nullptr,
                                                              cvec, gs, 0ull, 0, nullptr, nullptr, nullptr, 0.0,
                                                              (C*)nullptr);
   LAUNCH_OK(cudaGetLastError());
   count_launch();
-  pcg_tail_kernel<C><<<nb5, kVecThreads, sm_tail, stream>>>(d, w, y, U, s, gs, wy_part, st, 1, p);
+  pcg_tail_kernel<C><<<nb, kVecThreads, sm_tail, stream>>>(d, chunk, w, y, U, s, gs, wy_part, st, 1, p);
   LAUNCH_OK(cudaGetLastError());
 
   PcgState* hs = host_state();
@@ -476,15 +478,15 @@ nys_status pcg_run(const PcgProblem& pb, const PrecondView& P, const C* r, C* x,
     for (int c = 0; c < chunk_it && launched < cap; ++c, ++launched) {
       aa.p = p;
       LAUNCH_OK(apass_run(aa, pb.plan, apart, nullptr, dstat, stream));
-      MATVEC_REDUCE(pb.rho, pv_part, nbr);
+      MATVEC_REDUCE(pb.rho, pv_part);
       count_launch();
-      pcg_update_kernel<C><<<nb3, kVecThreads, sm_upd, stream>>>(0, d, chunk, x, w, r, v, p, U, s, pv_part, nbr,
-                                                                 wy_part, nb5, part_w2, part_r2, part_g, st, (C*)nullptr,
+      pcg_update_kernel<C><<<nb, kVecThreads, sm_upd, stream>>>(0, d, chunk, x, w, r, v, p, U, s, pv_part,
+                                                                 wy_part, part_w2, part_r2, part_g, st, (C*)nullptr,
                                                                  cvec, gs, 0ull, 0, nullptr, nullptr, nullptr, 0.0,
                                                                  (C*)nullptr);
       LAUNCH_OK(cudaGetLastError());
       count_launch();
-      pcg_tail_kernel<C><<<nb5, kVecThreads, sm_tail, stream>>>(d, w, y, U, s, gs, wy_part, st, 0, p);
+      pcg_tail_kernel<C><<<nb, kVecThreads, sm_tail, stream>>>(d, chunk, w, y, U, s, gs, wy_part, st, 0, p);
       LAUNCH_OK(cudaGetLastError());
     }
     LAUNCH_OK(cudaMemcpyAsync(hs, st, sizeof(PcgState), cudaMemcpyDeviceToHost, stream));
@@ -526,13 +528,14 @@ __global__ void admm_rhs_kernel(int64_t d, const double* __restrict__ q, const d
 
 // x <- xc (or x += xc), z_old = z, z = S_kappa(x + u), u += x - z, residual partials.
 template <typename C>
-__global__ void __launch_bounds__(kVecThreads) admm_zu_kernel(int64_t d, const C* __restrict__ xc, int accumulate,
+__global__ void __launch_bounds__(kVecThreads) admm_zu_kernel(int64_t d, int chunk, const C* __restrict__ xc, int accumulate,
                                                               double* __restrict__ x, double* __restrict__ z,
                                                               double* __restrict__ u, double kappa,
                                                               double* __restrict__ ztrace, double* part5) {
   __shared__ double sh[kVecThreads / 32];
   double a0 = 0, a1 = 0, a2 = 0, a3 = 0, a4 = 0;
-  for (int64_t j = blockIdx.x * (int64_t)kVecThreads + threadIdx.x; j < d; j += (int64_t)gridDim.x * kVecThreads) {
+  const int64_t j1 = min(d, (int64_t)(blockIdx.x + 1) * chunk);
+  for (int64_t j = blockIdx.x * (int64_t)chunk + threadIdx.x; j < j1; j += kVecThreads) {
     const double xj = accumulate ? x[j] + (double)xc[j] : (double)xc[j];
     const double zo = z[j];
     const double vj = xj + u[j];
@@ -603,13 +606,11 @@ __global__ void admm_scalar_kernel(int nb, const double* part5, double rho, int 
   }
 }
 
-int admm_blocks(int64_t d) { return reduce_blocks(d); }
-
 template <typename C>
 cudaError_t admm_rhs(int64_t d, const double* q, const double* z, const double* u, double rho, const double* x,
                      const double* yres, C* r, cudaStream_t st, double mu) {
   count_launch();
-  admm_rhs_kernel<C><<<admm_blocks(d), kVecThreads, 0, st>>>(d, q, z, u, rho, x, yres, r, mu);
+  admm_rhs_kernel<C><<<reduce_blocks(d), kVecThreads, 0, st>>>(d, q, z, u, rho, x, yres, r, mu);
   return cudaGetLastError();
 }
 template cudaError_t admm_rhs<double>(int64_t, const double*, const double*, const double*, double, const double*,
@@ -621,7 +622,7 @@ template <typename C>
 cudaError_t admm_zu(int64_t d, const C* xc, int accumulate, double* x, double* z, double* u, double kappa,
                     double* ztrace, double* part5, cudaStream_t st) {
   count_launch();
-  admm_zu_kernel<C><<<admm_blocks(d), kVecThreads, 0, st>>>(d, xc, accumulate, x, z, u, kappa, ztrace, part5);
+  admm_zu_kernel<C><<<vec_blocks(d), kVecThreads, 0, st>>>(d, vec_chunk(d), xc, accumulate, x, z, u, kappa, ztrace, part5);
   return cudaGetLastError();
 }
 template cudaError_t admm_zu<double>(int64_t, const double*, int, double*, double*, double*, double, double*,
@@ -632,7 +633,7 @@ template cudaError_t admm_zu<float>(int64_t, const float*, int, double*, double*
 cudaError_t admm_scalar(int64_t d, const double* part5, double rho, int k, double* rp, double* rd, double* eps_next,
                         double eps_abs, double eps_rel, int* stop, cudaStream_t st) {
   count_launch();
-  admm_scalar_kernel<<<1, 32, 0, st>>>(admm_blocks(d), part5, rho, k, rp, rd, eps_next, eps_abs, eps_rel, stop);
+  admm_scalar_kernel<<<1, 32, 0, st>>>(vec_blocks(d), part5, rho, k, rp, rd, eps_next, eps_abs, eps_rel, stop);
   return cudaGetLastError();
 }
 
@@ -797,7 +798,7 @@ __device__ void admm_scalar_g_body(int nb, const double* part5, double rho, int 
 }
 
 template <typename C>
-__global__ void __launch_bounds__(kVecThreads) admm_zu_g_kernel(int64_t d, const C* __restrict__ xc, int accumulate,
+__global__ void __launch_bounds__(kVecThreads) admm_zu_g_kernel(int64_t d, int chunk, const C* __restrict__ xc, int accumulate,
                                                                 double* __restrict__ x, double* __restrict__ z,
                                                                 double* __restrict__ u, double kappa,
                                                                 double* __restrict__ ztrace, AdmmCtl* ctl,
@@ -808,7 +809,8 @@ __global__ void __launch_bounds__(kVecThreads) admm_zu_g_kernel(int64_t d, const
                                                                 cudaGraphConditionalHandle cond) {
   double* zt = ztrace ? ztrace + (int64_t)ctl->k * d : nullptr;
   double a0 = 0, a1 = 0, a2 = 0, a3 = 0, a4 = 0;
-  for (int64_t j = blockIdx.x * (int64_t)kVecThreads + threadIdx.x; j < d; j += (int64_t)gridDim.x * kVecThreads) {
+  const int64_t j1 = min(d, (int64_t)(blockIdx.x + 1) * chunk);
+  for (int64_t j = blockIdx.x * (int64_t)chunk + threadIdx.x; j < j1; j += kVecThreads) {
     const double xj = accumulate ? x[j] + (double)xc[j] : (double)xc[j];
     const double zo = z[j];
     const double vj = xj + u[j];
@@ -859,30 +861,32 @@ __global__ void __launch_bounds__(kVecThreads) admm_zu_g_kernel(int64_t d, const
 // before it) and returns; the next launch continues at k.  The arithmetic and its order are
 // those of the general body, so the iterates are bitwise those of a solve without this
 // kernel.  Grid barriers are bounded (NYS_ETIMEOUT).
-// One PCG iteration after its A-pass as ONE cooperative launch (Alg. Nystrom PCG): the
-// reduction of the per-CTA A-pass partials (apass_reduce_kernel), the update of x, w and the
-// tracked (H + rho I) x with the partials of ||w||^2 and U^T w (pcg_update_kernel), the
-// scalar step (pcg_scalar_body), y = P^{-1} w (pcg_tail_kernel) and the next direction
-// p = y + beta p, separated by grid barriers instead of kernel boundaries.  Every element and
-// every partial is formed by the same code, block mapping and order as in those kernels, so
-// the result is bitwise theirs; data written by other blocks in the same launch is read
-// through L2.  With zu set, the iteration that ends the PCG loop also runs the prox / dual
+// One PCG iteration after its A-pass as ONE launch (Alg. Nystrom PCG): the reduction of the
+// per-CTA A-pass partials (apass_reduce_kernel), the update of x, w and the tracked
+// (H + rho I) x with the partials of ||w||^2 and U^T w (pcg_update_kernel), the scalar step
+// (pcg_scalar_body), y = P^{-1} w (pcg_tail_kernel) and the next direction p = y + beta p,
+// separated by barriers instead of kernel boundaries.  A block keeps its chunk of every vector
+// from step to step; only sums cross blocks, through L2.  Up to kClusterBlocks blocks run as one
+// cluster (hardware barrier), more as a cooperative grid.  Every element and every partial is
+// formed by the same code, block mapping and order as in the separate kernels, so the result
+// is bitwise theirs.  With zu set, the iteration that ends the PCG loop also runs the prox / dual
 // step and the scalars of the ADMM iteration (admm_zu_g_kernel, admm_scalar_g_body).
 template <typename C>
 struct PostArgs {
   int64_t d;
-  int chunk, nbr, nb3, nb5, nbz;
+  int chunk, nb;
   const C* partial;      // [G][dpad] A-pass partials
   int G;
   int64_t dpad;
   C rho;                 // rho + mu of the H-matvec
   const float* cscale;   // FP8 column scales, or null
-  C *p, *v, *x, *w, *hx, *y;
+  C *p, *x, *w, *hx, *y;
   const C* U;
   int s;
   const C* cvec;
   C* gs;
-  double *pv_part, *wy_part, *part_w2, *part_g;
+  double *pv_part, *wy_part, *part_w2;
+  C* part_g;
   PcgState* st;
   cudaGraphConditionalHandle cond;   // the PCG WHILE
   // prox / dual step (zu != 0)
@@ -896,18 +900,49 @@ struct PostArgs {
   int* dstat;            // NYS_ETIMEOUT when a grid barrier wait runs out
 };
 
-template <typename C>
-__global__ void __launch_bounds__(kVecThreads) pcg_post_kernel(const PostArgs<C> a) {
+// Barrier of a fused vector kernel's blocks: the cluster's when they form one (CL), else the
+// bounded grid barrier of the cooperative launch.
+template <bool CL>
+__device__ __forceinline__ bool vec_barrier(unsigned* count, unsigned* gen, unsigned nblk) {
+  if constexpr (CL) {
+    __syncthreads();
+    cluster_barrier();
+    return true;
+  } else {
+    return grid_barrier(count, gen, nblk);
+  }
+}
+
+// One element of the prox / dual step: z = S_kappa(x + u), u += x - z, the five residual sums.
+__device__ __forceinline__ void zu_element(double xj, double zo, double uo, double kappa, double& zj, double& uj,
+                                           double (&a)[5]) {
+  const double vj = xj + uo;
+  const double mag = fabs(vj) - kappa;
+  zj = mag > 0.0 ? copysign(mag, vj) : 0.0;
+  uj = uo + xj - zj;
+  a[0] += (xj - zj) * (xj - zj);
+  a[1] += (zj - zo) * (zj - zo);
+  a[2] += xj * xj;
+  a[3] += zj * zj;
+  a[4] += uj * uj;
+}
+
+template <typename C, bool CL>
+__global__ void __launch_bounds__(kVecThreads, 2) pcg_post_kernel(const PostArgs<C> a) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  C* wch = reinterpret_cast<C*>(sm_raw);   // chunk of w (U^T w), then g (y = w + U g)
+  C* vch = reinterpret_cast<C*>(sm_raw);   // the block's chunk of v, then of w
+  C* gsh = vch + a.chunk;                  // g
+  __shared__ C csh[8][kSumTiles][32];
   __shared__ double sh[kVecThreads / 32];
-  __shared__ double slot;
+  __shared__ double slots[2];
   PcgState* st = a.st;
   const int b = blockIdx.x;
   const unsigned nblk = gridDim.x;
   const int64_t d = a.d;
   const int s = a.s;
-  // every block reads the state before block 0 changes it below (after two barriers)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t j0 = min(d, (int64_t)b * a.chunk), j1 = min(d, j0 + a.chunk);
+  // every block reads the state before block 0 changes it below (after a barrier)
   const int done0 = st->done;
   const int iters0 = st->iters, fixed = st->fixed, maxit = st->maxit;
   const double thresh2 = st->thresh2;
@@ -923,51 +958,65 @@ __global__ void __launch_bounds__(kVecThreads) pcg_post_kernel(const PostArgs<C>
       if (a.zu) cudaGraphSetConditional(a.h_admm, 0u);
     }
   };
-  // ---- R: v = sum_g partial[g] + rho p, partials of p^T v (apass_reduce_kernel)
-  if (b < a.nbr) {
+  auto barrier = [&]() { return vec_barrier<CL>(&st->bar_count, &st->bar_gen, nblk); };
+  // ---- R: v = sum_g partial[g] + rho p over the block's chunk, partial of p^T v
+  // (apass_reduce_kernel)
+  {
     double dacc = 0.0;
-    for (int64_t j = b * (int64_t)kVecThreads + threadIdx.x; j < d; j += (int64_t)a.nbr * kVecThreads) {
-      C sj = sum_strided_fixed<false>(a.partial, a.G, a.dpad, j, C(0));
-      if (a.cscale) sj *= (C)a.cscale[j];
-      const C pj = a.p[j];
-      const C yj = fma(a.rho, pj, sj);
-      a.v[j] = yj;
-      dacc += (double)pj * (double)yj;
+    for (int64_t t0 = j0; t0 < j1; t0 += 32 * kSumTiles) {
+      C sum[kSumTiles];
+      pass_column_sums<C, kSumTiles>(a.partial, a.G, a.dpad, t0 + lane, j1, sum, csh);
+      if (warp == 0) {
+#pragma unroll
+        for (int t = 0; t < kSumTiles; ++t) {
+          const int64_t j = t0 + lane + 32 * t;
+          if (j < j1) {
+            C sj = sum[t];
+            if (a.cscale) sj *= (C)a.cscale[j];
+            const C pj = a.p[j];
+            const C yj = fma(a.rho, pj, sj);
+            vch[j - j0] = yj;
+            dacc += (double)pj * (double)yj;
+          }
+        }
+      }
     }
-    const double t = block_sum_t0<kVecThreads>(dacc, sh);
-    if (threadIdx.x == 0) a.pv_part[b] = t;
+    if (warp == 0) {
+      const double t = warp_sum(dacc);
+      if (lane == 0) a.pv_part[b] = t;
+    }
   }
-  if (!grid_barrier(&st->bar_count, &st->bar_gen, nblk)) return fail();
+  if (!barrier()) return fail();
   // ---- U: alpha = w^T y / p^T v, x += alpha p, w -= alpha v, hx += alpha v (pcg_update_kernel)
-  const double pv = block_fixed_sum_cg(a.pv_part, a.nbr, &slot);
-  const double wy = block_fixed_sum_cg(a.wy_part, a.nb5, &slot);
+  const double* const src[2] = {a.pv_part, a.wy_part};
+  double v2[2];
+  block_fixed_sums_cg<2>(src, a.nb, v2, slots);
+  const double pv = v2[0], wy = v2[1];
   const bool bad = !(pv > 0.0) || !isfinite(pv);
-  if (threadIdx.x == 0) slot = wy / pv;   // one division (the FP64 pipe is narrow), shared
+  if (threadIdx.x == 0) slots[0] = wy / pv;   // one division (the FP64 pipe is narrow), shared
   __syncthreads();
-  const double alpha = slot;
-  if (!bad && b < a.nb3) {
+  const double alpha = slots[0];
+  if (!bad) {
     const C al = (C)alpha;
-    const int64_t j0 = (int64_t)b * a.chunk;
-    const int64_t j1 = min(d, j0 + a.chunk);
     double lw2 = 0.0;
     for (int64_t j = j0 + threadIdx.x; j < j1; j += kVecThreads) {
-      const C vj = __ldcg(a.v + j);
+      const C vj = vch[j - j0];
       a.x[j] = fma(al, a.p[j], a.x[j]);
       const C wj = fma(-al, vj, a.w[j]);
       if (a.hx) a.hx[j] = fma(al, vj, a.hx[j]);
       a.w[j] = wj;
-      wch[j - j0] = wj;
+      vch[j - j0] = wj;
       lw2 += (double)wj * (double)wj;
     }
     const double tw2 = block_sum_t0<kVecThreads>(lw2, sh);
     if (threadIdx.x == 0) a.part_w2[b] = tw2;
   }
-  if (!grid_barrier(&st->bar_count, &st->bar_gen, nblk)) return fail();
+  if (!barrier()) return fail();
   // ---- S: ||w||^2, stop test, iteration count (pcg_scalar_body; every block takes the same
   // decision, block 0 records it).  U^T w and g = c o U^T w follow only if PCG goes on: the
   // iteration that ends the loop needs no P^{-1} w (the separate kernels form it regardless;
   // the values they use are the same).
-  const double w2 = block_fixed_sum_cg(a.part_w2, a.nb3, &slot);
+  const double w2 = block_fixed_sum_cg(a.part_w2, a.nb, &slots[1]);
   const bool stepped = !bad && isfinite(w2);
   int iters = iters0, done = 0, status = 0;
   if (!stepped) {
@@ -998,65 +1047,50 @@ __global__ void __launch_bounds__(kVecThreads) pcg_post_kernel(const PostArgs<C>
   if (!done) {
     // U^T w partials over this block's chunk of the new w, still in shared memory (every
     // block that stepped has !bad here)
-    if (b < a.nb3) {
-      const int64_t j0 = (int64_t)b * a.chunk;
-      const int64_t j1 = min(d, j0 + a.chunk);
-      utw_partials<C>(wch, (int)(j1 - j0), a.U, d, j0, s, a.part_g + (int64_t)b * s);
-    }
-    if (!grid_barrier(&st->bar_count, &st->bar_gen, nblk)) return fail();
+    utw_partials<C>(vch, (int)(j1 - j0), a.U, d, j0, s, a.part_g + (int64_t)b * s);
+    if (!barrier()) return fail();
     for (int i = threadIdx.x; i < s; i += kVecThreads) {
-      const double g = sum_strided_fixed<true>(a.part_g, a.nb3, s, i, 0.0);
-      const C gi = (C)((double)a.cvec[i] * g);
-      wch[i] = gi;
+      const C gi = g_entry<C>(a.part_g, a.nb, s, i, a.cvec[i]);
+      gsh[i] = gi;
       if (b == 0) a.gs[i] = gi;
     }
     __syncthreads();
     // ---- T: y = w + U g, partials of w^T y (pcg_tail_kernel)
-    if (b < a.nb5) {
+    {
       double lwy = 0.0;
-      for (int64_t j = b * (int64_t)kVecThreads + threadIdx.x; j < d; j += (int64_t)a.nb5 * kVecThreads) {
-        const C wj = __ldcg(a.w + j);
-        const C acc = urow_dot(a.U, d, j, s, wch, wj);
+      for (int64_t j = j0 + threadIdx.x; j < j1; j += kVecThreads) {
+        const C wj = vch[j - j0];
+        const C acc = urow_dot(a.U, d, j, s, gsh, wj);
         a.y[j] = acc;
         lwy += (double)wj * (double)acc;
       }
       const double t = block_sum_t0<kVecThreads>(lwy, sh);
       if (threadIdx.x == 0) a.wy_part[b] = t;
     }
-    if (!grid_barrier(&st->bar_count, &st->bar_gen, nblk)) return fail();
+    if (!barrier()) return fail();
     // ---- B: beta = (w^T y)_new / (w^T y)_old, p = y + beta p
-    const double wy_new = block_fixed_sum_cg(a.wy_part, a.nb5, &slot);
-    if (threadIdx.x == 0) slot = wy_new / wy;
+    const double wy_new = block_fixed_sum_cg(a.wy_part, a.nb, &slots[1]);
+    if (threadIdx.x == 0) slots[0] = wy_new / wy;
     __syncthreads();
-    const C bc = (C)slot;
-    for (int64_t j = b * (int64_t)kVecThreads + threadIdx.x; j < d; j += (int64_t)nblk * kVecThreads)
-      a.p[j] = fma(bc, a.p[j], __ldcg(a.y + j));
+    const C bc = (C)slots[0];
+    for (int64_t j = j0 + threadIdx.x; j < j1; j += kVecThreads) a.p[j] = fma(bc, a.p[j], a.y[j]);
     return;
   }
   if (!a.zu) return;
   // ---- Z: prox / dual step with the final x and the scalars of the ADMM iteration
-  // (admm_zu_g_kernel; x was written by other blocks above: read through L2)
-  if (b < a.nbz) {
+  // (admm_zu_g_kernel)
+  {
     double* zt = a.ztrace ? a.ztrace + (int64_t)a.ctl->k * d : nullptr;
-    double a0 = 0, a1 = 0, a2 = 0, a3 = 0, a4 = 0;
-    for (int64_t j = b * (int64_t)kVecThreads + threadIdx.x; j < d; j += (int64_t)a.nbz * kVecThreads) {
-      const double xj = (double)__ldcg(a.x + j);
-      const double zo = a.z[j];
-      const double vj = xj + a.u[j];
-      const double mag = fabs(vj) - a.kappa;
-      const double zj = mag > 0.0 ? copysign(mag, vj) : 0.0;
-      const double uj = a.u[j] + xj - zj;
+    double a5[5] = {0, 0, 0, 0, 0};
+    for (int64_t j = j0 + threadIdx.x; j < j1; j += kVecThreads) {
+      const double xj = (double)a.x[j];
+      double zj, uj;
+      zu_element(xj, a.z[j], a.u[j], a.kappa, zj, uj, a5);
       a.xd[j] = xj;
       a.z[j] = zj;
       a.u[j] = uj;
       if (zt) zt[j] = zj;
-      a0 += (xj - zj) * (xj - zj);
-      a1 += (zj - zo) * (zj - zo);
-      a2 += xj * xj;
-      a3 += zj * zj;
-      a4 += uj * uj;
     }
-    double a5[5] = {a0, a1, a2, a3, a4};
     block_sum5(a5);
     if (threadIdx.x == 0) {
       double* o = a.part5 + (int64_t)b * 5;
@@ -1064,19 +1098,19 @@ __global__ void __launch_bounds__(kVecThreads) pcg_post_kernel(const PostArgs<C>
       for (int t = 0; t < 5; ++t) o[t] = a5[t];
     }
   }
-  if (!grid_barrier(&st->bar_count, &st->bar_gen, nblk)) return fail();
+  if (!barrier()) return fail();
   if (b == 0 && threadIdx.x < 32)
-    admm_scalar_g_body(a.nbz, a.part5, a.rho_admm, a.K, a.eps_abs, a.eps_rel, a.rp, a.rd, a.pcg_it, st, a.ctl, 0, 2,
+    admm_scalar_g_body(a.nb, a.part5, a.rho_admm, a.K, a.eps_abs, a.eps_rel, a.rp, a.rd, a.pcg_it, st, a.ctl, 0, 2,
                        a.h_admm);
 }
 
 struct HeadArgs {
   int64_t d;
-  int chunk, nb3, nbz, nb5, s;
+  int chunk, nb, s;
   const double* q;
   double *x, *z, *u;
   double rho, kappa;
-  double *part_w2, *part_r2, *part_g, *wy_part, *part5;
+  double *part_w2, *part_r2, *wy_part, *part5;
   AdmmCtl* ctl;
   PcgState* st;
   double tol, tol_floor;
@@ -1089,16 +1123,19 @@ struct HeadArgs {
   int* dstat;
   cudaGraphConditionalHandle h_admm, h_pcg, h_zu, h_hx;
   int has_zu;   // 0: the PCG post kernel runs the prox / dual step, there is no IF (h_zu) node
+  int inline_hx;   // 1: the recompute pass precedes this kernel in every body pass (hx_refresh = 0)
 };
 
-template <typename C>
-__global__ void __launch_bounds__(kVecThreads) admm_head_kernel(HeadArgs a, const C* __restrict__ xc,
+template <typename C, bool CL>
+__global__ void __launch_bounds__(kVecThreads, 2) admm_head_kernel(HeadArgs a, const C* __restrict__ xc,
                                                                 const C* __restrict__ hx, C* __restrict__ w,
                                                                 C* __restrict__ rc, C* __restrict__ y,
                                                                 C* __restrict__ p, const C* __restrict__ U,
-                                                                const C* __restrict__ cvec, C* __restrict__ gs) {
+                                                                const C* __restrict__ cvec, C* __restrict__ gs,
+                                                                C* __restrict__ part_g) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  C* wch = reinterpret_cast<C*>(sm_raw);   // chunk of w (U^T w), then g (y = w + U g)
+  C* wch = reinterpret_cast<C*>(sm_raw);   // the block's chunk of w
+  C* gsh = wch + a.chunk;                  // g
   __shared__ double sh[kVecThreads / 32];
   __shared__ double slot;
   __shared__ double slot2[2];
@@ -1109,6 +1146,7 @@ __global__ void __launch_bounds__(kVecThreads) admm_head_kernel(HeadArgs a, cons
   const unsigned nblk = gridDim.x;
   const int64_t d = a.d;
   const int s = a.s;
+  const int64_t j0 = min(d, (int64_t)b * a.chunk), j1 = min(d, j0 + a.chunk);
   AdmmCtl* ctl = a.ctl;
   int k = ctl->k;
   double eps_next = ctl->eps_next;
@@ -1119,14 +1157,19 @@ __global__ void __launch_bounds__(kVecThreads) admm_head_kernel(HeadArgs a, cons
       cudaGraphSetConditional(a.h_admm, 0u);
       cudaGraphSetConditional(a.h_pcg, 0u);
       if (a.has_zu) cudaGraphSetConditional(a.h_zu, 0u);
-      cudaGraphSetConditional(a.h_hx, 0u);
+      if (!a.inline_hx) cudaGraphSetConditional(a.h_hx, 0u);
     }
   };
+  auto barrier = [&]() { return vec_barrier<CL>(&ctl->bar_count, &ctl->bar_gen, nblk); };
   bool first = true;
   for (;;) {
-    // ---- (H + rho I) x due for a recompute at iteration k: request it and return
-    if (!iter_hx_skip(0, k, a.hx_refresh) && !(first && refreshed)) {
-      if (b == 0 && threadIdx.x == 0) {
+    // ---- (H + rho I) x due for a recompute at iteration k: request it and return.  With
+    // inline_hx the body's next pass recomputes it before this kernel.
+    if (a.inline_hx ? !first : !iter_hx_skip(0, k, a.hx_refresh) && !(first && refreshed)) {
+      if (b == 0 && threadIdx.x == 0 && a.inline_hx) {
+        ctl->nodes += 3;
+        cudaGraphSetConditional(a.h_pcg, 0u);
+      } else if (b == 0 && threadIdx.x == 0) {
         ctl->hx_pending = 1;
         ctl->nodes += 1;
         cudaGraphSetConditional(a.h_hx, 1u);
@@ -1147,12 +1190,10 @@ __global__ void __launch_bounds__(kVecThreads) admm_head_kernel(HeadArgs a, cons
     const double tolk = s_tolk;
     const int tol_abs = s_tabs;
     // ---- 1. right-hand side, warm-start residual, ||w||^2, ||r||^2, U^T w partials
-    if (b < a.nb3) {
-      const int64_t j0 = (int64_t)b * a.chunk;
-      const int64_t j1 = min(d, j0 + a.chunk);
+    {
       double lw2 = 0.0, lr2 = 0.0;
       for (int64_t j = j0 + threadIdx.x; j < j1; j += kVecThreads) {
-        const C rj = (C)fma(a.rho, __ldcg(a.z + j) - __ldcg(a.u + j), a.q[j]);
+        const C rj = (C)fma(a.rho, a.z[j] - a.u[j], a.q[j]);
         rc[j] = rj;
         const C wj = rj - hx[j];
         lr2 += (double)rj * (double)rj;
@@ -1167,38 +1208,36 @@ __global__ void __launch_bounds__(kVecThreads) admm_head_kernel(HeadArgs a, cons
         a.part_r2[b] = tr2;
       }
     }
-    if (!grid_barrier(&ctl->bar_count, &ctl->bar_gen, nblk)) return fail();
-    if (first && refreshed && b == 0 && threadIdx.x == 0) ctl->hx_pending = 0;
+    if (!barrier()) return fail();
+    if (first && b == 0 && threadIdx.x == 0) {
+      if (refreshed) ctl->hx_pending = 0;
+      ctl->hx_skip = 0;   // inline_hx: x leaves 0 in this iteration, later passes recompute
+    }
     first = false;
     // ---- 2. stop decision of the warm start (every block, the order of pcg_scalar_body)
-    double w2, r2;
-    block_fixed_sum2_cg(a.part_w2, a.part_r2, a.nb3, &w2, &r2, slot2);
+    const double* const src[2] = {a.part_w2, a.part_r2};
+    double v2[2];
+    block_fixed_sums_cg<2>(src, a.nb, v2, slot2);
+    const double w2 = v2[0], r2 = v2[1];
     const double thresh2 = tol_abs ? tolk * tolk : tolk * tolk * r2;
     const int fixed = a.fixed_dev ? a.fixed_dev[k] : -1;
     const bool nostep = fixed >= 0 ? fixed == 0 : !(w2 > thresh2);
     if (!nostep) {
       // ---- 3b. P^{-1} w and the PCG state; the PCG WHILE node takes over.  U^T w partials
       // over the blocks' chunks of w (the mapping and order of pcg_update_kernel's init step)
-      if (b < a.nb3) {
-        const int64_t j0 = (int64_t)b * a.chunk;
-        const int64_t j1 = min(d, j0 + a.chunk);
-        for (int64_t j = j0 + threadIdx.x; j < j1; j += kVecThreads) wch[j - j0] = __ldcg(w + j);
-        __syncthreads();
-        utw_partials<C>(wch, (int)(j1 - j0), U, d, j0, s, a.part_g + (int64_t)b * s);
-      }
-      if (!grid_barrier(&ctl->bar_count, &ctl->bar_gen, nblk)) return fail();
+      utw_partials<C>(wch, (int)(j1 - j0), U, d, j0, s, part_g + (int64_t)b * s);
+      if (!barrier()) return fail();
       for (int i = threadIdx.x; i < s; i += kVecThreads) {
-        const double gsum = sum_strided_fixed<true>(a.part_g, a.nb3, s, i, 0.0);
-        const C gi = (C)((double)cvec[i] * gsum);
-        wch[i] = gi;
+        const C gi = g_entry<C>(part_g, a.nb, s, i, cvec[i]);
+        gsh[i] = gi;
         if (b == 0) gs[i] = gi;
       }
       __syncthreads();
-      if (b < a.nb5) {
+      {
         double lwy = 0.0;
-        for (int64_t j = b * (int64_t)kVecThreads + threadIdx.x; j < d; j += (int64_t)a.nb5 * kVecThreads) {
-          const C wj = __ldcg(w + j);
-          const C acc = urow_dot(U, d, j, s, wch, wj);
+        for (int64_t j = j0 + threadIdx.x; j < j1; j += kVecThreads) {
+          const C wj = wch[j - j0];
+          const C acc = urow_dot(U, d, j, s, gsh, wj);
           y[j] = acc;
           p[j] = acc;
           lwy += (double)wj * (double)acc;
@@ -1221,36 +1260,26 @@ __global__ void __launch_bounds__(kVecThreads) admm_head_kernel(HeadArgs a, cons
         st->fixed = fixed;
         st->ticket[0] = 0u;
         st->ticket[1] = 0u;
-        ctl->nodes += 1;
-        cudaGraphSetConditional(a.h_hx, 0u);
+        ctl->nodes += a.inline_hx ? 3 : 1;
+        if (!a.inline_hx) cudaGraphSetConditional(a.h_hx, 0u);
         cudaGraphSetConditional(a.h_pcg, 1u);
         if (a.has_zu) cudaGraphSetConditional(a.h_zu, 1u);
       }
       return;
     }
     // ---- 3a. prox / dual step with x unchanged, residual partials
-    if (b < a.nbz) {
+    {
       double* zt = a.ztrace ? a.ztrace + (int64_t)k * d : nullptr;
-      double a0 = 0, a1 = 0, a2 = 0, a3 = 0, a4 = 0;
-      for (int64_t j = b * (int64_t)kVecThreads + threadIdx.x; j < d; j += (int64_t)a.nbz * kVecThreads) {
+      double a5[5] = {0, 0, 0, 0, 0};
+      for (int64_t j = j0 + threadIdx.x; j < j1; j += kVecThreads) {
         const double xj = (double)xc[j];
-        const double zo = __ldcg(a.z + j);
-        const double uo = __ldcg(a.u + j);
-        const double vj = xj + uo;
-        const double mag = fabs(vj) - a.kappa;
-        const double zj = mag > 0.0 ? copysign(mag, vj) : 0.0;
-        const double uj = uo + xj - zj;
+        double zj, uj;
+        zu_element(xj, a.z[j], a.u[j], a.kappa, zj, uj, a5);
         a.x[j] = xj;
         a.z[j] = zj;
         a.u[j] = uj;
         if (zt) zt[j] = zj;
-        a0 += (xj - zj) * (xj - zj);
-        a1 += (zj - zo) * (zj - zo);
-        a2 += xj * xj;
-        a3 += zj * zj;
-        a4 += uj * uj;
       }
-      double a5[5] = {a0, a1, a2, a3, a4};
       block_sum5(a5);
       if (threadIdx.x == 0) {
         double* o = a.part5 + (int64_t)b * 5;
@@ -1258,11 +1287,11 @@ __global__ void __launch_bounds__(kVecThreads) admm_head_kernel(HeadArgs a, cons
         for (int t = 0; t < 5; ++t) o[t] = a5[t];
       }
     }
-    if (!grid_barrier(&ctl->bar_count, &ctl->bar_gen, nblk)) return fail();
+    if (!barrier()) return fail();
     // ---- 4. scalars of the iteration (every block; block 0 records them)
     if (threadIdx.x < 32) {
       double sums[5];
-      sum_part5(a.nbz, a.part5, sums);
+      sum_part5(a.nb, a.part5, sums);
       if (threadIdx.x == 0) {
         const double rp = sqrt(sums[0]);
         const double rd = a.rho * sqrt(sums[1]);
@@ -1292,9 +1321,9 @@ __global__ void __launch_bounds__(kVecThreads) admm_head_kernel(HeadArgs a, cons
     k += 1;
     if (!go) {
       if (b == 0 && threadIdx.x == 0) {
-        ctl->nodes += 1;
+        ctl->nodes += a.inline_hx ? 3 : 1;
         cudaGraphSetConditional(a.h_admm, 0u);
-        cudaGraphSetConditional(a.h_hx, 0u);
+        if (!a.inline_hx) cudaGraphSetConditional(a.h_hx, 0u);
         cudaGraphSetConditional(a.h_pcg, 0u);
         if (a.has_zu) cudaGraphSetConditional(a.h_zu, 0u);
       }
@@ -1388,28 +1417,25 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
   const int s = g.P.s;
   const C* U = reinterpret_cast<const C*>(g.P.U);
   const C* cvec = reinterpret_cast<const C*>(g.P.c);
-  const int chunk = upd_chunk(d);
-  const int nb3 = (int)((d + chunk - 1) / chunk);
-  const int nbr = reduce_blocks(d);
-  const int nb5 = nbr;
-  const int nbz = admm_blocks(d);
+  const int chunk = vec_chunk(d);
+  const int nb = vec_blocks(d);
   const int K = g.K;
   C* w = pool.alloc<C>(d);
   C* y = pool.alloc<C>(d);
   C* p = pool.alloc<C>(d);
   C* v = pool.alloc<C>(d);
   C* gs = pool.alloc<C>(std::max(1, s));
-  double* part_w2 = pool.alloc<double>(nb3);
-  double* part_r2 = pool.alloc<double>(nb3);
-  double* part_g = pool.alloc<double>((size_t)nb3 * std::max(1, s));
-  double* pv_part = pool.alloc<double>(nbr);
-  double* wy_part = pool.alloc<double>(nb5);
+  double* part_w2 = pool.alloc<double>(nb);
+  double* part_r2 = pool.alloc<double>(nb);
+  C* part_g = pool.alloc<C>((size_t)nb * std::max(1, s));
+  double* pv_part = pool.alloc<double>(nb);
+  double* wy_part = pool.alloc<double>(nb);
   void* apart = pool.alloc<unsigned char>(apass_partial_bytes(g.pb.A, g.pb.plan));
   void* apart_ref = g.Aref ? pool.alloc<unsigned char>(apass_partial_bytes(g.Aref, g.plan_ref)) : nullptr;
   PcgState* st = pool.alloc<PcgState>(1);
   AdmmCtl* ctl = pool.alloc<AdmmCtl>(1);
   int* dstat = pool.alloc<int>(1);
-  double* part5 = pool.alloc<double>((size_t)nbz * 5);
+  double* part5 = pool.alloc<double>((size_t)nb * 5);
   int* fixed_dev = g.fixed_host ? pool.alloc<int>(K) : nullptr;
   double* tolpow = g.tol_mode == NYS_TOL_RNORM_POW && K > 0 ? pool.alloc<double>(K) : nullptr;
   if (!pool.ok()) return NYS_ENOMEM;
@@ -1428,6 +1454,7 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
     }                                                                                        \
   } while (0)
   G_OK(cudaMemsetAsync(ctl, 0, sizeof(AdmmCtl), stream));
+  G_OK(cudaMemsetAsync(&ctl->hx_skip, 1, sizeof(int), stream));   // x = 0 at first: nothing to recompute
   G_OK(cudaMemsetAsync(st, 0, sizeof(PcgState), stream));   // the post kernel's barrier words start at 0
   G_OK(cudaMemsetAsync(dstat, 0, sizeof(int), stream));
   G_OK(cudaMemsetAsync(hx, 0, d * sizeof(C), stream));
@@ -1467,37 +1494,77 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
   aa.t_out = nullptr;
   aa.mode = g.pb.D ? MODE_DIAG : MODE_ID;
 
-  // One PCG iteration after its A-pass as one cooperative launch (pcg_post_kernel) instead of
-  // the reduce, update and tail kernels, for a single instance (its grid barriers want the
-  // grid co-resident; concurrent graph branches keep the separate kernels).  NYS_PCG_POST=0
-  // selects the separate kernels.
-  const int nbp = std::max(std::max(nbr, nb3), std::max(nb5, nbz));
-  const size_t sm_post = (size_t)std::max(chunk, std::max(1, s)) * sizeof(C);
-  bool use_post = g.allow_nostep && nbz <= kPart5Max;
+  // A fused vector kernel over nb blocks: one cluster when it fits, else a cooperative grid when
+  // the device can hold it at once (cl, ok).
+  struct Fused {
+    bool ok = false, cl = false;
+  };
+  auto fused_fits = [&](const void* fn_cl, const void* fn_grid, size_t smem, Fused* f) -> cudaError_t {
+    if (nb <= kClusterBlocks) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)nb);
+      cfg.blockDim = dim3(kVecThreads);
+      cfg.dynamicSmemBytes = smem;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = (unsigned)nb;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, fn_cl, &cfg) == cudaSuccess && n >= 1) {
+        f->ok = f->cl = true;
+        return cudaSuccess;
+      }
+      (void)cudaGetLastError();
+    }
+    int per_sm = 0, coop = 0;
+    NYS_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, current_device()));
+    NYS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn_grid, kVecThreads, smem));
+    f->ok = coop && (int64_t)per_sm * sm_count() >= nb;
+    return cudaSuccess;
+  };
+  auto fused_config = [&](const Fused& f, size_t smem, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at) {
+    *cfg = cudaLaunchConfig_t{};
+    cfg->gridDim = dim3((unsigned)nb);
+    cfg->blockDim = dim3(kVecThreads);
+    cfg->dynamicSmemBytes = smem;
+    cfg->stream = cap;
+    if (f.cl) {
+      at->id = cudaLaunchAttributeClusterDimension;
+      at->val.clusterDim.x = (unsigned)nb;
+      at->val.clusterDim.y = 1;
+      at->val.clusterDim.z = 1;
+    } else {
+      at->id = cudaLaunchAttributeCooperative;
+      at->val.cooperative = 1;
+    }
+    cfg->attrs = at;
+    cfg->numAttrs = 1;
+  };
+  // One PCG iteration after its A-pass as one launch (pcg_post_kernel) instead of the reduce,
+  // update and tail kernels.  A cooperative grid wants the device to itself, so concurrent graph
+  // branches take it only as a cluster.  NYS_PCG_POST=0 selects the separate kernels.
+  const size_t sm_post = ((size_t)chunk + std::max(1, s)) * sizeof(C);
+  Fused post;
   {
     const char* pe = std::getenv("NYS_PCG_POST");
-    if (pe && std::atoi(pe) == 0) use_post = false;
-    if (use_post) {
-      int per_sm = 0, coop = 0;
-      G_OK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, current_device()));
-      G_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pcg_post_kernel<C>, kVecThreads, sm_post));
-      use_post = coop && (int64_t)per_sm * sm_count() >= nbp;
-    }
+    if (nb <= kPart5Max && !(pe && std::atoi(pe) == 0))
+      G_OK(fused_fits((const void*)pcg_post_kernel<C, true>, (const void*)pcg_post_kernel<C, false>, sm_post, &post));
+    if (!g.allow_nostep && !post.cl) post.ok = false;
   }
+  const bool use_post = post.ok;
   PostArgs<C> pa = {};
   pa.d = d;
   pa.chunk = chunk;
-  pa.nbr = nbr;
-  pa.nb3 = nb3;
-  pa.nb5 = nb5;
-  pa.nbz = nbz;
+  pa.nb = nb;
   pa.partial = reinterpret_cast<const C*>(apart);
   pa.G = g.pb.plan.grid;
   pa.dpad = g.pb.plan.dpad;
   pa.rho = (C)(g.rho + g.mu);
   pa.cscale = g.pb.A->dtype == NYS_FP8E4M3 ? g.pb.A->col_scale : nullptr;
   pa.p = p;
-  pa.v = v;
   pa.x = xc;
   pa.w = w;
   pa.hx = hx;
@@ -1531,17 +1598,11 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
     q.cond = hc;
     q.zu = zu;
     q.h_admm = ha;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)nbp);
-    cfg.blockDim = dim3(kVecThreads);
-    cfg.dynamicSmemBytes = sm_post;
-    cfg.stream = cap;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, pcg_post_kernel<C>, q);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[1];
+    fused_config(post, sm_post, &cfg, at);
+    return post.cl ? cudaLaunchKernelEx(&cfg, pcg_post_kernel<C, true>, q)
+                   : cudaLaunchKernelEx(&cfg, pcg_post_kernel<C, false>, q);
   };
 
   // Fast body (tracked warm start, no refined step or warm-start model, a single instance):
@@ -1554,18 +1615,20 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
   {
     const bool use_model = (g.warm || g.warm_record) && s > 0;
     const char* env = std::getenv("NYS_ADMM_NOSTEP");
-    bool fast = !g.Aref && !use_model && g.hx_refresh > 0 && g.allow_nostep && !(env && std::atoi(env) == 0);
-    const int nbf = std::max(std::max(nb3, nbz), nbr);
-    const size_t sm_head = (size_t)std::max(chunk, std::max(1, s)) * sizeof(C);
+    // hx_refresh = 0 (the residual recomputed in every iteration): the pass runs ahead of the
+    // head kernel in every body pass, skipped while x = 0, and needs the post kernel's prox step
+    const bool inline_hx = g.hx_refresh == 0;
+    bool fast = !g.Aref && !use_model && (!inline_hx || use_post) && nb <= kPart5Max && !(env && std::atoi(env) == 0);
+    const size_t sm_head = ((size_t)chunk + std::max(1, s)) * sizeof(C);
+    Fused headf;
     if (fast) {
-      int per_sm = 0, coop = 0;
-      G_OK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, current_device()));
-      G_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, admm_head_kernel<C>, kVecThreads, sm_head));
-      fast = coop && (int64_t)per_sm * sm_count() >= nbf && nbz <= kPart5Max;
+      G_OK(fused_fits((const void*)admm_head_kernel<C, true>, (const void*)admm_head_kernel<C, false>, sm_head, &headf));
+      if (!g.allow_nostep && !headf.cl) headf.ok = false;
+      fast = headf.ok;
     }
     if (fast) {
-      cudaGraphConditionalHandle h_hx, h_zu = 0;
-      G_OK(cudaGraphConditionalHandleCreate(&h_hx, body, 0u, 0u));
+      cudaGraphConditionalHandle h_hx = 0, h_zu = 0;
+      if (!inline_hx) G_OK(cudaGraphConditionalHandleCreate(&h_hx, body, 0u, 0u));
       G_OK(cudaGraphConditionalHandleCreate(&h_pcg, body, 0u, 0u));
       // a handle must belong to a conditional node: h_zu only with the IF (h_zu) node
       if (!use_post) G_OK(cudaGraphConditionalHandleCreate(&h_zu, body, 0u, 0u));
@@ -1584,12 +1647,17 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
       // default, so no conditional node may be evaluated before the kernel has run)
       count_launch_suspend(true);
       G_OK(cudaStreamBeginCaptureToGraph(cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+      if (inline_hx) {
+        // (H + rho I) x with one pass over A, skipped in the first iteration (x = 0, hx = 0)
+        aa.p = xc;
+        aa.skip = &ctl->hx_skip;
+        G_OK(apass_run(aa, g.pb.plan, apart, nullptr, dstat, cap, true));
+        G_OK(apass_reduce(aa, g.pb.plan, apart, g.rho + g.mu, hx, nullptr, cap));
+      }
       HeadArgs ha;
       ha.d = d;
       ha.chunk = chunk;
-      ha.nb3 = nb3;
-      ha.nbz = nbz;
-      ha.nb5 = nb5;
+      ha.nb = nb;
       ha.s = s;
       ha.q = g.q;
       ha.x = g.x;
@@ -1599,7 +1667,6 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
       ha.kappa = g.gamma / g.rho;
       ha.part_w2 = part_w2;
       ha.part_r2 = part_r2;
-      ha.part_g = part_g;
       ha.wy_part = wy_part;
       ha.part5 = part5;
       ha.ctl = ctl;
@@ -1624,17 +1691,16 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
       ha.h_zu = h_zu;
       ha.has_zu = use_post ? 0 : 1;
       ha.h_hx = h_hx;
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)nbf);
-      cfg.blockDim = dim3(kVecThreads);
-      cfg.dynamicSmemBytes = sm_head;
-      cfg.stream = cap;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeCooperative;
-      attr[0].val.cooperative = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      G_OK(cudaLaunchKernelEx(&cfg, admm_head_kernel<C>, ha, (const C*)xc, (const C*)hx, w, rc, y, p, U, cvec, gs));
+      ha.inline_hx = inline_hx ? 1 : 0;
+      cudaLaunchConfig_t cfg;
+      cudaLaunchAttribute at[1];
+      fused_config(headf, sm_head, &cfg, at);
+      if (headf.cl)
+        G_OK(cudaLaunchKernelEx(&cfg, admm_head_kernel<C, true>, ha, (const C*)xc, (const C*)hx, w, rc, y, p, U, cvec, gs,
+                                part_g));
+      else
+        G_OK(cudaLaunchKernelEx(&cfg, admm_head_kernel<C, false>, ha, (const C*)xc, (const C*)hx, w, rc, y, p, U, cvec, gs,
+                                part_g));
       cudaStreamCaptureStatus cst0;
       const cudaGraphNode_t* deps0 = nullptr;
       size_t ndeps0 = 0;
@@ -1642,19 +1708,23 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
       std::vector<cudaGraphNode_t> leaf0(deps0, deps0 + ndeps0);
       G_OK(cudaStreamEndCapture(cap, &body));
       // IF (h_hx): (H + rho I) x with one pass over A, when the head kernel asked for it
-      cudaGraphNode_t n_hx;
-      cudaGraph_t hbody;
-      G_OK(add_cond(h_hx, cudaGraphCondTypeIf, leaf0, &n_hx, &hbody));
-      G_OK(cudaStreamBeginCaptureToGraph(cap, hbody, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-      aa.p = xc;
-      aa.skip = nullptr;
-      G_OK(apass_run(aa, g.pb.plan, apart, nullptr, dstat, cap, true));
-      G_OK(apass_reduce(aa, g.pb.plan, apart, g.rho + g.mu, hx, nullptr, 0, cap));
-      G_OK(cudaStreamEndCapture(cap, &hbody));
+      std::vector<cudaGraphNode_t> before_pcg = leaf0;
+      if (!inline_hx) {
+        cudaGraphNode_t n_hx;
+        cudaGraph_t hbody;
+        G_OK(add_cond(h_hx, cudaGraphCondTypeIf, leaf0, &n_hx, &hbody));
+        G_OK(cudaStreamBeginCaptureToGraph(cap, hbody, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+        aa.p = xc;
+        aa.skip = nullptr;
+        G_OK(apass_run(aa, g.pb.plan, apart, nullptr, dstat, cap, true));
+        G_OK(apass_reduce(aa, g.pb.plan, apart, g.rho + g.mu, hx, nullptr, cap));
+        G_OK(cudaStreamEndCapture(cap, &hbody));
+        before_pcg = {n_hx};
+      }
       // WHILE (h_pcg): PCG iterations
       cudaGraphNode_t n_pcg;
       cudaGraph_t pbody;
-      G_OK(add_cond(h_pcg, cudaGraphCondTypeWhile, {n_hx}, &n_pcg, &pbody));
+      G_OK(add_cond(h_pcg, cudaGraphCondTypeWhile, before_pcg, &n_pcg, &pbody));
       G_OK(cudaStreamBeginCaptureToGraph(cap, pbody, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
       aa.p = p;
       aa.skip = &st->done;
@@ -1664,11 +1734,11 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
         G_OK(launch_post(h_pcg, 1, h_admm));
         G_OK(cudaStreamEndCapture(cap, &pbody));
       } else {
-        G_OK(apass_reduce(aa, g.pb.plan, apart, g.rho + g.mu, v, pv_part, nbr, cap));
-        pcg_update_kernel<C><<<nb3, kVecThreads, (size_t)chunk * sizeof(C), cap>>>(
-            0, d, chunk, xc, w, rc, v, p, U, s, pv_part, nbr, wy_part, nb5, part_w2, part_r2, part_g, st, hx, cvec, gs,
+        G_OK(apass_reduce(aa, g.pb.plan, apart, g.rho + g.mu, v, pv_part, cap));
+        pcg_update_kernel<C><<<nb, kVecThreads, (size_t)chunk * sizeof(C), cap>>>(
+            0, d, chunk, xc, w, rc, v, p, U, s, pv_part, wy_part, part_w2, part_r2, part_g, st, hx, cvec, gs,
             h_pcg, 1, nullptr, nullptr, nullptr, 0.0, (C*)nullptr);
-        pcg_tail_kernel<C><<<nb5, kVecThreads, (size_t)std::max(1, s) * sizeof(C), cap>>>(d, w, y, U, s, gs, wy_part,
+        pcg_tail_kernel<C><<<nb, kVecThreads, (size_t)std::max(1, s) * sizeof(C), cap>>>(d, chunk, w, y, U, s, gs, wy_part,
                                                                                          st, 0, p);
         G_OK(cudaStreamEndCapture(cap, &pbody));
         // IF (h_zu): prox / dual step of an iteration that took PCG steps
@@ -1676,7 +1746,7 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
         cudaGraph_t zbody;
         G_OK(add_cond(h_zu, cudaGraphCondTypeIf, {n_pcg}, &n_zu, &zbody));
         G_OK(cudaStreamBeginCaptureToGraph(cap, zbody, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-        admm_zu_g_kernel<C><<<nbz, kVecThreads, 0, cap>>>(d, xc, 0, g.x, g.z, g.u, g.gamma / g.rho, g.ztrace, ctl,
+        admm_zu_g_kernel<C><<<nb, kVecThreads, 0, cap>>>(d, chunk, xc, 0, g.x, g.z, g.u, g.gamma / g.rho, g.ztrace, ctl,
                                                           part5, g.rho, K, g.eps_abs, g.eps_rel, g.rp, g.rd, g.pcg_it,
                                                           st, 1, 4, h_admm);
         G_OK(cudaStreamEndCapture(cap, &zbody));
@@ -1720,7 +1790,7 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
     G_OK(apass_run(ar, g.plan_ref, apart_ref, nullptr, dstat, cap, true));
     ApassArgs ar2 = ar;
     ar2.p = nullptr;
-    G_OK(apass_reduce(ar2, g.plan_ref, apart_ref, 0.0, g.yres, nullptr, 0, cap));
+    G_OK(apass_reduce(ar2, g.plan_ref, apart_ref, 0.0, g.yres, nullptr, cap));
     seg_nodes += 2;
   }
   const bool use_ws = (g.warm || g.warm_record) && s > 0;
@@ -1728,7 +1798,7 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
   // PCG-init update kernel itself (one launch fewer per iteration)
   const bool fuse_rhs = !refine && !use_ws;
   if (!fuse_rhs) {
-    admm_rhs_g_kernel<C><<<nbz, kVecThreads, 0, cap>>>(d, g.q, g.z, g.u, g.rho, g.mu, g.x, g.yres, refine, rc, xc,
+    admm_rhs_g_kernel<C><<<reduce_blocks(d), kVecThreads, 0, cap>>>(d, g.q, g.z, g.u, g.rho, g.mu, g.x, g.yres, refine, rc, xc,
                                                         hx);
     ++seg_nodes;
   }
@@ -1755,10 +1825,10 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
       if (!pool.ok()) return NYS_ENOMEM;
       ws_proj_kernel<C><<<s, kVecThreads, 0, cap>>>(d, s, U, xc, (const C*)nullptr, uxp);
       G_OK(mlp_forward_dev(g.warm, feat, 1, mlp_buf, mlp_buf + 1024, mlp_buf + 2048, mlp_buf + 3072, cout, cap));
-      ws_apply_kernel<C><<<nbz, kVecThreads, 0, cap>>>(d, s, U, cout, uxp, rnorm, g.rho, xc, xprev, ctl, h_hx, 2);
+      ws_apply_kernel<C><<<reduce_blocks(d), kVecThreads, 0, cap>>>(d, s, U, cout, uxp, rnorm, g.rho, xc, xprev, ctl, h_hx, 2);
       seg_nodes += 5;
     } else {
-      ws_copy_kernel<C><<<nbz, kVecThreads, 0, cap>>>(d, xc, xprev);
+      ws_copy_kernel<C><<<reduce_blocks(d), kVecThreads, 0, cap>>>(d, xc, xprev);
       ++seg_nodes;
     }
   }
@@ -1783,15 +1853,15 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
     aa.p = xc;
     aa.skip = nullptr;
     G_OK(apass_run(aa, g.pb.plan, apart, nullptr, dstat, cap, true));
-    G_OK(apass_reduce(aa, g.pb.plan, apart, g.rho + g.mu, hx, nullptr, 0, cap));
+    G_OK(apass_reduce(aa, g.pb.plan, apart, g.rho + g.mu, hx, nullptr, cap));
     G_OK(cudaStreamEndCapture(cap, &hbody));
     G_OK(cudaStreamBeginCaptureToGraph(cap, body, &n_hx, nullptr, 1, cudaStreamCaptureModeRelaxed));
   }
-  pcg_update_kernel<C><<<nb3, kVecThreads, sm_upd, cap>>>(1, d, chunk, xc, w, rc, hx, p, U, s, pv_part, nbr,
-                                                          wy_part, nb5, part_w2, part_r2, part_g, st, (C*)nullptr,
+  pcg_update_kernel<C><<<nb, kVecThreads, sm_upd, cap>>>(1, d, chunk, xc, w, rc, hx, p, U, s, pv_part,
+                                                          wy_part, part_w2, part_r2, part_g, st, (C*)nullptr,
                                                           cvec, gs, h_pcg, 1, fuse_rhs ? g.q : nullptr,
                                                           fuse_rhs ? g.z : nullptr, fuse_rhs ? g.u : nullptr, g.rho, rc);
-  pcg_tail_kernel<C><<<nb5, kVecThreads, sm_tail, cap>>>(d, w, y, U, s, gs, wy_part, st, 1, p);
+  pcg_tail_kernel<C><<<nb, kVecThreads, sm_tail, cap>>>(d, chunk, w, y, U, s, gs, wy_part, st, 1, p);
   seg_nodes += 2;
   cudaStreamCaptureStatus cst;
   const cudaGraphNode_t* deps = nullptr;
@@ -1817,11 +1887,11 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
     G_OK(launch_post(h_pcg, 0, h_admm));
     body_nodes = 2;
   } else {
-    G_OK(apass_reduce(aa, g.pb.plan, apart, g.rho + g.mu, v, pv_part, nbr, cap));
-    pcg_update_kernel<C><<<nb3, kVecThreads, sm_upd, cap>>>(0, d, chunk, xc, w, rc, v, p, U, s, pv_part, nbr, wy_part,
-                                                            nb5, part_w2, part_r2, part_g, st, hx, cvec, gs, h_pcg, 1,
+    G_OK(apass_reduce(aa, g.pb.plan, apart, g.rho + g.mu, v, pv_part, cap));
+    pcg_update_kernel<C><<<nb, kVecThreads, sm_upd, cap>>>(0, d, chunk, xc, w, rc, v, p, U, s, pv_part, wy_part,
+                                                            part_w2, part_r2, part_g, st, hx, cvec, gs, h_pcg, 1,
                                                             nullptr, nullptr, nullptr, 0.0, (C*)nullptr);
-    pcg_tail_kernel<C><<<nb5, kVecThreads, sm_tail, cap>>>(d, w, y, U, s, gs, wy_part, st, 0, p);
+    pcg_tail_kernel<C><<<nb, kVecThreads, sm_tail, cap>>>(d, chunk, w, y, U, s, gs, wy_part, st, 0, p);
     body_nodes = 4;
   }
   G_OK(cudaStreamEndCapture(cap, &pbody));
@@ -1834,7 +1904,7 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
     seg_nodes += 2;
   }
   seg_nodes += 1;
-  admm_zu_g_kernel<C><<<nbz, kVecThreads, 0, cap>>>(d, xc, refine, g.x, g.z, g.u, g.gamma / g.rho, g.ztrace, ctl,
+  admm_zu_g_kernel<C><<<nb, kVecThreads, 0, cap>>>(d, chunk, xc, refine, g.x, g.z, g.u, g.gamma / g.rho, g.ztrace, ctl,
                                                     part5, g.rho, K, g.eps_abs, g.eps_rel, g.rp, g.rd, g.pcg_it, st,
                                                     seg_nodes, body_nodes, h_admm);
   G_OK(cudaStreamEndCapture(cap, &body));

@@ -110,8 +110,6 @@ cudaError_t admm_zu(int64_t d, const C* xc, int accumulate, double* x, double* z
                     double* ztrace, double* part5, cudaStream_t st);
 cudaError_t admm_scalar(int64_t d, const double* part5, double rho, int k, double* rp, double* rd, double* eps_next,
                         double eps_abs, double eps_rel, int* stop, cudaStream_t st);
-int admm_blocks(int64_t d);
-int pcg_nb3(int64_t d);
 
 PcgState* host_state();
 
