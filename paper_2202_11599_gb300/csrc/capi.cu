@@ -114,6 +114,7 @@ nys_status cholqr2(double* Om, int64_t d, int m, cudaStream_t st, bool fp32_clas
   double* work = pool.alloc<double>(gram_work_bytes(d, m) / sizeof(double) + 1);
   int* info = pool.alloc<int>(2);   // Cholesky; waits of the products
   double* gap = pool.alloc<double>(1);
+  void* tw = pool.alloc<unsigned char>(trsm_work_bytes(d, m));
   if (!pool.ok()) return NYS_ENOMEM;
   NYS_CU(cudaMemsetAsync(info, 0, 2 * sizeof(int), st));
   for (int pass = 0; pass < 2; ++pass) {
@@ -133,7 +134,7 @@ nys_status cholqr2(double* Om, int64_t d, int m, cudaStream_t st, bool fp32_clas
     NYS_CU(cudaStreamSynchronize(st));
     if (info_h[1]) return (nys_status)info_h[1];
     if (info_h[0] != 0) return NYS_EINVAL;  // Omega has (numerically) dependent columns
-    NYS_CU(trsm_right_upper(G, m, Om, d, st));
+    NYS_CU(trsm_right_upper(G, m, Om, d, tw, info + 1, st));
   }
   return NYS_OK;
 }
@@ -208,6 +209,7 @@ nys_status nystrom_core(const double* Om, const double* Y, int64_t d, int s, dou
   double* V = pool.alloc<double>((size_t)N * N);
   double* jw = pool.alloc<double>(jacobi_work_bytes(s) / sizeof(double) + 1);
   double* fw = pool.alloc<double>(finish_work_bytes(d, s) / sizeof(double) + 1);
+  void* tw = pool.alloc<unsigned char>(trsm_work_bytes(d, s));
   if (!pool.ok()) return NYS_ENOMEM;
   NYS_CU(cudaMemsetAsync(info, 0, 2 * sizeof(int), st));
 
@@ -242,7 +244,7 @@ nys_status nystrom_core(const double* Om, const double* Y, int64_t d, int s, dou
   if (!ok) return NYS_ENOTSPD;
   {
     PhaseTimer pt("core: trsm + B^T B", st);
-    NYS_CU(trsm_right_upper(M, s, Ynu, d, st));       // B = Y_nu C^{-1} (in Ynu)
+    NYS_CU(trsm_right_upper(M, s, Ynu, d, tw, status, st));   // B = Y_nu C^{-1} (in Ynu)
     NYS_CU(gram_xty(Ynu, Ynu, d, s, G, gw, status, st));      // B^T B
   }
   int sweeps = 0;

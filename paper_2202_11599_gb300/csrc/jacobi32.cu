@@ -4,19 +4,19 @@
 //
 // A round of the FP64 sweeps costs ~4.3 us whatever the size (grid barrier, L2 loads, the FP64
 // square root of the rotation), so a 200 x 200 eigensolve took 9 x 199 of them, 8.1 ms.  Here
-// everything stays on chip in FP32: L L^T = G + eps I (one CTA, packed in shared memory), then
-// one-sided Jacobi (Hestenes) on the columns of L in one thread-block cluster, one warp per pair
-// of columns, the columns in registers.  A round is three dot products, a rotation and the
-// systolic exchange of the round-robin order (each warp passes one column to each neighbour
-// through the neighbour's shared memory, across CTAs through distributed shared memory), with one
-// cluster barrier.  The left singular vectors of L -- the normalised columns at the end -- are the
-// eigenvectors of G, so no V is carried, and starting from the Cholesky factor saves a third of
-// the sweeps (Drmac and Veselic, SIAM J. Matrix Anal. Appl. 29, 2008).  eps = 1e-3 trace(G)
-// leaves the eigenvectors as they are and keeps the small columns above FP32 rounding.
-// V0 is then orthonormalised in FP64 (three Newton-Schulz steps: the columns leave the FP32
-// stage orthogonal to 1e-6 .. 3e-4 over spectra from flat to (1 + j)^-4) and checked on the
-// device: if V0^T V0 is off the identity by more than 1e-13 the sweeps start from the identity
-// instead, as they do without this stage.  The accuracy of the result is that of the sweeps.
+// everything stays on chip in FP32: one-sided Jacobi (Hestenes) on the columns of the Cholesky
+// factor L of G + eps I in one thread-block cluster, one warp per pair of columns, the columns in
+// registers.  A round is three dot products, a rotation and the systolic exchange of the
+// round-robin order (each warp passes one column to each neighbour through the neighbour's shared
+// memory, across CTAs through distributed shared memory), with one cluster barrier.  The left
+// singular vectors of L -- the normalised columns at the end -- are the eigenvectors of G, so no
+// V is carried, and starting from the Cholesky factor saves a third of the sweeps (Drmac and
+// Veselic, SIAM J. Matrix Anal. Appl. 29, 2008).  L is factored in FP64 and rounded, and the
+// rotation test is relative, so small eigenpairs are as accurate as large ones; eps = 1e-7
+// trace(G) leaves the eigenvectors as they are and keeps a singular G's columns above rounding.
+// V0 is then orthonormalised in FP64 (two Newton-Schulz steps: the columns leave the FP32 stage
+// orthogonal to 1e-6 .. 1e-4) and checked on the device: if V0^T V0 is off the identity by more
+// than 1e-13 the sweeps start from the identity instead, as they do without this stage.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -28,74 +28,9 @@ namespace nys {
 namespace {
 namespace cg = cooperative_groups;
 
-constexpr float kJacRidge = 1e-3f;   // eps / trace(G)
-constexpr float kJacSkip = 1e-8f;    // entries of L^T L (largest diagonal of G: 1) below rounding
-constexpr float kJacAgain = 1e-5f;   // a sweep that met none above this was the last (quadratic)
-
-// L (N x N FP32, column-major, lower) with L L^T = 2^-ex (G + eps I), G symmetrised, 2^ex the
-// scale of its largest diagonal entry; zero when that is zero or not finite.  Rows and columns
-// from s on are those of the identity times sqrt(eps).  Right-looking, packed by columns.
-__global__ void __launch_bounds__(1024) chol32_kernel(const double* __restrict__ G, int s, int N, float* __restrict__ L) {
-  extern __shared__ float lo[];
-  __shared__ double smx[32], str[32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  auto at = [N](int i, int c) { return c * N - c * (c - 1) / 2 + (i - c); };
-  double mx = 0.0, tr = 0.0;
-  for (int i = tid; i < s; i += blockDim.x) {
-    const double g = G[i + (int64_t)i * s];
-    tr += g;
-    mx = fabs(g) > mx || g != g ? fabs(g) : mx;
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    const double m2 = __shfl_xor_sync(0xffffffffu, mx, o);
-    mx = m2 > mx || m2 != m2 ? m2 : mx;
-    tr += __shfl_xor_sync(0xffffffffu, tr, o);
-  }
-  if (lane == 0) {
-    smx[warp] = mx;
-    str[warp] = tr;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    mx = tr = 0.0;
-    for (int w = 0; w < nw; ++w) {
-      mx = smx[w] > mx || smx[w] != smx[w] ? smx[w] : mx;
-      tr += str[w];
-    }
-    smx[0] = mx;
-    str[0] = tr;
-  }
-  __syncthreads();
-  mx = smx[0];
-  tr = str[0];
-  const bool plain = mx > 0.0 && isfinite(mx) && isfinite(tr);
-  int ex = 0;
-  if (plain) frexp(mx, &ex);
-  const float eps = plain ? kJacRidge * (float)scalbn(tr, -ex) : 0.f;
-  for (int c = warp; c < N; c += nw)
-    for (int i = c + lane; i < N; i += 32) {
-      float v = (plain && i < s && c < s)
-                    ? (float)scalbn(0.5 * (G[i + (int64_t)c * s] + G[c + (int64_t)i * s]), -ex) : 0.f;
-      if (i == c) v += eps;
-      lo[at(i, c)] = v;
-    }
-  __syncthreads();
-  for (int j = 0; j < N && plain; ++j) {
-    // pivots stay above eps / 4: G is positive semidefinite up to rounding
-    const float r = rsqrtf(fmaxf(lo[at(j, j)], 0.25f * eps));
-    const float* col = lo + at(j, j) - j;   // col[i] = entry (i, j), not yet scaled
-    for (int c = j + 1 + warp; c < N; c += nw) {
-      const float f = col[c] * r * r;
-      float* dst = lo + at(c, c) - c;
-      for (int i = c + lane; i < N; i += 32) dst[i] = fmaf(-f, col[i], dst[i]);
-    }
-    __syncthreads();
-    for (int i = j + tid; i < N; i += blockDim.x) lo[at(i, j)] *= r;   // nobody reads column j again
-  }
-  __syncthreads();
-  for (int c = warp; c < N; c += nw)
-    for (int i = lane; i < N; i += 32) L[i + (int64_t)c * N] = i >= c && plain ? lo[at(i, c)] : 0.f;
-}
+constexpr double kJacRidge = 1e-7;     // eps / trace(G)
+constexpr float kJacSkip2 = 1e-14f;    // squared cosine below which two columns are orthogonal to rounding
+constexpr float kJacAgain2 = 1e-6f;    // a sweep that met none above this was the last (quadratic)
 
 // Warp sums of three values, in every lane: a reduce-scatter over the first two lane bits, one
 // value per lane after that, and a broadcast of each (9 exchanges for 15).
@@ -161,8 +96,9 @@ __global__ void jacobi32_kernel(const float* __restrict__ L, int N, double* __re
           g = fmaf(t[l], b[l], g);
         }
         sum3(a, c2, g, lane);
-        if (fabsf(g) > kJacSkip) {
-          if (fabsf(g) > kJacAgain) again = true;
+        const float ab = a * c2, gg = g * g;
+        if (gg > kJacSkip2 * ab) {
+          if (gg > kJacAgain2 * ab) again = true;
           // the smaller root, by h = |b|^2 - |t|^2, r = sqrt(h^2 + 4 g^2): c^2 = (1 + |h| / r) / 2,
           // s = sign(h g) |g| / (r c): two reciprocal square roots and a reciprocal
           const float h = c2 - a, g2 = 2.f * g;
@@ -273,6 +209,44 @@ __global__ void exp2_kernel(const double* __restrict__ E, const double* __restri
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)N * N; e += (int64_t)gridDim.x * blockDim.x)
     U[e] = (e % N == e / N ? 1.0 : 0.0) + E[e] + 0.5 * E2[e];
 }
+// Z = op(X) Y for N x N column-major matrices, op the transpose with kc.  Up to kSmallProduct on the FP64
+// pipe, a 16 x 16 tile per CTA (100 x 100: 49 CTAs, 6 us; the tensor-core product's stages and
+// split take ~17 us there), beyond as the FP64 product on the tensor cores (200 x 200: ~20 us
+// either way, 320: 30 for 60).  ex, ey: exponents of op(X)'s rows and Y's columns (tensor cores).
+constexpr int kSmallProduct = 128;
+__global__ void __launch_bounds__(256) small_product_kernel(const double* __restrict__ X, int kc,
+                                                            const double* __restrict__ Y, double* __restrict__ Z, int N) {
+  __shared__ double As[16][17], Bs[16][17];   // [k][m], [k][n]
+  const int lo = threadIdx.x & 15, hi = threadIdx.x >> 4;
+  const int m0 = blockIdx.x * 16, n0 = blockIdx.y * 16;
+  auto load = [&](int k0, double& a, double& b) {
+    // kc: K runs along X's columns' storage
+    const int am = m0 + (kc ? hi : lo), ak = k0 + (kc ? lo : hi), bn = n0 + hi, bk = k0 + lo;
+    a = am < N && ak < N ? X[kc ? (int64_t)am * N + ak : (int64_t)ak * N + am] : 0.0;
+    b = bn < N && bk < N ? Y[(int64_t)bn * N + bk] : 0.0;
+  };
+  double a, b, acc = 0.0;
+  load(0, a, b);
+  for (int k0 = 0; k0 < N; k0 += 16) {
+    if (kc) As[lo][hi] = a;
+    else As[hi][lo] = a;
+    Bs[lo][hi] = b;
+    __syncthreads();
+    if (k0 + 16 < N) load(k0 + 16, a, b);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) acc = fma(As[k][lo], Bs[k][hi], acc);
+    __syncthreads();
+  }
+  if (m0 + lo < N && n0 + hi < N) Z[(int64_t)(n0 + hi) * N + m0 + lo] = acc;
+}
+cudaError_t square_product(const double* X, bool kc, const unsigned* ex, const double* Y, const unsigned* ey, double* Z,
+                           int N, void* gw, int* status, cudaStream_t st) {
+  if (N > kSmallProduct) return gemm64(X, kc, N, ex, N, Y, N, ey, N, N, nullptr, Z, N, gw, status, st);
+  count_launch();
+  small_product_kernel<<<dim3((N + 15) / 16, (N + 15) / 16), 256, 0, st>>>(X, kc ? 1 : 0, Y, Z, N);
+  return cudaGetLastError();
+}
+
 // Cluster shape: one CTA while its 32 warps hold every pair, else eight CTAs.
 int jac_ctas(int H) { return H <= 32 ? 1 : 8; }
 
@@ -308,7 +282,7 @@ size_t up256(size_t b) { return (b + 255) / 256 * 256; }
 
 }  // namespace
 
-// Ranks the start covers: the packed factor of 320 columns takes 205 KB of shared memory.
+// Ranks the start covers: 10 elements per lane, the warps of 320 columns in eight CTAs.
 bool jacobi_start_supported(int s) { return s >= 8 && s <= 320; }
 
 // Scratch of the start and of the correction: two N x N matrices, exponents, the products' own.
@@ -344,27 +318,22 @@ cudaError_t jacobi_start(const double* G, int s, double* A, double* V, void* wor
   const int64_t nn = (int64_t)N * N;
   const StartWork w(work, N);
   float* L = reinterpret_cast<float*>(w.S);
-  const size_t tri = (size_t)N * (N + 1) / 2 * sizeof(float);
-  NYS_CUDA_TRY(ensure_max_dyn_smem((const void*)chol32_kernel, 206 * 1024));
-  count_launch();
-  chol32_kernel<<<1, 1024, tri, st>>>(G, s, N, L);
-  NYS_CUDA_TRY(cudaGetLastError());
-  // three orthonormalisation steps alternate between P and V, so V0 goes to P
-  if (N <= 64) NYS_CUDA_TRY(launch_jacobi32<2>(L, N, w.P, st, ran));
-  else if (N <= 128) NYS_CUDA_TRY(launch_jacobi32<4>(L, N, w.P, st, ran));
-  else if (N <= 224) NYS_CUDA_TRY(launch_jacobi32<7>(L, N, w.P, st, ran));
-  else NYS_CUDA_TRY(launch_jacobi32<10>(L, N, w.P, st, ran));
+  NYS_CUDA_TRY(chol_lower_f32(G, s, kJacRidge, L, N, st));
+  // two orthonormalisation steps, V -> P -> V
+  if (N <= 64) NYS_CUDA_TRY(launch_jacobi32<2>(L, N, V, st, ran));
+  else if (N <= 128) NYS_CUDA_TRY(launch_jacobi32<4>(L, N, V, st, ran));
+  else if (N <= 224) NYS_CUDA_TRY(launch_jacobi32<7>(L, N, V, st, ran));
+  else NYS_CUDA_TRY(launch_jacobi32<10>(L, N, V, st, ran));
   if (!*ran) return cudaSuccess;
   const unsigned grid = (unsigned)std::min<int64_t>(1024, (nn + 255) / 256);
   count_launch();
   fill_kernel<<<(N + 127) / 128, 128, 0, st>>>(w.e1, N, 0x40000000u);
   NYS_CUDA_TRY(cudaMemsetAsync(w.bad, 0, sizeof(int), st));
-  // Z = op(X) Y (columns of Y are K-contiguous); ex, ey: exponents of X's rows, of Y's columns
   auto mul = [&](const double* X, bool kc, const unsigned* ex, const double* Y, const unsigned* ey, double* Z) {
-    return gemm64(X, kc, N, ex, N, Y, N, ey, N, N, nullptr, Z, N, w.gw, status, st);
+    return square_product(X, kc, ex, Y, ey, Z, N, w.gw, status, st);
   };
-  double *cur = w.P, *nxt = V;
-  for (int k = 0; k < 3; ++k) {
+  double *cur = V, *nxt = w.P;
+  for (int k = 0; k < 2; ++k) {
     NYS_CUDA_TRY(mul(cur, true, w.e1, cur, w.e1, w.S));
     count_launch();
     schulz_kernel<<<grid, 256, 0, st>>>(w.S, N);
@@ -377,9 +346,9 @@ cudaError_t jacobi_start(const double* G, int s, double* A, double* V, void* wor
   gap_kernel<<<grid, 256, 0, st>>>(w.S, N, 1e-13, w.bad);
   NYS_CUDA_TRY(cudaGetLastError());
   // A <- V^T A V
-  NYS_CUDA_TRY(absmax_f64(A, N, N, N, w.eg, nullptr, st));
+  if (N > kSmallProduct) NYS_CUDA_TRY(absmax_f64(A, N, N, N, w.eg, nullptr, st));
   NYS_CUDA_TRY(mul(A, true, w.eg, V, w.e1, w.S));
-  NYS_CUDA_TRY(absmax_f64(w.S, N, N, N, w.et, nullptr, st));
+  if (N > kSmallProduct) NYS_CUDA_TRY(absmax_f64(w.S, N, N, N, w.et, nullptr, st));
   NYS_CUDA_TRY(mul(V, true, w.e1, w.S, w.et, w.P));
   count_launch();
   accept_kernel<<<grid, 256, 0, st>>>(w.P, N, w.bad, 1, A, V, V);
@@ -392,7 +361,7 @@ cudaError_t jacobi_polish(const double* G, int N, double* A, double* T, double* 
   const StartWork w(work, N);   // e1 and eg as jacobi_start left them
   const unsigned grid = (unsigned)std::min<int64_t>(1024, (nn + 255) / 256);
   auto mul = [&](const double* X, bool kc, const unsigned* ex, const double* Y, const unsigned* ey, double* Z) {
-    return gemm64(X, kc, N, ex, N, Y, N, ey, N, N, nullptr, Z, N, w.gw, status, st);
+    return square_product(X, kc, ex, Y, ey, Z, N, w.gw, status, st);
   };
   // exp(E) to second order, its departure from orthogonality (E^4 / 4) squared away by one
   // Newton-Schulz step; checked like the start's V, and left out when it fails
@@ -413,7 +382,7 @@ cudaError_t jacobi_polish(const double* G, int N, double* A, double* T, double* 
   gap_kernel<<<grid, 256, 0, st>>>(w.S, N, 1e-13, w.bad);
   NYS_CUDA_TRY(cudaGetLastError());
   NYS_CUDA_TRY(mul(G, true, w.eg, T, w.e1, w.S));
-  NYS_CUDA_TRY(absmax_f64(w.S, N, N, N, w.et, nullptr, st));
+  if (N > kSmallProduct) NYS_CUDA_TRY(absmax_f64(w.S, N, N, N, w.et, nullptr, st));
   NYS_CUDA_TRY(mul(T, true, w.e1, w.S, w.et, w.P));
   count_launch();
   accept_kernel<<<grid, 256, 0, st>>>(w.P, N, w.bad, 0, A, T, V);

@@ -119,8 +119,13 @@ size_t gram_work_bytes(int64_t d, int s);
 // k+1 if the k-th pivot is not positive, or not above rel_tol times the largest diagonal
 // entry of M (numerically dependent columns).  M is symmetrised as (M + M^T)/2 first.
 cudaError_t chol_upper(double* M, int s, int* info, cudaStream_t st, double rel_tol = 0.0);
-// B (d x s) = Y C^{-1} with C upper (s x s); B may alias Y.
-cudaError_t trsm_right_upper(const double* C, int s, double* Y, int64_t d, cudaStream_t st);
+// L (N x N FP32, column-major): lower factor of (G + ridge trace(G) I) 2^-e for a symmetric positive
+// semidefinite G (s x s), e even and the largest diagonal entry scaled to [1/2, 2); zero when G is
+// not finite.  s <= 448.
+cudaError_t chol_lower_f32(const double* G, int s, double ridge, float* L, int N, cudaStream_t st);
+// Y (d x s, column-major, in place) <- Y C^{-1} with C upper (s x s); *status as for gemm64.
+size_t trsm_work_bytes(int64_t d, int s);
+cudaError_t trsm_right_upper(const double* C, int s, double* Y, int64_t d, void* work, int* status, cudaStream_t st);
 // Y += nu * X  (d x s)
 cudaError_t axpy_panel(double nu, const double* X, double* Y, int64_t n, cudaStream_t st);
 // lambda_max of a symmetric s x s matrix by power iteration (device scalar out)
