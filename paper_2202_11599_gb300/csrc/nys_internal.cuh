@@ -168,6 +168,7 @@ size_t sketch_atw_work_bytes(const nys_matrix* A, int s);
 // three BF16 terms): tc_prepare builds the operands once (transposed copy of A; for FP32
 // also the terms) in caller-owned scratch of tc_prepare_bytes(A) bytes.
 struct TcPrepared {
+  bool direct = false;           // A is converted inside the products: no copies
   int at = 1;                    // A terms: 1 (BF16) or 3 (FP32 split)
   const uint16_t* A = nullptr;   // row-major terms, n x lda, term stride aterm
   int64_t lda = 0, aterm = 0;

@@ -89,6 +89,20 @@ __device__ __forceinline__ void split3(float x, uint16_t (&t)[3]) {
   const float r2 = r1 - bf16_val(t[1]);
   t[2] = bf16_bits(r2);
 }
+// The same terms of two values, packed (x0 in the low half): one conversion for both.
+__device__ __forceinline__ void split3_pair(float x0, float x1, uint32_t& t0, uint32_t& t1, uint32_t& t2) {
+  auto pack = [](float a, float b) -> uint32_t {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+  };
+  t0 = pack(x0, x1);
+  x0 -= __uint_as_float(t0 << 16);
+  x1 -= __uint_as_float(t0 & 0xffff0000u);
+  t1 = pack(x0, x1);
+  x0 -= __uint_as_float(t1 << 16);
+  x1 -= __uint_as_float(t1 & 0xffff0000u);
+  t2 = pack(x0, x1);
+}
 
 // AT, BT = number of BF16 terms of the A and B operands: 1 (BF16 values) or 3 (FP32 values
 // split exactly into three BF16 terms).  A K step issues the MMAs a_i x b_j with i + j <= 2
@@ -398,6 +412,243 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 
+// ---- A converted in the kernel.  FP32 storage needs its three BF16 terms and GEMM 2 needs A^T with K
+// contiguous; prepared copies of both cost a pass over A each (FP32: 3 terms and 3 transposes,
+// 24 bytes moved per element, and 6 bytes read per element and product instead of 4).  Here the raw
+// tile of A ({32 K, R rows}, or {R columns, 32 rows} for A^T) arrives by TMA in a ring of its own,
+// and a group of eight warps converts it for the MMAs; the stage's B box comes by TMA with the
+// 64-byte swizzle as in sketch_tc_tma_kernel.  One thread each issues the raw copies, the B copies
+// and the MMAs.  The terms and the MMAs and their order are those of the prepared form, so the
+// bits are too.
+//
+// FP32 storage: the three terms of a stage go to TMEM (48 columns beside the accumulator) and the
+// MMAs take A from there, which leaves shared memory to the raw ring (up to eight tiles) and B.
+// 50,000 x 4,000 by 64 columns: 256 us, A^T of it 212 us (terms in shared memory, one group of
+// eight warps: 336 and 268; two groups: 267 and 222).  An MMA of 64 columns onto one accumulator
+// then takes ~100 clocks, three times its multiplication, and that sets the pace; the read of A
+// is 118 us.  The order of the MMAs, and with it the rounding, is kept, so they stay in one chain.
+// BF16 storage (A^T only): repacked into the K-major core-matrix layout of a stage (8 rows x 16 bytes
+// contiguous, K chunks 128 B and row groups 512 B apart); its two accumulators fill TMEM, and
+// at 200 columns the MMAs bound it (100,000 x 10,000: 0.65 ms; transposing A first cost 0.81 ms
+// more).
+constexpr int TD_G = 2;                             // groups of eight converting warps: stage kt is group kt % TD_G's
+constexpr int TD_THREADS = (8 * TD_G + 3) * 32;     // and the raw, B and MMA issuers
+template <int DT, int BM2> constexpr int td_raw_bytes() { return BM2 * TC_BM * TC_BK * (DT == NYS_F32 ? 4 : 2); }
+template <int AT, int BT, int BM2, int NM> constexpr int td_stage_max() {   // AT = 3: the terms are in TMEM
+  return (AT == 3 ? 0 : BM2 * AT * TC_BM * TC_BK * 2) + BT * NM * TC_BK * 2;
+}
+constexpr int kTdSmem = 222 * 1024;
+template <int AT> constexpr int td_raw_min() { return AT == 3 ? 4 : 3; }
+template <int DT, int AT, int BT, int BM2, int NM> constexpr int td_stages() {   // converted stages: up to 3 (TMEM: 5)
+  constexpr int fit = (kTdSmem - td_raw_min<AT>() * td_raw_bytes<DT, BM2>()) / td_stage_max<AT, BT, BM2, NM>();
+  return fit < (AT == 3 ? 5 : 3) ? fit : (AT == 3 ? 5 : 3);
+}
+template <int DT, int AT, int BT, int BM2, int NM> constexpr int td_raw_stages() {   // raw stages: up to 8
+  constexpr int fit = (kTdSmem - td_stages<DT, AT, BT, BM2, NM>() * td_stage_max<AT, BT, BM2, NM>()) / td_raw_bytes<DT, BM2>();
+  return fit < 8 ? fit : 8;
+}
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+          dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(smem_u32(bar))
+      : "memory");
+}
+__device__ __forceinline__ bool warp_wait_tc(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity)) != 0;
+}
+
+template <int EPI, int DT, int AT, int BT, int BM2, int NM>
+__global__ void __launch_bounds__(TD_THREADS, 1)
+    sketch_tc_direct_kernel(const __grid_constant__ TcArgs a, const __grid_constant__ CUtensorMap tmA,
+                            const __grid_constant__ CUtensorMap tmB) {
+  constexpr bool TRANS = EPI == 1;
+  constexpr int ST = td_stages<DT, AT, BT, BM2, NM>(), RT = td_raw_stages<DT, AT, BT, BM2, NM>();
+  static_assert(ST >= 2 && RT >= 3, "shared memory holds too few stages");
+  static_assert(DT == NYS_F32 || TRANS, "BF16 rows need no conversion");
+  constexpr bool TA = DT == NYS_F32;   // A's terms in TMEM, 16 columns per term of a stage
+  static_assert(!TA || (BM2 == 1 && AT == 3 && TC_NMAX + 48 * ST <= 512), "TMEM columns");
+  constexpr uint32_t kTmemCols = 2 * TC_NMAX;
+  constexpr int R = TC_BM * BM2;
+  constexpr uint32_t RAW = td_raw_bytes<DT, BM2>();
+  constexpr uint32_t A_TERM = TA ? 0 : R * TC_BK * 2;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t raw_full[RT], raw_empty[RT], full_bar[ST], empty_bar[ST];
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int s_fail;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t m0 = (int64_t)blockIdx.x * R;
+  const int64_t kt0 = (int64_t)blockIdx.y * a.kslice;
+  const int64_t kt1 = min(a.ktiles, kt0 + a.kslice);
+  const int nkt = (int)max((int64_t)0, kt1 - kt0);
+  const uint32_t b_term = (uint32_t)(a.NP * 64), b_bytes = BT * b_term;
+  const uint32_t stage_bytes = AT * A_TERM + b_bytes;   // a multiple of 1 KB: NP is a multiple of 16
+  const uint32_t rbase = smem_u32(smem), sbase = rbase + RT * RAW;
+  const uint32_t idesc = mma_idesc_bf16(TC_BM, a.NP);
+  if (warp == 0) {
+    tmem_alloc(&tmem_slot, kTmemCols);
+    tmem_relinquish();
+  }
+  if (tid == 0) {
+    for (int s = 0; s < RT; ++s) {
+      mbar_init(&raw_full[s], 1);
+      mbar_init(&raw_empty[s], 8);
+    }
+    for (int s = 0; s < ST; ++s) {
+      mbar_init(&full_bar[s], 9);   // the group's eight warps and the B copy
+      mbar_init(&empty_bar[s], 1);
+    }
+    s_fail = 0;
+    fence_mbar_init();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+
+  if (warp < 8 * TD_G) {
+    const int gt = tid & 255;   // thread of the group
+    for (int kt = warp >> 3; kt < nkt && !s_fail; kt += TD_G) {
+      const int rs = kt % RT, s = kt % ST;
+      const uint32_t raw = rbase + rs * RAW, st = sbase + (uint32_t)s * stage_bytes;
+      if ((kt >= ST && !warp_wait_tc(&empty_bar[s], (uint32_t)((kt / ST - 1) & 1))) ||
+          !warp_wait_tc(&raw_full[rs], (uint32_t)((kt / RT) & 1))) {
+        s_fail = 1;
+        break;
+      }
+      tc_fence_after();   // the stage's last MMAs are done with it
+      if constexpr (DT == NYS_F32) {
+        // warp w: rows 32 (w % 4) + lane (its lanes of TMEM), K 16 (w / 4) .. + 15
+        const int row = 32 * (warp & 3) + lane, half = (warp >> 2) & 1;
+        float x[16];
+        if constexpr (TRANS) {
+#pragma unroll
+          for (int e = 0; e < 16; ++e)
+            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x[e]) : "r"(raw + (uint32_t)(((16 * half + e) * R + row) * 4)));
+        } else {
+          // 128-byte rows with the 128-byte swizzle: 16-byte chunk c of row r sits at c ^ (r & 7)
+#pragma unroll
+          for (int h = 0; h < 4; ++h)
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                         : "=f"(x[4 * h]), "=f"(x[4 * h + 1]), "=f"(x[4 * h + 2]), "=f"(x[4 * h + 3])
+                         : "r"(raw + (uint32_t)(row * 128 + ((4 * half + h) ^ (row & 7)) * 16)));
+        }
+        uint32_t w[3][8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) split3_pair(x[2 * e], x[2 * e + 1], w[0][e], w[1][e], w[2][e]);
+        const uint32_t ta = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(TC_NMAX + 48 * s + 8 * half);
+#pragma unroll
+        for (int t = 0; t < 3; ++t) tmem_st8(ta + (uint32_t)(16 * t), w[t]);
+        tmem_st_wait();
+      } else {
+        auto put = [&](int term, int row, int chunk, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                           st + term * A_TERM + (uint32_t)((row >> 3) * 512 + chunk * 128 + (row & 7) * 16)),
+                       "r"(w0), "r"(w1), "r"(w2), "r"(w3)
+                       : "memory");
+        };
+        // BF16 A^T: raw [32 K][R columns]; unit u: columns 2 (u % (R / 2)) and + 1, K chunk
+        for (int u = gt; u < (R / 2) * (TC_BK / 8); u += 256) {
+          const int cp = u % (R / 2), chunk = u / (R / 2);
+          uint32_t v[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v[e]) : "r"(raw + (uint32_t)(((8 * chunk + e) * R + 2 * cp) * 2)));
+          uint32_t lo[4], hi[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            lo[e] = __byte_perm(v[2 * e], v[2 * e + 1], 0x5410);
+            hi[e] = __byte_perm(v[2 * e], v[2 * e + 1], 0x7632);
+          }
+          put(0, 2 * cp, chunk, lo[0], lo[1], lo[2], lo[3]);
+          put(0, 2 * cp + 1, chunk, hi[0], hi[1], hi[2], hi[3]);
+        }
+      }
+      // the stores, before the tensor core reads them
+      if constexpr (TA) tc_fence_before();
+      else fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&full_bar[s]);
+        mbar_arrive(&raw_empty[rs]);
+      }
+    }
+  } else if (warp == 8 * TD_G && lane == 0) {
+    int kt = 0;
+    for (; kt < nkt && !s_fail; ++kt) {
+      const int rs = kt % RT;
+      if (kt >= RT && !mbar_wait_bounded(&raw_empty[rs], (uint32_t)((kt / RT - 1) & 1))) {
+        s_fail = 1;
+        break;
+      }
+      const int k0 = (int)((kt0 + kt) * TC_BK);
+      mbar_arrive_expect_tx(&raw_full[rs], RAW);
+      if (TRANS) tma_load_2d(rbase + rs * RAW, &tmA, (int)m0, k0, &raw_full[rs]);
+      else tma_load_2d(rbase + rs * RAW, &tmA, k0, (int)m0, &raw_full[rs]);
+    }
+    // copies still in flight land in this CTA's shared memory: wait for them (bounded)
+    for (int j = max(0, kt - RT); j < kt; ++j) (void)mbar_wait_bounded(&raw_full[j % RT], (uint32_t)((j / RT) & 1));
+  } else if (warp == 8 * TD_G + 1 && lane == 0) {
+    int kt = 0;
+    for (; kt < nkt && !s_fail; ++kt) {
+      const int s = kt % ST;
+      if (kt >= ST && !mbar_wait_bounded(&empty_bar[s], (uint32_t)((kt / ST - 1) & 1))) {
+        s_fail = 1;
+        break;
+      }
+      mbar_arrive_expect_tx(&full_bar[s], b_bytes);
+      tma_load_3d(sbase + (uint32_t)s * stage_bytes + AT * A_TERM, &tmB, (int)((kt0 + kt) * TC_BK), 0, 0, &full_bar[s]);
+    }
+    // (when a wait gave up the converting warps may not complete the stage: the bound ends this)
+    for (int j = max(0, kt - ST); j < kt; ++j) (void)mbar_wait_bounded(&full_bar[j % ST], (uint32_t)((j / ST) & 1));
+  } else if (warp == 8 * TD_G + 2 && lane == 0) {
+    for (int kt = 0; kt < nkt && !s_fail; ++kt) {
+      const int s = kt % ST;
+      if (!mbar_wait_bounded(&full_bar[s], (uint32_t)((kt / ST) & 1))) {
+        s_fail = 1;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t st = sbase + (uint32_t)s * stage_bytes;
+#pragma unroll
+      for (int kk = 0; kk < TC_BK / 16; ++kk) {
+#pragma unroll
+        for (int h = 0; h < BM2; ++h) {
+#pragma unroll
+          for (int pr = 0; pr < tc_npairs<AT, BT>(); ++pr) {
+            const uint64_t bd = smem_desc_sw64(st + AT * A_TERM + (uint32_t)tc_pair_b<AT, BT>(pr) * b_term + (uint32_t)(kk * 32),
+                                               512u);
+            const uint32_t acc = (kt | kk | pr) != 0 ? 1u : 0u;
+            if constexpr (TA) {
+              mma_bf16_ta(tmem, tmem + (uint32_t)(TC_NMAX + 48 * s + 16 * tc_pair_a<AT, BT>(pr) + 8 * kk), bd, idesc, acc);
+            } else {
+              const uint64_t ad = smem_desc(st + (uint32_t)tc_pair_a<AT, BT>(pr) * A_TERM + (uint32_t)(h * 16 * 512 + kk * 256),
+                                            TC_LBO, TC_SBO);
+              mma_bf16(tmem + (uint32_t)(h * TC_NMAX), ad, bd, idesc, acc);
+            }
+          }
+        }
+      }
+      mma_commit(&empty_bar[s]);
+    }
+  }
+  __syncthreads();
+  bool ok = s_fail == 0;
+  // the last commit tracks every MMA this CTA issued
+  if (ok && nkt > 0) ok = mbar_wait_bounded(&empty_bar[(nkt - 1) % ST], (uint32_t)(((nkt - 1) / ST) & 1));
+  ok = __syncthreads_and(ok);
+  tc_fence_after();
+  if (ok) {
+    if (warp < 8) tc_epilogue<EPI, BM2>(a, tmem, m0, nkt, warp, lane);
+  } else if (tid == 0) {
+    atomicExch(a.status, (int)NYS_ETIMEOUT);
+    if (nkt > 0) (void)mbar_wait_bounded(&empty_bar[(nkt - 1) % ST], (uint32_t)(((nkt - 1) / ST) & 1));
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, kTmemCols);
+}
+
 // Operand terms: Ot[t][c][k] (c < NP, k < KP) = t-th BF16 term of float(X[k + (c0 + c) d]),
 // zero outside c < mp, k < d.  X is d x m column-major (FP64 or FP32).
 // NT = 1: X holds BF16 values (the rounded test matrix of the sketch), its one term is exact.
@@ -535,6 +786,23 @@ cudaError_t make_tile_map(CUtensorMap* m, const uint16_t* base, int64_t K, int64
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// 2-D map of A itself (n rows of d elements, row stride ld) with the raw box of the converting
+// kernel: {32 K, rows} with the 128-byte swizzle, or {rows (columns of A), 32} for A^T.
+cudaError_t make_raw_map(CUtensorMap* m, const nys_matrix* A, bool trans, int rows) {
+  EncodeTiledFn enc = encode_tiled_fn();
+  if (!enc) return cudaErrorNotSupported;
+  const bool f32 = A->dtype == NYS_F32;
+  const cuuint64_t dims[2] = {(cuuint64_t)A->d, (cuuint64_t)A->n};
+  const cuuint64_t strides[1] = {(cuuint64_t)A->ld * (f32 ? 4 : 2)};
+  const cuuint32_t box[2] = {(cuuint32_t)(trans ? rows : TC_BK), (cuuint32_t)(trans ? TC_BK : rows)};
+  const cuuint32_t estr[2] = {1u, 1u};
+  const CUresult r = enc(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                         const_cast<void*>(A->data), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                         trans ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
+                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 // TMA staging unless NYS_TC_TMA=0 or the driver offers no tensor-map encoder (then the
 // cp.async form: the same MMAs, the same bits).
 bool tc_use_tma() {
@@ -547,21 +815,46 @@ template <int EPI, int AT, int BT, int BM2>
 cudaError_t launch_tc(const TcArgs& a, dim3 grid, cudaStream_t st) {
   constexpr int ST = tc_stages<AT, BT, BM2>();
   const size_t smem = (size_t)ST * (BM2 * AT * TC_BM * TC_BK * 2 + (size_t)BT * a.NP * TC_BK * 2);
-  if (tc_use_tma()) {
-    CUtensorMap tmA, tmB;
-    NYS_CUDA_TRY(make_tile_map(&tmA, a.A, a.Kvalid, a.Mrows, a.lda, AT, a.aterm, TC_BM * BM2));
-    NYS_CUDA_TRY(make_tile_map(&tmB, a.B, a.ktiles * TC_BK, a.NP, a.ldb, BT, a.bterm, a.NP));
-    NYS_CUDA_TRY(ensure_max_dyn_smem((const void*)sketch_tc_tma_kernel<EPI, AT, BT, BM2>,
-                                     ST * tc_stage_max_bytes<AT, BT, BM2>()));
-    count_launch();
-    sketch_tc_tma_kernel<EPI, AT, BT, BM2><<<grid, TC_THREADS, smem, st>>>(a, tmA, tmB);
-    return cudaGetLastError();
+  if constexpr (EPI == 0 && AT == 1) {   // BF16 rows; the other products convert A (launch_direct)
+    if (tc_use_tma()) {
+      CUtensorMap tmA, tmB;
+      NYS_CUDA_TRY(make_tile_map(&tmA, a.A, a.Kvalid, a.Mrows, a.lda, AT, a.aterm, TC_BM * BM2));
+      NYS_CUDA_TRY(make_tile_map(&tmB, a.B, a.ktiles * TC_BK, a.NP, a.ldb, BT, a.bterm, a.NP));
+      NYS_CUDA_TRY(ensure_max_dyn_smem((const void*)sketch_tc_tma_kernel<EPI, AT, BT, BM2>,
+                                       ST * tc_stage_max_bytes<AT, BT, BM2>()));
+      count_launch();
+      sketch_tc_tma_kernel<EPI, AT, BT, BM2><<<grid, TC_THREADS, smem, st>>>(a, tmA, tmB);
+      return cudaGetLastError();
+    }
   }
   NYS_CUDA_TRY(ensure_max_dyn_smem((const void*)sketch_tc_kernel<EPI, AT, BT, BM2>,
                                    ST * tc_stage_max_bytes<AT, BT, BM2>()));
   count_launch();
   sketch_tc_kernel<EPI, AT, BT, BM2><<<grid, TC_THREADS, smem, st>>>(a);
   return cudaGetLastError();
+}
+
+template <int EPI, int DT, int AT, int BT, int BM2, int NM>
+cudaError_t launch_direct_nm(const nys_matrix* A, const TcArgs& a, dim3 grid, cudaStream_t st) {
+  constexpr int ST = td_stages<DT, AT, BT, BM2, NM>(), RT = td_raw_stages<DT, AT, BT, BM2, NM>();
+  const size_t smem = (size_t)RT * td_raw_bytes<DT, BM2>() +
+                      (size_t)ST * ((AT == 3 ? 0 : BM2 * AT * TC_BM * TC_BK * 2) + (size_t)BT * a.NP * TC_BK * 2);
+  CUtensorMap tmA, tmB;
+  NYS_CUDA_TRY(make_raw_map(&tmA, A, EPI == 1, TC_BM * BM2));
+  NYS_CUDA_TRY(make_tile_map(&tmB, a.B, a.ktiles * TC_BK, a.NP, a.ldb, BT, a.bterm, a.NP));
+  auto fn = sketch_tc_direct_kernel<EPI, DT, AT, BT, BM2, NM>;
+  NYS_CUDA_TRY(ensure_max_dyn_smem((const void*)fn, kTdSmem));
+  count_launch();
+  fn<<<grid, TD_THREADS, smem, st>>>(a, tmA, tmB);
+  return cudaGetLastError();
+}
+// stage counts from the columns: at most 64, 128, 208 (rank 200: three stages of GEMM 2 just fit), 256
+template <int EPI, int DT, int AT, int BT, int BM2>
+cudaError_t launch_direct(const nys_matrix* A, const TcArgs& a, dim3 grid, cudaStream_t st) {
+  if (a.NP <= 64) return launch_direct_nm<EPI, DT, AT, BT, BM2, 64>(A, a, grid, st);
+  if (a.NP <= 128) return launch_direct_nm<EPI, DT, AT, BT, BM2, 128>(A, a, grid, st);
+  if (a.NP <= 208) return launch_direct_nm<EPI, DT, AT, BT, BM2, 208>(A, a, grid, st);
+  return launch_direct_nm<EPI, DT, AT, BT, BM2, 256>(A, a, grid, st);
 }
 
 // Output rows per CTA: two 128-row accumulators, except for FP32 x FP32 (six MMA pairs),
@@ -609,7 +902,7 @@ TcShape tc_shape(const nys_matrix* A, const TcPrepared& prep, int m, int xterms)
   TcShape h;
   h.dP = (A->d + TC_BK - 1) / TC_BK * TC_BK;
   h.NPmax = std::min(TC_NMAX, (m + 15) / 16 * 16);
-  h.rows1 = tc_cta_rows(prep.at, xterms);
+  h.rows1 = prep.direct && prep.at == 3 ? TC_BM : tc_cta_rows(prep.at, xterms);
   h.rows2 = tc_cta_rows(prep.at, TC_TERMS);
   h.mt2 = (A->d + h.rows2 - 1) / h.rows2;
   h.kt2 = prep.nP / TC_BK;
@@ -668,7 +961,12 @@ cudaError_t tc_enqueue(const nys_matrix* A, const TcPrepared& prep, const double
     g1.wrows = nP;
     g1.desc_swap = swap;
     g1.status = status;
-    NYS_CUDA_TRY(launch_tc_at<0>(prep.at, xterms, g1, dim3((unsigned)((n + h.rows1 - 1) / h.rows1), 1), st));
+    const dim3 grid1((unsigned)((n + h.rows1 - 1) / h.rows1), 1), grid2((unsigned)h.mt2, (unsigned)h.Zeff);
+    if (prep.direct && prep.at == 3)
+      NYS_CUDA_TRY(xterms == 3 ? (launch_direct<0, NYS_F32, 3, 3, 1>(A, g1, grid1, st))
+                               : (launch_direct<0, NYS_F32, 3, 1, 1>(A, g1, grid1, st)));
+    else
+      NYS_CUDA_TRY(launch_tc_at<0>(prep.at, xterms, g1, grid1, st));
     if (c0 == 0) mark();
 
     TcArgs g2 = {};
@@ -687,7 +985,11 @@ cudaError_t tc_enqueue(const nys_matrix* A, const TcPrepared& prep, const double
     g2.ldp = d;
     g2.desc_swap = swap;
     g2.status = status;
-    NYS_CUDA_TRY(launch_tc_at<1>(prep.at, TC_TERMS, g2, dim3((unsigned)h.mt2, (unsigned)h.Zeff), st));
+    if (prep.direct)
+      NYS_CUDA_TRY(prep.at == 3 ? (launch_direct<1, NYS_F32, 3, 3, 1>(A, g2, grid2, st))
+                                : (launch_direct<1, NYS_BF16, 1, 3, 2>(A, g2, grid2, st)));
+    else
+      NYS_CUDA_TRY(launch_tc_at<1>(prep.at, TC_TERMS, g2, grid2, st));
     if (c0 == 0) mark();
 
     count_launch();
@@ -757,10 +1059,11 @@ bool sketch_tc_supported(const nys_matrix* A) {
   return true;
 }
 
-// Scratch of the prepared operands: BF16 storage keeps A itself and adds the transposed
-// copy (d x nP); FP32 storage adds its three BF16 terms (n x ldS each) and their
-// transposes (d x nP each).
+// Scratch of the prepared operands of the cp.async form (the TMA form converts A as it reads it
+// and needs none): BF16 storage keeps A itself and adds the transposed copy (d x nP); FP32
+// storage adds its three BF16 terms (n x ldS each) and their transposes (d x nP each).
 size_t tc_prepare_bytes(const nys_matrix* A) {
+  if (tc_use_tma()) return 0;
   const int64_t nP = (A->n + TC_BK - 1) / TC_BK * TC_BK;
   const int64_t ldS = (A->d + 7) / 8 * 8;
   if (A->dtype == NYS_BF16) return (size_t)A->d * nP * 2;
@@ -773,6 +1076,17 @@ cudaError_t tc_prepare(const nys_matrix* A, void* scratch, TcPrepared* prep, cud
   const dim3 tgrid((unsigned)((nP + 63) / 64), (unsigned)((d + 63) / 64));
   uint16_t* buf = reinterpret_cast<uint16_t*>(scratch);
   prep->nP = nP;
+  prep->direct = tc_use_tma();
+  if (prep->direct) {
+    if (A->dtype != NYS_BF16 && A->dtype != NYS_F32) return cudaErrorInvalidValue;
+    prep->at = A->dtype == NYS_BF16 ? 1 : 3;
+    prep->A = reinterpret_cast<const uint16_t*>(A->data);   // BF16: the rows of the first product
+    prep->lda = A->ld;
+    prep->aterm = 0;
+    prep->At = nullptr;
+    prep->atterm = 0;
+    return cudaSuccess;
+  }
   if (A->dtype == NYS_BF16) {
     prep->at = 1;
     prep->A = reinterpret_cast<const uint16_t*>(A->data);
