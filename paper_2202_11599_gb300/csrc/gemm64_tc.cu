@@ -20,15 +20,17 @@
 // against 1e-16 to 8e-15 for a chain of FP64 FMAs.  A row holding a NaN or an infinity gives NaN.
 //
 // Measured (FP64 pipe before, this kernel after): the two products of a 40,000 x 4,000 sketch of
-// rank 100, 36.1 + 40.4 ms -> 2.7 + 2.7 ms; X^T Y at 10,000 x 200, 0.52 (symmetric) and 0.90 ms
-// -> 0.05 ms; U = B V at 10,000 x 200, 1.09 -> 0.06 ms.
+// rank 100, 36.1 + 40.4 ms -> 1.85 + 1.85 ms; X^T Y at 10,000 x 200, 0.52 (symmetric) and 0.90 ms
+// -> 0.11 ms; U = B V at 10,000 x 200, 1.09 -> 0.06 ms.
 //
-// What bounds it: at N = 64 an MMA reads its 4 KB A tile and 2 KB B tile from shared memory in
-// 48 clocks and multiplies in 39, so shared memory does (36 MMAs x 2 per 32 K: ~3,400 clocks
-// plus 500 to store the digits); making the digits (30 integer operations an element, 512
-// threads) runs beside the MMAs of the previous stage.  Both operands are converted in the
-// kernel: the digits are never written to memory, and an operand stored along M (A^T) is
-// transposed on the way into shared memory.
+// What bounds it: per 32 K a tile makes the digits of 6,144 elements (~30 integer operations each)
+// and issues 72 MMAs (multiplying takes 2,300 clocks, reading A and B from shared memory 3,500);
+// together it takes 6,700.  So sixteen warps convert, one thread issues the MMAs, and they meet
+// only through mbarriers; the read-out of a 256-K group runs after the next stage's digits are
+// written; MMAs that share an A tile follow each other and keep it in the collector.  (With one
+// warp doing both and a barrier per stage: 9,200 clocks, tensor pipe 26 % active.)  Both operands
+// are converted in the kernel: the digits are never written to memory, and an operand stored
+// along M (A^T) is transposed on the way into shared memory.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -40,7 +42,8 @@ namespace nys {
 namespace {
 
 constexpr int EM = 128, EN = 64, EK = 32;     // tile and K of one stage
-constexpr int ET = 512;                       // threads
+constexpr int ECW = 16;                       // converting warps
+constexpr int ET = 32 * (ECW + 4);            // and a warpgroup of which one thread issues the MMAs
 constexpr int ESL = 8;                        // digits per operand = orders kept
 constexpr int EFLUSH = 8;                     // stages between read-outs (256 K)
 constexpr uint32_t EA_SLICE = EM * EK * 2, EB_SLICE = EN * EK * 2;
@@ -63,16 +66,22 @@ struct EmuArgs {
 };
 
 // Fixed-point value of x at the scale of its row (largest exponent field emax), each byte the
-// digit + 128.
-__device__ __forceinline__ uint64_t digits(double x, int emax) {
+// digit + 128: (lo, hi) words.
+__device__ __forceinline__ void digits(double x, int emax, uint32_t& lo, uint32_t& hi) {
   const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
   const int e = (int)((h >> 20) & 0x7ffu);
-  const uint32_t mh = (h & 0xfffffu) | (e ? 0x100000u : 0u);
-  const uint64_t m = (((uint64_t)mh << 32) | l) << 9;
-  const int sh = emax - max(e, 1);
-  uint64_t q = (unsigned)sh < 64u ? m >> sh : 0ull;
-  if ((int)h < 0) q = 0ull - q;
-  return q + 0x8080808080808080ull;
+  // significand at bits 9 .. 61 (its leading one, implicit unless e = 0, at 61)
+  uint32_t mh = (__funnelshift_l(l, h, 9) & 0x1fffffffu) | 0x20000000u;
+  int sh = min(emax - e, 63);   // 62 bits shifted by 62 or more are zero: no test for e = 0, unless
+  if (emax < 64) {              // the row's maximum is itself within 2^64 of the denormals
+    if (e == 0) mh &= 0x1fffffffu;
+    sh = emax - max(e, 1);
+  }
+  if (sh < 0) sh = 63;          // a value above its row's bound: only where the caller discards the result
+  const uint64_t q = (((uint64_t)mh << 32) | (uint64_t)(l << 9)) >> sh;
+  const uint32_t sg = (uint32_t)((int)h >> 31);
+  const uint32_t a = (uint32_t)q ^ sg, c = (uint32_t)(q >> 32) ^ sg;
+  asm("add.cc.u32 %0, %2, %3;\n addc.u32 %1, %4, 0x80808080;" : "=r"(lo), "=r"(hi) : "r"(a), "r"(0x80808080u - sg), "r"(c));
 }
 
 // Digit b (0 = lowest byte) of two biased values as a BF16 pair: with d + 128 = 128 u + v
@@ -116,7 +125,8 @@ __device__ __forceinline__ double fixed_to_double(__int128 v, int sh) {
 template <bool KC>
 __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  __shared__ __align__(8) uint64_t bars[2];
+  __shared__ __align__(8) uint64_t full_bar[2], empty_bar[2], drained, done;
+  __shared__ volatile int s_fail;
   __shared__ uint32_t tmem_slot;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t m0 = (int64_t)blockIdx.y * EM;
@@ -129,8 +139,13 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
     tmem_relinquish();
   }
   if (tid == 0) {
-    mbar_init(&bars[0], 1);
-    mbar_init(&bars[1], 1);
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&full_bar[q], ECW);
+      mbar_init(&empty_bar[q], 1);
+    }
+    mbar_init(&drained, ECW);
+    mbar_init(&done, 1);
+    s_fail = 0;
     fence_mbar_init();
   }
   tc_fence_before();
@@ -143,13 +158,13 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
   // so the 16-byte stores of eight lanes fill one.
   int ar, ac;
   if (KC) {
-    ar = 8 * warp + (lane & 7);
+    ar = (8 * warp + (lane & 7)) % EM;
     ac = lane >> 3;
   } else {
     ar = 32 * (warp & 3) + lane;
     ac = warp >> 2;
   }
-  const int br = 4 * warp + (lane >> 3), bc = lane & 7;
+  const int br = (4 * warp + (lane >> 3)) % EN, bc = lane & 7;   // (the issuing warp converts nothing)
   const int64_t am = m0 + ar;
   const bool aok = am < a.M, bok = n0 + br < a.N;
   const int emA = aok ? max(1, (int)(a.ea[am] >> 20)) : 1;
@@ -193,9 +208,7 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
       uint32_t lo[8], hi[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
-        const uint64_t q = digits(ra[e], emA);
-        lo[e] = (uint32_t)q;
-        hi[e] = (uint32_t)(q >> 32);
+        digits(ra[e], emA, lo[e], hi[e]);
       }
       auto put = [&](int slice, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(st + slice * EA_SLICE + aoff), "r"(w0), "r"(w1),
@@ -218,9 +231,7 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
       uint32_t lo[4], hi[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const uint64_t q = digits(rb[e], emB);
-        lo[e] = (uint32_t)q;
-        hi[e] = (uint32_t)(q >> 32);
+        digits(rb[e], emB, lo[e], hi[e]);
       }
       auto put = [&](int slice, uint32_t w0, uint32_t w1) {
         asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(st + ESL * EA_SLICE + slice * EB_SLICE + boff), "r"(w0),
@@ -240,12 +251,12 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
     }
   };
 
-  // Read-out: warp w holds rows 32 (w % 4) + lane, columns 16 (w / 4) .. + 15.  hi collects
-  // orders 0-3 (in units of order 3), lo orders 4-7 (in units of order 7).
+  // Read-out: warp w holds rows 32 (w % 4) + lane, columns 16 (w / 4) .. + 15, each as a 96-bit
+  // integer in units of order 7: orders 0-3 times 2^32 plus orders 4-7.
   const int quad = warp & 3, cg = (warp >> 2) * 16;
-  int64_t hi[16], lo[16];
+  uint32_t w0[16], w1[16], w2[16];
 #pragma unroll
-  for (int e = 0; e < 16; ++e) hi[e] = lo[e] = 0;
+  for (int e = 0; e < 16; ++e) w0[e] = w1[e] = w2[e] = 0u;
   const uint32_t trow = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)cg;
   auto flush = [&]() {
 #pragma unroll
@@ -265,77 +276,119 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
           }
         }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) (half ? lo : hi)[8 * h + e] += s[e];
+        for (int e = 0; e < 8; ++e) {
+          const int x = 8 * h + e;
+          const uint32_t s0 = (uint32_t)s[e], s1 = (uint32_t)((uint64_t)s[e] >> 32);
+          if (half == 0)
+            asm("add.cc.u32 %0, %0, %2;\n addc.u32 %1, %1, %3;" : "+r"(w1[x]), "+r"(w2[x]) : "r"(s0), "r"(s1));
+          else
+            asm("add.cc.u32 %0, %0, %3;\n addc.cc.u32 %1, %1, %4;\n addc.u32 %2, %2, %5;"
+                : "+r"(w0[x]), "+r"(w1[x]), "+r"(w2[x])
+                : "r"(s0), "r"(s1), "r"((uint32_t)((int)s1 >> 31)));
+        }
       }
     }
   };
 
   constexpr uint32_t idesc = mma_idesc_bf16(EM, EN);
-  bool ok = true;
-  if (nt > 0) load(0);
-  for (int t = 0; t < nt; ++t) {
-    const int s = t & 1;
-    const uint32_t st = sbase + (uint32_t)s * E_STAGE;
-    // the MMAs of this stage's previous use must be done reading it
-    if (t >= 2) ok = ok && mbar_wait_bounded(&bars[s], (uint32_t)(((t >> 1) - 1) & 1));
-    store(st);
-    if (t + 1 < nt) load(t + 1);
-    fence_proxy_async_smem();
-    tc_fence_before();
-    ok = __syncthreads_and(ok) != 0;
-    if (!ok) break;
-    const bool first = t % EFLUSH == 0;
-    if (tid == 0) {
+  // 20 warps of 96 registers; the issuing warpgroup gives up what the converting ones take
+  // (512 x 112 + 128 x 24 = 60,416 of 640 x 96 = 61,440)
+  if (warp < ECW) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+    // step t's accumulators are complete once the commit of step t has arrived
+    auto drain = [&](int t) -> bool {
+      if (!__all_sync(0xffffffffu, mbar_wait_bounded(&empty_bar[t & 1], (uint32_t)((t >> 1) & 1)))) return false;
       tc_fence_after();
+      flush();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&drained);
+      return true;
+    };
+    if (nt > 0) load(0);
+    for (int t = 0; t < nt; ++t) {
+      const int s = t & 1;
+      // the MMAs of this stage's previous use must be done reading it
+      const bool bad = s_fail || (t >= 2 && !mbar_wait_bounded(&empty_bar[s], (uint32_t)(((t >> 1) - 1) & 1)));
+      if (__any_sync(0xffffffffu, bad)) {
+        s_fail = 1;
+        break;
+      }
+      store(sbase + (uint32_t)s * E_STAGE);
+      const bool group = t > 0 && t % EFLUSH == 0;
+      if (t + 1 < nt && !group) load(t + 1);   // (not across a read-out: registers)
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&full_bar[s]);
+      // the group that ended with step t - 1 (the MMAs of step t wait for its read-out)
+      if (group) {
+        if (!drain(t - 1)) {
+          s_fail = 1;
+          break;
+        }
+        if (t + 1 < nt) load(t + 1);
+      }
+    }
+    const bool whole = !__any_sync(0xffffffffu, s_fail != 0) && (nt == 0 || drain(nt - 1));
+    if (!whole) s_fail = 1;
+    const int64_t m = m0 + 32 * quad + lane;
+    if (m < a.M) {
+      const unsigned wa = a.ea[m];
+      const double dm = a.D ? a.D[m] : 1.0;
+      double* out = a.C + (int64_t)blockIdx.z * a.cslice + m;
+  #pragma unroll
+      for (int e = 0; e < 16; ++e) {
+        const int n = n0 + cg + e;
+        if (n < a.N) {
+          const unsigned wb = a.eb[n];
+          const uint64_t low = ((uint64_t)w1[e] << 32) | w0[e];
+          double x = fixed_to_double((((__int128)(int)w2[e]) << 64) | (__int128)(unsigned __int128)low,
+                                     56 - 2168 + max(1, (int)(wa >> 20)) + max(1, (int)(wb >> 20)));
+          if (!whole || (wa >> 20) == 0x7ffu || (wb >> 20) == 0x7ffu) x = __longlong_as_double(0x7ff8000000000000ll);
+          out[(int64_t)n * a.ldc] = a.D ? dm * x : x;
+        }
+      }
+    }
+  } else {
+   asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");
+   if (tid == 32 * ECW) {
+    for (int t = 0; t < nt && !s_fail; ++t) {
+      const int s = t & 1;
+      if (!mbar_wait_bounded(&full_bar[s], (uint32_t)((t >> 1) & 1)) ||
+          (t > 0 && t % EFLUSH == 0 && !mbar_wait_bounded(&drained, (uint32_t)((t / EFLUSH - 1) & 1)))) {
+        s_fail = 1;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t st = sbase + (uint32_t)s * E_STAGE;
+      const bool first = t % EFLUSH == 0;
       const uint64_t ad0 = smem_desc(st, 128u, 512u), bd0 = smem_desc(st + ESL * EA_SLICE, 128u, 512u);
 #pragma unroll 1
       for (int kk = 0; kk < EK / 16; ++kk) {
+        // digit i of A against digits 0 .. 7 - i of B, each onto another order's accumulator: A stays
+        // in the collector, and no MMA waits for the one before (the sums are exact in any order)
 #pragma unroll
-        for (int o = 0; o < ESL; ++o) {
+        for (int i = 0; i < ESL; ++i) {
+          const uint64_t ad = ad0 + (uint64_t)((i * EA_SLICE + kk * 256u) >> 4);
+          const uint32_t acc = (first && kk == 0 && i == 0) ? 0u : 1u;
+          mma_bf16_same_a<true>(tmem + (uint32_t)(i * EN), ad, bd0 + (uint64_t)((kk * 256u) >> 4), idesc, acc);
 #pragma unroll
-          for (int i = 0; i <= o; ++i) {
-            mma_bf16(tmem + (uint32_t)(o * EN), ad0 + (uint64_t)((i * EA_SLICE + kk * 256u) >> 4),
-                     bd0 + (uint64_t)(((o - i) * EB_SLICE + kk * 256u) >> 4), idesc,
-                     (first && kk == 0 && i == 0) ? 0u : 1u);
-          }
+          for (int o = i + 1; o < ESL; ++o)
+            mma_bf16_same_a<false>(tmem + (uint32_t)(o * EN), ad, bd0 + (uint64_t)(((o - i) * EB_SLICE + kk * 256u) >> 4),
+                                   idesc, acc);
         }
       }
-      mma_commit(&bars[s]);
+      mma_commit(&empty_bar[s]);
     }
-    if (t % EFLUSH == EFLUSH - 1 || t == nt - 1) {
-      ok = mbar_wait_bounded(&bars[s], (uint32_t)((t >> 1) & 1));
-      tc_fence_after();
-      if (__all_sync(0xffffffffu, ok)) flush();
+    if (s_fail) {   // MMAs still queued: they finish before TMEM is freed
+      mma_commit(&done);
+      (void)mbar_wait_bounded(&done, 0u);
     }
-  }
-  tc_fence_before();
-  ok = __syncthreads_and(ok) != 0;
-  tc_fence_after();
-  if (!ok && tid == 0) {
-    // a wait gave up: report, and give the MMAs still queued a bounded last chance to finish
-    atomicExch(a.status, (int)NYS_ETIMEOUT);
-    const int last = nt - 1;
-    (void)mbar_wait_bounded(&bars[last & 1], (uint32_t)((last >> 1) & 1));
-  }
-  const int64_t m = m0 + 32 * quad + lane;
-  if (m < a.M) {
-    const unsigned wa = a.ea[m];
-    const double dm = a.D ? a.D[m] : 1.0;
-    double* out = a.C + (int64_t)blockIdx.z * a.cslice + m;
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-      const int n = n0 + cg + e;
-      if (n < a.N) {
-        const unsigned wb = a.eb[n];
-        double x = fixed_to_double((((__int128)hi[e]) << 32) + (__int128)lo[e],
-                                   56 - 2168 + max(1, (int)(wa >> 20)) + max(1, (int)(wb >> 20)));
-        if (!ok || (wa >> 20) == 0x7ffu || (wb >> 20) == 0x7ffu) x = __longlong_as_double(0x7ff8000000000000ll);
-        out[(int64_t)n * a.ldc] = a.D ? dm * x : x;
-      }
-    }
+   }
   }
   tc_fence_before();
   __syncthreads();
+  if (s_fail && tid == 0) atomicExch(a.status, (int)NYS_ETIMEOUT);
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
