@@ -297,13 +297,14 @@ __global__ void __launch_bounds__(kVecThreads) apass_reduce_kernel(const C* __re
   }
 }
 
-// Elements per block of the PCG / ADMM vector steps.  Up to 2,048 elements: at most eight blocks,
-// so that the fused steps run as one cluster (its barrier costs a fraction of the grid's
-// 1.6 us), but never under 64; up to 19,456: 128, for up to 152 blocks; beyond: 256 and
-// more, at most 304 blocks.
+// Elements per block of the PCG / ADMM vector steps.  Up to 2,048 elements: at most sixteen
+// blocks, so that the fused steps run as one cluster (its barrier costs a fraction of the grid's
+// 1.6 us), but never under 32: the steps of an FP64 block are bound by its SM's FP64 pipe (the
+// partials of A^T u alone, 500 columns: 9 us on eight SMs).  Up to 19,456: 128, for up to 152
+// blocks; beyond: 256 and more, at most 304 blocks.
 int vec_chunk(int64_t d) {
   int64_t c;
-  if (d <= 256 * kClusterBlocks) c = std::max<int64_t>(64, (d + kClusterBlocks - 1) / kClusterBlocks);
+  if (d <= 128 * kClusterBlocks) c = std::max<int64_t>(32, (d + kClusterBlocks - 1) / kClusterBlocks);
   else if (d <= 128 * 152) c = 128;
   else c = std::max<int64_t>(256, (d + 303) / 304);
   return (int)((c + 31) / 32 * 32);

@@ -208,6 +208,21 @@ __device__ __forceinline__ double block_sum_t0(double v, double* sh /* >= NT/32 
   return s;
 }
 
+// block_sum_t0 when only the first nw warps hold anything but zeros (the same value: the FP64
+// additions of the others' zeros are left out).
+template <int NT>
+__device__ __forceinline__ double block_sum_t0(double v, double* sh, int nw) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (w < nw) v = warp_sum(v);
+  __syncthreads();
+  if (lane == 0 && w < nw) sh[w] = v;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < nw; ++i) s += sh[i];
+  return s;
+}
+
 // Block-wide sum in fixed order (deterministic); every thread gets the result.
 template <int NT>
 __device__ __forceinline__ double block_sum(double v, double* sh /* >= NT/32 */) {
@@ -228,10 +243,11 @@ constexpr int kLoadBatch = sizeof(T) == 4 ? 64 : 32;
 
 // sum_{g < n} a[g * stride + j] added in increasing g (the order of a plain loop), the loads
 // issued kLoadBatch at a time so that a thread keeps that many reads in flight.  CG: read
-// through L2, for data written by other blocks of the running kernel.
+// through L2, for data written by other blocks of the running kernel.  The additions run in
+// groups of eight behind a branch for FP64: a predicated-off one still takes its 64 clocks.
 template <bool CG, typename T>
 __device__ __forceinline__ T sum_strided_fixed(const T* a, int n, int64_t stride, int64_t j, T s) {
-  constexpr int B = kLoadBatch<T>;
+  constexpr int B = kLoadBatch<T>, W = sizeof(T) == 8 ? 8 : B;
   for (int g = 0; g < n; g += B) {
     T v[B];
 #pragma unroll
@@ -241,13 +257,17 @@ __device__ __forceinline__ T sum_strided_fixed(const T* a, int n, int64_t stride
         v[q] = CG ? __ldcg(ptr) : *ptr;
       }
 #pragma unroll
-    for (int q = 0; q < B; ++q)
-      if (g + q < n) s += v[q];
+    for (int o = 0; o < B; o += W)
+      if (g + o < n) {
+#pragma unroll
+        for (int q = o; q < o + W; ++q)
+          if (g + q < n) s += v[q];
+      }
   }
   return s;
 }
 
-// Column sums of the A-pass partials [G][dpad] by a block of 256 threads, for NT (four, or one) tiles
+// Column sums of the A-pass partials [G][dpad] by a block of 256 threads, for NT (four, two or one) tiles
 // of 32 columns (tile t: columns j + 32 t, j = first column + lane): warp w adds the partials g = w,
 // w + 8, ... in increasing g, then warp 0 adds the eight warps' sums in order and holds the
 // result (one FP64 addition per 64 clocks and SM quarter: 152 partials added by one thread
@@ -257,7 +277,7 @@ template <typename C, int NT>
 __device__ __forceinline__ void pass_column_sums(const C* partial, int G, int64_t dpad, int64_t j, int64_t j1,
                                                  C (&sum)[NT], C (*sh)[NT][32]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int U = NT == 1 ? 20 : (sizeof(C) == 4 ? 10 : 5);   // partials per tile in flight
+  constexpr int U = NT == 1 ? 20 : (NT == 2 || sizeof(C) == 4 ? 10 : 5);   // partials per tile in flight
 #pragma unroll
   for (int t = 0; t < NT; ++t) sum[t] = C(0);
   for (int g0 = warp; g0 < G; g0 += 8 * U) {
@@ -290,21 +310,53 @@ __device__ __forceinline__ void pass_column_sums(const C* partial, int G, int64_
   __syncthreads();
 }
 
-// acc + sum_{i < s} U[i * d + j] g[i] as one fma chain in increasing i (the row of U g, for
-// y = w + U g), the loads of U issued kLoadBatch at a time.
+// acc + sum_{i0 <= i < i1} U[i * d + j] g[i] as one fma chain in increasing i, the loads of U
+// issued kLoadBatch at a time (groups of eight as in sum_strided_fixed).
 template <typename C>
-__device__ __forceinline__ C urow_dot(const C* __restrict__ U, int64_t d, int64_t j, int s, const C* g, C acc) {
-  constexpr int B = kLoadBatch<C>;
-  for (int i = 0; i < s; i += B) {
+__device__ __forceinline__ C urow_dot(const C* __restrict__ U, int64_t d, int64_t j, int i0, int i1, const C* g, C acc) {
+  constexpr int B = kLoadBatch<C>, W = sizeof(C) == 8 ? 8 : B;
+  for (int i = i0; i < i1; i += B) {
     C u[B];
 #pragma unroll
     for (int q = 0; q < B; ++q)
-      if (i + q < s) u[q] = U[(int64_t)(i + q) * d + j];
+      if (i + q < i1) u[q] = U[(int64_t)(i + q) * d + j];
 #pragma unroll
-    for (int q = 0; q < B; ++q)
-      if (i + q < s) acc = fma(u[q], g[i + q], acc);
+    for (int o = 0; o < B; o += W)
+      if (i + o < i1) {
+#pragma unroll
+        for (int q = o; q < o + W; ++q)
+          if (i + q < i1) acc = fma(u[q], g[i + q], acc);
+      }
   }
   return acc;
+}
+
+// y = w + U g over a block's chunk of `len` elements from j0 (w at w[0 .. len)): done(jj, w, y) in
+// thread jj % kVecThreads.  Bound by the latency of the chain over s and its loads (rank 50, FP64:
+// 9,800 clocks as one chain per element), so a chunk of up to 128 elements gives each element
+// kVecThreads / chunk threads, added in order.
+template <typename C, typename F>
+__device__ __forceinline__ void u_times_g(const C* __restrict__ U, int64_t d, int64_t j0, int len, int chunk, int s,
+                                          const C* g, const C* w, F done) {
+  __shared__ C red[kVecThreads];
+  if (chunk > kVecThreads / 2) {
+    for (int jj = threadIdx.x; jj < len; jj += kVecThreads) {
+      const C wj = w[jj];
+      done(jj, wj, urow_dot(U, d, j0 + jj, 0, s, g, wj));
+    }
+    return;
+  }
+  const int cw = (chunk + 31) / 32 * 32, parts = kVecThreads / cw, per = (s + parts - 1) / parts;
+  const int jj = threadIdx.x % cw, part = threadIdx.x / cw;
+  const C wj = jj < len ? w[jj] : C(0);
+  C acc = part == 0 ? wj : C(0);
+  if (part < parts && jj < len) acc = urow_dot(U, d, j0 + jj, min(s, part * per), min(s, part * per + per), g, acc);
+  red[threadIdx.x] = acc;
+  __syncthreads();
+  if (part == 0 && jj < len) {
+    for (int q = 1; q < parts; ++q) acc += red[q * cw + jj];
+    done(jj, wj, acc);
+  }
 }
 
 }  // namespace nys

@@ -89,7 +89,7 @@ int reduce_blocks(int64_t d);
 // vector data between blocks, only of sums.
 int vec_chunk(int64_t d);
 int vec_blocks(int64_t d);
-constexpr int kClusterBlocks = 8;   // vec_blocks(d) up to this: the fused kernels run as one cluster
+constexpr int kClusterBlocks = 16;   // vec_blocks(d) up to this: the fused kernels run as one cluster
 
 // ---------------------------------------------------------------- small dense FP64 kernels
 // FP64 products on the tensor cores (gemm64_tc.cu).  absmax_f64: per row and / or column of the

@@ -16,6 +16,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
+#include <type_traits>
 
 namespace nys {
 
@@ -58,27 +59,33 @@ __device__ __forceinline__ void block_fixed_sums_cg(const double* const (&a)[N],
   __syncthreads();
 }
 
-// Five block_sum<kVecThreads> reductions with one pair of barriers (same values as five calls),
-// results in thread 0 only.
-__device__ __forceinline__ void block_sum5(double (&v)[5]) {
+// Warps of a block that hold elements of its chunk.
+__device__ __forceinline__ int vec_warps(int chunk) { return min(kVecThreads, chunk + 31) / 32; }
+
+// Five block sums with one pair of barriers (the values of five block_sum calls), results in
+// thread 0 only; only the first nw warps hold anything but zeros.
+__device__ __forceinline__ void block_sum5(double (&v)[5], int nw) {
   __shared__ double sh5[5][kVecThreads / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (w < nw) {
 #pragma unroll
-  for (int t = 0; t < 5; ++t) v[t] = warp_sum(v[t]);
+    for (int t = 0; t < 5; ++t) v[t] = warp_sum(v[t]);
+  }
   __syncthreads();
-  if (lane == 0) {
+  if (lane == 0 && w < nw) {
 #pragma unroll
     for (int t = 0; t < 5; ++t) sh5[t][w] = v[t];
   }
   __syncthreads();
+  if (lane == 0 && w < 5) {   // one warp per sum: the five chains run side by side
+    double s = 0.0;
+    for (int i = 0; i < nw; ++i) s += sh5[w][i];
+    sh5[w][0] = s;
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
 #pragma unroll
-    for (int t = 0; t < 5; ++t) {
-      double s = 0.0;
-#pragma unroll
-      for (int i = 0; i < kVecThreads / 32; ++i) s += sh5[t][i];
-      v[t] = s;
-    }
+    for (int t = 0; t < 5; ++t) v[t] = sh5[t][0];
   }
   __syncthreads();
 }
@@ -326,14 +333,12 @@ __global__ void __launch_bounds__(kVecThreads) pcg_tail_kernel(int64_t d, int ch
   for (int i = threadIdx.x; i < s; i += kVecThreads) g[i] = gs[i];
   __syncthreads();
   double lwy = 0.0;
-  const int64_t j1 = min(d, (int64_t)(blockIdx.x + 1) * chunk);
-  for (int64_t j = blockIdx.x * (int64_t)chunk + threadIdx.x; j < j1; j += kVecThreads) {
-    const C wj = w[j];
-    const C acc = urow_dot(U, d, j, s, g, wj);
-    y[j] = acc;
+  const int64_t j0 = blockIdx.x * (int64_t)chunk, j1 = min(d, j0 + chunk);
+  u_times_g(U, d, j0, (int)(j1 - j0), chunk, s, g, w + j0, [&](int jj, C wj, C acc) {
+    y[j0 + jj] = acc;
     lwy += (double)wj * (double)acc;
-  }
-  const double t = block_sum_t0<kVecThreads>(lwy, sh);
+  });
+  const double t = block_sum_t0<kVecThreads>(lwy, sh, vec_warps(chunk));
   if (threadIdx.x == 0) part_wy[blockIdx.x] = t;
   if (!p) return;
   if (!last_block_done(&st->ticket[1])) return;
@@ -828,7 +833,7 @@ __global__ void __launch_bounds__(kVecThreads) admm_zu_g_kernel(int64_t d, int c
     a4 += uj * uj;
   }
   double a5[5] = {a0, a1, a2, a3, a4};
-  block_sum5(a5);
+  block_sum5(a5, vec_warps(chunk));
   if (threadIdx.x == 0) {
     double* o = part5 + (int64_t)blockIdx.x * 5;
 #pragma unroll
@@ -932,7 +937,7 @@ __global__ void __launch_bounds__(kVecThreads, 2) pcg_post_kernel(const PostArgs
   extern __shared__ __align__(16) unsigned char sm_raw[];
   C* vch = reinterpret_cast<C*>(sm_raw);   // the block's chunk of v, then of w
   C* gsh = vch + a.chunk;                  // g
-  __shared__ C csh[8][kSumTiles][32];
+  __shared__ C csh[8 * kSumTiles * 32];
   __shared__ double sh[kVecThreads / 32];
   __shared__ double slots[2];
   PcgState* st = a.st;
@@ -963,24 +968,30 @@ __global__ void __launch_bounds__(kVecThreads, 2) pcg_post_kernel(const PostArgs
   // (apass_reduce_kernel)
   {
     double dacc = 0.0;
-    for (int64_t t0 = j0; t0 < j1; t0 += 32 * kSumTiles) {
-      C sum[kSumTiles];
-      pass_column_sums<C, kSumTiles>(a.partial, a.G, a.dpad, t0 + lane, j1, sum, csh);
-      if (warp == 0) {
+    auto columns = [&](auto tiles) {   // tiles of 32 columns at a time: as many as the chunk has, up to four
+      constexpr int NT = decltype(tiles)::value;
+      for (int64_t t0 = j0; t0 < j1; t0 += 32 * NT) {
+        C sum[NT];
+        pass_column_sums<C, NT>(a.partial, a.G, a.dpad, t0 + lane, j1, sum, reinterpret_cast<C(*)[NT][32]>(csh));
+        if (warp == 0) {
 #pragma unroll
-        for (int t = 0; t < kSumTiles; ++t) {
-          const int64_t j = t0 + lane + 32 * t;
-          if (j < j1) {
-            C sj = sum[t];
-            if (a.cscale) sj *= (C)a.cscale[j];
-            const C pj = a.p[j];
-            const C yj = fma(a.rho, pj, sj);
-            vch[j - j0] = yj;
-            dacc += (double)pj * (double)yj;
+          for (int t = 0; t < NT; ++t) {
+            const int64_t j = t0 + lane + 32 * t;
+            if (j < j1) {
+              C sj = sum[t];
+              if (a.cscale) sj *= (C)a.cscale[j];
+              const C pj = a.p[j];
+              const C yj = fma(a.rho, pj, sj);
+              vch[j - j0] = yj;
+              dacc += (double)pj * (double)yj;
+            }
           }
         }
       }
-    }
+    };
+    if (a.chunk <= 32) columns(std::integral_constant<int, 1>{});
+    else if (a.chunk <= 64) columns(std::integral_constant<int, 2>{});
+    else columns(std::integral_constant<int, kSumTiles>{});
     if (warp == 0) {
       const double t = warp_sum(dacc);
       if (lane == 0) a.pv_part[b] = t;
@@ -1008,7 +1019,7 @@ __global__ void __launch_bounds__(kVecThreads, 2) pcg_post_kernel(const PostArgs
       vch[j - j0] = wj;
       lw2 += (double)wj * (double)wj;
     }
-    const double tw2 = block_sum_t0<kVecThreads>(lw2, sh);
+    const double tw2 = block_sum_t0<kVecThreads>(lw2, sh, vec_warps(a.chunk));
     if (threadIdx.x == 0) a.part_w2[b] = tw2;
   }
   if (!barrier()) return fail();
@@ -1058,13 +1069,11 @@ __global__ void __launch_bounds__(kVecThreads, 2) pcg_post_kernel(const PostArgs
     // ---- T: y = w + U g, partials of w^T y (pcg_tail_kernel)
     {
       double lwy = 0.0;
-      for (int64_t j = j0 + threadIdx.x; j < j1; j += kVecThreads) {
-        const C wj = vch[j - j0];
-        const C acc = urow_dot(a.U, d, j, s, gsh, wj);
-        a.y[j] = acc;
+      u_times_g(a.U, d, j0, (int)(j1 - j0), a.chunk, s, gsh, vch, [&](int jj, C wj, C acc) {
+        a.y[j0 + jj] = acc;
         lwy += (double)wj * (double)acc;
-      }
-      const double t = block_sum_t0<kVecThreads>(lwy, sh);
+      });
+      const double t = block_sum_t0<kVecThreads>(lwy, sh, vec_warps(a.chunk));
       if (threadIdx.x == 0) a.wy_part[b] = t;
     }
     if (!barrier()) return fail();
@@ -1091,7 +1100,7 @@ __global__ void __launch_bounds__(kVecThreads, 2) pcg_post_kernel(const PostArgs
       a.u[j] = uj;
       if (zt) zt[j] = zj;
     }
-    block_sum5(a5);
+    block_sum5(a5, vec_warps(a.chunk));
     if (threadIdx.x == 0) {
       double* o = a.part5 + (int64_t)b * 5;
 #pragma unroll
@@ -1201,8 +1210,8 @@ __global__ void __launch_bounds__(kVecThreads, 2) admm_head_kernel(HeadArgs a, c
         wch[j - j0] = wj;
         lw2 += (double)wj * (double)wj;
       }
-      const double tw2 = block_sum_t0<kVecThreads>(lw2, sh);
-      const double tr2 = block_sum_t0<kVecThreads>(lr2, sh);
+      const double tw2 = block_sum_t0<kVecThreads>(lw2, sh, vec_warps(a.chunk));
+      const double tr2 = block_sum_t0<kVecThreads>(lr2, sh, vec_warps(a.chunk));
       if (threadIdx.x == 0) {
         a.part_w2[b] = tw2;
         a.part_r2[b] = tr2;
@@ -1235,14 +1244,12 @@ __global__ void __launch_bounds__(kVecThreads, 2) admm_head_kernel(HeadArgs a, c
       __syncthreads();
       {
         double lwy = 0.0;
-        for (int64_t j = j0 + threadIdx.x; j < j1; j += kVecThreads) {
-          const C wj = wch[j - j0];
-          const C acc = urow_dot(U, d, j, s, gsh, wj);
-          y[j] = acc;
-          p[j] = acc;
+        u_times_g(U, d, j0, (int)(j1 - j0), a.chunk, s, gsh, wch, [&](int jj, C wj, C acc) {
+          y[j0 + jj] = acc;
+          p[j0 + jj] = acc;
           lwy += (double)wj * (double)acc;
-        }
-        const double t = block_sum_t0<kVecThreads>(lwy, sh);
+        });
+        const double t = block_sum_t0<kVecThreads>(lwy, sh, vec_warps(a.chunk));
         if (threadIdx.x == 0) a.wy_part[b] = t;
       }
       if (b == 0 && threadIdx.x == 0) {
@@ -1280,7 +1287,7 @@ __global__ void __launch_bounds__(kVecThreads, 2) admm_head_kernel(HeadArgs a, c
         a.u[j] = uj;
         if (zt) zt[j] = zj;
       }
-      block_sum5(a5);
+      block_sum5(a5, vec_warps(a.chunk));
       if (threadIdx.x == 0) {
         double* o = a.part5 + (int64_t)b * 5;
 #pragma unroll
@@ -1500,7 +1507,9 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
     bool ok = false, cl = false;
   };
   auto fused_fits = [&](const void* fn_cl, const void* fn_grid, size_t smem, Fused* f) -> cudaError_t {
-    if (nb <= kClusterBlocks) {
+    // more than eight blocks: beyond the portable cluster size, where the device offers it
+    if (nb <= kClusterBlocks &&
+        (nb <= 8 || cudaFuncSetAttribute(fn_cl, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3((unsigned)nb);
       cfg.blockDim = dim3(kVecThreads);
@@ -1517,8 +1526,8 @@ nys_status admm_graph_add(cudaGraph_t graph, const GraphLoopArgs& g, cudaStream_
         f->ok = f->cl = true;
         return cudaSuccess;
       }
-      (void)cudaGetLastError();
     }
+    (void)cudaGetLastError();
     int per_sm = 0, coop = 0;
     NYS_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, current_device()));
     NYS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn_grid, kVecThreads, smem));
