@@ -461,15 +461,19 @@ bool apass_plan(const nys_matrix* A, ApassPlan* plan) {
     // warp-specialised: 2 rows per stage by default (1 for rows over 64 KB, 4 under 8 KB)
     int R = rowbytes > 64 * 1024 ? 1 : (rowbytes < 8 * 1024 ? 4 : 2);
     if (A->dtype == NYS_F64 && R > 2) R = 2;
-    if (const int tr = tuned_rows(A->dtype, vkey < 0 ? 99 : vkey, rowbytes)) R = tr;
+    int env_or_tuned = 0;   // a choice of rows that was made, not the rule's
+    if (const int tr = tuned_rows(A->dtype, vkey < 0 ? 99 : vkey, rowbytes)) R = env_or_tuned = tr;
     if (R != 1 && R != 2 && R != 4) R = 2;
     if (A->dtype == NYS_F64 && R > 2) R = 2;
     if (const char* env = std::getenv("NYS_APASS_ROWS")) {
       const int r = std::atoi(env);
-      if (r == 1 || r == 2 || (r == 4 && A->dtype != NYS_F64)) R = r;
+      if (r == 1 || r == 2 || (r == 4 && A->dtype != NYS_F64)) R = env_or_tuned = r;
     }
     while (R > 1 && ws_stages(rowbytes, R) < 3) R /= 2;
     const int S = ws_stages(rowbytes, R);
+    // FP64 (apass_wide64.cu): R rows a warp at a time, p in shared memory, no stages
+    const bool wide64 = A->dtype == NYS_F64;
+    if (wide64) R = env_or_tuned == 1 ? 1 : 2;
     if (S >= 2) {
       plan->ws = true;
       plan->rows_per_step = R;
@@ -477,7 +481,7 @@ bool apass_plan(const nys_matrix* A, ApassPlan* plan) {
       plan->threads = wthreads;
       plan->vpt = wvpt;
       plan->onebar = false;
-      plan->smem = (size_t)S * R * rowbytes;
+      plan->smem = wide64 ? (size_t)nvec * 16 : (size_t)S * R * rowbytes;
       plan->dpad = nvec * vec;
       const int64_t steps_total = (A->n + R - 1) / R;
       plan->grid = (int)std::max<int64_t>(1, std::min<int64_t>(sm_count(), steps_total));

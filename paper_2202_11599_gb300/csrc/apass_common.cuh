@@ -13,7 +13,6 @@ constexpr int kMaxStages = 8;
 constexpr int kSmemBudget = 200 * 1024;
 constexpr int kWsGroupWarps = 8;   // warp-specialised float pass: dot warps = update warps
 constexpr int kRows64Max = 32;     // FP64 pass for narrow rows: rows per stage
-constexpr int kWs64DotWarps = 8;   // warp-specialised FP64 pass: dot warps (update warps: twice as many)
 
 struct ApassKArgs {
   const unsigned char* A;
@@ -218,7 +217,11 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity) {
 bool apass_ws_layout(int dtype, int64_t d, int* threads, int* vpt);
 cudaError_t apass_ws_launch(const ApassKArgs& k, const ApassPlan& plan, int dtype, cudaStream_t st,
                             bool prepare_only);
-// FP64 pass for the widths the warp-specialised one does not take (apass_rows64.cu): column
+// FP64 pass for wide rows (apass_wide64.cu): column vectors per thread (-1: too wide), threads, launch.
+int apass_wide64_vpt(int64_t d);
+int apass_wide64_threads();
+cudaError_t apass_wide64_launch(const ApassKArgs& k, const ApassPlan& plan, cudaStream_t st, bool prepare_only);
+// FP64 pass for the widths the wide one is not chosen for (apass_rows64.cu): column
 // vectors per thread (-1: too wide), and the launch.
 int apass_rows64_vpt(int64_t d);
 cudaError_t apass_rows64_launch(const ApassKArgs& k, const ApassPlan& plan, cudaStream_t st, bool prepare_only);

@@ -1,5 +1,4 @@
-// Fused FP64 A-pass for narrow rows (the pass for FP64 matrices the warp-specialised one does
-// not take): y = A^T phi(A p) with one read of A, the result layout of apass.cu.
+// Fused FP64 A-pass for narrow rows (the pass for FP64 matrices apass_wide64.cu does not take): y = A^T phi(A p) with one read of A, the result layout of apass.cu.
 //
 // The FP64 pipe bounds it: an SM quarter issues one FP64 warp instruction per 64 clocks, so
 // the rows' n d products and n d updates set the pace and any FP64 instruction beside them

@@ -57,8 +57,8 @@ struct ApassPlan {
   int threads = 512;     // CTA size (float path: 512 or 640)
   int vpt = 0;           // 16-byte column vectors owned per thread
   bool onebar = false;   // float path, H-matvec modes: one barrier per step
-  bool ws = false;       // warp-specialised pass (apass_ws.cu): threads / vpt / R / S of its layout
-                         // (FP64 without it: apass_rows64.cu)
+  bool ws = false;       // wide rows: the warp-specialised pass (apass_ws.cu), threads / vpt / R / S of
+                         // its layout; FP64: apass_wide64.cu (without: apass_rows64.cu)
 };
 
 bool apass_plan(const nys_matrix* A, ApassPlan* plan);
