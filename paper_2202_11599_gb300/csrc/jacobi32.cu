@@ -7,8 +7,10 @@
 // everything stays on chip in FP32: one-sided Jacobi (Hestenes) on the columns of the Cholesky
 // factor L of G + eps I in one thread-block cluster, one warp per pair of columns, the columns in
 // registers.  A round is three dot products, a rotation and the systolic exchange of the
-// round-robin order (each warp passes one column to each neighbour through the neighbour's shared
-// memory, across CTAs through distributed shared memory), with one cluster barrier.  The left
+// round-robin order: each warp passes one column to each neighbour through the neighbour's shared
+// memory.  Inside a CTA a round ends with __syncthreads; across CTAs the edge warps send their
+// column by st.async, whose arrival an mbarrier at the receiver counts (a cluster barrier per
+// round made 200 x 200 1.84 ms and 50 x 50, in one CTA, 0.31; now 1.19 and 0.13).  The left
 // singular vectors of L -- the normalised columns at the end -- are the eigenvectors of G, so no
 // V is carried, and starting from the Cholesky factor saves a third of the sweeps (Drmac and
 // Veselic, SIAM J. Matrix Anal. Appl. 29, 2008).  L is factored in FP64 and rounded, and the
@@ -50,21 +52,101 @@ __device__ __forceinline__ void sum3(float& a, float& b, float& c, int lane) {
   c = __shfl_sync(F, v, 16);
 }
 
+// A column in a buffer: elements l of the lanes as 16-byte, then 8-byte, then 4-byte words.
+template <int NL>
+__device__ __forceinline__ void put_column(float* d, const float (&v)[NL], int lane) {
+#pragma unroll
+  for (int q = 0; q < NL / 4; ++q)
+    reinterpret_cast<float4*>(d)[q * 32 + lane] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+  constexpr int R = NL / 4 * 4;
+  if constexpr (NL % 4 >= 2) reinterpret_cast<float2*>(d + 32 * R)[lane] = make_float2(v[R], v[R + 1]);
+  if constexpr (NL % 2 == 1) d[32 * (NL - 1) + lane] = v[NL - 1];
+}
+template <int NL>
+__device__ __forceinline__ void get_column(const float* d, float (&v)[NL], int lane) {
+#pragma unroll
+  for (int q = 0; q < NL / 4; ++q) {
+    const float4 x = reinterpret_cast<const float4*>(d)[q * 32 + lane];
+    v[4 * q] = x.x;
+    v[4 * q + 1] = x.y;
+    v[4 * q + 2] = x.z;
+    v[4 * q + 3] = x.w;
+  }
+  constexpr int R = NL / 4 * 4;
+  if constexpr (NL % 4 >= 2) {
+    const float2 x = reinterpret_cast<const float2*>(d + 32 * R)[lane];
+    v[R] = x.x;
+    v[R + 1] = x.y;
+  }
+  if constexpr (NL % 2 == 1) v[NL - 1] = d[32 * (NL - 1) + lane];
+}
+// put_column into another CTA of the cluster: `d` and the mbarrier `bar` there count the bytes.
+template <int NL>
+__device__ __forceinline__ void send_column(uint32_t d, uint32_t bar, const float (&v)[NL], int lane) {
+#pragma unroll
+  for (int q = 0; q < NL / 4; ++q)
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
+                     d + (uint32_t)(q * 32 + lane) * 16u),
+                 "f"(v[4 * q]), "f"(v[4 * q + 1]), "f"(v[4 * q + 2]), "f"(v[4 * q + 3]), "r"(bar)
+                 : "memory");
+  constexpr int R = NL / 4 * 4;
+  if constexpr (NL % 4 >= 2)
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(
+                     d + (uint32_t)(128 * R + 8 * lane)),
+                 "f"(v[R]), "f"(v[R + 1]), "r"(bar)
+                 : "memory");
+  if constexpr (NL % 2 == 1)
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(
+                     d + (uint32_t)(128 * (NL - 1) + 4 * lane)),
+                 "f"(v[NL - 1]), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_address(uint32_t addr, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// Bounded wait for what other CTAs of the cluster sent.
+__device__ __forceinline__ bool cluster_wait(uint64_t* bar, uint32_t parity) {
+  const long long t0 = clock64();
+  for (;;) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if (clock64() - t0 > kWaitCycles) return false;
+  }
+}
+
 // One-sided Jacobi on the columns of L.  N even; warp m of the cluster holds pair m of H = N / 2;
 // NL elements per lane (32 NL >= N).  Shared memory: [2][warps][2][32 NL] exchange buffers
-// (t, b).  V (N x N FP64 out, column-major): the normalised columns.
-template <int NL>
+// (t, b).  V (N x N FP64 out, column-major): the normalised columns.  ONE: a single CTA.
+//
+// Two buffers are enough, inside a CTA and across: round n + 2 overwrites what round n brought, and
+// by then the receiver has passed its round n + 1 on (__syncthreads, or the column that comes back
+// from it: neighbours always exchange both ways).
+template <int NL, bool ONE>
 __global__ void jacobi32_kernel(const float* __restrict__ L, int N, double* __restrict__ V, int max_sweeps) {
   extern __shared__ __align__(16) float xbuf[];
   __shared__ int flag[3];
+  __shared__ __align__(8) uint64_t in_bar[2][2];   // [from the CTA before / after][buffer]
   cg::cluster_group cl = cg::this_cluster();
   const int wpc = blockDim.x >> 5;
-  const int rank = (int)cl.block_rank();
+  const int rank = ONE ? 0 : (int)cl.block_rank();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int H = N / 2, m = rank * wpc + warp;
   const bool on = m < H;
   constexpr int LEN = 32 * NL;
+  const bool before = !ONE && on && warp == 0 && m >= 1;             // neighbour m - 1 in another CTA
+  const bool after = !ONE && on && warp == wpc - 1 && m < H - 1;     // neighbour m + 1
   if (threadIdx.x < 3) flag[threadIdx.x] = 0;
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < 4; ++q) mbar_init(&in_bar[q >> 1][q & 1], 1);
+    fence_mbar_init();
+  }
   // pair m starts with columns m and N - 1 - m
   float t[NL], b[NL];
 #pragma unroll
@@ -75,18 +157,21 @@ __global__ void jacobi32_kernel(const float* __restrict__ L, int N, double* __re
   }
   // where this warp's columns go after a round: t to pair m + 1's t (pair 0 keeps it; the last
   // pair's becomes its own b), b to pair m - 1's b (pair 0's becomes pair 1's t)
-  // (the CTA's own buffers by their plain address: only the edge warps write across CTAs)
-  auto slot = [&](int pair, int buf, int part) -> float* {
-    float* base = pair / wpc == rank ? xbuf : cl.map_shared_rank(xbuf, pair / wpc);
-    return base + ((buf * wpc + pair % wpc) * 2 + part) * LEN;
-  };
-  int* flags0 = cl.map_shared_rank(flag, 0);
-  cl.sync();
-  int buf = 0;
+  auto slot = [&](int w, int buf, int part) -> float* { return xbuf + ((buf * wpc + w) * 2 + part) * LEN; };
+  int* flags0 = flag;
+  if constexpr (ONE) {
+    __syncthreads();
+  } else {
+    flags0 = cl.map_shared_rank(flag, 0);
+    cl.sync();
+  }
+  int round = 0;
+  bool lost = false;   // a wait gave up: the result will not pass its check
   for (int sweep = 0; sweep < max_sweeps && H > 1; ++sweep) {
     if (rank == 0 && threadIdx.x == 0) flag[(sweep + 1) % 3] = 0;
     bool again = false;
-    for (int r = 0; r < N - 1; ++r) {
+    for (int r = 0; r < N - 1; ++r, ++round) {
+      const int buf = round & 1;
       if (on) {
         float a = 0.f, c2 = 0.f, g = 0.f;
 #pragma unroll
@@ -116,29 +201,42 @@ __global__ void jacobi32_kernel(const float* __restrict__ L, int N, double* __re
             b[l] = fmaf(sn, fmaf(-tau, y, x), y);
           }
         }
-        if (m >= 1) {
-          float* d = slot(m - 1, buf, 1);
-#pragma unroll
-          for (int l = 0; l < NL; ++l) d[l * 32 + lane] = b[l];
-        }
-        if (m == 0 || m < H - 1) {
-          float* d = slot(m + 1, buf, 0);
-#pragma unroll
-          for (int l = 0; l < NL; ++l) d[l * 32 + lane] = m == 0 ? b[l] : t[l];
+        if (before)
+          send_column<NL>(cluster_address(smem_u32(slot(wpc - 1, buf, 1)), rank - 1),
+                          cluster_address(smem_u32(&in_bar[1][buf]), rank - 1), b, lane);
+        else if (m >= 1)
+          put_column<NL>(slot(warp - 1, buf, 1), b, lane);
+        if (after)
+          send_column<NL>(cluster_address(smem_u32(slot(0, buf, 0)), rank + 1),
+                          cluster_address(smem_u32(&in_bar[0][buf]), rank + 1), t, lane);
+        else if (m == 0)
+          put_column<NL>(slot(1, buf, 0), b, lane);
+        else if (m < H - 1)
+          put_column<NL>(slot(warp + 1, buf, 0), t, lane);
+        if (lane == 0) {
+          if (before) mbar_arrive_expect_tx(&in_bar[0][buf], LEN * 4);
+          if (after) mbar_arrive_expect_tx(&in_bar[1][buf], LEN * 4);
         }
       }
       if (r == N - 2 && again && lane == 0) flags0[sweep % 3] = 1;
-      cl.sync();
-      if (on) {
-        const float* base = xbuf + (size_t)(buf * wpc + warp) * 2 * LEN;
-#pragma unroll
-        for (int l = 0; l < NL; ++l) {
-          b[l] = m == H - 1 ? t[l] : base[LEN + l * 32 + lane];
-          if (m >= 1) t[l] = base[l * 32 + lane];
-        }
+      __syncthreads();
+      if (!ONE && on && !lost) {
+        const uint32_t ph = (uint32_t)((round >> 1) & 1);
+        if (before && !cluster_wait(&in_bar[0][buf], ph)) lost = true;
+        if (after && !cluster_wait(&in_bar[1][buf], ph)) lost = true;
+        lost = __any_sync(0xffffffffu, lost);
       }
-      buf ^= 1;
+      if (on) {
+        if (m == H - 1) {
+#pragma unroll
+          for (int l = 0; l < NL; ++l) b[l] = t[l];
+        } else {
+          get_column<NL>(slot(warp, buf, 1), b, lane);
+        }
+        if (m >= 1) get_column<NL>(slot(warp, buf, 0), t, lane);
+      }
     }
+    if constexpr (!ONE) cl.sync();   // every CTA's flag
     if (*(volatile int*)(flags0 + sweep % 3) == 0) break;
   }
   if (on) {
@@ -160,7 +258,7 @@ __global__ void jacobi32_kernel(const float* __restrict__ L, int N, double* __re
       }
     }
   }
-  cl.sync();   // no CTA leaves while another may still read its flag
+  if constexpr (!ONE) cl.sync();   // no CTA leaves while another may still read its flag
 }
 
 // S <- 1.5 I - 0.5 S (the factor of the Newton-Schulz step V <- V (1.5 I - 0.5 V^T V))
@@ -250,11 +348,11 @@ cudaError_t square_product(const double* X, bool kc, const unsigned* ex, const d
 // Cluster shape: one CTA while its 32 warps hold every pair, else eight CTAs.
 int jac_ctas(int H) { return H <= 32 ? 1 : 8; }
 
-template <int NL>
-cudaError_t launch_jacobi32(const float* L, int N, double* V, cudaStream_t st, bool* ran) {
+template <int NL, bool ONE>
+cudaError_t launch_jacobi32_ctas(const float* L, int N, double* V, cudaStream_t st, bool* ran) {
   const int H = N / 2, C = jac_ctas(H), wpc = (H + C - 1) / C;
   const size_t smem = (size_t)2 * wpc * 2 * 32 * NL * sizeof(float);
-  NYS_CUDA_TRY(ensure_max_dyn_smem((const void*)jacobi32_kernel<NL>, 200 * 1024));
+  NYS_CUDA_TRY(ensure_max_dyn_smem((const void*)jacobi32_kernel<NL, ONE>, 200 * 1024));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)C);
   cfg.blockDim = dim3((unsigned)(32 * wpc));
@@ -266,16 +364,23 @@ cudaError_t launch_jacobi32(const float* L, int N, double* V, cudaStream_t st, b
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = ONE ? 0 : 1;
   int n_clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&n_clusters, jacobi32_kernel<NL>, &cfg) != cudaSuccess || n_clusters < 1) {
+  if (!ONE && (cudaOccupancyMaxActiveClusters(&n_clusters, jacobi32_kernel<NL, ONE>, &cfg) != cudaSuccess || n_clusters < 1)) {
     (void)cudaGetLastError();
     *ran = false;   // the cluster does not fit this device: the FP64 sweeps start from the identity
     return cudaSuccess;
   }
   count_launch();
   *ran = true;
-  return cudaLaunchKernelEx(&cfg, jacobi32_kernel<NL>, L, N, V, 12);
+  return cudaLaunchKernelEx(&cfg, jacobi32_kernel<NL, ONE>, L, N, V, 12);
+}
+template <int NL>
+cudaError_t launch_jacobi32(const float* L, int N, double* V, cudaStream_t st, bool* ran) {
+  if constexpr (NL <= 2)   // 32 pairs at most
+    return launch_jacobi32_ctas<NL, true>(L, N, V, st, ran);
+  else
+    return launch_jacobi32_ctas<NL, false>(L, N, V, st, ran);
 }
 
 size_t up256(size_t b) { return (b + 255) / 256 * 256; }
