@@ -129,14 +129,14 @@ template <int AT, int BT, int BM2> constexpr int tc_stages() {
 // Epilogue of both staging forms: TMEM -> registers (tcgen05.ld; warp w reads lanes
 // 32 (w % 4) .. + 31 and half the columns), then W's three BF16 terms (EPI 0, rows scaled
 // by D) or the split-K slice's FP32 partial (EPI 1).
-template <int EPI, int BM2>
+template <int EPI, int BM2, int ACC = TC_NMAX>
 __device__ __forceinline__ void tc_epilogue(const TcArgs& a, uint32_t tmem, int64_t m0, int nkt, int warp, int lane) {
   const int quad = warp & 3;
   const int half = a.NP / 2;
   const int cb = (warp >> 2) * half;
   for (int h = 0; h < BM2; ++h) {
     const int64_t row = m0 + h * TC_BM + 32 * quad + lane;
-    const uint32_t trow = tmem + (uint32_t)(h * TC_NMAX) + ((uint32_t)(32 * quad) << 16);
+    const uint32_t trow = tmem + (uint32_t)(h * ACC) + ((uint32_t)(32 * quad) << 16);
     double dr = 1.0;
     if (EPI == 0 && a.D && row < a.Mrows) dr = a.D[row];
     for (int c0 = cb; c0 < cb + half; c0 += 8) {
@@ -423,10 +423,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 //
 // FP32 storage: the three terms of a stage go to TMEM (48 columns beside the accumulator) and the
 // MMAs take A from there, which leaves shared memory to the raw ring (up to eight tiles) and B.
-// 50,000 x 4,000 by 64 columns: 256 us, A^T of it 212 us (terms in shared memory, one group of
-// eight warps: 336 and 268; two groups: 267 and 222).  An MMA of 64 columns onto one accumulator
-// then takes ~100 clocks, three times its multiplication, and that sets the pace; the read of A
-// is 118 us.  The order of the MMAs, and with it the rounding, is kept, so they stay in one chain.
+// With one tile of 128 rows per CTA a stage takes ~1,240 clocks, 12 MMAs of 64 columns onto one
+// accumulator (three groups of warps instead of two: no change; terms in shared memory: 5 % more);
+// up to three tiles per CTA take turns and share the B stage: 950 a tile (td_tiles).  The order of the
+// MMAs of an accumulator, and with it the rounding, is kept.
 // BF16 storage (A^T only): repacked into the K-major core-matrix layout of a stage (8 rows x 16 bytes
 // contiguous, K chunks 128 B and row groups 512 B apart); its two accumulators fill TMEM, and
 // at 200 columns the MMAs bound it (100,000 x 10,000: 0.65 ms; transposing A first cost 0.81 ms
@@ -439,9 +439,12 @@ template <int AT, int BT, int BM2, int NM> constexpr int td_stage_max() {   // A
 }
 constexpr int kTdSmem = 222 * 1024;
 template <int AT> constexpr int td_raw_min() { return AT == 3 ? 4 : 3; }
-template <int DT, int AT, int BT, int BM2, int NM> constexpr int td_stages() {   // converted stages: up to 3 (TMEM: 5)
+template <int AT, int NM> constexpr int td_acc() { return AT == 3 && NM <= 128 ? (NM <= 64 ? 64 : 128) : TC_NMAX; }   // columns
+template <int DT, int AT, int BT, int BM2, int NM> constexpr int td_stages() {   // converted stages
   constexpr int fit = (kTdSmem - td_raw_min<AT>() * td_raw_bytes<DT, BM2>()) / td_stage_max<AT, BT, BM2, NM>();
-  return fit < (AT == 3 ? 5 : 3) ? fit : (AT == 3 ? 5 : 3);
+  constexpr int most = AT == 3 ? (512 - BM2 * td_acc<AT, NM>()) / (48 * BM2) : 3;   // (FP32: the terms' TMEM)
+  constexpr int cap = most < 5 ? most : 5;
+  return fit < cap ? fit : cap;
 }
 template <int DT, int AT, int BT, int BM2, int NM> constexpr int td_raw_stages() {   // raw stages: up to 8
   constexpr int fit = (kTdSmem - td_stages<DT, AT, BT, BM2, NM>() * td_stage_max<AT, BT, BM2, NM>()) / td_raw_bytes<DT, BM2>();
@@ -464,10 +467,11 @@ __global__ void __launch_bounds__(TD_THREADS, 1)
                             const __grid_constant__ CUtensorMap tmB) {
   constexpr bool TRANS = EPI == 1;
   constexpr int ST = td_stages<DT, AT, BT, BM2, NM>(), RT = td_raw_stages<DT, AT, BT, BM2, NM>();
-  static_assert(ST >= 2 && RT >= 3, "shared memory holds too few stages");
+  static_assert(ST >= 2 && RT >= 3 && RT >= ST, "shared memory holds too few stages");
   static_assert(DT == NYS_F32 || TRANS, "BF16 rows need no conversion");
   constexpr bool TA = DT == NYS_F32;   // A's terms in TMEM, 16 columns per term of a stage
-  static_assert(!TA || (BM2 == 1 && AT == 3 && TC_NMAX + 48 * ST <= 512), "TMEM columns");
+  constexpr int ACC = td_acc<AT, NM>();   // columns from one accumulator to the next; the terms follow the last
+  static_assert(!TA || (AT == 3 && BM2 * (ACC + 48 * ST) <= 512), "TMEM columns");
   constexpr uint32_t kTmemCols = 2 * TC_NMAX;
   constexpr int R = TC_BM * BM2;
   constexpr uint32_t RAW = td_raw_bytes<DT, BM2>();
@@ -506,6 +510,9 @@ __global__ void __launch_bounds__(TD_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
 
+  // A group turns to stage kt + TD_G knowing that the MMAs up to kt - ST are done, and the wait for the
+  // slot's last use tells that use only from the one before.
+  static_assert(TD_G <= ST, "more groups than converted stages");
   if (warp < 8 * TD_G) {
     const int gt = tid & 255;   // thread of the group
     for (int kt = warp >> 3; kt < nkt && !s_fail; kt += TD_G) {
@@ -518,27 +525,32 @@ __global__ void __launch_bounds__(TD_THREADS, 1)
       }
       tc_fence_after();   // the stage's last MMAs are done with it
       if constexpr (DT == NYS_F32) {
-        // warp w: rows 32 (w % 4) + lane (its lanes of TMEM), K 16 (w / 4) .. + 15
+        // warp w: rows 32 (w % 4) + lane of each 128-row tile (its lanes of TMEM), K 16 (w / 4) .. + 15
         const int row = 32 * (warp & 3) + lane, half = (warp >> 2) & 1;
-        float x[16];
-        if constexpr (TRANS) {
+#pragma unroll 1
+        for (int h = 0; h < BM2; ++h) {
+          const uint32_t rt = raw + (uint32_t)(h * TC_BM * TC_BK * 4);
+          float x[16];
+          if constexpr (TRANS) {
 #pragma unroll
-          for (int e = 0; e < 16; ++e)
-            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x[e]) : "r"(raw + (uint32_t)(((16 * half + e) * R + row) * 4)));
-        } else {
-          // 128-byte rows with the 128-byte swizzle: 16-byte chunk c of row r sits at c ^ (r & 7)
+            for (int e = 0; e < 16; ++e)
+              asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x[e]) : "r"(rt + (uint32_t)(((16 * half + e) * TC_BM + row) * 4)));
+          } else {
+            // 128-byte rows with the 128-byte swizzle: 16-byte chunk c of row r sits at c ^ (r & 7)
 #pragma unroll
-          for (int h = 0; h < 4; ++h)
-            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                         : "=f"(x[4 * h]), "=f"(x[4 * h + 1]), "=f"(x[4 * h + 2]), "=f"(x[4 * h + 3])
-                         : "r"(raw + (uint32_t)(row * 128 + ((4 * half + h) ^ (row & 7)) * 16)));
+            for (int c = 0; c < 4; ++c)
+              asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                           : "=f"(x[4 * c]), "=f"(x[4 * c + 1]), "=f"(x[4 * c + 2]), "=f"(x[4 * c + 3])
+                           : "r"(rt + (uint32_t)(row * 128 + ((4 * half + c) ^ (row & 7)) * 16)));
+          }
+          uint32_t w[3][8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) split3_pair(x[2 * e], x[2 * e + 1], w[0][e], w[1][e], w[2][e]);
+          const uint32_t ta = tmem + ((uint32_t)(32 * (warp & 3)) << 16) +
+                              (uint32_t)(BM2 * ACC + 48 * (s * BM2 + h) + 8 * half);
+#pragma unroll
+          for (int t = 0; t < 3; ++t) tmem_st8(ta + (uint32_t)(16 * t), w[t]);
         }
-        uint32_t w[3][8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) split3_pair(x[2 * e], x[2 * e + 1], w[0][e], w[1][e], w[2][e]);
-        const uint32_t ta = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(TC_NMAX + 48 * s + 8 * half);
-#pragma unroll
-        for (int t = 0; t < 3; ++t) tmem_st8(ta + (uint32_t)(16 * t), w[t]);
         tmem_st_wait();
       } else {
         auto put = [&](int term, int row, int chunk, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
@@ -583,8 +595,15 @@ __global__ void __launch_bounds__(TD_THREADS, 1)
       }
       const int k0 = (int)((kt0 + kt) * TC_BK);
       mbar_arrive_expect_tx(&raw_full[rs], RAW);
-      if (TRANS) tma_load_2d(rbase + rs * RAW, &tmA, (int)m0, k0, &raw_full[rs]);
-      else tma_load_2d(rbase + rs * RAW, &tmA, k0, (int)m0, &raw_full[rs]);
+      // FP32: a box of 128 rows (columns of A^T) per tile; BF16: one of 256
+      constexpr int BOXES = TA ? BM2 : 1;
+#pragma unroll
+      for (int h = 0; h < BOXES; ++h) {
+        const uint32_t dst = rbase + rs * RAW + (uint32_t)(h * TC_BM * TC_BK * 4);
+        const int mh = (int)m0 + h * TC_BM;
+        if (TRANS) tma_load_2d(dst, &tmA, mh, k0, &raw_full[rs]);
+        else tma_load_2d(dst, &tmA, k0, mh, &raw_full[rs]);
+      }
     }
     // copies still in flight land in this CTA's shared memory: wait for them (bounded)
     for (int j = max(0, kt - RT); j < kt; ++j) (void)mbar_wait_bounded(&raw_full[j % RT], (uint32_t)((j / RT) & 1));
@@ -610,17 +629,19 @@ __global__ void __launch_bounds__(TD_THREADS, 1)
       }
       tc_fence_after();
       const uint32_t st = sbase + (uint32_t)s * stage_bytes;
+      // the tiles take turns: an MMA need not wait for the one before it on the same accumulator
 #pragma unroll
       for (int kk = 0; kk < TC_BK / 16; ++kk) {
 #pragma unroll
-        for (int h = 0; h < BM2; ++h) {
+        for (int pr = 0; pr < tc_npairs<AT, BT>(); ++pr) {
+          const uint64_t bd = smem_desc_sw64(st + AT * A_TERM + (uint32_t)tc_pair_b<AT, BT>(pr) * b_term + (uint32_t)(kk * 32),
+                                             512u);
+          const uint32_t acc = (kt | kk | pr) != 0 ? 1u : 0u;
 #pragma unroll
-          for (int pr = 0; pr < tc_npairs<AT, BT>(); ++pr) {
-            const uint64_t bd = smem_desc_sw64(st + AT * A_TERM + (uint32_t)tc_pair_b<AT, BT>(pr) * b_term + (uint32_t)(kk * 32),
-                                               512u);
-            const uint32_t acc = (kt | kk | pr) != 0 ? 1u : 0u;
+          for (int h = 0; h < BM2; ++h) {
             if constexpr (TA) {
-              mma_bf16_ta(tmem, tmem + (uint32_t)(TC_NMAX + 48 * s + 16 * tc_pair_a<AT, BT>(pr) + 8 * kk), bd, idesc, acc);
+              mma_bf16_ta(tmem + (uint32_t)(h * ACC),
+                          tmem + (uint32_t)(BM2 * ACC + 48 * (s * BM2 + h) + 16 * tc_pair_a<AT, BT>(pr) + 8 * kk), bd, idesc, acc);
             } else {
               const uint64_t ad = smem_desc(st + (uint32_t)tc_pair_a<AT, BT>(pr) * A_TERM + (uint32_t)(h * 16 * 512 + kk * 256),
                                             TC_LBO, TC_SBO);
@@ -639,7 +660,7 @@ __global__ void __launch_bounds__(TD_THREADS, 1)
   ok = __syncthreads_and(ok);
   tc_fence_after();
   if (ok) {
-    if (warp < 8) tc_epilogue<EPI, BM2>(a, tmem, m0, nkt, warp, lane);
+    if (warp < 8) tc_epilogue<EPI, BM2, ACC>(a, tmem, m0, nkt, warp, lane);
   } else if (tid == 0) {
     atomicExch(a.status, (int)NYS_ETIMEOUT);
     if (nkt > 0) (void)mbar_wait_bounded(&empty_bar[(nkt - 1) % ST], (uint32_t)(((nkt - 1) / ST) & 1));
@@ -835,26 +856,61 @@ cudaError_t launch_tc(const TcArgs& a, dim3 grid, cudaStream_t st) {
 }
 
 template <int EPI, int DT, int AT, int BT, int BM2, int NM>
-cudaError_t launch_direct_nm(const nys_matrix* A, const TcArgs& a, dim3 grid, cudaStream_t st) {
+cudaError_t launch_direct_nm(const nys_matrix* A, const TcArgs& a, int64_t slices, cudaStream_t st) {
   constexpr int ST = td_stages<DT, AT, BT, BM2, NM>(), RT = td_raw_stages<DT, AT, BT, BM2, NM>();
   const size_t smem = (size_t)RT * td_raw_bytes<DT, BM2>() +
                       (size_t)ST * ((AT == 3 ? 0 : BM2 * AT * TC_BM * TC_BK * 2) + (size_t)BT * a.NP * TC_BK * 2);
   CUtensorMap tmA, tmB;
-  NYS_CUDA_TRY(make_raw_map(&tmA, A, EPI == 1, TC_BM * BM2));
+  NYS_CUDA_TRY(make_raw_map(&tmA, A, EPI == 1, DT == NYS_F32 ? TC_BM : TC_BM * BM2));
   NYS_CUDA_TRY(make_tile_map(&tmB, a.B, a.ktiles * TC_BK, a.NP, a.ldb, BT, a.bterm, a.NP));
   auto fn = sketch_tc_direct_kernel<EPI, DT, AT, BT, BM2, NM>;
   NYS_CUDA_TRY(ensure_max_dyn_smem((const void*)fn, kTdSmem));
   count_launch();
+  const dim3 grid((unsigned)((a.Mrows + TC_BM * BM2 - 1) / (TC_BM * BM2)), (unsigned)slices);
   fn<<<grid, TD_THREADS, smem, st>>>(a, tmA, tmB);
   return cudaGetLastError();
 }
+// FP32: 128-row tiles per CTA, up to `most`, that finish the product's waves over the SMs first.  A wave
+// of CTAs of one tile, two and three takes 1 : 1.6 : 2.2 with up to 64 columns (50,000 x 4,000 by 64: 85,
+// 135, 187 us) and 1 : 1.9 with up to 128, so three tiles fill the chip where one leaves 3 waves
+// (391 CTAs: 256 -> 187 us; A^T of it, 32 tiles in 19 slices: 212 -> 170 us with two).
+int td_tiles(int64_t mtiles, int64_t slices, int most, int sms) {
+  const double cost[4] = {0.0, 1.0, most == 3 ? 1.6 : 1.9, 2.2};
+  int best = 1;
+  double t = 0.0;
+  for (int q = 1; q <= most; ++q) {
+    const int64_t ctas = (mtiles + q - 1) / q * slices;
+    const double tq = (double)((ctas + sms - 1) / sms) * cost[q];
+    if (q == 1 || tq < t) {
+      best = q;
+      t = tq;
+    }
+  }
+  return best;
+}
 // stage counts from the columns: at most 64, 128, 208 (rank 200: three stages of GEMM 2 just fit), 256
-template <int EPI, int DT, int AT, int BT, int BM2>
-cudaError_t launch_direct(const nys_matrix* A, const TcArgs& a, dim3 grid, cudaStream_t st) {
-  if (a.NP <= 64) return launch_direct_nm<EPI, DT, AT, BT, BM2, 64>(A, a, grid, st);
-  if (a.NP <= 128) return launch_direct_nm<EPI, DT, AT, BT, BM2, 128>(A, a, grid, st);
-  if (a.NP <= 208) return launch_direct_nm<EPI, DT, AT, BT, BM2, 208>(A, a, grid, st);
-  return launch_direct_nm<EPI, DT, AT, BT, BM2, 256>(A, a, grid, st);
+template <int EPI, int DT, int AT, int BT>
+cudaError_t launch_direct(const nys_matrix* A, const TcArgs& a, int64_t slices, cudaStream_t st) {
+  if constexpr (DT == NYS_F32) {
+    const int64_t mtiles = (a.Mrows + TC_BM - 1) / TC_BM;
+    if (a.NP <= 64) {
+      switch (td_tiles(mtiles, slices, 3, sm_count_tc())) {
+        case 3: return launch_direct_nm<EPI, DT, AT, BT, 3, 64>(A, a, slices, st);
+        case 2: return launch_direct_nm<EPI, DT, AT, BT, 2, 64>(A, a, slices, st);
+        default: return launch_direct_nm<EPI, DT, AT, BT, 1, 64>(A, a, slices, st);
+      }
+    }
+    if (a.NP <= 128)
+      return td_tiles(mtiles, slices, 2, sm_count_tc()) == 2 ? launch_direct_nm<EPI, DT, AT, BT, 2, 128>(A, a, slices, st)
+                                                             : launch_direct_nm<EPI, DT, AT, BT, 1, 128>(A, a, slices, st);
+    if (a.NP <= 208) return launch_direct_nm<EPI, DT, AT, BT, 1, 208>(A, a, slices, st);
+    return launch_direct_nm<EPI, DT, AT, BT, 1, 256>(A, a, slices, st);
+  } else {
+    if (a.NP <= 64) return launch_direct_nm<EPI, DT, AT, BT, 2, 64>(A, a, slices, st);
+    if (a.NP <= 128) return launch_direct_nm<EPI, DT, AT, BT, 2, 128>(A, a, slices, st);
+    if (a.NP <= 208) return launch_direct_nm<EPI, DT, AT, BT, 2, 208>(A, a, slices, st);
+    return launch_direct_nm<EPI, DT, AT, BT, 2, 256>(A, a, slices, st);
+  }
 }
 
 // Output rows per CTA: two 128-row accumulators, except for FP32 x FP32 (six MMA pairs),
@@ -963,8 +1019,8 @@ cudaError_t tc_enqueue(const nys_matrix* A, const TcPrepared& prep, const double
     g1.status = status;
     const dim3 grid1((unsigned)((n + h.rows1 - 1) / h.rows1), 1), grid2((unsigned)h.mt2, (unsigned)h.Zeff);
     if (prep.direct && prep.at == 3)
-      NYS_CUDA_TRY(xterms == 3 ? (launch_direct<0, NYS_F32, 3, 3, 1>(A, g1, grid1, st))
-                               : (launch_direct<0, NYS_F32, 3, 1, 1>(A, g1, grid1, st)));
+      NYS_CUDA_TRY(xterms == 3 ? (launch_direct<0, NYS_F32, 3, 3>(A, g1, 1, st))
+                               : (launch_direct<0, NYS_F32, 3, 1>(A, g1, 1, st)));
     else
       NYS_CUDA_TRY(launch_tc_at<0>(prep.at, xterms, g1, grid1, st));
     if (c0 == 0) mark();
@@ -986,8 +1042,8 @@ cudaError_t tc_enqueue(const nys_matrix* A, const TcPrepared& prep, const double
     g2.desc_swap = swap;
     g2.status = status;
     if (prep.direct)
-      NYS_CUDA_TRY(prep.at == 3 ? (launch_direct<1, NYS_F32, 3, 3, 1>(A, g2, grid2, st))
-                                : (launch_direct<1, NYS_BF16, 1, 3, 2>(A, g2, grid2, st)));
+      NYS_CUDA_TRY(prep.at == 3 ? (launch_direct<1, NYS_F32, 3, 3>(A, g2, h.Zeff, st))
+                                : (launch_direct<1, NYS_BF16, 1, 3>(A, g2, h.Zeff, st)));
     else
       NYS_CUDA_TRY(launch_tc_at<1>(prep.at, TC_TERMS, g2, grid2, st));
     if (c0 == 0) mark();
