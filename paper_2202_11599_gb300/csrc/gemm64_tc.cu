@@ -1,11 +1,11 @@
-// FP64 matrix products on the BF16 tensor cores.
+// FP64 matrix products on the FP16 tensor cores.
 //
 //   C (M x N) = diag(D) A B^T,   A(m, k), B(n, k) FP64
 //
-// GB300's FP64 pipe retires about 2 FMA per clock and SM; its BF16 tensor cores ~3,400 MAC.
+// GB300's FP64 pipe retires about 2 FMA per clock and SM; its tensor cores ~3,400 MAC.
 // Each operand row is written in fixed point relative to its own largest exponent, as eight
 // signed 8-bit digits (62 bits below the row's maximum):
-//   A(m, k) = 2^(ea_m - 1084) sum_i a_i 256^(7 - i),  a_i in [-128, 127] (exact in BF16),
+//   A(m, k) = 2^(ea_m - 1084) sum_i a_i 256^(7 - i),  a_i in [-128, 127] (exact in FP16),
 // so a product of digits is an integer of at most 2^14, and the tensor core's FP32
 // accumulators add them exactly while |sum| < 2^24.  The digit products of equal weight
 // (order o = i + j = 0 .. 7, o + 1 pairs) share one TMEM accumulator: 36 MMAs per K step for
@@ -20,18 +20,20 @@
 // against 1e-16 to 8e-15 for a chain of FP64 FMAs.  A row holding a NaN or an infinity gives NaN.
 //
 // Measured (FP64 pipe before, this kernel after): the two products of a 40,000 x 4,000 sketch of
-// rank 100, 36.1 + 40.4 ms -> 1.85 + 1.85 ms; X^T Y at 10,000 x 200, 0.52 (symmetric) and 0.90 ms
-// -> 0.11 ms; U = B V at 10,000 x 200, 1.09 -> 0.06 ms.
+// rank 100, 36.1 + 40.4 ms -> 1.7 + 1.7 ms; X^T Y at 10,000 x 200, 0.52 (symmetric) and 0.90 ms
+// -> 0.1 ms; U = B V at 10,000 x 200, 1.09 -> 0.05 ms.
 //
-// What bounds it: per 32 K a tile makes the digits of 6,144 elements (~30 integer operations each)
-// and issues 72 MMAs (multiplying takes 2,300 clocks, reading A and B from shared memory 3,500);
-// together it takes 6,700.  So sixteen warps convert, one thread issues the MMAs, and they meet
-// only through mbarriers; the read-out of a 256-K group runs after the next stage's digits are
-// written; MMAs that share an A tile follow each other and keep it in the collector.  (With one
-// warp doing both and a barrier per stage: 9,200 clocks, tensor pipe 26 % active.)  Both operands
-// are converted in the kernel: the digits are never written to memory, and an operand stored
-// along M (A^T) is transposed on the way into shared memory.
-#include <cuda_bf16.h>
+// What bounds it: per 32 K a tile makes the digits of 6,144 elements (~40 integer operations each at
+// 64 lanes per clock: 3,900 clocks) and issues 72 MMAs (multiplying takes 2,300, reading A and B
+// from shared memory 3,500); together it takes 6,100.  So sixteen warps convert, one thread
+// issues the MMAs, and they meet only through mbarriers; the read-out of a 256-K group runs after
+// the next stage's digits are written; MMAs that share an A tile follow each other and keep it
+// in the collector; a digit is one byte in the significand of an FP16 number and one
+// subtraction (in BF16 pairs: three integer operations more per two digits, 8 % of the kernel).
+// (One warp doing both and a barrier per stage: 9,200 clocks, tensor pipe 26 % active.)  Both
+// operands are converted in the kernel: the digits are never written to memory, and an operand
+// stored along M (A^T) is transposed on the way into shared memory.
+#include <cuda_fp16.h>
 
 #include <algorithm>
 
@@ -84,16 +86,18 @@ __device__ __forceinline__ void digits(double x, int emax, uint32_t& lo, uint32_
   asm("add.cc.u32 %0, %2, %3;\n addc.u32 %1, %4, 0x80808080;" : "=r"(lo), "=r"(hi) : "r"(a), "r"(0x80808080u - sg), "r"(c));
 }
 
-// Digit b (0 = lowest byte) of two biased values as a BF16 pair: with d + 128 = 128 u + v
-// (v < 128), (128 + v) - (u ? 128 : 256) = d, all exact in BF16.
-template <int B>
-__device__ __forceinline__ uint32_t digit_pair(uint32_t x0, uint32_t x1) {
-  const uint32_t p = __byte_perm(x0, x1, B | (B << 4) | ((4 + B) << 8) | ((4 + B) << 12));
-  const uint32_t a = (p & 0x007f007fu) | 0x43004300u;
-  const uint32_t s = (~p & 0x00800080u) | 0x43004300u;
-  const __nv_bfloat162 r = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&a),
-                                   *reinterpret_cast<const __nv_bfloat162*>(&s));
-  return *reinterpret_cast<const uint32_t*>(&r);
+// The four digits of a word of two biased values as FP16 pairs, lowest byte first: 1,024 + (d + 128)
+// is the FP16 number 0x6400 | byte, so a byte needs no more than its place and one subtraction.
+__device__ __forceinline__ void digit_pairs(uint32_t x0, uint32_t x1, uint32_t (&d)[4]) {
+  const uint32_t lo = __byte_perm(x0, x1, 0x5140), hi = __byte_perm(x0, x1, 0x7362);   // bytes 0 0' 1 1', 2 2' 3 3'
+  const uint32_t m = 0x64646464u, off = 0x64806480u;                                   // off: 1,152 twice
+  const uint32_t p[4] = {__byte_perm(lo, m, 0x4140), __byte_perm(lo, m, 0x4342), __byte_perm(hi, m, 0x4140),
+                         __byte_perm(hi, m, 0x4342)};
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const __half2 r = __hsub2(*reinterpret_cast<const __half2*>(&p[b]), *reinterpret_cast<const __half2*>(&off));
+    d[b] = *reinterpret_cast<const uint32_t*>(&r);
+  }
 }
 
 // v 2^sh rounded once to FP64 (to nearest, ties to even).
@@ -164,7 +168,8 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
     ar = 32 * (warp & 3) + lane;
     ac = warp >> 2;
   }
-  const int br = (4 * warp + (lane >> 3)) % EN, bc = lane & 7;   // (the issuing warp converts nothing)
+  // (B: 16 lanes fill the two halves of eight rows; the issuing warpgroup converts nothing)
+  const int br = (8 * (warp >> 1) + ((lane >> 1) & 7)) % EN, bc = 2 * (2 * (warp & 1) + (lane >> 4)) + (lane & 1);
   const int64_t am = m0 + ar;
   const bool aok = am < a.M, bok = n0 + br < a.N;
   const int emA = aok ? max(1, (int)(a.ea[am] >> 20)) : 1;
@@ -215,17 +220,15 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
                      "r"(w2), "r"(w3)
                      : "memory");
       };
-#define NYS_PUT(SL, B, W) \
-  put(SL, digit_pair<B>(W[0], W[1]), digit_pair<B>(W[2], W[3]), digit_pair<B>(W[4], W[5]), digit_pair<B>(W[6], W[7]))
-      NYS_PUT(0, 3, hi);
-      NYS_PUT(1, 2, hi);
-      NYS_PUT(2, 1, hi);
-      NYS_PUT(3, 0, hi);
-      NYS_PUT(4, 3, lo);
-      NYS_PUT(5, 2, lo);
-      NYS_PUT(6, 1, lo);
-      NYS_PUT(7, 0, lo);
-#undef NYS_PUT
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        const uint32_t* w = half == 0 ? hi : lo;
+        uint32_t dg[4][4];   // [pair of elements][byte]
+#pragma unroll
+        for (int q = 0; q < 4; ++q) digit_pairs(w[2 * q], w[2 * q + 1], dg[q]);
+#pragma unroll
+        for (int b = 3; b >= 0; --b) put(4 * half + 3 - b, dg[0][b], dg[1][b], dg[2][b], dg[3][b]);
+      }
     }
     {
       uint32_t lo[4], hi[4];
@@ -238,16 +241,15 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
                      "r"(w1)
                      : "memory");
       };
-#define NYS_PUT(SL, B, W) put(SL, digit_pair<B>(W[0], W[1]), digit_pair<B>(W[2], W[3]))
-      NYS_PUT(0, 3, hi);
-      NYS_PUT(1, 2, hi);
-      NYS_PUT(2, 1, hi);
-      NYS_PUT(3, 0, hi);
-      NYS_PUT(4, 3, lo);
-      NYS_PUT(5, 2, lo);
-      NYS_PUT(6, 1, lo);
-      NYS_PUT(7, 0, lo);
-#undef NYS_PUT
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        const uint32_t* w = half == 0 ? hi : lo;
+        uint32_t dg[2][4];
+        digit_pairs(w[0], w[1], dg[0]);
+        digit_pairs(w[2], w[3], dg[1]);
+#pragma unroll
+        for (int b = 3; b >= 0; --b) put(4 * half + 3 - b, dg[0][b], dg[1][b]);
+      }
     }
   };
 
@@ -290,7 +292,7 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
     }
   };
 
-  constexpr uint32_t idesc = mma_idesc_bf16(EM, EN);
+  constexpr uint32_t idesc = mma_idesc_f16(EM, EN);
   // 20 warps of 96 registers; the issuing warpgroup gives up what the converting ones take
   // (512 x 112 + 128 x 24 = 60,416 of 640 x 96 = 61,440)
   if (warp < ECW) {
@@ -371,10 +373,10 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
         for (int i = 0; i < ESL; ++i) {
           const uint64_t ad = ad0 + (uint64_t)((i * EA_SLICE + kk * 256u) >> 4);
           const uint32_t acc = (first && kk == 0 && i == 0) ? 0u : 1u;
-          mma_bf16_same_a<true>(tmem + (uint32_t)(i * EN), ad, bd0 + (uint64_t)((kk * 256u) >> 4), idesc, acc);
+          mma_same_a<true>(tmem + (uint32_t)(i * EN), ad, bd0 + (uint64_t)((kk * 256u) >> 4), idesc, acc);
 #pragma unroll
           for (int o = i + 1; o < ESL; ++o)
-            mma_bf16_same_a<false>(tmem + (uint32_t)(o * EN), ad, bd0 + (uint64_t)(((o - i) * EB_SLICE + kk * 256u) >> 4),
+            mma_same_a<false>(tmem + (uint32_t)(o * EN), ad, bd0 + (uint64_t)(((o - i) * EB_SLICE + kk * 256u) >> 4),
                                    idesc, acc);
         }
       }

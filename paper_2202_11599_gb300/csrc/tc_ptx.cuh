@@ -38,6 +38,10 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr, uint32_t sbo) 
 __host__ __device__ constexpr uint32_t mma_idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
+// The same with A and B FP16 (formats 0).
+__host__ __device__ constexpr uint32_t mma_idesc_f16(int M, int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
 __device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate) {
   asm volatile(
@@ -46,10 +50,10 @@ __device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t adesc, uint64_
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// The same for a run of MMAs with one A tile: the first keeps it in the collector buffer, the next
+// kind::f16 again (BF16 or FP16 by the descriptor), for a run of MMAs with one A tile: the first keeps it in the collector buffer, the next
 // use it from there instead of reading it from shared memory again.
 template <bool FIRST>
-__device__ __forceinline__ void mma_bf16_same_a(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+__device__ __forceinline__ void mma_same_a(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                                 uint32_t accumulate) {
   if constexpr (FIRST)
     asm volatile(
