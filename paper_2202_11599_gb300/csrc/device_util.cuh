@@ -242,12 +242,11 @@ template <typename T>
 constexpr int kLoadBatch = sizeof(T) == 4 ? 64 : 32;
 
 // sum_{g < n} a[g * stride + j] added in increasing g (the order of a plain loop), the loads
-// issued kLoadBatch at a time so that a thread keeps that many reads in flight.  CG: read
-// through L2, for data written by other blocks of the running kernel.  The additions run in
-// groups of eight behind a branch for FP64: a predicated-off one still takes its 64 clocks.
-template <bool CG, typename T>
+// issued B at a time so that a thread keeps that many reads in flight.  CG: read through L2, for
+// data written by other blocks of the running kernel.  Short sums take a smaller B: the
+// additions past n are predicated off, and in FP64 each still takes its 64 clocks.
+template <bool CG, typename T, int B = kLoadBatch<T>>
 __device__ __forceinline__ T sum_strided_fixed(const T* a, int n, int64_t stride, int64_t j, T s) {
-  constexpr int B = kLoadBatch<T>, W = sizeof(T) == 8 ? 8 : B;
   for (int g = 0; g < n; g += B) {
     T v[B];
 #pragma unroll
@@ -257,12 +256,8 @@ __device__ __forceinline__ T sum_strided_fixed(const T* a, int n, int64_t stride
         v[q] = CG ? __ldcg(ptr) : *ptr;
       }
 #pragma unroll
-    for (int o = 0; o < B; o += W)
-      if (g + o < n) {
-#pragma unroll
-        for (int q = o; q < o + W; ++q)
-          if (g + q < n) s += v[q];
-      }
+    for (int q = 0; q < B; ++q)
+      if (g + q < n) s += v[q];
   }
   return s;
 }
@@ -311,22 +306,17 @@ __device__ __forceinline__ void pass_column_sums(const C* partial, int G, int64_
 }
 
 // acc + sum_{i0 <= i < i1} U[i * d + j] g[i] as one fma chain in increasing i, the loads of U
-// issued kLoadBatch at a time (groups of eight as in sum_strided_fixed).
-template <typename C>
+// issued B at a time.
+template <typename C, int B = kLoadBatch<C>>
 __device__ __forceinline__ C urow_dot(const C* __restrict__ U, int64_t d, int64_t j, int i0, int i1, const C* g, C acc) {
-  constexpr int B = kLoadBatch<C>, W = sizeof(C) == 8 ? 8 : B;
   for (int i = i0; i < i1; i += B) {
     C u[B];
 #pragma unroll
     for (int q = 0; q < B; ++q)
       if (i + q < i1) u[q] = U[(int64_t)(i + q) * d + j];
 #pragma unroll
-    for (int o = 0; o < B; o += W)
-      if (i + o < i1) {
-#pragma unroll
-        for (int q = o; q < o + W; ++q)
-          if (i + q < i1) acc = fma(u[q], g[i + q], acc);
-      }
+    for (int q = 0; q < B; ++q)
+      if (i + q < i1) acc = fma(u[q], g[i + q], acc);
   }
   return acc;
 }
@@ -350,7 +340,10 @@ __device__ __forceinline__ void u_times_g(const C* __restrict__ U, int64_t d, in
   const int jj = threadIdx.x % cw, part = threadIdx.x / cw;
   const C wj = jj < len ? w[jj] : C(0);
   C acc = part == 0 ? wj : C(0);
-  if (part < parts && jj < len) acc = urow_dot(U, d, j0 + jj, min(s, part * per), min(s, part * per + per), g, acc);
+  if (part < parts && jj < len) {
+    const int i0 = min(s, part * per), i1 = min(s, part * per + per);
+    acc = per <= 8 ? urow_dot<C, 8>(U, d, j0 + jj, i0, i1, g, acc) : urow_dot(U, d, j0 + jj, i0, i1, g, acc);
+  }
   red[threadIdx.x] = acc;
   __syncthreads();
   if (part == 0 && jj < len) {

@@ -172,7 +172,7 @@ __device__ __forceinline__ void utw_partials(const C* wch, int len, const C* __r
 template <typename C>
 __device__ __forceinline__ C g_entry(const C* part, int nb, int s, int i, C ci) {
   if constexpr (sizeof(C) == 8) {
-    return ci * sum_strided_fixed<true>(part, nb, s, i, 0.0);
+    return ci * (nb <= 16 ? sum_strided_fixed<true, double, 16>(part, nb, s, i, 0.0) : sum_strided_fixed<true>(part, nb, s, i, 0.0));
   } else {
     constexpr int B = 32;
     float hi = 0.f, lo = 0.f;
@@ -871,7 +871,10 @@ __global__ void __launch_bounds__(kVecThreads) admm_zu_g_kernel(int64_t d, int c
 // (H + rho I) x with the partials of ||w||^2 and U^T w (pcg_update_kernel), the scalar step
 // (pcg_scalar_body), y = P^{-1} w (pcg_tail_kernel) and the next direction p = y + beta p,
 // separated by barriers instead of kernel boundaries.  A block keeps its chunk of every vector
-// from step to step; only sums cross blocks, through L2.  Up to kClusterBlocks blocks run as one
+// from step to step; only sums cross blocks, through L2.  What bounds it is latency: at d = 500, rank
+// 50 in FP64 15.6 us (30,000 clocks: the partial sums 6,400, three or four barriers of 1,250, the
+// rest the FP64 chains and L2 reads of each phase), with one column of partials or of U per
+// thread and a barrier more 45 us.  Up to kClusterBlocks blocks run as one
 // cluster (hardware barrier), more as a cooperative grid.  Every element and every partial is
 // formed by the same code, block mapping and order as in the separate kernels, so the result
 // is bitwise theirs.  With zu set, the iteration that ends the PCG loop also runs the prox / dual
@@ -964,6 +967,15 @@ __global__ void __launch_bounds__(kVecThreads, 2) pcg_post_kernel(const PostArgs
     }
   };
   auto barrier = [&]() { return vec_barrier<CL>(&st->bar_count, &st->bar_gen, nblk); };
+  // this thread's first element of x, p, w and hx, on their way while the sums are formed
+  const int64_t jf = j0 + threadIdx.x;
+  C x0 = C(0), p0 = C(0), w0 = C(0), h0 = C(0);
+  if (jf < j1) {
+    x0 = a.x[jf];
+    p0 = a.p[jf];
+    w0 = a.w[jf];
+    if (a.hx) h0 = a.hx[jf];
+  }
   // ---- R: v = sum_g partial[g] + rho p over the block's chunk, partial of p^T v
   // (apass_reduce_kernel)
   {
@@ -1012,21 +1024,25 @@ __global__ void __launch_bounds__(kVecThreads, 2) pcg_post_kernel(const PostArgs
     double lw2 = 0.0;
     for (int64_t j = j0 + threadIdx.x; j < j1; j += kVecThreads) {
       const C vj = vch[j - j0];
-      a.x[j] = fma(al, a.p[j], a.x[j]);
-      const C wj = fma(-al, vj, a.w[j]);
-      if (a.hx) a.hx[j] = fma(al, vj, a.hx[j]);
+      const bool f = j == jf;
+      a.x[j] = fma(al, f ? p0 : a.p[j], f ? x0 : a.x[j]);
+      const C wj = fma(-al, vj, f ? w0 : a.w[j]);
+      if (a.hx) a.hx[j] = fma(al, vj, f ? h0 : a.hx[j]);
       a.w[j] = wj;
       vch[j - j0] = wj;
       lw2 += (double)wj * (double)wj;
     }
     const double tw2 = block_sum_t0<kVecThreads>(lw2, sh, vec_warps(a.chunk));
     if (threadIdx.x == 0) a.part_w2[b] = tw2;
+    // U^T w partials over this block's chunk of the new w.  A cluster forms them here whether PCG goes on
+    // or not (small d: 2,200 clocks, and a barrier less when it does); a grid only if it does.
+    if constexpr (CL) utw_partials<C>(vch, (int)(j1 - j0), a.U, d, j0, s, a.part_g + (int64_t)b * s);
   }
   if (!barrier()) return fail();
   // ---- S: ||w||^2, stop test, iteration count (pcg_scalar_body; every block takes the same
-  // decision, block 0 records it).  U^T w and g = c o U^T w follow only if PCG goes on: the
-  // iteration that ends the loop needs no P^{-1} w (the separate kernels form it regardless;
-  // the values they use are the same).
+  // decision, block 0 records it).  g = c o U^T w follows only if PCG goes on: the iteration that
+  // ends the loop needs no P^{-1} w (the separate kernels form it regardless; the values they
+  // use are the same).
   const double w2 = block_fixed_sum_cg(a.part_w2, a.nb, &slots[1]);
   const bool stepped = !bad && isfinite(w2);
   int iters = iters0, done = 0, status = 0;
@@ -1056,10 +1072,10 @@ __global__ void __launch_bounds__(kVecThreads, 2) pcg_post_kernel(const PostArgs
     cudaGraphSetConditional(a.cond, done ? 0u : 1u);
   }
   if (!done) {
-    // U^T w partials over this block's chunk of the new w, still in shared memory (every
-    // block that stepped has !bad here)
-    utw_partials<C>(vch, (int)(j1 - j0), a.U, d, j0, s, a.part_g + (int64_t)b * s);
-    if (!barrier()) return fail();
+    if constexpr (!CL) {   // (every block that stepped has !bad here)
+      utw_partials<C>(vch, (int)(j1 - j0), a.U, d, j0, s, a.part_g + (int64_t)b * s);
+      if (!barrier()) return fail();
+    }
     for (int i = threadIdx.x; i < s; i += kVecThreads) {
       const C gi = g_entry<C>(a.part_g, a.nb, s, i, a.cvec[i]);
       gsh[i] = gi;
@@ -1067,10 +1083,12 @@ __global__ void __launch_bounds__(kVecThreads, 2) pcg_post_kernel(const PostArgs
     }
     __syncthreads();
     // ---- T: y = w + U g, partials of w^T y (pcg_tail_kernel)
+    C y0 = C(0);
     {
       double lwy = 0.0;
       u_times_g(a.U, d, j0, (int)(j1 - j0), a.chunk, s, gsh, vch, [&](int jj, C wj, C acc) {
         a.y[j0 + jj] = acc;
+        if (jj < kVecThreads) y0 = acc;   // jj = this thread
         lwy += (double)wj * (double)acc;
       });
       const double t = block_sum_t0<kVecThreads>(lwy, sh, vec_warps(a.chunk));
@@ -1082,7 +1100,7 @@ __global__ void __launch_bounds__(kVecThreads, 2) pcg_post_kernel(const PostArgs
     if (threadIdx.x == 0) slots[0] = wy_new / wy;
     __syncthreads();
     const C bc = (C)slots[0];
-    for (int64_t j = j0 + threadIdx.x; j < j1; j += kVecThreads) a.p[j] = fma(bc, a.p[j], a.y[j]);
+    for (int64_t j = jf; j < j1; j += kVecThreads) a.p[j] = j == jf ? fma(bc, p0, y0) : fma(bc, a.p[j], a.y[j]);
     return;
   }
   if (!a.zu) return;
