@@ -251,7 +251,7 @@ nys_status batched_pcg_run(const PcgProblem& pb, const TcPrepared* tcp, const Pr
   const dim3 cgrid((unsigned)nb, (unsigned)k);
   if (f64) B_OK(hmm64_prepare(pb.A, k, tcw, st));
   // BF16 and FP32 storage: the k-column products run on the tensor cores (the same tcgen05
-  // GEMMs as the sketch, FP32 operand as three BF16 terms) from operands prepared once per solve;
+  // GEMMs as the sketch, FP32 operand as three BF16 terms);
   // FP64 storage on the FP64 products of the sketch.
   // V = A^T (A P) + rho P for the k columns of P (reads A once)
   auto bmatvec = [&](const C* Pin, C* Vout) -> bool {

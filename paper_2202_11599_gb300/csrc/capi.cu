@@ -815,8 +815,8 @@ nys_status lasso_path(const nys_matrix* A, const nys_matrix* Ain, const double* 
   double* Om = pool.alloc<double>((size_t)d * rank);
   double* Y = pool.alloc<double>((size_t)d * rank);
   if (!pool.ok()) return NYS_ENOMEM;
-  // the tensor-core operands of A (FP32: three BF16 terms and their transposes), made once for
-  // the sketch and every matvec of the path (50,000 x 4,000: 1.05 ms each time)
+  // the tensor-core operands of A for the sketch and every matvec of the path: A itself, or in the
+  // cp.async form (NYS_TC_TMA=0) copies made once (50,000 x 4,000 FP32: 1.05 ms)
   TcPrepared tcp;
   const TcPrepared* tcpp = nullptr;
   if (sizeof(C) == 4 && sketch_tc_supported(Ain)) {
@@ -1078,8 +1078,8 @@ nys_status logistic_admm(const nys_matrix* A, const nys_matrix* Ain, const doubl
   const int maxit = o.pcg_maxit > 0 ? o.pcg_maxit : (int)std::min<int64_t>(d, 1000);
   int total_pcg = 0, cur_rank = 0;
   nys_status result = NYS_OK;
-  // the curvature D changes every iteration but A does not: prepare its tensor-core
-  // operands once for all re-sketches
+  // the curvature D changes every iteration but A does not: its tensor-core operands (copies in the
+  // cp.async form only) serve all re-sketches
   TcPrepared tcp;
   const TcPrepared* tcpp = nullptr;
   if (sketch_tc_supported(Ain)) {

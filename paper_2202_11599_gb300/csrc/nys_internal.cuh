@@ -165,8 +165,9 @@ cudaError_t sketch_atw(const nys_matrix* A, const void* W, int s, double* Y, voi
                        size_t work_bytes, cudaStream_t st);
 size_t sketch_atw_work_bytes(const nys_matrix* A, int s);
 // Tensor-core (tcgen05) products for BF16 storage and for FP32 storage (split exactly into
-// three BF16 terms): tc_prepare builds the operands once (transposed copy of A; for FP32
-// also the terms) in caller-owned scratch of tc_prepare_bytes(A) bytes.
+// three BF16 terms): A is converted inside the products, or in the cp.async form tc_prepare builds
+// the operands once (transposed copy of A; for FP32 also the terms) in caller-owned scratch of
+// tc_prepare_bytes(A) bytes (0 when A serves as it is).
 struct TcPrepared {
   bool direct = false;           // A is converted inside the products: no copies
   int at = 1;                    // A terms: 1 (BF16) or 3 (FP32 split)

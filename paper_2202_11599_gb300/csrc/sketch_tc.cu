@@ -13,10 +13,10 @@
 //
 // Kernel design (one CTA = two 128-row tiles of the output sharing each staged B tile, the
 // full N = s <= 256 of each in TMEM):
-//   * both operands are K-major: GEMM 1 reads the rows of A directly, GEMM 2 reads a
-//     transposed copy of A made once per sketch (2 GB of the 280 GB HBM for the paper's
-//     largest single-GPU problem); W is written by GEMM 1 already in the K-major layout
-//     GEMM 2 wants;
+//   * both operands are K-major: GEMM 1 reads the rows of A directly, GEMM 2 (and GEMM 1 for FP32
+//     storage) converts A as it reads it (sketch_tc_direct_kernel below; the cp.async form
+//     of NYS_TC_TMA=0, described next, takes a transposed copy made beforehand); W is written by
+//     GEMM 1 already in the K-major layout GEMM 2 wants;
 //   * tiles are staged by cp.async (16-byte chunks, zero-filled outside the matrix) into
 //     the canonical no-swizzle core-matrix layout (8 rows x 16 bytes per core matrix;
 //     core matrices 128 B apart along K, 512 B apart along M/N), 4 stages of 32 K;
@@ -971,8 +971,8 @@ TcShape tc_shape(const nys_matrix* A, const TcPrepared& prep, int m, int xterms)
   return h;
 }
 
-// Y (d x m, column-major) = A^T diag(D) A X (+ rho X) on the tensor cores, given the
-// transposed copy At (d x nP) of A.  X and Y are FP64 (sketch) or FP32 (batched PCG).
+// Y (d x m, column-major) = A^T diag(D) A X (+ rho X) on the tensor cores, given A as tc_prepare
+// left it.  X and Y are FP64 (sketch) or FP32 (batched PCG).
 // xterms = 1: X holds BF16 values (the sketch's rounded test matrix), so the first product
 // takes one MMA term of X instead of three.  Enqueues on `st` only: work (tc_shape's bytes) and
 // status (a device int the caller zeroed; NYS_ETIMEOUT when a wait ran out) are the caller's.
