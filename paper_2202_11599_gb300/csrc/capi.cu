@@ -371,10 +371,16 @@ int mant_bits_of(const nys_matrix* A) { return A->dtype == NYS_F64 ? 52 : 23; }
 // given back when the thread ends.
 struct HostStatus {
   int* p = nullptr;
-  HostStatus() {
-    if (cudaHostAlloc(reinterpret_cast<void**>(&p), sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) !=
-        cudaSuccess)
+  HostStatus() = default;
+  // the word, allocated on first use (a call that could not get it, inside a stream capture for
+  // instance, leaves the next one to try again); null when there is none
+  int* get() {
+    if (!p && cudaHostAlloc(reinterpret_cast<void**>(&p), sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) !=
+                  cudaSuccess) {
       p = nullptr;
+      (void)cudaGetLastError();
+    }
+    return p;
   }
   ~HostStatus() {
     if (p) cudaFreeHost(p);
@@ -388,12 +394,13 @@ template <typename C>
 nys_status hmatvec_t(const nys_matrix* A, const double* D, double rho, const void* p, void* y, cudaStream_t st) {
   ApassPlan plan;
   apass_plan(A, &plan);
-  static thread_local HostStatus status;
-  if (!status.p) return NYS_ENOMEM;
+  static thread_local HostStatus host_status;
+  int* const status = host_status.get();
+  if (!status) return NYS_ENOMEM;
   Pool pool(st);
   void* part = pool.alloc<unsigned char>(apass_partial_bytes(A, plan));
   if (!pool.ok()) return NYS_ENOMEM;
-  *status.p = 0;
+  *status = 0;
   ApassArgs a;
   a.A = A->data;
   a.n = A->n;
@@ -407,10 +414,10 @@ nys_status hmatvec_t(const nys_matrix* A, const double* D, double rho, const voi
   a.D_out = nullptr;
   a.t_out = nullptr;
   a.mode = D ? MODE_DIAG : MODE_ID;
-  NYS_CU(apass_run(a, plan, part, nullptr, status.p, st));
+  NYS_CU(apass_run(a, plan, part, nullptr, status, st));
   NYS_CU(apass_reduce(a, plan, part, rho, y, nullptr, st));
   NYS_CU(cudaStreamSynchronize(st));
-  const int h = *static_cast<volatile int*>(status.p);
+  const int h = *static_cast<volatile int*>(status);
   return h ? (nys_status)h : NYS_OK;
 }
 
