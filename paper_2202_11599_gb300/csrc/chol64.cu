@@ -336,7 +336,7 @@ cudaError_t trsm_right_upper(const double* C, int s, double* Y, int64_t d, void*
   NYS_CUDA_TRY(cudaGetLastError());
   NYS_CUDA_TRY(absmax_f64(X, s, s, s, ex, nullptr, st));
   NYS_CUDA_TRY(absmax_f64(Y, s, d, d, nullptr, ed, st));
-  NYS_CUDA_TRY(gemm64(Y, false, d, ed, d, X, s, ex, s, s, nullptr, B, d, b, status, st));
+  NYS_CUDA_TRY(gemm64(Y, false, d, ed, d, X, s, ex, s, s, nullptr, B, d, b, status, st, /*any_scale=*/false));
   return cudaMemcpyAsync(Y, B, (size_t)d * s * sizeof(double), cudaMemcpyDeviceToDevice, st);
 }
 

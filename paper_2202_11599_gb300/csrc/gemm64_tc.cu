@@ -12,12 +12,20 @@
 // 64 output columns x 8 orders = all 512 TMEM columns.  Every 256 K the accumulators are read
 // out as integers and added to two 64-bit integer sums per output: at 256 K orders 0-3 cannot
 // leave 2^24 for any input, and orders 4-7, below 2^-32 of the product's scale, could round
-// only for inputs whose low digits all agree in sign.  The dropped orders lie below 2^-60.
-// The final integer is rounded to FP64 once.  (Fixed-point splitting of a product into exact
-// low-precision ones: Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 59, 2012.)  The error is
-// that of rounding each operand to 2^-62 of its row's maximum plus the final rounding: on random,
-// graded, constant and one-signed rows of up to 600 terms it is 1e-18 to 7e-17 of sum |a||b|,
-// against 1e-16 to 8e-15 for a chain of FP64 FMAs.  A row holding a NaN or an infinity gives NaN.
+// only for inputs whose low digits all agree in sign.  The final integer is rounded to FP64 once.
+// (Fixed-point splitting of a product into exact low-precision ones: Ozaki, Ogita, Oishi, Rump,
+// Numer. Algorithms 59, 2012.)
+//
+// Error: with |a| < 2 x 2^ea and |b| < 2 x 2^eb over the rows, cutting the digits off (toward zero, below
+// 2^-61) and dropping the orders from 8 on (order 8: 7 x 2^-60) leaves at most
+//   9.1 K 2^-60 2^ea 2^eb + 2^-53 |C|,
+// which is relative to the rows' largest entries, not to the entries that meet: where large ones of A only
+// meet small ones of B a chain of FMAs, K 2^-53 sum |a||b|, is better, by any factor.  So for products
+// with a caller's matrix (hmm64) gemm64_check_kernel first finds the outputs with sum |a||b| <
+// 9.1/128 2^ea 2^eb, where the FMAs' bound is the smaller, and this kernel forms those (in columns of 32 rows)
+// by FMAs.  Of A Omega and A^T W with columns decaying like 1/j there are none, with 1/j^2 5 % of the
+// columns; rows scaled against their weights have all.  (Sketch of 40,000 x 4,000, rank 100: 6.6 ms, 0.1 of it the
+// check; 13 with columns like 1/j^2, 44 with the rows so scaled; 83 on the FP64 pipe alone.)
 //
 // Measured (FP64 pipe before, this kernel after): the two products of a 40,000 x 4,000 sketch of
 // rank 100, 36.1 + 40.4 ms -> 1.7 + 1.7 ms; X^T Y at 10,000 x 200, 0.52 (symmetric) and 0.90 ms
@@ -33,6 +41,7 @@
 // (One warp doing both and a barrier per stage: 9,200 clocks, tensor pipe 26 % active.)  Both
 // operands are converted in the kernel: the digits are never written to memory, and an operand
 // stored along M (A^T) is transposed on the way into shared memory.
+#include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -51,6 +60,7 @@ constexpr int EFLUSH = 8;                     // stages between read-outs (256 K
 constexpr uint32_t EA_SLICE = EM * EK * 2, EB_SLICE = EN * EK * 2;
 constexpr uint32_t E_STAGE = ESL * (EA_SLICE + EB_SLICE);   // 96 KB
 constexpr int E_MINSTEPS = 2;                 // K steps a split slice has at least
+constexpr int ESPREAD = (EM / 32) * (EN / 8); // bytes of a tile in EmuArgs::spread
 
 struct EmuArgs {
   const double* A;
@@ -64,6 +74,9 @@ struct EmuArgs {
   const double* D;      // row factors, applied when the K range is not split
   double* C;            // slice z at C + z * cslice, column n at + n * ldc
   int64_t ldc, cslice;
+  // which outputs the FMAs form: per tile 4 x 8 bytes, bit n % 8 of byte (m / 32, n / 8) for column n of the
+  // 32 rows; or null (none)
+  unsigned char* spread;
   int* status;
 };
 
@@ -125,6 +138,80 @@ __device__ __forceinline__ double fixed_to_double(__int128 v, int sh) {
   return neg ? -x : x;
 }
 
+// C(m, n) over [kb, ke) by FMAs in increasing k for m = mb + lane and the columns n = nb + (bits of `cols`);
+// of two warps, `part` takes every other column.  Four columns at a time; A(m, k) from each lane's own row or column,
+// eight K ahead of their use, B(n, k) by lanes over k.  Bound by the FP64 pipe where all columns are formed here, by
+// latency where a few are.  Zeros in B (triangular factors) are passed over while A is finite.
+template <bool KC>
+__device__ __forceinline__ void fma_columns(const EmuArgs& a, int64_t mb, int nb, uint32_t cols, int part, int64_t kb, int64_t ke) {
+  constexpr int AHEAD = 8;
+  const int lane = threadIdx.x & 31;
+  const int64_t m = mb + lane;
+  const bool mok = m < a.M;
+  const double* Ap = KC ? a.A + (mok ? m : 0) * a.lda : a.A + (mok ? m : 0);
+  const int64_t step = KC ? 1 : a.lda;
+  const bool finite = !__any_sync(0xffffffffu, mok && (a.ea[m] >> 20) == 0x7ffu);
+  const double dm = a.D && mok ? a.D[m] : 1.0;
+  double* out = a.C + (int64_t)blockIdx.z * a.cslice + m;
+  if (part && cols) cols &= cols - 1;
+  while (cols) {
+    int n[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      n[j] = cols ? nb + __ffs(cols) - 1 : -1;
+      cols &= cols - 1;   // this one
+      cols &= cols - 1;   // the other warp's
+    }
+    double acc[4] = {0.0, 0.0, 0.0, 0.0}, bn[4];
+    auto load_b = [&](int64_t k0) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        bn[j] = n[j] >= 0 && k0 + lane < ke ? __ldg(a.B + (int64_t)n[j] * a.ldb + k0 + lane) : 0.0;
+    };
+    load_b(kb);
+    for (int64_t k0 = kb; k0 < ke; k0 += 32) {
+      double bv[4];
+      uint32_t some = 0u;   // the K that count
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        bv[j] = bn[j];
+        some |= __ballot_sync(0xffffffffu, bv[j] != 0.0);
+      }
+      if (k0 + 32 < ke) load_b(k0 + 32);
+      if (!finite) some = ke - k0 >= 32 ? 0xffffffffu : (1u << (ke - k0)) - 1u;
+      const double* Ak = Ap + k0 * step;
+      uint32_t ahead = some;
+      double an[AHEAD];
+      auto load_a = [&]() {
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) {
+          an[u] = ahead && mok ? __ldg(Ak + (__ffs(ahead) - 1) * step) : 0.0;
+          ahead &= ahead - 1;
+        }
+      };
+      load_a();
+      while (some) {
+        double av[AHEAD];
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) av[u] = an[u];
+        if (ahead) load_a();
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) {
+          if (some) {
+            const int k = __ffs(some) - 1;
+            some &= some - 1;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[j] = fma(av[u], __shfl_sync(0xffffffffu, bv[j], k), acc[j]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (mok && n[j] >= 0) out[(int64_t)n[j] * a.ldc] = a.D ? dm * acc[j] : acc[j];
+  }
+}
+
 // KC: A(m, k) = A[m lda + k]; else A(m, k) = A[k lda + m].  B(n, k) = B[n ldb + k].
 template <bool KC>
 __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
@@ -136,7 +223,18 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
   const int64_t m0 = (int64_t)blockIdx.y * EM;
   const int n0 = blockIdx.x * EN;
   const int64_t kb = (int64_t)blockIdx.z * a.kslice, ke = min(a.K, kb + a.kslice);
-  const int nt = (int)((ke - kb + EK - 1) / EK);
+  const uint32_t* spread =
+      a.spread ? reinterpret_cast<const uint32_t*>(a.spread) + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * (ESPREAD / 4)
+               : nullptr;
+  int nt = (int)((ke - kb + EK - 1) / EK);
+  if (spread) {   // a tile all of FMAs needs no digits
+    bool all = true;
+    for (int w = 0; w < ESPREAD / 4; ++w) {
+      const int nv = min(32, max(0, a.N - n0 - 32 * (w & 1)));
+      if (m0 + 32 * (w >> 1) < a.M && nv > 0) all = all && spread[w] == 0xffffffffu >> (32 - nv);
+    }
+    if (all) nt = 0;
+  }
   const uint32_t sbase = smem_u32(smem);
   if (warp == 0) {
     tmem_alloc(&tmem_slot, 512);
@@ -334,6 +432,7 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
     const bool whole = !__any_sync(0xffffffffu, s_fail != 0) && (nt == 0 || drain(nt - 1));
     if (!whole) s_fail = 1;
     const int64_t m = m0 + 32 * quad + lane;
+    const uint32_t fma_cols = spread && whole ? spread[2 * quad + (cg >> 5)] >> (cg & 31) : 0u;
     if (m < a.M) {
       const unsigned wa = a.ea[m];
       const double dm = a.D ? a.D[m] : 1.0;
@@ -341,7 +440,7 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
   #pragma unroll
       for (int e = 0; e < 16; ++e) {
         const int n = n0 + cg + e;
-        if (n < a.N) {
+        if (n < a.N && !(fma_cols >> e & 1)) {
           const unsigned wb = a.eb[n];
           const uint64_t low = ((uint64_t)w1[e] << 32) | w0[e];
           double x = fixed_to_double((((__int128)(int)w2[e]) << 64) | (__int128)(unsigned __int128)low,
@@ -351,6 +450,8 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
         }
       }
     }
+    // two warps per 32 x 32 part of the tile share its columns of FMAs
+    if (spread && whole) fma_columns<KC>(a, m0 + 32 * (warp >> 2), n0 + 32 * ((warp >> 1) & 1), spread[warp >> 1], warp & 1, kb, ke);
   } else {
    asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");
    if (tid == 32 * ECW) {
@@ -394,10 +495,192 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
+// Fills EmuArgs::spread: the outputs of a tile with sum_k |a||b| < kSpread 2^ea 2^eb.  The sum is taken over the
+// entries' magnitudes in FP16 at the scale of their rows, cut to 11 bits (2^-14 of the row's scale and
+// smaller count as zero), so it is a lower bound, on mma.sync with FP32 sums.
+//
+// What bounds it is latency: the sums of ordinary rows pass within the first 64 K, so the CTAs of a tile's
+// cluster (one to eight, a slice of K each, so that few tiles fill the chip too) look at 64 K
+// each, add their sums up in one order and stop when every output has passed; only else they go on to
+// the end of their slices.  Only the top words of the FP64 values are used.
+constexpr float kSpread = 9.1f / 128.f;
+constexpr int CK = 64, CPITCH = CK + 8;   // K of a step; halves from one row to the next
+template <bool KC>
+__global__ void __launch_bounds__(256, 2) gemm64_check_kernel(const EmuArgs a) {
+  namespace cg = cooperative_groups;
+  __shared__ __align__(16) unsigned char sm[EM * EN * sizeof(float)];
+  static_assert((EM + EN) * CPITCH * sizeof(__half) <= sizeof(sm), "stage and sums share shared memory");
+  __shared__ unsigned s_ea[EM], s_eb[EN];
+  __shared__ unsigned s_fail[EM / 32][EN / 8];   // as EmuArgs::spread
+  __shared__ int s_pass[8];
+  unsigned short* As = reinterpret_cast<unsigned short*>(sm);
+  unsigned short* Bs = As + EM * CPITCH;
+  float* S = reinterpret_cast<float*>(sm);
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), nrank = (int)cl.num_blocks();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t m0 = (int64_t)blockIdx.y * EM;
+  const int n0 = blockIdx.x * EN;
+  const int64_t steps = (a.K + CK - 1) / CK, per = (steps + nrank - 1) / nrank;
+  const int64_t s0 = min(steps, rank * per), s1 = min(steps, s0 + per);
+  if (tid < EM) s_ea[tid] = m0 + tid < a.M ? a.ea[m0 + tid] : 0u;
+  if (tid < EN) s_eb[tid] = n0 + tid < a.N ? a.eb[n0 + tid] : 0u;
+  __syncthreads();
+  // This thread's entries of a step: of A rows warp + 8 i at K lane and lane + 32 (KC), else columns lane + 32 j at K
+  // warp + 8 i; of B rows warp + 8 i at K lane and lane + 32.
+  unsigned ra[32], rb[16];
+  auto top = [](const double* p) { return __ldg(reinterpret_cast<const unsigned*>(p) + 1) & 0x7fffffffu; };
+  const double* pa = KC ? a.A + (m0 + warp) * a.lda + lane : a.A + (int64_t)warp * a.lda + m0 + lane;
+  const double* pb = a.B + (int64_t)(n0 + warp) * a.ldb + lane;
+  const int mv = (int)min((int64_t)EM, a.M - m0), nv = min(EN, a.N - n0);
+  auto load = [&](int64_t st) {
+    const int64_t k0 = st * CK;
+    const int kv = (int)min((int64_t)CK, a.K - k0);
+    const double* q = KC ? pa + k0 : pa + k0 * a.lda;
+#pragma unroll
+    for (int i = 0; i < (KC ? 16 : 8); ++i, q += 8 * a.lda) {
+      if (KC) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) ra[2 * i + j] = warp + 8 * i < mv && lane + 32 * j < kv ? top(q + 32 * j) : 0u;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ra[4 * i + j] = warp + 8 * i < kv && lane + 32 * j < mv ? top(q + 32 * j) : 0u;
+      }
+    }
+    q = pb + k0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i, q += 8 * a.ldb)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) rb[2 * i + j] = warp + 8 * i < nv && lane + 32 * j < kv ? top(q + 32 * j) : 0u;
+  };
+  // FP16 bits of a magnitude at the scale of its row (largest entries in [1, 2)); rows below 2^-959 and
+  // rows that are not finite are decided without their sums
+  auto scale_of = [](unsigned e) { return (max((int)(e >> 20), 64) - 15) << 20; };
+  auto half_bits = [](unsigned h, int base) {
+    const int v = (int)h - base;
+    return (unsigned short)(v >= 1 << 20 ? min(v >> 10, 0x7bff) : 0);
+  };
+  auto store = [&]() {
+#pragma unroll
+    for (int i = 0; i < (KC ? 16 : 4); ++i) {
+      const int r = KC ? warp + 8 * i : lane + 32 * i, base = scale_of(s_ea[r]);
+#pragma unroll
+      for (int j = 0; j < (KC ? 2 : 8); ++j) {
+        const int k = KC ? lane + 32 * j : warp + 8 * j;
+        As[r * CPITCH + k] = half_bits(ra[KC ? 2 * i + j : 4 * j + i], base);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = warp + 8 * i, base = scale_of(s_eb[r]);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) Bs[r * CPITCH + lane + 32 * j] = half_bits(rb[2 * i + j], base);
+    }
+  };
+  // warp w: rows 16 w .. + 15, all columns; the fragments of mma.m16n8k16
+  float acc[EN / 8][4] = {};
+  const int g = lane >> 2, t = lane & 3;
+  auto multiply = [&]() {
+#pragma unroll
+    for (int kk = 0; kk < CK; kk += 16) {
+      auto frag = [&](const unsigned short* X, int r, int k) {
+        return *reinterpret_cast<const uint32_t*>(X + r * CPITCH + kk + k + 2 * t);
+      };
+      const uint32_t x0 = frag(As, 16 * warp + g, 0), x1 = frag(As, 16 * warp + g + 8, 0);
+      const uint32_t x2 = frag(As, 16 * warp + g, 8), x3 = frag(As, 16 * warp + g + 8, 8);
+#pragma unroll
+      for (int j = 0; j < EN / 8; ++j) {
+        const uint32_t y0 = frag(Bs, 8 * j + g, 0), y1 = frag(Bs, 8 * j + g, 8);
+        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                     : "+f"(acc[j][0]), "+f"(acc[j][1]), "+f"(acc[j][2]), "+f"(acc[j][3])
+                     : "r"(x0), "r"(x1), "r"(x2), "r"(x3), "r"(y0), "r"(y1));
+      }
+    }
+  };
+  auto run = [&](int64_t from, int64_t to) {
+    if (from < to) load(from);
+    for (int64_t st = from; st < to; ++st) {
+      __syncthreads();
+      store();
+      __syncthreads();
+      if (st + 1 < to) load(st + 1);
+      multiply();
+    }
+  };
+  // Whether every output of the tile has passed.  The columns 8 j .. 8 j + 7 are decided by CTA j / (8 / nrank),
+  // from the sums of all CTAs in rank order.
+  const int jper = (EN / 8) / nrank;
+  auto decide = [&]() -> bool {
+    __syncthreads();
+    if (tid < EM / 32 * (EN / 8)) s_fail[tid >> 3][tid & 7] = 0u;
+    if (nrank > 1) {
+#pragma unroll
+      for (int j = 0; j < EN / 8; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) S[(4 * j + q) * 256 + tid] = acc[j][q];
+      cl.sync();
+    } else {
+      __syncthreads();
+    }
+    unsigned any = 0u;
+    auto columns = [&](int j, const float (&sum)[4]) {
+      unsigned lanes[2] = {0u, 0u};   // of columns 8 j + 2 t and 8 j + 2 t + 1
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int m = 16 * warp + g + 8 * (q >> 1), n = 8 * j + 2 * t + (q & 1);
+        const unsigned ea = s_ea[m], eb = s_eb[n], wa = ea >> 20, wb = eb >> 20;
+        const bool pass = wa != 0x7ffu && wb != 0x7ffu && (ea == 0u || eb == 0u || (wa >= 64u && wb >= 64u && sum[q] >= kSpread));
+        lanes[q & 1] |= __ballot_sync(0xffffffffu, m < mv && n < nv && !pass);
+      }
+      unsigned byte = 0u;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) byte |= (unsigned)((lanes[c & 1] & (0x11111111u << (c >> 1))) != 0u) << c;
+      if (byte && lane == 0) atomicOr(&s_fail[warp >> 1][j], byte);
+      any |= byte;
+    };
+    if (nrank == 1) {
+#pragma unroll
+      for (int j = 0; j < EN / 8; ++j) columns(j, acc[j]);
+    } else {
+      for (int j = rank * jper; j < (rank + 1) * jper; ++j) {
+        float sum[4] = {0.f, 0.f, 0.f, 0.f}, part[8][4];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const float* Sr = cl.map_shared_rank(S, r < nrank ? r : rank);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) part[r][q] = r < nrank ? Sr[(4 * j + q) * 256 + tid] : 0.f;
+        }
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) sum[q] += part[r][q];
+        columns(j, sum);
+      }
+    }
+    const int fail = __syncthreads_or((int)any);
+    if (nrank == 1) return !fail;
+    if (tid < nrank) cl.map_shared_rank(s_pass, tid)[rank] = !fail;
+    cl.sync();
+    bool all = true;
+    for (int r = 0; r < nrank; ++r) all = all && s_pass[r];
+    return all;
+  };
+  run(s0, min(s0 + 1, s1));
+  if (!decide() && per > 1) {
+    run(min(s0 + 1, s1), s1);
+    (void)decide();
+  }
+  if (tid < EM / 32 * (EN / 8) && (tid & 7) / jper == rank)
+    a.spread[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * ESPREAD + tid] = (unsigned char)s_fail[tid >> 3][tid & 7];
+}
+
 // Largest magnitude (top word: order and exponent; a NaN or an infinity is above every finite
-// value) of each row and / or column of the row-major rows x cols matrix X.  Block (bx, by):
+// value; zero only for zeros) of each row and / or column of the row-major rows x cols matrix X.  Block (bx, by):
 // columns 512 bx .. + 511 (two per thread), `slab` rows from by * slab; rowmax and colmax are
 // zeroed by the caller.  Bound by the one read of X.
+__device__ __forceinline__ unsigned top_word(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7fffffffu) | (__double2loint(x) != 0 ? 1u : 0u);
+}
 constexpr int kAbsCols = 512;
 constexpr int kAbsMaxSlab = 256;
 __global__ void __launch_bounds__(256) absmax_kernel(const double* __restrict__ X, int64_t rows, int64_t cols,
@@ -418,11 +701,11 @@ __global__ void __launch_bounds__(256) absmax_kernel(const double* __restrict__ 
         const double* p = X + (r0 + b + q) * ld + c;
         if (vec) {
           const double2 v = __ldg(reinterpret_cast<const double2*>(p));
-          h0[q] = (unsigned)__double2hiint(v.x) & 0x7fffffffu;
-          h1[q] = (unsigned)__double2hiint(v.y) & 0x7fffffffu;
+          h0[q] = top_word(v.x);
+          h1[q] = top_word(v.y);
         } else {
-          if (c < cols) h0[q] = (unsigned)__double2hiint(__ldg(p)) & 0x7fffffffu;
-          if (c + 1 < cols) h1[q] = (unsigned)__double2hiint(__ldg(p + 1)) & 0x7fffffffu;
+          if (c < cols) h0[q] = top_word(__ldg(p));
+          if (c + 1 < cols) h1[q] = top_word(__ldg(p + 1));
         }
       }
     }
@@ -523,16 +806,40 @@ cudaError_t absmax_f64(const double* X, int64_t rows, int64_t cols, int64_t ld, 
   return cudaSuccess;
 }
 
+static size_t spread_bytes(const EmuPlan& p) { return ((size_t)p.mt * p.ntl * ESPREAD + 255) / 256 * 256; }
+
 size_t gemm64_work_bytes(int64_t M, int N, int64_t K) {
   const EmuPlan p = emu_plan(M, N, K);
-  return p.nz > 1 ? (size_t)p.nz * M * N * sizeof(double) : 0;
+  return spread_bytes(p) + (p.nz > 1 ? (size_t)p.nz * M * N * sizeof(double) : 0);
+}
+
+// The check over one launch's tiles, in clusters of up to eight CTAs that split K: about one CTA per SM or more.
+template <bool KC>
+static cudaError_t launch_check(const EmuArgs& a, dim3 tiles, cudaStream_t st) {
+  int c = 1;
+  while (c < 8 && (int64_t)tiles.x * tiles.y * c < 152 && (int64_t)2 * c * CK <= a.K) c *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(tiles.x, tiles.y, (unsigned)c);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = (unsigned)c;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, gemm64_check_kernel<KC>, a);
 }
 
 cudaError_t gemm64(const double* A, bool k_contiguous, int64_t lda, const unsigned* ea, int64_t M, const double* B,
                    int64_t ldb, const unsigned* eb, int N, int64_t K, const double* D, double* C, int64_t ldc,
-                   void* work, int* status, cudaStream_t st) {
+                   void* work, int* status, cudaStream_t st, bool any_scale) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
   const EmuPlan p = emu_plan(M, N, K);
+  unsigned char* spread = reinterpret_cast<unsigned char*>(work);
+  double* part = reinterpret_cast<double*>(spread + spread_bytes(p));
   if (p.ntl > INT32_MAX) return cudaErrorInvalidValue;
   EmuArgs a;
   a.A = A;
@@ -555,9 +862,11 @@ cudaError_t gemm64(const double* A, bool k_contiguous, int64_t lda, const unsign
     a.A = A + (k_contiguous ? m0 * lda : m0);
     a.ea = ea + m0;
     a.M = std::min<int64_t>(M - m0, nt * EM);
-    a.C = (p.nz == 1 ? C : reinterpret_cast<double*>(work)) + m0;
+    a.C = (p.nz == 1 ? C : part) + m0;
     a.D = p.nz == 1 && D ? D + m0 : nullptr;
     const dim3 grid((unsigned)p.ntl, (unsigned)nt, (unsigned)p.nz);
+    a.spread = any_scale ? spread + t0 * p.ntl * ESPREAD : nullptr;
+    if (any_scale) NYS_CUDA_TRY(k_contiguous ? launch_check<true>(a, grid, st) : launch_check<false>(a, grid, st));
     count_launch();
     if (k_contiguous) gemm64_tc_kernel<true><<<grid, ET, 2 * E_STAGE, st>>>(a);
     else gemm64_tc_kernel<false><<<grid, ET, 2 * E_STAGE, st>>>(a);
@@ -567,7 +876,7 @@ cudaError_t gemm64(const double* A, bool k_contiguous, int64_t lda, const unsign
     const int64_t len = M * (int64_t)N;
     count_launch();
     emu_sum_kernel<<<(unsigned)std::min<int64_t>(4096, (len + 127) / 128), 128, 0, st>>>(
-        reinterpret_cast<const double*>(work), p.nz, M, len, D, C, ldc);
+        part, p.nz, M, len, D, C, ldc);
     NYS_CUDA_TRY(cudaGetLastError());
   }
   return cudaSuccess;
@@ -625,9 +934,9 @@ cudaError_t hmm64(const nys_matrix* A, const double* D, const double* X, int m, 
   void* work = b + h.w + ((size_t)A->n * m * sizeof(double) + 255) / 256 * 256;
   const int64_t n = A->n, d = A->d;
   NYS_CUDA_TRY(absmax_f64(X, m, d, d, ex, nullptr, st));
-  NYS_CUDA_TRY(gemm64(Ad, true, A->ld, row, n, X, d, ex, m, d, D, W, n, work, status, st));
+  NYS_CUDA_TRY(gemm64(Ad, true, A->ld, row, n, X, d, ex, m, d, D, W, n, work, status, st, /*any_scale=*/true));
   NYS_CUDA_TRY(absmax_f64(W, m, n, n, ew, nullptr, st));
-  return gemm64(Ad, false, A->ld, col, d, W, n, ew, m, n, nullptr, Y, d, work, status, st);
+  return gemm64(Ad, false, A->ld, col, d, W, n, ew, m, n, nullptr, Y, d, work, status, st, /*any_scale=*/true);
 }
 
 }  // namespace nys

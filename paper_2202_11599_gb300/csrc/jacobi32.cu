@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(256) small_product_kernel(const double* __rest
 }
 cudaError_t square_product(const double* X, bool kc, const unsigned* ex, const double* Y, const unsigned* ey, double* Z,
                            int N, void* gw, int* status, cudaStream_t st) {
-  if (N > kSmallProduct) return gemm64(X, kc, N, ex, N, Y, N, ey, N, N, nullptr, Z, N, gw, status, st);
+  if (N > kSmallProduct) return gemm64(X, kc, N, ex, N, Y, N, ey, N, N, nullptr, Z, N, gw, status, st, false);
   count_launch();
   small_product_kernel<<<dim3((N + 15) / 16, (N + 15) / 16), 256, 0, st>>>(X, kc ? 1 : 0, Y, Z, N);
   return cudaGetLastError();

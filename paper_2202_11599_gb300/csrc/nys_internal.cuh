@@ -99,11 +99,13 @@ cudaError_t absmax_f64(const double* X, int64_t rows, int64_t cols, int64_t ld, 
 // C (M x N, column-major, ldc) = diag(D) A B^T with A(m, k) = A[m lda + k] (k_contiguous) or
 // A[k lda + m], B(n, k) = B[n ldb + k]; ea / eb: absmax of A over k for each m, of B for each n.
 // D (length M) may be NULL.  *status (device, caller-zeroed): NYS_ETIMEOUT when a bounded wait ran
-// out (the outputs are then NaN).
+// out (the outputs are then NaN).  |error| <= 9.1 K 2^-60 2^ea 2^eb + 2^-53 |C| with ea, eb the exponents; with
+// any_scale every output is moreover as accurate as a chain of FMAs, K 2^-53 sum |a||b|, however the scales of
+// the entries that meet differ (then ea and eb are the maxima, not bounds of them).
 size_t gemm64_work_bytes(int64_t M, int N, int64_t K);
 cudaError_t gemm64(const double* A, bool k_contiguous, int64_t lda, const unsigned* ea, int64_t M, const double* B,
                    int64_t ldb, const unsigned* eb, int N, int64_t K, const double* D, double* C, int64_t ldc,
-                   void* work, int* status, cudaStream_t st);
+                   void* work, int* status, cudaStream_t st, bool any_scale);
 // Y (d x m, column-major) = A^T diag(D) A X for an FP64 matrix; scratch of hmm64_bytes, prepared
 // once per matrix and m (the exponents of A; zeroes the status word).
 size_t hmm64_bytes(const nys_matrix* A, int m);

@@ -1,0 +1,34 @@
+// Entry points for the tests only, not part of nysadmm.h: single device functions that the library otherwise
+// runs inside a sketch, so that their results can be compared entry by entry.
+#include "nys_internal.cuh"
+#include "solver.cuh"
+
+namespace {
+nys_status read_status(const int* status, cudaStream_t st) {
+  int h = 0;
+  if (cudaMemcpyAsync(&h, status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return NYS_ECUDA;
+  return (nys_status)h;
+}
+}  // namespace
+
+// gemm64: C (M x N, column-major) = diag(D) A B^T with the exponents taken from A and B here.  k_contiguous: A is
+// M x K row-major, else K x M; B is N x K row-major; all arrays on the device.
+extern "C" nys_status nys_test_gemm64(const double* A, int32_t k_contiguous, int64_t lda, int64_t M, const double* B,
+                                      int64_t ldb, int32_t N, int64_t K, const double* D, double* C, void* stream) {
+  using namespace nys;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  Pool pool(st);
+  unsigned* ea = pool.alloc<unsigned>(M);
+  unsigned* eb = pool.alloc<unsigned>(N);
+  void* work = pool.alloc<unsigned char>(gemm64_work_bytes(M, N, K));
+  int* status = pool.alloc<int>(1);
+  if (!pool.ok()) return NYS_ENOMEM;
+  if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return NYS_ECUDA;
+  if ((k_contiguous ? absmax_f64(A, M, K, lda, ea, nullptr, st) : absmax_f64(A, K, M, lda, nullptr, ea, st)) != cudaSuccess ||
+      absmax_f64(B, N, K, ldb, eb, nullptr, st) != cudaSuccess ||
+      gemm64(A, k_contiguous != 0, lda, ea, M, B, ldb, eb, N, K, D, C, M, work, status, st, /*any_scale=*/true) != cudaSuccess)
+    return NYS_ECUDA;
+  return read_status(status, st);
+}
