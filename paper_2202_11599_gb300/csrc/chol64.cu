@@ -240,10 +240,14 @@ __global__ void __launch_bounds__(1024) chol_upper_kernel(double* M, int s, int*
     for (int i = j + 1 + lane; i < s; i += 32) M[i + (int64_t)j * s] = 0.0;
 }
 
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }   // |e| < 1023
+
 // X = C^{-1} for an upper triangular C (both s x s column-major): warp c solves C x = e_c from the
 // last row up, column by column of C (the next column's entries are loaded a step ahead).
 constexpr int kInvAhead = 8;   // entries of a column a lane holds: 256 rows; more are read in place
-__global__ void __launch_bounds__(32) tri_inverse_kernel(const double* __restrict__ C, int s, double* __restrict__ X) {
+// Row i of the result is scaled by 2^t_i.
+__global__ void __launch_bounds__(32) tri_inverse_kernel(const double* __restrict__ C, int s, const int* __restrict__ t,
+                                                         double* __restrict__ X) {
   extern __shared__ double y[];
   const int c = s - 1 - (int)blockIdx.x;   // the longest solves first
   const int lane = threadIdx.x;
@@ -278,7 +282,26 @@ __global__ void __launch_bounds__(32) tri_inverse_kernel(const double* __restric
     if (lane == 0) y[k] = xk;
     __syncwarp();
   }
-  for (int i = lane; i < s; i += 32) X[i + (int64_t)c * s] = i <= c ? y[i] : 0.0;
+  for (int i = lane; i < s; i += 32) X[i + (int64_t)c * s] = i <= c ? y[i] * pow2(t[i]) : 0.0;
+}
+
+// T(:, k) = 2^-t_k Y(:, k) (d x s), t_k the exponent of the largest entry of C's column k; block (rows, k).
+__global__ void __launch_bounds__(256) scale_columns_kernel(const double* __restrict__ C, int s, const double* __restrict__ Y,
+                                                            int64_t d, double* __restrict__ T, int* __restrict__ t) {
+  __shared__ unsigned top[8];
+  const int k = blockIdx.y;
+  unsigned h = 0u;
+  for (int i = threadIdx.x; i <= k; i += 256) h = max(h, (unsigned)__double2hiint(__ldg(C + i + (int64_t)k * s)) & 0x7fffffffu);
+  h = __reduce_max_sync(0xffffffffu, h);
+  if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = h;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) h = max(h, top[w]);
+  const int e = min(max((int)(h >> 20) - 1023, -1000), 1000);
+  if (blockIdx.x == 0 && threadIdx.x == 0) t[k] = e;
+  const double f = pow2(-e);
+  const int64_t base = (int64_t)k * d;
+  for (int64_t i = blockIdx.x * 256ll + threadIdx.x; i < d; i += gridDim.x * 256ll) T[base + i] = Y[base + i] * f;
 }
 
 size_t up256(size_t b) { return (b + 255) / 256 * 256; }
@@ -316,28 +339,33 @@ cudaError_t chol_lower_f32(const double* G, int s, double ridge, float* L, int N
 // cores.  (Substitution row by row on the FP64 pipe: 0.75 ms at 10,000 x 200;
 // the inverse takes 83 us there and the product 55.)  Each column x of
 // the computed inverse satisfies |C x - e| <= eps s |C| |x|, so B = Y X has the error bound of
-// substitution, B (I + F) with |F| <= eps s |C| |C^{-1}|.
+// substitution, B (I + F) with |F| <= eps s |C| |C^{-1}|.  The product's error is relative to the largest
+// entries of Y's rows and X's columns, so the columns of Y are brought to one scale first, by powers of two
+// that X's rows take up (test matrices and their images need not have columns of one scale).
 size_t trsm_work_bytes(int64_t d, int s) {
   return up256((size_t)d * s * sizeof(double)) + up256((size_t)s * s * sizeof(double)) +
-         up256((size_t)(d + s) * sizeof(unsigned)) + gemm64_work_bytes(d, s, s);
+         up256((size_t)(d + 2 * s) * sizeof(unsigned)) + gemm64_work_bytes(d, s, s);
 }
 
 cudaError_t trsm_right_upper(const double* C, int s, double* Y, int64_t d, void* work, int* status, cudaStream_t st) {
   unsigned char* b = reinterpret_cast<unsigned char*>(work);
-  double* B = reinterpret_cast<double*>(b);
+  double* T = reinterpret_cast<double*>(b);
   b += up256((size_t)d * s * sizeof(double));
   double* X = reinterpret_cast<double*>(b);
   b += up256((size_t)s * s * sizeof(double));
   unsigned* ed = reinterpret_cast<unsigned*>(b);
   unsigned* ex = ed + d;
-  b += up256((size_t)(d + s) * sizeof(unsigned));
+  int* t = reinterpret_cast<int*>(ex + s);
+  b += up256((size_t)(d + 2 * s) * sizeof(unsigned));
   count_launch();
-  tri_inverse_kernel<<<s, 32, 2 * (size_t)s * sizeof(double), st>>>(C, s, X);
+  scale_columns_kernel<<<dim3((unsigned)std::min<int64_t>(8, (d + 255) / 256), (unsigned)s), 256, 0, st>>>(C, s, Y, d, T, t);
+  NYS_CUDA_TRY(cudaGetLastError());
+  count_launch();
+  tri_inverse_kernel<<<s, 32, 2 * (size_t)s * sizeof(double), st>>>(C, s, t, X);
   NYS_CUDA_TRY(cudaGetLastError());
   NYS_CUDA_TRY(absmax_f64(X, s, s, s, ex, nullptr, st));
-  NYS_CUDA_TRY(absmax_f64(Y, s, d, d, nullptr, ed, st));
-  NYS_CUDA_TRY(gemm64(Y, false, d, ed, d, X, s, ex, s, s, nullptr, B, d, b, status, st, /*any_scale=*/false));
-  return cudaMemcpyAsync(Y, B, (size_t)d * s * sizeof(double), cudaMemcpyDeviceToDevice, st);
+  NYS_CUDA_TRY(absmax_f64(T, s, d, d, nullptr, ed, st));
+  return gemm64(T, false, d, ed, d, X, s, ex, s, s, nullptr, Y, d, b, status, st, /*any_scale=*/false);
 }
 
 }  // namespace nys

@@ -32,3 +32,19 @@ extern "C" nys_status nys_test_gemm64(const double* A, int32_t k_contiguous, int
     return NYS_ECUDA;
   return read_status(status, st);
 }
+
+// chol_upper of M (s x s, column-major, in place: C^T C = M) and, when Y is given, Y <- Y C^{-1} (d x s, column-major).
+// *info (host): chol_upper's.
+extern "C" nys_status nys_test_triangular(double* M, int32_t s, double* Y, int64_t d, int32_t* info, void* stream) {
+  using namespace nys;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  Pool pool(st);
+  int* words = pool.alloc<int>(2);   // info, status
+  void* work = pool.alloc<unsigned char>(Y ? trsm_work_bytes(d, s) : 1);
+  if (!pool.ok()) return NYS_ENOMEM;
+  if (cudaMemsetAsync(words, 0, 2 * sizeof(int), st) != cudaSuccess || chol_upper(M, s, words, st) != cudaSuccess ||
+      (Y && trsm_right_upper(M, s, Y, d, work, words + 1, st) != cudaSuccess) ||
+      cudaMemcpyAsync(info, words, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+    return NYS_ECUDA;
+  return read_status(words + 1, st);
+}
