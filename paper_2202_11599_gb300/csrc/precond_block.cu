@@ -22,12 +22,15 @@ namespace {
 constexpr int BT_M = 64, BT_K = 16;
 constexpr int kSmallCols = 4;
 constexpr int kSmallChunk = 256;   // rows of one partial of the small-block form
+constexpr int kPairRows = 256;
 constexpr int kRowThreads = 64;    // step 3 of the small-block form: rows per CTA
 
 // part[z][c][i] = sum over the rows j of chunk z of U[j, i] V[j, c]; U and V column-major,
 // ld d.  Tile 64 (i) x TN (c), 256 threads, 4 x TN / 16 outputs each.  FP32 sums are formed in
-// runs of 64 rows that are then added up, so a chunk's rounding does not grow with its length.
-template <typename T, int TN>
+// runs of 64 rows; PAIR adds these up as a pair (two-sum), for chunks of more than kPairRows rows: wide
+// blocks have chunks of thousands (rank 200, 4,096 columns: all rows in one), whose rounding must
+// not grow with their length.
+template <typename T, int TN, bool PAIR>
 __global__ void __launch_bounds__(256) utv_tile_kernel(const T* __restrict__ U, const T* __restrict__ V, int64_t d,
                                                        int s, int k, int64_t kc, T* __restrict__ part) {
   constexpr int RN = TN / 16;
@@ -51,7 +54,7 @@ __global__ void __launch_bounds__(256) utv_tile_kernel(const T* __restrict__ U, 
       rb[l] = (j < ke && c < k) ? V[j + (int64_t)c * d] : T(0);
     }
   };
-  T acc[4][RN] = {}, run[4][RN] = {};
+  T acc[4][RN] = {}, run[4][RN] = {}, low[4][RN] = {};   // low: what the additions to acc rounded off
   load(kb);
   int in_run = 0;
   for (int64_t k0 = kb; k0 < ke; k0 += BT_K) {
@@ -79,7 +82,13 @@ __global__ void __launch_bounds__(256) utv_tile_kernel(const T* __restrict__ U, 
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < RN; ++j) {
-          acc[i][j] += run[i][j];
+          if constexpr (PAIR) {
+            const T t = acc[i][j] + run[i][j], z = t - acc[i][j];
+            low[i][j] += (acc[i][j] - (t - z)) + (run[i][j] - z);
+            acc[i][j] = t;
+          } else {
+            acc[i][j] += run[i][j];
+          }
           run[i][j] = T(0);
         }
     }
@@ -91,7 +100,8 @@ __global__ void __launch_bounds__(256) utv_tile_kernel(const T* __restrict__ U, 
 #pragma unroll
     for (int j = 0; j < RN; ++j) {
       const int m = m0 + tx + 16 * i, c = n0 + ty + 16 * j;
-      if (m < s && c < k) out[(int64_t)c * s + m] = acc[i][j];
+      // (a sum that overflowed has no low part)
+      if (m < s && c < k) out[(int64_t)c * s + m] = PAIR && isfinite(acc[i][j]) ? acc[i][j] + low[i][j] : acc[i][j];
     }
 }
 
@@ -293,7 +303,9 @@ cudaError_t launch_tile(const T* U, const T* cvec, const double* lam, double rho
   const int nz = (int)((d + kc - 1) / kc);
   const unsigned nt = (unsigned)((k + TN - 1) / TN);
   count_launch();
-  utv_tile_kernel<T, TN><<<dim3((s + BT_M - 1) / BT_M, nt, (unsigned)nz), 256, 0, st>>>(U, V, d, s, k, kc, part);
+  const dim3 tiles((s + BT_M - 1) / BT_M, nt, (unsigned)nz);
+  if (sizeof(T) == 4 && kc > kPairRows) utv_tile_kernel<T, TN, sizeof(T) == 4><<<tiles, 256, 0, st>>>(U, V, d, s, k, kc, part);
+  else utv_tile_kernel<T, TN, false><<<tiles, 256, 0, st>>>(U, V, d, s, k, kc, part);
   NYS_CUDA_TRY(cudaGetLastError());
   count_launch();
   block_g_kernel<T><<<(unsigned)std::min<int64_t>(2048, ((int64_t)s * k + 127) / 128), 128, 0, st>>>(
