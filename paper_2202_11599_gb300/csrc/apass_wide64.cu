@@ -59,8 +59,9 @@ __global__ void __launch_bounds__(kW64Threads, 1) apass_wide64_kernel(const Apas
   for (int kk = 0; kk < VPT; ++kk) acc[kk] = make_double2(0.0, 0.0);
   double loss = 0.0;
 
-  // dots of NR rows, kW64Warps apart, from Ar on (lanes over the column vectors)
-  auto dots = [&](auto nr, const double2* Ar) -> double {
+  // dots of NR rows, kW64Warps apart, from Ar on (lanes over the column vectors); of `share` warps on the same
+  // rows, this is number `part` and takes every share-th batch of columns
+  auto dots = [&](auto nr, const double2* Ar, int part, int share) -> double {
     constexpr int NR = decltype(nr)::value, U = (VPT <= 6 ? 8 : 4) / NR;
     double sx[NR], sy[NR];
 #pragma unroll
@@ -89,10 +90,11 @@ __global__ void __launch_bounds__(kW64Threads, 1) apass_wide64_kernel(const Apas
         }
       }
     };
-    int v0 = lane;
+    int v0 = lane + 32 * U * part;
+    const int step = 32 * U * share;
     const int whole = (nvec - 1) / (32 * U) * (32 * U);   // batches that end before the last vector
-    for (; v0 < whole; v0 += 32 * U) batch(v0, std::true_type{});
-    for (; v0 < nvec; v0 += 32 * U) batch(v0, std::false_type{});
+    for (; v0 < whole; v0 += step) batch(v0, std::true_type{});
+    for (; v0 < nvec; v0 += step) batch(v0, std::false_type{});
 #pragma unroll
     for (int r = 0; r < NR; ++r) sx[r] += sy[r];
     __syncwarp();
@@ -133,18 +135,22 @@ __global__ void __launch_bounds__(kW64Threads, 1) apass_wide64_kernel(const Apas
     const int nr = (int)min((int64_t)B, r1 - base);
     const double2* Ab = A + base * ldv;
     const double rin = warp == 0 && lane < nr ? row_input(a, base + lane) : 0.0;
-    if (!nodot && warp < nr) {
+    // Few rows: 2, 4, 8 or all warps share one (152 x 10,000, a row per CTA: 13.1 us a pass, 23.2 with a warp a row)
+    const int share = nr > 8 ? 1 : (nr > 4 ? 2 : (nr > 2 ? 4 : (nr > 1 ? 8 : 16)));
+    if (!nodot && warp < nr * share) {
       if (warp + kW64Warps < nr) {
-        const double t = dots(std::integral_constant<int, 2>{}, Ab + warp * ldv);
+        const double t = dots(std::integral_constant<int, 2>{}, Ab + warp * ldv, 0, 1);
         if ((lane & 15) == 0) ts[warp + (lane >> 4) * kW64Warps] = t;
       } else {
-        const double t = dots(std::integral_constant<int, 1>{}, Ab + warp * ldv);
+        const double t = dots(std::integral_constant<int, 1>{}, Ab + warp / share * ldv, warp % share, share);
         if (lane == 0) ts[warp] = t;
       }
     }
     __syncthreads();
     if (warp == 0 && lane < nr) {
-      const double t = nodot ? 0.0 : ts[lane];
+      double t = nodot ? 0.0 : ts[lane * share];
+      if (!nodot)
+        for (int w = 1; w < share; ++w) t += ts[lane * share + w];
       us[lane] = row_phi_d(a, base + lane, t, rin, loss);
       if (!nodot && a.t_out) a.t_out[base + lane] = t;
     }
