@@ -420,7 +420,8 @@ static int ws_stages(int64_t rowbytes, int R) {
 
 // Rows-per-stage values the kernels support for this matrix (float path: bounded by
 // the register budget of the raw vectors; all: at least two stages must fit; the
-// warp-specialised pass: 1, 2 or 4 rows with at least three stages, or two for 1 row).
+// warp-specialised pass: 1, 2 or 4 rows with at least three stages, or two for 1 row; FP64 rows from 2,048
+// columns: 1 or 2 rows a warp).
 int apass_row_candidates(const nys_matrix* A, int* out) {
   const int64_t esz = (int64_t)dtype_size(A->dtype);
   const int64_t nvec = (A->d + (16 / esz) - 1) / (16 / esz);
@@ -429,15 +430,14 @@ int apass_row_candidates(const nys_matrix* A, int* out) {
   int wthreads = 0, wvpt = 0;
   if (ws_wanted(A) && apass_ws_layout(A->dtype, A->d, &wthreads, &wvpt)) {
     for (int r : {1, 2, 4}) {
-      if (A->dtype == NYS_F64 && r == 4) continue;
-      const int S = ws_stages(rowbytes, r);
-      if (S >= (r == 1 ? 2 : 3)) out[n++] = r;
+      if (A->dtype == NYS_F64 ? r <= 2 && 2 * rowbytes <= kSmemBudget : ws_stages(rowbytes, r) >= (r == 1 ? 2 : 3))
+        out[n++] = r;
     }
     return n;
   }
   if (A->dtype == NYS_F64) {
-    // narrow FP64 rows: the stage depth follows from the rows per CTA; a warp takes four rows
-    out[n++] = 4;
+    // narrow FP64 rows: the stage depth follows from the rows per CTA and nothing is chosen; a warp takes four rows
+    if (2 * rowbytes <= kSmemBudget) out[n++] = 4;
     return n;
   }
   int threads = kApassThreads, vpt = vpt_bucket(nvec);
@@ -458,22 +458,26 @@ bool apass_plan(const nys_matrix* A, ApassPlan* plan) {
   const int64_t rowbytes = A->ld * esz;
   int wthreads = 0, wvpt = 0;
   if (ws_wanted(A) && apass_ws_layout(A->dtype, A->d, &wthreads, &wvpt)) {
-    // warp-specialised: 2 rows per stage by default (1 for rows over 64 KB, 4 under 8 KB)
-    int R = rowbytes > 64 * 1024 ? 1 : (rowbytes < 8 * 1024 ? 4 : 2);
-    if (A->dtype == NYS_F64 && R > 2) R = 2;
-    int env_or_tuned = 0;   // a choice of rows that was made, not the rule's
-    if (const int tr = tuned_rows(A->dtype, vkey < 0 ? 99 : vkey, rowbytes)) R = env_or_tuned = tr;
-    if (R != 1 && R != 2 && R != 4) R = 2;
-    if (A->dtype == NYS_F64 && R > 2) R = 2;
+    int chosen = tuned_rows(A->dtype, vkey < 0 ? 99 : vkey, rowbytes);   // by the autotuner or the environment, or 0
     if (const char* env = std::getenv("NYS_APASS_ROWS")) {
       const int r = std::atoi(env);
-      if (r == 1 || r == 2 || (r == 4 && A->dtype != NYS_F64)) R = env_or_tuned = r;
+      if (r == 1 || r == 2 || (r == 4 && A->dtype != NYS_F64)) chosen = r;
     }
-    while (R > 1 && ws_stages(rowbytes, R) < 3) R /= 2;
-    const int S = ws_stages(rowbytes, R);
-    // FP64 (apass_wide64.cu): R rows a warp at a time, p in shared memory, no stages
-    const bool wide64 = A->dtype == NYS_F64;
-    if (wide64) R = env_or_tuned == 1 ? 1 : 2;
+    int R, S;
+    if (A->dtype == NYS_F64) {
+      // apass_wide64.cu: R rows a warp at a time, p in shared memory, no stages; two rows unless one was chosen.
+      // (Rows beyond half the budget are refused, here as by the narrow rows' kernel.)
+      R = chosen == 1 ? 1 : 2;
+      S = 2 * rowbytes <= kSmemBudget ? 2 : 0;
+      plan->smem = (size_t)nvec * 16;
+    } else {
+      // warp-specialised: 2 rows per stage by default (1 for rows over 64 KB, 4 under 8 KB)
+      R = chosen ? chosen : (rowbytes > 64 * 1024 ? 1 : (rowbytes < 8 * 1024 ? 4 : 2));
+      if (R != 1 && R != 2 && R != 4) R = 2;
+      while (R > 1 && ws_stages(rowbytes, R) < 3) R /= 2;
+      S = ws_stages(rowbytes, R);
+      plan->smem = (size_t)S * R * rowbytes;
+    }
     if (S >= 2) {
       plan->ws = true;
       plan->rows_per_step = R;
@@ -481,7 +485,6 @@ bool apass_plan(const nys_matrix* A, ApassPlan* plan) {
       plan->threads = wthreads;
       plan->vpt = wvpt;
       plan->onebar = false;
-      plan->smem = wide64 ? (size_t)nvec * 16 : (size_t)S * R * rowbytes;
       plan->dpad = nvec * vec;
       const int64_t steps_total = (A->n + R - 1) / R;
       plan->grid = (int)std::max<int64_t>(1, std::min<int64_t>(sm_count(), steps_total));

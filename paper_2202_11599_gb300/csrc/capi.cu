@@ -1536,7 +1536,6 @@ nys_status nys_autotune_apass(const nys_matrix* A, int32_t* rows_out, double* ms
   int cand[3];
   const int nc = apass_row_candidates(A, cand);
   if (nc == 0) return NYS_EINVAL;
-  const bool f64 = A->dtype == NYS_F64;
   Pool pool(st);
   void* p = pool.alloc<unsigned char>((size_t)A->d * 8);
   int* dstat = pool.alloc<int>(1);
@@ -1583,8 +1582,7 @@ nys_status nys_autotune_apass(const nys_matrix* A, int32_t* rows_out, double* ms
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  (void)f64;
-  apass_set_tuned_rows(A, best);
+  apass_set_tuned_rows(A, nc > 1 ? best : 0);   // (a single form is no choice)
   // then the row slabs of the warp-specialised float pass, balanced over the CTAs
   double ms_eq = 0.0, ms_split = 0.0;
   NYS_CU(apass_balance_rows(A, p, part, dstat, st, &ms_eq, &ms_split));

@@ -48,3 +48,13 @@ extern "C" nys_status nys_test_triangular(double* M, int32_t s, double* Y, int64
     return NYS_ECUDA;
   return read_status(words + 1, st);
 }
+
+// Rows per step the autotuner would time on A (rows[0 .. return value)) and the one that the plan takes now (*planned; 0: no plan).
+extern "C" int32_t nys_test_rows(const nys_matrix* A, int32_t* rows, int32_t* planned) {
+  int cand[3] = {0, 0, 0};
+  const int n = nys::apass_row_candidates(A, cand);
+  for (int i = 0; i < n; ++i) rows[i] = cand[i];
+  nys::ApassPlan plan;
+  *planned = nys::apass_plan(A, &plan) ? plan.rows_per_step : 0;
+  return n;
+}
