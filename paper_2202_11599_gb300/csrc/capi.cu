@@ -117,26 +117,29 @@ nys_status cholqr2(double* Om, int64_t d, int m, cudaStream_t st, bool fp32_clas
   void* tw = pool.alloc<unsigned char>(trsm_work_bytes(d, m));
   if (!pool.ok()) return NYS_ENOMEM;
   NYS_CU(cudaMemsetAsync(info, 0, 2 * sizeof(int), st));
+  int info_h[2] = {0, 0};
   for (int pass = 0; pass < 2; ++pass) {
     NYS_CU(gram_xty(Om, Om, d, m, G, work, info + 1, st));
     if (pass == 1 && fp32_class) {
       NYS_CU(identity_gap(G, m, gap, st));
       double gap_h = 1.0;
       NYS_CU(cudaMemcpyAsync(&gap_h, gap, sizeof(double), cudaMemcpyDeviceToHost, st));
+      NYS_CU(cudaMemcpyAsync(info_h, info, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
       NYS_CU(cudaStreamSynchronize(st));
-      if (gap_h <= 0x1p-20) break;
+      if (info_h[1]) return (nys_status)info_h[1];
+      if (gap_h <= 0x1p-20) return NYS_OK;
     }
     // a pivot below 1e-10 of the largest column norm^2: columns dependent to ~1e-5, which
     // CholQR cannot orthonormalise -- refused as a bad test matrix
     NYS_CU(chol_upper(G, m, info, st, 1e-10));
-    int info_h[2] = {0, 0};
     NYS_CU(cudaMemcpyAsync(info_h, info, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     NYS_CU(cudaStreamSynchronize(st));
-    if (info_h[1]) return (nys_status)info_h[1];
-    if (info_h[0] != 0) return NYS_EINVAL;  // Omega has (numerically) dependent columns
+    NYS_TRY(step_status(info_h[1], info_h[0] == 0, NYS_EINVAL));  // Omega has (numerically) dependent columns
     NYS_CU(trsm_right_upper(G, m, Om, d, tw, info + 1, st));
   }
-  return NYS_OK;
+  NYS_CU(cudaMemcpyAsync(info_h, info, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+  NYS_CU(cudaStreamSynchronize(st));
+  return (nys_status)info_h[1];
 }
 
 // Y (d x m, FP64) = (A^T diag(D) A + shift I) Om for an FP64 orthonormal panel Om.
@@ -220,9 +223,11 @@ nys_status nystrom_core(const double* Om, const double* Y, int64_t d, int s, dou
     NYS_CU(power_lambda_max(G, s, lmax, pw, st));
   }
   double lmax_h = 0.0;
+  int info_h[2] = {0, 0};
   NYS_CU(cudaMemcpyAsync(&lmax_h, lmax, sizeof(double), cudaMemcpyDeviceToHost, st));
+  NYS_CU(cudaMemcpyAsync(info_h, info, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
   NYS_CU(cudaStreamSynchronize(st));
-  if (!is_fin(lmax_h)) return NYS_EINVAL;
+  NYS_TRY(step_status(info_h[1], is_fin(lmax_h), NYS_EINVAL));
   double nu = shift_scale * eps_host(std::sqrt(std::max(lmax_h, 0.0)), mant_bits);
   bool ok = false;
   PhaseTimer* pt_chol = new PhaseTimer("core: shift + chol", st);
@@ -231,17 +236,14 @@ nys_status nystrom_core(const double* Om, const double* Y, int64_t d, int s, dou
     NYS_CU(axpy_panel(nu, Om, Ynu, d * s, st));
     NYS_CU(gram_xty(Om, Ynu, d, s, M, gw, status, st));
     NYS_CU(chol_upper(M, s, info, st));
-    int info_h = 0;
-    NYS_CU(cudaMemcpyAsync(&info_h, info, sizeof(int), cudaMemcpyDeviceToHost, st));
+    NYS_CU(cudaMemcpyAsync(info_h, info, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     NYS_CU(cudaStreamSynchronize(st));
-    if (info_h == 0) {
-      ok = true;
-      break;
-    }
+    ok = info_h[0] == 0;
+    if (ok || info_h[1]) break;
     nu *= 10.0;
   }
   delete pt_chol;
-  if (!ok) return NYS_ENOTSPD;
+  NYS_TRY(step_status(info_h[1], ok, NYS_ENOTSPD));
   {
     PhaseTimer pt("core: trsm + B^T B", st);
     NYS_CU(trsm_right_upper(M, s, Ynu, d, tw, status, st));   // B = Y_nu C^{-1} (in Ynu)

@@ -92,6 +92,11 @@ int vec_blocks(int64_t d);
 constexpr int kClusterBlocks = 16;   // vec_blocks(d) up to this: the fused kernels run as one cluster
 
 // ---------------------------------------------------------------- small dense FP64 kernels
+// What a step of the core returns, given the status word of its products and whether its result is usable: a
+// wait that ran out leaves NaN, which must not be taken for the caller's bad data.
+inline nys_status step_status(int wait, bool usable, nys_status if_not) {
+  return wait ? static_cast<nys_status>(wait) : (usable ? NYS_OK : if_not);
+}
 // FP64 products on the tensor cores (gemm64_tc.cu).  absmax_f64: per row and / or column of the
 // row-major rows x cols matrix X, the top word of its largest magnitude.
 cudaError_t absmax_f64(const double* X, int64_t rows, int64_t cols, int64_t ld, unsigned* rowmax, unsigned* colmax,

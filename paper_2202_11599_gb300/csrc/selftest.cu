@@ -58,3 +58,7 @@ extern "C" int32_t nys_test_rows(const nys_matrix* A, int32_t* rows, int32_t* pl
   *planned = nys::apass_plan(A, &plan) ? plan.rows_per_step : 0;
   return n;
 }
+
+extern "C" nys_status nys_test_step_status(int32_t wait, int32_t usable, int32_t if_not) {
+  return nys::step_status(wait, usable != 0, (nys_status)if_not);
+}
