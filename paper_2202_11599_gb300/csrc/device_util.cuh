@@ -321,6 +321,39 @@ __device__ __forceinline__ C urow_dot(const C* __restrict__ U, int64_t d, int64_
   return acc;
 }
 
+// g_i = c_i sum_b part[b][i] (U^T w over the blocks), the partials read through L2 and added in increasing b: in
+// FP64, or for FP32 partials as three FP32 words by two-sums, ~70 bits of the sum, so no fewer than FP64 holds, without the
+// FP64 pipe (79 blocks x 200 rows: 4.4 us of FP64 additions in every block).  A sum beyond FP32's range is formed in FP64.
+template <typename C>
+__device__ __forceinline__ C g_entry(const C* part, int nb, int s, int i, C ci) {
+  if constexpr (sizeof(C) == 8) {
+    return ci * (nb <= 16 ? sum_strided_fixed<true, double, 16>(part, nb, s, i, 0.0) : sum_strided_fixed<true>(part, nb, s, i, 0.0));
+  } else {
+    constexpr int B = 32;
+    float hi = 0.f, lo = 0.f, last = 0.f;
+    for (int b = 0; b < nb; b += B) {
+      float v[B];
+#pragma unroll
+      for (int q = 0; q < B; ++q) v[q] = b + q < nb ? __ldcg(part + (int64_t)(b + q) * s + i) : 0.f;
+#pragma unroll
+      for (int q = 0; q < B; ++q) {
+        const float t = hi + v[q], z = t - hi;
+        const float e = (hi - (t - z)) + (v[q] - z);
+        hi = t;
+        const float u = lo + e, y = u - lo;
+        last += (lo - (u - y)) + (e - y);
+        lo = u;
+      }
+    }
+    double sum = (double)hi + ((double)lo + (double)last);
+    if (!isfinite(sum)) {
+      sum = 0.0;
+      for (int b = 0; b < nb; ++b) sum += (double)__ldcg(part + (int64_t)b * s + i);
+    }
+    return (float)((double)ci * sum);
+  }
+}
+
 // y = w + U g over a block's chunk of `len` elements from j0 (w at w[0 .. len)): done(jj, w, y) in
 // thread jj % kVecThreads.  Bound by the latency of the chain over s and its loads (rank 50, FP64:
 // 9,800 clocks as one chain per element), so a chunk of up to 128 elements gives each element

@@ -165,32 +165,6 @@ __device__ __forceinline__ void utw_partials(const C* wch, int len, const C* __r
   }
 }
 
-// g_i = c_i sum_b part[b][i], the partials read through L2 and added in increasing b: in FP64, or
-// for FP32 partials as an error-compensated FP32 pair (two-sum; 48 bits of the sum for values
-// of 24), which keeps FP64 accuracy after the rounding to FP32 without the FP64 pipe (79
-// blocks x 200 rows: 4.4 us of FP64 additions in every block).
-template <typename C>
-__device__ __forceinline__ C g_entry(const C* part, int nb, int s, int i, C ci) {
-  if constexpr (sizeof(C) == 8) {
-    return ci * (nb <= 16 ? sum_strided_fixed<true, double, 16>(part, nb, s, i, 0.0) : sum_strided_fixed<true>(part, nb, s, i, 0.0));
-  } else {
-    constexpr int B = 32;
-    float hi = 0.f, lo = 0.f;
-    for (int b = 0; b < nb; b += B) {
-      float v[B];
-#pragma unroll
-      for (int q = 0; q < B; ++q) v[q] = b + q < nb ? __ldcg(part + (int64_t)(b + q) * s + i) : 0.f;
-#pragma unroll
-      for (int q = 0; q < B; ++q) {
-        const float t = hi + v[q], z = t - hi;
-        lo += (hi - (t - z)) + (v[q] - z);
-        hi = t;
-      }
-    }
-    return (float)((double)ci * ((double)hi + (double)lo));
-  }
-}
-
 // Scalar step of a PCG iteration (run by the last block of the update): ||w||^2, stop test,
 // iteration count, g = c o U^T w.
 template <typename C>

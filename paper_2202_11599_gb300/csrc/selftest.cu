@@ -1,9 +1,14 @@
 // Entry points for the tests only, not part of nysadmm.h: single device functions that the library otherwise
 // runs inside a sketch, so that their results can be compared entry by entry.
+#include "device_util.cuh"
 #include "nys_internal.cuh"
 #include "solver.cuh"
 
 namespace {
+__global__ void g_entry_kernel(const float* part, int nb, int s, float c, float* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < s) out[i] = nys::g_entry<float>(part, nb, s, i, c);
+}
 nys_status read_status(const int* status, cudaStream_t st) {
   int h = 0;
   if (cudaMemcpyAsync(&h, status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -61,4 +66,11 @@ extern "C" int32_t nys_test_rows(const nys_matrix* A, int32_t* rows, int32_t* pl
 
 extern "C" nys_status nys_test_step_status(int32_t wait, int32_t usable, int32_t if_not) {
   return nys::step_status(wait, usable != 0, (nys_status)if_not);
+}
+
+// out[i] = c sum_b part[b][i] as the fused vector steps form it (part nb x s).
+extern "C" nys_status nys_test_g_entry(const float* part, int32_t nb, int32_t s, float c, float* out, void* stream) {
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  g_entry_kernel<<<(s + 127) / 128, 128, 0, st>>>(part, nb, s, c, out);
+  return cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess ? NYS_OK : NYS_ECUDA;
 }
