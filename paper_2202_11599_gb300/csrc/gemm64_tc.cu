@@ -483,15 +483,18 @@ __global__ void __launch_bounds__(ET, 1) gemm64_tc_kernel(const EmuArgs a) {
       }
       mma_commit(&empty_bar[s]);
     }
-    if (s_fail) {   // MMAs still queued: they finish before TMEM is freed
-      mma_commit(&done);
-      (void)mbar_wait_bounded(&done, 0u);
-    }
    }
   }
   tc_fence_before();
   __syncthreads();
-  if (s_fail && tid == 0) atomicExch(a.status, (int)NYS_ETIMEOUT);
+  if (s_fail) {   // whoever gave up: MMAs still queued finish before their operands and TMEM are given back
+    if (tid == 32 * ECW && nt > 0) {
+      mma_commit(&done);
+      (void)mbar_wait_bounded(&done, 0u);
+    }
+    if (tid == 0) atomicExch(a.status, (int)NYS_ETIMEOUT);
+    __syncthreads();
+  }
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
