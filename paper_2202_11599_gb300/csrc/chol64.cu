@@ -22,20 +22,6 @@ constexpr int kCholCtas = 8;
 constexpr int kCholThreads = 256;
 constexpr int kCholMax = 448;   // 56 columns of 448 and three buffers: 211 KB of shared memory
 
-// 1 / sqrt(d) for a positive normal d: an FP32 estimate r of the significand's, whose error e = 1 - m r^2
-// (2^-21) one step of Householder's third-order method, r + r e (1/2 + 3/8 e), takes to FP64 bits: four
-// dependent instructions, 64 clocks each on this GPU.  (The library function's chain of ~20 set
-// the pace of a step.)
-__device__ __forceinline__ double rsqrt_householder(double d) {
-  const int hi = __double2hiint(d), e = (hi >> 20) - 1023;
-  const int k = e >> 1;   // d = m 4^k, m in [1, 4)
-  const double m = __hiloint2double(hi - (2 * k << 20), __double2loint(d));
-  double r = (double)rsqrtf((float)m);
-  const double err = fma(-(m * r), r, 1.0);
-  r = fma(fma(0.375, err, 0.5), err * r, r);
-  return __hiloint2double(__double2hiint(r) - (k << 20), __double2loint(r));
-}
-
 struct CholArgs {
   const double* M;   // s x s column-major, symmetrised as (M + M^T) / 2
   int s;
@@ -87,8 +73,7 @@ __global__ void __launch_bounds__(kCholThreads) chol_cluster_kernel(const CholAr
     if (warp == 0) {
       const double d = col[j];
       const bool ok = d > 0.0 && d > thresh && isfinite(d);
-      // denormal pivots are scaled into range first
-      const double r = !ok ? 0.0 : (d < 0x1p-1000 ? rsqrt_householder(d * 0x1p200) * 0x1p100 : rsqrt_householder(d));
+      const double r = ok ? rsqrt(d) : 0.0;
       if (lane == 0) {
         s_r = r;
         if (!ok)

@@ -25,8 +25,7 @@ def _run(M, Y=None):
 
 
 def test_pivots_of_every_exponent():
-    """C_kk of a diagonal matrix: the reciprocal root is off by at most 1.5 u (its last FMA and half the rounding
-    of m r), the product adds u."""
+    """C_kk of a diagonal matrix: the library's reciprocal root is within an ulp (2 u), the product adds u."""
     vals = [np.ldexp(m, e) for e in range(-1070, 1020, 19) for m in (1.0, 1.0 + 2.0 ** -52, 1.5, 2.0 - 2.0 ** -52)]
     vals = np.array(vals + [5e-324, 2.0 ** -1022, np.nextafter(2.0 ** -1022, 0), 2.0 ** -1000, np.nextafter(2.0 ** -1000, 0), 1.7e308])
     for e in (-1000, -2, -1, 0, 1, 2, 3, 4):   # beside powers of two and four
@@ -35,7 +34,7 @@ def test_pivots_of_every_exponent():
         info, C, _ = _run(np.diag(part))
         assert info == 0
         assert np.array_equal(C, np.diag(np.diag(C)))
-        assert np.max(np.abs(np.diag(C) / np.sqrt(part.astype(LD)) - 1)) <= 2.6 * U
+        assert np.max(np.abs(np.diag(C) / np.sqrt(part.astype(LD)) - 1)) <= 3 * U
 
 
 @pytest.mark.parametrize("s", [1, 9, 64, 200, 448, 449])
@@ -46,7 +45,7 @@ def test_factor(s):
     M = 0.5 * (M + M.T)
     info, C, _ = _run(M)
     assert info == 0 and np.array_equal(C, np.triu(C))
-    # |C^T C - M| <= gamma_{s+1} |C|^T |C| with a division of 2 u in the place of one of u / 2
+    # |C^T C - M| <= gamma_{s+1} |C|^T |C|, with the reciprocal root's ulp and a product in the place of a division
     R = C.T.astype(LD) @ C.astype(LD) - M.astype(LD)
     assert np.max(np.abs(R) / (np.abs(C).T @ np.abs(C))) <= (s + 4) * U
 
