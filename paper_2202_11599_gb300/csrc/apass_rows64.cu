@@ -1,4 +1,5 @@
-// Fused FP64 A-pass for narrow rows (the pass for FP64 matrices apass_wide64.cu does not take): y = A^T phi(A p) with one read of A, the result layout of apass.cu.
+// Fused FP64 A-pass for narrow rows (the pass for FP64 matrices apass_wide64.cu does not take):
+// y = A^T phi(A p) with one read of A, the result layout of apass.cu.
 //
 // The FP64 pipe bounds it: an SM quarter issues one FP64 warp instruction per 64 clocks, so
 // the rows' n d products and n d updates set the pace and any FP64 instruction beside them
@@ -7,10 +8,8 @@
 //     additions for the four rows), a row's columns split over WS warps when R < 32;
 //   * lanes r < R of one warp add a row's WS partials and apply phi;
 //   * every thread applies the rank-R update to the column vectors it owns.
-// The kernel it replaces had every thread add the 16 warp partials of every row: 64 dependent
-// FP64 additions per thread and four-row step, 52 us for the 2,000 x 500 pass whose products
-// take 3.3 us.  With this one nys_hmatvec there went from 112 to 67 us a call and a 2,000 x 500
-// lasso of 1,700 passes from 190 to 107 ms.
+// With every thread adding the 16 warp partials of every row (64 dependent FP64 additions per
+// thread and four-row step) the 2,000 x 500 pass, whose products take 3.3 us, took 52 us; it takes 8.6.
 #include "apass_common.cuh"
 #include "apass_ws.cuh"
 

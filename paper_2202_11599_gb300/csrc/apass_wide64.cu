@@ -8,11 +8,9 @@
 // reading the rows again, through L2 or HBM.  Beside the FMAs a block of 32 rows costs one
 // reduction per warp and one evaluation of phi.
 //
-// The kernel before it kept each row in shared memory between roles that ran side by side (dot warps,
-// a finisher, update warps, R <= 2 rows a stage): eight reductions and one phi per stage, each
-// FP64 instruction of the finisher's chain queueing with five other warps for the pipe:
-// 39,999 x 4,001 684 us, 200,000 x 5,000 logistic 5.55 ms (FMAs alone: 527 us, 3.3 ms).  Now 567 us
-// and 3.46 ms.
+// 39,999 x 4,001: 567 us (FMAs alone 527), 200,000 x 5,000 in logistic mode 3.42 ms (3.3).  With dot, finishing
+// and update warps side by side over a ring of stages it was 684 us and 5.55 ms: each FP64 instruction of the
+// finisher's chain queues for the pipe behind every other warp's.
 #include "apass_common.cuh"
 #include "apass_ws.cuh"
 

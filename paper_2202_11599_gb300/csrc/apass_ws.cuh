@@ -110,14 +110,13 @@ __device__ __forceinline__ int ws_produce(const ApassKArgs& a, WsBars& b, unsign
 // Finisher warp: u_i = phi(t_i) for the rows of each stage, t_i summed over the G dot
 // warps' partials in a fixed order.  Returns this lane's share of the pass's loss term.
 //
-// The logistic modes take two stages per step: exp and the division are ~40 FP64 warp
-// instructions of 64 pipe clocks each whether one lane or all take part, so with one wide
-// row per stage (R = 1) the finisher, not the FP64 dot products beside it, set the pace
-// (200,000 x 5,000 FP64, logistic mode: 6.9 -> 5.6 ms a pass; before, one row at a time with a
-// second exp and the log1p of an unwanted loss).  Lane q R + r takes row r of stage k + q.
-template <typename C, int R, int G>
-__device__ __forceinline__ double ws_finish(const ApassKArgs& a, WsBars& b, const C (*red)[G][R], C (*us)[R],
-                                            int nsteps, int S, int64_t r0, int64_t r1, volatile int* abort_flag,
+// The logistic modes take two stages per step: exp and the division go through the FP64 pipe, 64 clocks a
+// warp instruction whether one lane or all take part, and with few rows per stage the finisher sets the
+// pace (logistic regression on 200,000 x 5,000 FP32, eight iterations: 69.5 ms with one stage per step,
+// 65.8 with two).  Lane q R + r takes row r of stage k + q.
+template <int R, int G>
+__device__ __forceinline__ double ws_finish(const ApassKArgs& a, WsBars& b, const float (*red)[G][R],
+                                            float (*us)[R], int nsteps, int S, int64_t r0, int64_t r1, volatile int* abort_flag,
                                             int kbase = 0) {
   const int lane = threadIdx.x & 31;
   const bool nodot = a.mode == MODE_CONST;
@@ -144,18 +143,14 @@ __device__ __forceinline__ double ws_finish(const ApassKArgs& a, WsBars& b, cons
     }
     if (mine) {
       const int sq = q == 0 ? st : st1;
-      C u = C(0);
+      float u = 0.f;
       if (live) {
-        C t = C(0);
+        float t = 0.f;
         if (!nodot) {
 #pragma unroll
           for (int w = 0; w < G; ++w) t += red[sq][w][r];
         }
-        if constexpr (sizeof(C) == 4) {
-          u = row_phi(a, row, t, rin, loss);
-        } else {
-          u = (C)row_phi_d(a, row, (double)t, rin, loss);
-        }
+        u = row_phi(a, row, t, rin, loss);
         if (!nodot && a.t_out) a.t_out[row] = (double)t;
       }
       us[sq][r] = u;
@@ -340,7 +335,7 @@ __device__ __forceinline__ bool ws_pass_float(const ApassKArgs& a, WsFloatSmem<R
     if (lane == 0) issued = ws_produce(a, bars, smem, nsteps, R, S, rowbytes, r0, r1, abort_v, kbase);
   } else {
     // ---------------- finisher
-    double l = ws_finish<float, R, G>(a, bars, sm.red, sm.us, nsteps, S, r0, r1, abort_v, kbase);
+    double l = ws_finish<R, G>(a, bars, sm.red, sm.us, nsteps, S, r0, r1, abort_v, kbase);
     l = warp_sum(l);
     if (lane == 0) sm.loss = l;
   }

@@ -10,9 +10,10 @@
 // accumulators add them exactly while |sum| < 2^24.  The digit products of equal weight
 // (order o = i + j = 0 .. 7, o + 1 pairs) share one TMEM accumulator: 36 MMAs per K step for
 // 64 output columns x 8 orders = all 512 TMEM columns.  Every 256 K the accumulators are read
-// out as integers and added to two 64-bit integer sums per output: at 256 K orders 0-3 cannot
-// leave 2^24 for any input, and orders 4-7, below 2^-32 of the product's scale, could round
-// only for inputs whose low digits all agree in sign.  The final integer is rounded to FP64 once.
+// out as integers and added to a 96-bit integer sum per output.  In 256 K orders 0-4 cannot leave 2^24 for
+// any input; orders 5-7 can in the last MMAs of a group whose digits are nearly all at their largest and of
+// one sign (sum |a||b| is above 2^-4 2^ea 2^eb then), and round by at most 2^-47 2^ea 2^eb, less than
+// a chain of FMAs there.  The final integer is rounded to FP64 once.
 // (Fixed-point splitting of a product into exact low-precision ones: Ozaki, Ogita, Oishi, Rump,
 // Numer. Algorithms 59, 2012.)
 //

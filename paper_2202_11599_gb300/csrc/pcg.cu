@@ -820,26 +820,6 @@ __global__ void __launch_bounds__(kVecThreads) admm_zu_g_kernel(int64_t d, int c
                        nodes_per_iter, nodes_per_pcg_iter, cond);
 }
 
-
-// Head of the device loop's ADMM iteration, one cooperative launch (tracked warm start,
-// no refined step or warm-start model).  It replaces the begin / right-hand side / PCG-init
-// (P^{-1} w) launches of the general body, and it runs the iterations whose x-subproblem
-// needs no PCG step -- the common case under the decaying schedules of Sec. 5, where the
-// tracked warm start often already meets the iteration's tolerance -- back to back:
-//   1. r = q + rho (z - u), w = r - (H + rho I) x (tracked), partial ||w||^2, ||r||^2 and
-//      U^T w (blocks, thread mapping and order of pcg_update_kernel's init step);
-//   2. every block sums the partials in the order of pcg_scalar_body and takes the same stop
-//      decision;
-//   3a. no step: x stays; z = S_kappa(x + u), u += x - z and the residual partials (blocks of
-//      admm_zu_g_kernel); every block forms r_p, r_d, the stop test and the next tolerance as
-//      admm_scalar_g_body does (block 0 records them) and goes on with iteration k + 1;
-//   3b. a step: g = c o U^T w (order of pcg_scalar_body), y = w + U g, p = y and the partials
-//      of w^T y (blocks and order of pcg_tail_kernel), the PCG state as the begin and init
-//      kernels leave it; the PCG WHILE node and the prox/dual kernel finish iteration k.
-// When (H + rho I) x is due for a recompute at iteration k the kernel requests it (IF node
-// before it) and returns; the next launch continues at k.  The arithmetic and its order are
-// those of the general body, so the iterates are bitwise those of a solve without this
-// kernel.  Grid barriers are bounded (NYS_ETIMEOUT).
 // One PCG iteration after its A-pass as ONE launch (Alg. Nystrom PCG): the reduction of the
 // per-CTA A-pass partials (apass_reduce_kernel), the update of x, w and the tracked
 // (H + rho I) x with the partials of ||w||^2 and U^T w (pcg_update_kernel), the scalar step
@@ -1105,6 +1085,26 @@ __global__ void __launch_bounds__(kVecThreads, 2) pcg_post_kernel(const PostArgs
                        a.h_admm);
 }
 
+// Head of the device loop's ADMM iteration as one launch, a cluster or a cooperative grid like the post
+// kernel (no refined step or warm-start model; (H + rho I) x tracked, or formed anew by the pass ahead of
+// this kernel when inline_hx).  It replaces the begin / right-hand side / PCG-init
+// (P^{-1} w) launches of the general body, and it runs the iterations whose x-subproblem
+// needs no PCG step -- the common case under the decaying schedules of Sec. 5, where the
+// tracked warm start often already meets the iteration's tolerance -- back to back:
+//   1. r = q + rho (z - u), w = r - (H + rho I) x (tracked), partial ||w||^2, ||r||^2 and
+//      U^T w (blocks, thread mapping and order of pcg_update_kernel's init step);
+//   2. every block sums the partials in the order of pcg_scalar_body and takes the same stop
+//      decision;
+//   3a. no step: x stays; z = S_kappa(x + u), u += x - z and the residual partials (blocks of
+//      admm_zu_g_kernel); every block forms r_p, r_d, the stop test and the next tolerance as
+//      admm_scalar_g_body does (block 0 records them) and goes on with iteration k + 1;
+//   3b. a step: g = c o U^T w (order of pcg_scalar_body), y = w + U g, p = y and the partials
+//      of w^T y (blocks and order of pcg_tail_kernel), the PCG state as the begin and init
+//      kernels leave it; the PCG WHILE node and the prox/dual kernel finish iteration k.
+// When (H + rho I) x is due for a recompute at iteration k the kernel requests it (the IF node
+// after it; with inline_hx the next pass of the body) and returns; the next launch continues at k.  The arithmetic and its order are
+// those of the general body, so the iterates are bitwise those of a solve without this
+// kernel.  Grid barriers are bounded (NYS_ETIMEOUT).
 struct HeadArgs {
   int64_t d;
   int chunk, nb, s;
