@@ -258,7 +258,8 @@ nys_status nystrom_core(const double* Om, const double* Y, int64_t d, int s, dou
   }
   {
     PhaseTimer pt("core: finish (U = BV)", st);
-    NYS_CU(nystrom_finish(Ynu, d, s, jw, V, nu, U, lam_d, fw, status, st));
+    // (the shift of an FP32-class sketch bounds B's scales to 1 : 10^3)
+    NYS_CU(nystrom_finish(Ynu, d, s, jw, V, nu, U, lam_d, fw, status, st, /*any_scale=*/mant_bits == 52));
   }
   if (std::getenv("NYS_TRACE")) std::fprintf(stderr, "[nys] jacobi sweeps %d (s = %d)\n", sweeps, s);
   lam_h.resize(s);

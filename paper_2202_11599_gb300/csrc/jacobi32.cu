@@ -19,6 +19,13 @@
 // V0 is then orthonormalised in FP64 (two Newton-Schulz steps: the columns leave the FP32 stage
 // orthogonal to 1e-6 .. 1e-4) and checked on the device: if V0^T V0 is off the identity by more
 // than 1e-13 the sweeps start from the identity instead, as they do without this stage.
+//
+// So they do for a steep spectrum (kJacSteep).  Orthonormalising and A = V^T G V are accurate
+// relative to lam_1, so what is left of eigenvalue i's row carries eps lam_1 / lam_i, while sweeps from the
+// identity keep the relative accuracy of a graded G.  With columns decaying like j^-p, FP64, ranks 100 to 300,
+// U^T U - I is 1e-15 .. 3e-13 with this start down to lam_s / lam_1 = 3e-9 (4e-14 .. 2e-7 from the identity),
+// but 3e-4 at 2e-10 (1e-6); on rows or columns scaled by 10^+-6, where the ratio is 1e-14 and below, PCG with the
+// result no longer converged.  An FP32-class sketch's shift keeps the ratio above 1e-6.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -31,6 +38,7 @@ namespace {
 namespace cg = cooperative_groups;
 
 constexpr double kJacRidge = 1e-7;     // eps / trace(G)
+constexpr double kJacSteep = 0x1p-24;  // lam_s / lam_1 below which the sweeps start from the identity
 constexpr float kJacSkip2 = 1e-14f;    // squared cosine below which two columns are orthogonal to rounding
 constexpr float kJacAgain2 = 1e-6f;    // a sweep that met none above this was the last (quadratic)
 
@@ -273,11 +281,40 @@ __global__ void gap_kernel(const double* __restrict__ S, int N, double tol, int*
     b |= !(fabs(S[e] - (e % N == e / N ? 1.0 : 0.0)) <= tol);
   if (__syncthreads_or(b) && threadIdx.x == 0) atomicOr(bad, 1);
 }
-// A <- (T + T^T) / 2, V <- Vn; when Vn failed its check A stays, and V too (V = I with `reset`).
-// Vn may be V.
+// bad[1] = the spectrum on the diagonal of T = V^T G V is steep.  The padding row's own eigenvector (N > s), if
+// any, is left out.
+__global__ void __launch_bounds__(512) steep_kernel(const double* __restrict__ T, const double* __restrict__ V, int N, int s,
+                                                    int* bad) {
+  __shared__ double lo[16], hi[16];
+  double mn = INFINITY, mx = 0.0;
+  for (int i = threadIdx.x; i < N; i += 512)
+    if (N == s || fabs(V[(N - 1) + (int64_t)i * N]) < 0.5) {
+      const double t = T[i + (int64_t)i * N];
+      mn = fmin(mn, t);
+      mx = fmax(mx, t);
+    }
+  for (int o = 16; o > 0; o >>= 1) {
+    mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+    mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    lo[threadIdx.x >> 5] = mn;
+    hi[threadIdx.x >> 5] = mx;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 16; ++w) {
+      mn = fmin(mn, lo[w]);
+      mx = fmax(mx, hi[w]);
+    }
+    bad[1] = !(mn >= kJacSteep * mx);
+  }
+}
+// A <- (T + T^T) / 2, V <- Vn; when Vn failed its check (bad[0]) or the spectrum is steep (bad[1]) A stays, and V too
+// (V = I with `reset`).  Vn may be V.
 __global__ void accept_kernel(const double* __restrict__ T, int N, const int* __restrict__ bad, int reset,
                               double* __restrict__ A, const double* Vn, double* V) {
-  const bool no = *bad != 0;
+  const bool no = (bad[0] | bad[1]) != 0;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)N * N; e += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(e % N), j = (int)(e / N);
     if (no) {
@@ -395,7 +432,7 @@ namespace {
 struct StartWork {
   double *S, *P;
   unsigned *e1, *eg, *et;   // exponents: of entries below 4, of G's rows, of a product's columns
-  int* bad;
+  int* bad;                 // the check of V; a steep spectrum (of the start, kept through the corrections)
   void* gw;
   StartWork(void* work, int N) {
     unsigned char* b = reinterpret_cast<unsigned char*>(work);
@@ -406,14 +443,14 @@ struct StartWork {
     eg = e1 + N;
     et = eg + N;
     bad = reinterpret_cast<int*>(et + N);
-    gw = b + 2 * m + up256(3 * (size_t)N * sizeof(unsigned) + sizeof(int));
+    gw = b + 2 * m + up256(3 * (size_t)N * sizeof(unsigned) + 2 * sizeof(int));
   }
 };
 }  // namespace
 
 size_t jacobi_start_work_bytes(int s) {
   const size_t N = s + (s & 1);
-  return 2 * up256(N * N * sizeof(double)) + up256(3 * N * sizeof(unsigned) + sizeof(int)) +
+  return 2 * up256(N * N * sizeof(double)) + up256(3 * N * sizeof(unsigned) + 2 * sizeof(int)) +
          gemm64_work_bytes(N, (int)N, N);
 }
 
@@ -455,6 +492,9 @@ cudaError_t jacobi_start(const double* G, int s, double* A, double* V, void* wor
   NYS_CUDA_TRY(mul(A, true, w.eg, V, w.e1, w.S));
   if (N > kSmallProduct) NYS_CUDA_TRY(absmax_f64(w.S, N, N, N, w.et, nullptr, st));
   NYS_CUDA_TRY(mul(V, true, w.e1, w.S, w.et, w.P));
+  count_launch();
+  steep_kernel<<<1, 512, 0, st>>>(w.P, V, N, s, w.bad);
+  NYS_CUDA_TRY(cudaGetLastError());
   count_launch();
   accept_kernel<<<grid, 256, 0, st>>>(w.P, N, w.bad, 1, A, V, V);
   return cudaGetLastError();

@@ -157,9 +157,11 @@ cudaError_t jacobi_polish(const double* G, int N, double* A, double* T, double* 
 size_t jacobi_work_bytes(int s);
 // *out (device) = max_ij |G_ij - delta_ij| of the m x m matrix G.
 cudaError_t identity_gap(const double* G, int m, double* out, cudaStream_t st);
-// After Jacobi: sort eigenpairs descending, U = B V Sigma^{-1}, lam = max(0, sigma^2 - nu).
+// After Jacobi: sort eigenpairs descending, U = B V Sigma^{-1}, lam = max(0, sigma^2 - nu).  any_scale: the product's
+// (gemm64), for spectra whose small columns of B V an error relative to the largest entries of B would reach.
 cudaError_t nystrom_finish(const double* B, int64_t d, int s, const double* G, const double* V,
-                           double nu, double* U, double* lam, double* work, int* status, cudaStream_t st);
+                           double nu, double* U, double* lam, double* work, int* status, cudaStream_t st,
+                           bool any_scale);
 size_t finish_work_bytes(int64_t d, int s);
 
 // ---------------------------------------------------------------- sketch GEMMs
