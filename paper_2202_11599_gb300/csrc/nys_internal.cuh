@@ -144,14 +144,14 @@ cudaError_t jacobi_eig(double* G, double* V, int s, double* work, int* sweeps, i
                        double tol = 1e-12);
 // FP32 start of the sweeps (jacobi32.cu): V = an orthogonal matrix that makes V^T G V diagonal to
 // FP32 accuracy and A <- V^T A V, for A = the zero-padded symmetrised G.  *ran = false: nothing
-// was changed; a V that fails its orthogonality check on the device leaves V = I and A alone.
+// was changed; a V that fails its orthogonality check on the device, or a steep spectrum, leaves V = I and A alone.
 bool jacobi_start_supported(int s);
 size_t jacobi_start_work_bytes(int s);
 cudaError_t jacobi_start(const double* G, int s, double* A, double* V, void* work, int* status, cudaStream_t st,
                          bool* ran);
 // First-order correction of a nearly diagonal A = V^T G V: V <- V exp(E) with E_ij = A_ij / (A_jj -
 // A_ii) where that is below 2e-3, A <- V^T G V; nothing changes when the new V fails its
-// orthogonality check.  G: N x N symmetric; T: N x N scratch; work of jacobi_start.
+// orthogonality check or the start found the spectrum steep.  G: N x N symmetric; T: N x N scratch; work of jacobi_start.
 cudaError_t jacobi_polish(const double* G, int N, double* A, double* T, double* V, void* work, int* status,
                           cudaStream_t st);
 size_t jacobi_work_bytes(int s);
